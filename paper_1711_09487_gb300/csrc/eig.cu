@@ -3,8 +3,10 @@
 // bisection on Sturm counts for the eigenvalues of the tridiagonal matrix, inverse iteration
 // with Gram-Schmidt inside clusters of close eigenvalues, back-transformation.
 #include "eig.cuh"
+#include "dense.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 
@@ -169,61 +171,134 @@ __device__ inline double recip_nr(double q) {
   return fma(r, fma(-q, r, 1.0), r);
 }
 
-__device__ inline int sturm_count_nr(const double *__restrict__ d, const double *__restrict__ e, int n, double x,
-                                     double pivmin) {
+// Number of eigenvalues below x.  e2[k] = e[k]^2 (tri_prep_kernel).  The FP64 pipe issues one warp
+// instruction in 16 cycles, so a step has four FP64 instructions: the shift, the Newton pair and the
+// recurrence; the guard |q| < pivmin and the sign are read off the high word with integer
+// instructions.
+__device__ __forceinline__ int sturm_count_nr(const double *__restrict__ d, const double *__restrict__ e2, int n,
+                                              double x, double pivmin) {
+  const int pv_hi = __double2hiint(pivmin);
   int cnt = 0;
   double q = d[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  cnt += q < 0.0;
+  if ((__double2hiint(q) & 0x7fffffff) < pv_hi) q = -pivmin;
+  cnt += (int)((unsigned)__double2hiint(q) >> 31);
+#pragma unroll 4
   for (int k = 1; k < n; ++k) {
-    const double ek = e[k - 1];
-    q = fma(-ek * ek, recip_nr(q), d[k] - x);
-    if (fabs(q) < pivmin) q = -pivmin;
-    cnt += q < 0.0;
+    q = fma(-e2[k - 1], recip_nr(q), d[k] - x);
+    if ((__double2hiint(q) & 0x7fffffff) < pv_hi) q = -pivmin;
+    cnt += (int)((unsigned)__double2hiint(q) >> 31);
   }
   return cnt;
 }
 
-// BIS_G lanes per eigenvalue: each round the lanes take the Sturm counts at BIS_G points that cut
-// [lo, hi] into BIS_G + 1 equal parts, and the part holding eigenvalue i becomes the new interval
-// (log2(BIS_G + 1) bits per round instead of one, at BIS_G times the counting work).
-constexpr int BIS_G = 8;
+// Per item: e2 = e^2 into work, and into info the Gershgorin bounds of the spectrum, the smallest
+// pivot of the counts and the largest absolute row sum.
+constexpr int TRI_INFO = 4;
+__global__ void __launch_bounds__(256) tri_prep_kernel(SymBatchP b, double *info) {
+  const SymItem it = b.it[blockIdx.x];
+  const int n = it.n;
+  double gl = INFINITY, gu = -INFINITY, em = 0.0, tn = 0.0;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const double dk = it.d[k], el = k > 0 ? fabs(it.e[k - 1]) : 0.0, er = k < n - 1 ? fabs(it.e[k]) : 0.0;
+    gl = fmin(gl, dk - (el + er));
+    gu = fmax(gu, dk + (el + er));
+    tn = fmax(tn, fabs(dk) + el + er);
+    em = fmax(em, er * er);
+    it.work[k] = er * er;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    gl = fmin(gl, __shfl_xor_sync(0xffffffffu, gl, o));
+    gu = fmax(gu, __shfl_xor_sync(0xffffffffu, gu, o));
+    em = fmax(em, __shfl_xor_sync(0xffffffffu, em, o));
+    tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+  }
+  __shared__ double red[4][8];
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    red[0][w] = gl;
+    red[1][w] = gu;
+    red[2][w] = em;
+    red[3][w] = tn;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) {
+      gl = fmin(gl, red[0][q]);
+      gu = fmax(gu, red[1][q]);
+      em = fmax(em, red[2][q]);
+      tn = fmax(tn, red[3][q]);
+    }
+    double *o = info + (int64_t)blockIdx.x * TRI_INFO;
+    o[0] = gl;
+    o[1] = gu;
+    o[2] = 2.2250738585072014e-308 * fmax(1.0, em);
+    o[3] = tn;
+  }
+}
 
-__global__ void __launch_bounds__(256) bisect_kernel(SymBatchP b) {
+// G lanes per eigenvalue: each round the lanes take the Sturm counts at G points that cut [lo, hi]
+// into G + 1 equal parts, and the part holding eigenvalue i becomes the new interval (log2(G + 1)
+// bits per round instead of one, at G times the counting work).  One warp per CTA: the FP64 pipe of
+// an SM serves one warp as fast as it does eight, so the warps are spread over all SMs (with eight
+// warps a CTA the order-120 problem ran on 4 SMs: 1.23 ms, and order 1885 on 59: 19.8 ms).
+template <int G>
+__global__ void __launch_bounds__(32) bisect_kernel(SymBatchP b, const double *__restrict__ info) {
   const SymItem it = b.it[blockIdx.y];
   const int n = it.n;
-  const int g = threadIdx.x % BIS_G;                                   // lane within the group
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) / BIS_G;       // eigenvalue index
-  const unsigned gmask = ((1u << BIS_G) - 1u) << ((threadIdx.x & 31) & ~(BIS_G - 1));
+  const int lane = threadIdx.x, base = lane & ~(G - 1), g = lane - base;
+  const int i = blockIdx.x * (32 / G) + lane / G;  // eigenvalue index
+  const unsigned gmask = (G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u)) << base;
   if (i >= n) return;  // the lanes of a group share i, so a group leaves together
-  const double *d = it.d, *e = it.e;
-  double gl = d[0], gu = d[0], emax2 = 0.0;
-  for (int k = 0; k < n; ++k) {
-    const double r = (k > 0 ? fabs(e[k - 1]) : 0.0) + (k < n - 1 ? fabs(e[k]) : 0.0);
-    gl = fmin(gl, d[k] - r);
-    gu = fmax(gu, d[k] + r);
-    if (k < n - 1) emax2 = fmax(emax2, e[k] * e[k]);
-  }
+  const double *f = info + (int64_t)blockIdx.y * TRI_INFO;
+  const double gl = f[0], gu = f[1], pivmin = f[2];
   const double eps = 2.220446049250313e-16;
-  const double pivmin = 2.2250738585072014e-308 * fmax(1.0, emax2);
   const double span = fmax(fabs(gl), fabs(gu));
   double lo = gl - 2.0 * eps * span * n - pivmin, hi = gu + 2.0 * eps * span * n + pivmin;
   for (int round = 0; round < 100; ++round) {
     if (hi - lo <= 2.0 * eps * fmax(fabs(lo), fabs(hi)) + 4.0 * pivmin) break;
-    const double step = (hi - lo) / (BIS_G + 1);
+    const double step = (hi - lo) / (G + 1);
     const double x = lo + step * (g + 1);
-    const bool above = (x > lo && x < hi) ? sturm_count_nr(d, e, n, x, pivmin) > i : (x >= hi);
+    const bool above = (x > lo && x < hi) ? sturm_count_nr(it.d, it.work, n, x, pivmin) > i : (x >= hi);
     // the first cut point whose count exceeds i bounds the eigenvalue from above
     const unsigned m = __ballot_sync(gmask, above) & gmask;
-    const int base = (threadIdx.x & 31) & ~(BIS_G - 1);
-    const int first = m ? (__ffs(m) - 1 - base) : BIS_G;
+    const int first = m ? (__ffs(m) - 1 - base) : G;
     const double nlo = first > 0 ? lo + step * first : lo;
-    const double nhi = first < BIS_G ? lo + step * (first + 1) : hi;
+    const double nhi = first < G ? lo + step * (first + 1) : hi;
     if (!(nlo > lo || nhi < hi)) break;  // no progress in floating point
     lo = nlo;
     hi = nhi;
   }
   if (g == 0) it.lam[i] = 0.5 * (lo + hi);
+}
+
+// Eigenvalues of the tridiagonal matrices (d, e) of the batch.  G is the lanes per eigenvalue with
+// the least estimated time: rounds (52 bits at log2(G + 1) a round) times a step, which takes the
+// chain of dependent instructions (about 150 cycles) or, with w warps on an SM, 64 cycles of FP64
+// issue for each.
+static void tridiagonal_values(cudaStream_t st, const SymBatchP &b, int cnt, int nmax) {
+  double *info = nullptr;
+  RFDD_CUDA(cudaMallocAsync((void **)&info, (size_t)cnt * TRI_INFO * sizeof(double), st));
+  tri_prep_kernel<<<cnt, 256, 0, st>>>(b, info);
+  RFDD_CHECK_LAUNCH();
+  int64_t total = 0;
+  for (int i = 0; i < cnt; ++i) total += b.it[i].n;
+  int G = 4;
+  double best = 0.0;
+  for (int c = 4; c <= 32; c *= 2) {
+    const double w = std::ceil((double)total * c / 32.0 / sm_count());
+    const double t = std::ceil(52.0 / std::log2(c + 1.0)) * std::max(150.0, 64.0 * w);
+    if (c == 4 || t < best) {
+      best = t;
+      G = c;
+    }
+  }
+  const dim3 grid(ceil_div((int64_t)nmax * G, 32), cnt);
+  if (G == 4) bisect_kernel<4><<<grid, 32, 0, st>>>(b, info);
+  else if (G == 8) bisect_kernel<8><<<grid, 32, 0, st>>>(b, info);
+  else if (G == 16) bisect_kernel<16><<<grid, 32, 0, st>>>(b, info);
+  else bisect_kernel<32><<<grid, 32, 0, st>>>(b, info);
+  RFDD_CHECK_LAUNCH();
+  RFDD_CUDA(cudaFreeAsync(info, st));
 }
 
 // Householder reduction of every item of the batch to tridiagonal form (d, e)
@@ -281,10 +356,7 @@ void sym_eig_values(cudaStream_t st, const std::vector<SymItem> &items, int *sta
     for (int i = 0; i < cnt; ++i) { b.it[i] = items[s0 + i]; nmax = std::max(nmax, b.it[i].n); }
     if (nmax == 0) continue;
     tridiagonalize(st, b, cnt, nmax);
-    // e[n-1] = 0 for every item (house_kernel leaves it undefined)
-    // BIS_G lanes per eigenvalue, 256 / BIS_G eigenvalues per block
-    bisect_kernel<<<dim3(ceil_div((int64_t)nmax * BIS_G, 256), cnt), 256, 0, st>>>(b);
-    RFDD_CHECK_LAUNCH();
+    tridiagonal_values(st, b, cnt, nmax);
   }
 }
 
@@ -425,6 +497,142 @@ __global__ void __launch_bounds__(256) inviter_kernel(InvIterP p, const Cluster 
   (void)ctol;
 }
 
+// Inverse iteration for eigenvalues that stand alone (clusters of one), one lane per eigenvalue:
+// the factorisation and the triangular solves are serial chains, so a warp runs 32 of them at the
+// cost of one (one thread of a CTA per eigenvalue took 14.2 ms for all vectors of order 1885).
+// Scratch is lane-interleaved (entry k of lane l at k * 32 + l), so every access is coalesced, and
+// IV_U steps are loaded ahead of the chain.  Same start vectors, factorisation and number of
+// iterations as inviter_kernel.
+struct SingleWarp {
+  int item, first, count;  // rows[first .. first + count): positions in the item's selection list
+};
+constexpr int IV_ARRAYS = 5;
+constexpr int IV_U = 8;
+__global__ void __launch_bounds__(32) inviter_single_kernel(InvIterP p, const SingleWarp *__restrict__ sw,
+                                                            const int *__restrict__ rows, double *scratch,
+                                                            int64_t per_warp, unsigned *flags, int64_t flags_per_warp) {
+  const SingleWarp c = sw[blockIdx.x];
+  const SymItem it = p.it[c.item];
+  const int n = it.n, lane = threadIdx.x;
+  const int row = rows[c.first + min(lane, c.count - 1)];
+  const int ei = p.sel[c.item][row];
+  const double lam = it.lam[ei];
+  const double *__restrict__ d = it.d, *__restrict__ e = it.e;
+  const int64_t len = (int64_t)n * 32;
+  double *__restrict__ ru = scratch + (int64_t)blockIdx.x * per_warp + lane;
+  double *__restrict__ u2 = ru + len, *__restrict__ u3 = u2 + len, *__restrict__ ml = u3 + len,
+         *__restrict__ x = ml + len;
+  unsigned *__restrict__ fl = flags + (int64_t)blockIdx.x * flags_per_warp;
+  double tn = 0.0;
+  for (int k = lane; k < n; k += 32)
+    tn = fmax(tn, fabs(d[k]) + (k > 0 ? fabs(e[k - 1]) : 0.0) + (k < n - 1 ? fabs(e[k]) : 0.0));
+  for (int o = 16; o > 0; o >>= 1) tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
+  const double delta = 2.220446049250313e-16 * fmax(tn, 1e-300);
+  auto hash = [&](int k) {
+    uint64_t z = (uint64_t)(ei + 1) * 0x9E3779B97F4A7C15ull + (uint64_t)(k + 1) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    z ^= z >> 31;
+    return (double)(z >> 11) * 0x1p-53 + 0.5;
+  };
+  // T - lam I = P L U with row interchanges of neighbours; ru = 1 / U_kk
+  double cd = d[0] - lam, ce1 = n > 1 ? e[0] : 0.0, ce2 = 0.0;
+  for (int k = 0; k < n - 1; ++k) {
+    const double sub = e[k], an = d[k + 1] - lam, bn = (k + 1 < n - 1) ? e[k + 1] : 0.0;
+    const bool piv = fabs(cd) < fabs(sub);
+    if (!piv && cd == 0.0) cd = delta;
+    double u = piv ? sub : cd;
+    const double l = (piv ? cd : sub) / u;
+    if (fabs(u) < delta) u = u < 0 ? -delta : delta;
+    ru[(int64_t)k * 32] = 1.0 / u;
+    u2[(int64_t)k * 32] = piv ? an : ce1;
+    u3[(int64_t)k * 32] = piv ? bn : ce2;
+    ml[(int64_t)k * 32] = l;
+    x[(int64_t)k * 32] = hash(k);
+    const unsigned f = __ballot_sync(0xffffffffu, piv);
+    if (lane == 0) fl[k] = f;
+    const double nd = piv ? ce1 - l * an : an - l * ce1;
+    ce1 = piv ? ce2 - l * bn : bn - l * ce2;
+    ce2 = 0.0;
+    cd = nd;
+  }
+  {
+    const double u = (fabs(cd) < delta) ? (cd < 0 ? -delta : delta) : cd;
+    ru[(int64_t)(n - 1) * 32] = 1.0 / u;
+    u2[(int64_t)(n - 1) * 32] = u3[(int64_t)(n - 1) * 32] = 0.0;
+    x[(int64_t)(n - 1) * 32] = hash(n - 1);
+  }
+  __syncwarp();
+  double scale = 1.0, ss = 0.0;
+  for (int iter = 0; iter < 3; ++iter) {
+    // forward: the largest entry of the last solve is scaled to one on the way in
+    double cur = x[0] * scale;
+    for (int k0 = 0; k0 < n - 1; k0 += IV_U) {
+      double xn[IV_U], mk[IV_U];
+      unsigned fk[IV_U];
+#pragma unroll
+      for (int q = 0; q < IV_U; ++q)
+        if (k0 + q < n - 1) {
+          xn[q] = x[(int64_t)(k0 + q + 1) * 32];
+          mk[q] = ml[(int64_t)(k0 + q) * 32];
+          fk[q] = fl[k0 + q];
+        }
+#pragma unroll
+      for (int q = 0; q < IV_U; ++q)
+        if (k0 + q < n - 1) {
+          const double nx = xn[q] * scale;
+          const bool piv = (fk[q] >> lane) & 1u;
+          const double top = piv ? nx : cur, bot = piv ? cur : nx;
+          x[(int64_t)(k0 + q) * 32] = top;
+          cur = bot - mk[q] * top;
+        }
+    }
+    // backward
+    double x1 = cur * ru[(int64_t)(n - 1) * 32], x2 = 0.0, mx = fabs(x1);
+    x[(int64_t)(n - 1) * 32] = x1;
+    for (int k0 = n - 2; k0 >= 0; k0 -= IV_U) {
+      double xk[IV_U], a2[IV_U], a3[IV_U], rk[IV_U];
+#pragma unroll
+      for (int q = 0; q < IV_U; ++q)
+        if (k0 - q >= 0) {
+          const int64_t o = (int64_t)(k0 - q) * 32;
+          xk[q] = x[o];
+          a2[q] = u2[o];
+          a3[q] = u3[o];
+          rk[q] = ru[o];
+        }
+#pragma unroll
+      for (int q = 0; q < IV_U; ++q)
+        if (k0 - q >= 0) {
+          const double v = (xk[q] - a2[q] * x1 - a3[q] * x2) * rk[q];
+          x[(int64_t)(k0 - q) * 32] = v;
+          x2 = x1;
+          x1 = v;
+          mx = fmax(mx, fabs(v));
+        }
+    }
+    scale = mx > 0.0 ? 1.0 / mx : 1.0;
+  }
+  for (int k = 0; k < n; ++k) {
+    const double v = x[(int64_t)k * 32] * scale;
+    ss = fma(v, v, ss);
+  }
+  const double sc = ss > 0.0 ? scale / sqrt(ss) : 0.0;
+  // rows of Zt through shared memory, so that the stores run along them
+  __shared__ double tile[32][33];
+  double *Zt = it.Zt;
+  for (int k0 = 0; k0 < n; k0 += 32) {
+    const int w = min(32, n - k0);
+    for (int q = 0; q < w; ++q) tile[lane][q] = x[(int64_t)(k0 + q) * 32] * sc;
+    __syncwarp();
+    for (int r = 0; r < c.count; ++r) {
+      const int rr = __shfl_sync(0xffffffffu, row, r);
+      if (lane < w) Zt[(int64_t)rr * n + k0 + lane] = tile[r][lane];
+    }
+    __syncwarp();
+  }
+}
+
 // x = H_0 H_1 ... H_{n-3} z for each tridiagonal eigenvector z (row of Zt); one CTA per vector,
 // the vector in shared memory.
 struct BackBatchP {
@@ -467,6 +675,8 @@ void sym_eig_vectors(cudaStream_t st, const std::vector<BackItem> &items, double
     BackBatchP bb;
     memset(&bb, 0, sizeof(bb));
     std::vector<Cluster> clusters;
+    std::vector<SingleWarp> singles;  // eigenvalues that stand alone, 32 of one item to a warp
+    std::vector<int> srows;
     std::vector<int> allsel;
     std::vector<size_t> seloff(cnt);
     int nmax = 1, selmax = 0;
@@ -496,32 +706,59 @@ void sym_eig_vectors(cudaStream_t st, const std::vector<BackItem> &items, double
       int start = 0;
       for (int q = 1; q <= (int)bi.sel.size(); ++q) {
         if (q == (int)bi.sel.size() || lam[bi.sel[q]] - lam[bi.sel[q - 1]] > ctol * tnorm) {
-          clusters.push_back({i, start, q - start});
+          if (q - start == 1) {
+            if (singles.empty() || singles.back().item != i || singles.back().count == 32)
+              singles.push_back({i, (int)srows.size(), 0});
+            ++singles.back().count;
+            srows.push_back(start);
+          } else {
+            clusters.push_back({i, start, q - start});
+          }
           start = q;
         }
       }
     }
-    if (clusters.empty()) continue;
+    if (clusters.empty() && singles.empty()) continue;
     int *sel_dev = nullptr;
-    Cluster *cl_dev = nullptr;
-    double *scratch = nullptr;
-    const int64_t per = (int64_t)7 * nmax;
     RFDD_CUDA(cudaMallocAsync((void **)&sel_dev, allsel.size() * sizeof(int), st));
-    RFDD_CUDA(cudaMallocAsync((void **)&cl_dev, clusters.size() * sizeof(Cluster), st));
-    RFDD_CUDA(cudaMallocAsync((void **)&scratch, (size_t)clusters.size() * per * sizeof(double), st));
     RFDD_CUDA(cudaMemcpyAsync(sel_dev, allsel.data(), allsel.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    RFDD_CUDA(cudaMemcpyAsync(cl_dev, clusters.data(), clusters.size() * sizeof(Cluster), cudaMemcpyHostToDevice, st));
     for (int i = 0; i < cnt; ++i) ip.sel[i] = sel_dev + seloff[i];
-    inviter_kernel<<<(unsigned)clusters.size(), 256, 0, st>>>(ip, cl_dev, scratch, per, ctol);
-    RFDD_CHECK_LAUNCH();
+    if (!clusters.empty()) {
+      Cluster *cl_dev = nullptr;
+      double *scratch = nullptr;
+      const int64_t per = (int64_t)7 * nmax;
+      RFDD_CUDA(cudaMallocAsync((void **)&cl_dev, clusters.size() * sizeof(Cluster), st));
+      RFDD_CUDA(cudaMallocAsync((void **)&scratch, (size_t)clusters.size() * per * sizeof(double), st));
+      RFDD_CUDA(cudaMemcpyAsync(cl_dev, clusters.data(), clusters.size() * sizeof(Cluster), cudaMemcpyHostToDevice, st));
+      inviter_kernel<<<(unsigned)clusters.size(), 256, 0, st>>>(ip, cl_dev, scratch, per, ctol);
+      RFDD_CHECK_LAUNCH();
+      RFDD_CUDA(cudaFreeAsync(cl_dev, st));
+      RFDD_CUDA(cudaFreeAsync(scratch, st));
+    }
+    if (!singles.empty()) {
+      SingleWarp *sw_dev = nullptr;
+      int *rows_dev = nullptr;
+      double *scratch = nullptr;
+      const int64_t per = (int64_t)IV_ARRAYS * 32 * nmax, fper = nmax;
+      RFDD_CUDA(cudaMallocAsync((void **)&sw_dev, singles.size() * sizeof(SingleWarp), st));
+      RFDD_CUDA(cudaMallocAsync((void **)&rows_dev, srows.size() * sizeof(int), st));
+      RFDD_CUDA(cudaMallocAsync((void **)&scratch,
+                                singles.size() * ((size_t)per * sizeof(double) + (size_t)fper * sizeof(unsigned)), st));
+      RFDD_CUDA(cudaMemcpyAsync(sw_dev, singles.data(), singles.size() * sizeof(SingleWarp), cudaMemcpyHostToDevice, st));
+      RFDD_CUDA(cudaMemcpyAsync(rows_dev, srows.data(), srows.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+      inviter_single_kernel<<<(unsigned)singles.size(), 32, 0, st>>>(
+          ip, sw_dev, rows_dev, scratch, per, reinterpret_cast<unsigned *>(scratch + singles.size() * per), fper);
+      RFDD_CHECK_LAUNCH();
+      RFDD_CUDA(cudaFreeAsync(sw_dev, st));
+      RFDD_CUDA(cudaFreeAsync(rows_dev, st));
+      RFDD_CUDA(cudaFreeAsync(scratch, st));
+    }
     const size_t smem = (size_t)nmax * sizeof(double);
     RFDD_REQUIRE(smem <= 200 * 1024, RFDD_EINVAL, "sym_eig: order too large");
     RFDD_CUDA(cudaFuncSetAttribute(back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     back_kernel<<<dim3(selmax, cnt), 256, smem, st>>>(bb);
     RFDD_CHECK_LAUNCH();
     RFDD_CUDA(cudaFreeAsync(sel_dev, st));
-    RFDD_CUDA(cudaFreeAsync(cl_dev, st));
-    RFDD_CUDA(cudaFreeAsync(scratch, st));
     // host vectors referenced by async copies must outlive them
     RFDD_CUDA(cudaStreamSynchronize(st));
   }

@@ -152,6 +152,7 @@ enum DevStatus : int {
   DS_NONFINITE = 2,
   DS_BAD_SIZE = 4,
   DS_WAIT_TIMEOUT = 8,
+  DS_GRID_TIMEOUT = 16,  // a barrier among the CTAs of a cooperative kernel ran out
 };
 
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }

@@ -18,6 +18,16 @@ struct SymBatchP {
   SymItem it[EIG_MAXB];
 };
 
+// 1/q by the hardware's approximate reciprocal refined with one Newton-Raphson step
+// (r <- r + r (1 - q r)), which doubles the number of correct bits: relative error about 2^-44,
+// far below what a Sturm count needs (it is a tiny backward perturbation of e_k^2).  |q| >= pivmin
+// keeps q a normal number.
+__device__ inline double recip_nr(double q) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
+  return fma(r, fma(-q, r, 1.0), r);
+}
+
 // Block-wide sum, the same value in every thread.  One thread adds the warp partials (FP64
 // arithmetic is scarce on this GPU: every thread adding them would cost nw FP64 adds each).
 __device__ double block_sum(double v, double *red) {
@@ -161,16 +171,6 @@ __device__ inline int sturm_count(const double *d, const double *e, int n, doubl
   return cnt;
 }
 
-// 1/q by the hardware's approximate reciprocal refined with one Newton-Raphson step
-// (r <- r + r (1 - q r)), which doubles the number of correct bits: relative error about 2^-44,
-// far below what a Sturm count needs (it is a tiny backward perturbation of e_k^2).  |q| >= pivmin
-// keeps q a normal number.
-__device__ inline double recip_nr(double q) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
-  return fma(r, fma(-q, r, 1.0), r);
-}
-
 // Number of eigenvalues below x.  e2[k] = e[k]^2 (tri_prep_kernel).  The FP64 pipe issues one warp
 // instruction in 16 cycles, so a step has four FP64 instructions: the shift, the Newton pair and the
 // recurrence; the guard |q| < pivmin and the sign are read off the high word with integer
@@ -302,7 +302,239 @@ static void tridiagonal_values(cudaStream_t st, const SymBatchP &b, int cnt, int
 }
 
 // Householder reduction of every item of the batch to tridiagonal form (d, e)
-static void tridiagonalize(cudaStream_t st, const SymBatchP &b, int cnt, int nmax) {
+//
+// Up to order TRD_NMAX one cooperative launch does every step: G CTAs per item, row r of the
+// trailing block held by CTA r % G (its own rows stay in that SM's L1 / L2), one barrier among the
+// item's CTAs per step.  After the barrier every CTA forms q_{i-1}, the updated row i and the
+// Householder vector from it for itself (O(n) work, cheaper than a second barrier), then updates its
+// rows and their entries of p_i.  p alternates between two buffers, and row i takes v_i one step
+// late, so that no CTA overwrites what a slower one still reads.  Bound: below order 400 the chain of
+// one step (barrier, two block reductions, the reflector's scalars: about 6 us), above it the three
+// FP64 operations per trailing entry (1885 FMA-cubed is 11 ms of the chip's FP64 rate).  Measured:
+// order 120 0.74 ms (1.04 ms in 240 launches, 1.7 ms with their gaps), order 1885 32.9 ms (37.2 in
+// 3769 launches, 44 with gaps).
+constexpr int TRD_THREADS = 512;  // at most; 256 below order 512
+constexpr int TRD_NMAX = 8192;  // three vectors of the order in shared memory
+constexpr int TRD_SPIN = 1 << 22;
+__device__ __forceinline__ bool trd_barrier(unsigned *cnt, unsigned target) {
+  __shared__ int ok_s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("fence.acq_rel.gpu;\n\tred.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
+    unsigned v = 0;
+    int k = 0;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+    } while (v < target && ++k < TRD_SPIN);
+    ok_s = v >= target;
+  }
+  __syncthreads();
+  return ok_s != 0;
+}
+
+// Block-wide sum over the first nact warps, the same value in every thread.  A warp's FP64 add takes
+// 16 cycles of an SM's FP64 pipe, so warps without data add nothing and the warp partials are added
+// as a tree by one warp.
+__device__ __forceinline__ double trd_sum(double v, double *red, int nact) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < nact) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) red[w] = v;
+  }
+  __syncthreads();
+  if (w == 0) {
+    v = lane < nact ? red[lane] : 0.0;
+    for (int o = nact > 8 ? 8 : nact > 4 ? 4 : nact > 2 ? 2 : 1; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) red[32] = v;
+  }
+  __syncthreads();
+  return red[32];
+}
+
+// The Householder reflector of a vector with first entry alpha and the sum of squares sig of the
+// others: beta = -sign(alpha) ||x||, tau = 1 + |alpha| / ||x||, scale = 1 / (alpha - beta).  1 / ||x|| and the
+// scale come from the hardware's approximate (reciprocal) square root refined by Newton's
+// iteration, half the dependent FP64 operations of a square root and two divisions; far from 1 the
+// plain operations.
+__device__ __forceinline__ void householder(double alpha, double sig, double &beta, double &tau, double &sc) {
+  beta = alpha;
+  tau = sc = 0.0;
+  if (sig == 0.0) return;
+  const double S = fma(alpha, alpha, sig);
+  if (S > 1e-280 && S < 1e280) {
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(S));
+    r = fma(0.5 * r, fma(-S * r, r, 1.0), r);
+    r = fma(0.5 * r, fma(-S * r, r, 1.0), r);
+    const double a = fabs(alpha), nrm = S * r, D = a + nrm;
+    beta = alpha <= 0.0 ? nrm : -nrm;
+    tau = fma(a, r, 1.0);
+    double t = recip_nr(D);
+    t = fma(t, fma(-D, t, 1.0), t);
+    sc = alpha <= 0.0 ? -t : t;
+  } else {
+    const double nrm = sqrt(S);
+    beta = alpha <= 0.0 ? nrm : -nrm;
+    tau = (beta - alpha) / beta;
+    sc = 1.0 / (alpha - beta);
+  }
+}
+
+// CTAs off[j] .. off[j+1]-1 of the grid work on item j.
+struct TridSplit {
+  int off[EIG_MAXB + 1];
+};
+
+__global__ void __launch_bounds__(TRD_THREADS) tridiag_kernel(SymBatchP b, TridSplit sp, int nmax, double *pbuf,
+                                                              unsigned *bars, int *status) {
+  int item = 0;
+  while (sp.off[item + 1] <= (int)blockIdx.x) ++item;
+  const int me = (int)blockIdx.x - sp.off[item], G = sp.off[item + 1] - sp.off[item];
+  const SymItem it = b.it[item];
+  const int n = it.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nthr = blockDim.x, NW = nthr >> 5;
+  extern __shared__ double sm[];
+  double *vp = sm, *q = sm + nmax, *v = sm + 2 * nmax;  // v_{i-1}, q_{i-1}, v_i, indexed by row
+  __shared__ double red[33];
+  double *p0 = pbuf + (int64_t)item * 2 * nmax;
+  unsigned *bar = bars + item;
+  double taup = 0.0;  // tau of the current reflector (of step i-1 until it is formed)
+  for (int i = 0; i < n; ++i) {
+    // q_{i-1} and row i
+    double *row = it.H + (int64_t)i * it.ld;
+    const bool upd = i >= 1 && i - 1 < n - 2;
+    const int nact = min(NW, (n - i + 31) >> 5);
+    double ss = 0.0;
+    if (upd) {
+      const double *p = p0 + (int64_t)((i - 1) & 1) * nmax;
+      for (int k = i + tid; k < n; k += nthr) {
+        const double pk = __ldcg(p + k);
+        q[k] = pk;
+        ss = fma(pk, vp[k], ss);
+        v[k] = __ldcg(row + k);
+      }
+      const double K = 0.5 * taup * trd_sum(ss, red, nact);
+      const double vi = vp[i], qi = q[i] - K * vi;
+      ss = 0.0;
+      for (int k = i + tid; k < n; k += nthr) {
+        const double qk = q[k] - K * vp[k];
+        const double x = fma(-qi, vp[k], fma(-vi, qk, v[k]));
+        if (k > i) q[k] = qk;  // q[i] stays as it is: other threads may still read it
+        v[k] = x;
+        if (k > i + 1) ss = fma(x, x, ss);
+      }
+    } else {  // the first row, and the last one (complete after the pass of step n - 2)
+      for (int k = i + tid; k < n; k += nthr) {
+        const double x = __ldcg(row + k);
+        v[k] = x;
+        if (k > i + 1) ss = fma(x, x, ss);
+      }
+    }
+    const double sig = trd_sum(ss, red, nact);
+    const double di = v[i];
+    if (i >= n - 1) {
+      if (me == 0 && tid == 0) { it.d[i] = di; it.tau[i] = 0.0; }
+    } else {
+      const double alpha = v[i + 1];
+      double beta, sc;
+      householder(alpha, sig, beta, taup, sc);
+      if (me == 0 && tid == 0) { it.d[i] = di; it.e[i] = beta; it.tau[i] = taup; }
+      __syncthreads();
+      for (int k = i + 2 + tid; k < n; k += nthr) v[k] *= sc;
+      if (tid == 0) v[i + 1] = 1.0;
+      __syncthreads();
+    }
+    // v_{i-1} into row i-1, for the back-transformation (every CTA has read that row)
+    if (me == 0 && i >= 1)
+      for (int k = i + tid; k < n; k += nthr) it.H[(int64_t)(i - 1) * it.ld + k] = vp[k];
+    if (i > n - 2) break;
+    // this CTA's rows of the trailing block: pending rank-2 update, then p_i
+    const bool sym = i < n - 2;
+    double *pn = p0 + (int64_t)(i & 1) * nmax;
+    const int first = i + 1 + ((me - (i + 1)) % G + G) % G;
+    for (int r = first + warp * G; r < n; r += NW * G) {
+      double *h = it.H + (int64_t)r * it.ld;
+      const double vr = upd ? vp[r] : 0.0, qr = upd ? q[r] : 0.0;
+      double s0 = 0.0, s1 = 0.0;
+      int c = i + 1 + lane;
+      if (upd) {
+        double h4[4];
+        if (c + 96 < n) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) h4[u] = h[c + 32 * u];
+        }
+        for (; c + 96 < n; c += 128) {
+          const bool more = c + 224 < n;  // the next four entries are loaded ahead of this four's chain
+          double g4[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) g4[u] = more ? h[c + 128 + 32 * u] : 0.0;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            h4[u] = fma(-qr, vp[c + 32 * u], fma(-vr, q[c + 32 * u], h4[u]));
+            h[c + 32 * u] = h4[u];
+          }
+          s0 = fma(h4[0], v[c], s0);
+          s1 = fma(h4[1], v[c + 32], s1);
+          s0 = fma(h4[2], v[c + 64], s0);
+          s1 = fma(h4[3], v[c + 96], s1);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) h4[u] = g4[u];
+        }
+        for (; c < n; c += 32) {
+          const double x = fma(-qr, vp[c], fma(-vr, q[c], h[c]));
+          h[c] = x;
+          s0 = fma(x, v[c], s0);
+        }
+      } else {
+        for (; c < n; c += 32) s0 = fma(h[c], v[c], s0);
+      }
+      if (sym) {
+        double t = s0 + s1;
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) pn[r] = taup * t;
+      }
+    }
+    if (!trd_barrier(bar, (unsigned)(G * (i + 1)))) {
+      if (tid == 0) atomicOr(status, DS_GRID_TIMEOUT);
+      return;
+    }
+    double *t = vp;  // v_i is the next step's v_{i-1}
+    vp = v;
+    v = t;
+  }
+}
+
+static void tridiagonalize(cudaStream_t st, const SymBatchP &b, int cnt, int nmax, int *status) {
+  if (nmax > 2 && nmax <= TRD_NMAX && status) {
+    // one CTA per SM over all items, shared in proportion to n^2 (the work of a step), at least four
+    // rows to a CTA at the start
+    TridSplit sp;
+    double sq = 0.0;
+    for (int j = 0; j < cnt; ++j) sq += (double)b.it[j].n * b.it[j].n;
+    sp.off[0] = 0;
+    for (int j = 0; j < cnt; ++j) {
+      const double nj = b.it[j].n;
+      const int g = 1 + (int)(std::max(0, sm_count() - cnt) * nj * nj / sq);
+      sp.off[j + 1] = sp.off[j] + std::max(1, std::min(g, b.it[j].n / 4));
+    }
+    for (int j = cnt; j < EIG_MAXB; ++j) sp.off[j + 1] = sp.off[cnt];
+    const int nv = (nmax + 1) & ~1;
+    const size_t smem = (size_t)3 * nv * sizeof(double);
+    RFDD_CUDA(cudaFuncSetAttribute(tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    double *pbuf = nullptr;
+    const size_t pb = (size_t)cnt * 2 * nv * sizeof(double);
+    RFDD_CUDA(cudaMallocAsync((void **)&pbuf, pb + (size_t)cnt * sizeof(unsigned), st));
+    unsigned *bars = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(pbuf) + pb);
+    RFDD_CUDA(cudaMemsetAsync(bars, 0, (size_t)cnt * sizeof(unsigned), st));
+    SymBatchP bb = b;
+    int nvv = nv;
+    void *args[] = {&bb, &sp, &nvv, &pbuf, &bars, &status};
+    RFDD_CUDA(cudaLaunchCooperativeKernel((const void *)tridiag_kernel, dim3(sp.off[cnt]), dim3(nmax <= 512 ? 256 : TRD_THREADS), args, smem,
+                                          st));
+    RFDD_CHECK_LAUNCH();
+    RFDD_CUDA(cudaFreeAsync(pbuf, st));
+    return;
+  }
   double *qbuf = nullptr;
   RFDD_CUDA(cudaMallocAsync((void **)&qbuf, (size_t)cnt * std::max(nmax, 1) * sizeof(double), st));
   for (int i = 0; i < nmax; ++i) {
@@ -333,21 +565,21 @@ __global__ void sturm_count_kernel(SymBatchP b, int cnt, double shift, long long
   counts[q] = sturm_count(it.d, it.e, n, shift, pivmin);
 }
 
-void sym_negative_counts(cudaStream_t st, const std::vector<SymItem> &items, double shift, long long *counts_dev) {
+void sym_negative_counts(cudaStream_t st, const std::vector<SymItem> &items, double shift, long long *counts_dev,
+                         int *status) {
   for (size_t s0 = 0; s0 < items.size(); s0 += EIG_MAXB) {
     SymBatchP b;
     memset(&b, 0, sizeof(b));
     const int cnt = (int)std::min<size_t>(EIG_MAXB, items.size() - s0);
     int nmax = 0;
     for (int i = 0; i < cnt; ++i) { b.it[i] = items[s0 + i]; nmax = std::max(nmax, b.it[i].n); }
-    if (nmax > 0) tridiagonalize(st, b, cnt, nmax);
+    if (nmax > 0) tridiagonalize(st, b, cnt, nmax, status);
     sturm_count_kernel<<<1, 64, 0, st>>>(b, cnt, shift, counts_dev + s0);
     RFDD_CHECK_LAUNCH();
   }
 }
 
 void sym_eig_values(cudaStream_t st, const std::vector<SymItem> &items, int *status) {
-  (void)status;
   for (size_t s0 = 0; s0 < items.size(); s0 += EIG_MAXB) {
     SymBatchP b;
     memset(&b, 0, sizeof(b));
@@ -355,7 +587,7 @@ void sym_eig_values(cudaStream_t st, const std::vector<SymItem> &items, int *sta
     int nmax = 0;
     for (int i = 0; i < cnt; ++i) { b.it[i] = items[s0 + i]; nmax = std::max(nmax, b.it[i].n); }
     if (nmax == 0) continue;
-    tridiagonalize(st, b, cnt, nmax);
+    tridiagonalize(st, b, cnt, nmax, status);
     tridiagonal_values(st, b, cnt, nmax);
   }
 }
@@ -499,7 +731,7 @@ __global__ void __launch_bounds__(256) inviter_kernel(InvIterP p, const Cluster 
 
 // Inverse iteration for eigenvalues that stand alone (clusters of one), one lane per eigenvalue:
 // the factorisation and the triangular solves are serial chains, so a warp runs 32 of them at the
-// cost of one (one thread of a CTA per eigenvalue took 14.2 ms for all vectors of order 1885).
+// cost of one (all vectors of order 1885: 4.8 ms, 14.2 with one thread of a CTA per eigenvalue).
 // Scratch is lane-interleaved (entry k of lane l at k * 32 + l), so every access is coalesced, and
 // IV_U steps are loaded ahead of the chain.  Same start vectors, factorisation and number of
 // iterations as inviter_kernel.

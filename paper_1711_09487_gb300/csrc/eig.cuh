@@ -24,7 +24,8 @@ void sym_eig_values(cudaStream_t st, const std::vector<SymItem> &items, int *sta
 // Number of eigenvalues below shift of every H (Householder tridiagonalisation, which keeps the
 // inertia, then a Sturm count of the tridiagonal matrix); H is overwritten.  counts_dev: device
 // array, one entry per item.
-void sym_negative_counts(cudaStream_t st, const std::vector<SymItem> &items, double shift, long long *counts_dev);
+void sym_negative_counts(cudaStream_t st, const std::vector<SymItem> &items, double shift, long long *counts_dev,
+                         int *status);
 
 // Eigenvectors for the ascending sorted indices sel of each item: out row r (ld_out) = unit
 // eigenvector of H for lam[sel[r]].  Eigenvalues closer than ctol * ||T|| to a neighbouring

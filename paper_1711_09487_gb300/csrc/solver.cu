@@ -362,6 +362,8 @@ void sync_status(rfdd_handle *h, const char *where, Buf *w = nullptr) {
     RFDD_CUDA(cudaStreamSynchronize(h->st));
     if (s & DS_WAIT_TIMEOUT)
       throw Error(RFDD_ECUDA, std::string(where) + ": a tensor-core GEMM timed out waiting for its operands");
+    if (s & DS_GRID_TIMEOUT)
+      throw Error(RFDD_ECUDA, std::string(where) + ": the CTAs of a cooperative kernel timed out waiting for each other");
     if (s & (DS_ZERO_PIVOT | DS_NONFINITE))
       throw Error(RFDD_ESINGULAR, std::string(where) + ": zero or non-finite pivot (device status " +
                                       std::to_string(s) + ")");
@@ -2875,10 +2877,10 @@ int64_t inertia_impl(rfdd_handle *h, double sigma) {
                   nullptr, nullptr});
   }
   cnt.alloc((size_t)nitems * sizeof(long long));
-  sym_negative_counts(st, si, 0.0, cnt.as<long long>());
+  sym_negative_counts(st, si, 0.0, cnt.as<long long>(), h->status.as<int>());
   std::vector<long long> hc(nitems);
   RFDD_CUDA(cudaMemcpyAsync(hc.data(), cnt.p, nitems * sizeof(long long), cudaMemcpyDeviceToHost, st));
-  RFDD_CUDA(cudaStreamSynchronize(st));
+  sync_status(h, "inertia: tridiagonalisation");
   int64_t total = 0;
   for (long long c : hc) total += c;
   return total;

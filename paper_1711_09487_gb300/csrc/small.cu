@@ -73,14 +73,128 @@ __global__ void __launch_bounds__(512) chol_inv_kernel(CholBatchP bp, double tol
   }
 }
 
+// 1/sqrt(x): the hardware's approximation refined by two Newton steps; the plain operations far
+// from 1
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  if (!(x > 1e-280 && x < 1e280)) return 1.0 / sqrt(x);
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(0.5 * r, fma(-x * r, r, 1.0), r);
+  return fma(0.5 * r, fma(-x * r, r, 1.0), r);
+}
+
+// Up to order CH_SMALL (the widths of the Krylov and V_j blocks) the matrix lives in shared memory
+// and the work is split in two launches: the factorisation, one CTA per matrix (b^3 / 6 FMAs at the 2
+// per cycle of one SM, and a chain of about 0.5 us a step), then the inverse with CHI_COLS columns
+// per CTA, so that its b^3 / 6 FMAs spread over the chip.  Order 120: 0.22 + 0.06 ms; 0.77 ms with
+// chol_inv_kernel, whose inverse is one global-memory chain per column.
+constexpr int CH_SMALL = 160;
+constexpr int CHI_COLS = 8;
+__global__ void __launch_bounds__(512) chol_small_kernel(CholBatchP bp, double tol, double *dinv_all) {
+  const CholItem it = bp.it[blockIdx.x];
+  const int b = it.b, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  extern __shared__ double S[];
+  __shared__ double diag[CH_SMALL], dinv[CH_SMALL];
+  __shared__ double thr_s;
+  for (int e = tid; e < b * b; e += blockDim.x) S[e] = it.G[e];
+  __syncthreads();
+  if (warp == 0) {
+    double m = 0.0;
+    for (int i = lane; i < b; i += 32) m = fmax(m, S[i * b + i]);
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) thr_s = tol * m;
+  }
+  __syncthreads();
+  const double thr = thr_s;
+  // warp 0 turns row t (complete) into a row of R; one warp, because every warp that computes the
+  // scalars takes 16 cycles of the SM's FP64 pipe per instruction
+  auto finish_row = [&](int t) {
+    const double pv = S[t * b + t];
+    const bool dead = !(pv > thr) || !isfinite(pv);
+    const double r = dead ? 0.0 : rsqrt_nr(pv);
+    for (int c = t + 1 + lane; c < b; c += 32) S[t * b + c] *= r;
+    if (lane == 0) {
+      diag[t] = dead ? 0.0 : pv * r;
+      dinv[t] = r;
+      it.dead[t] = dead;
+    }
+  };
+  if (warp == 0 && b > 0) finish_row(0);
+  __syncthreads();
+  for (int t = 0; t + 1 < b; ++t) {
+    const bool live = dinv[t] != 0.0;
+    // row t + 1 by warp 0, the others by the other warps
+    for (int i = t + 1 + warp; i < b; i += warp == 0 ? b : nw - 1) {
+      if (live) {
+        const double g = S[t * b + i];
+        for (int c = i + lane; c < b; c += 32) S[i * b + c] = fma(-g, S[t * b + c], S[i * b + c]);
+      }
+    }
+    if (warp == 0) {
+      __syncwarp();
+      finish_row(t + 1);
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < b * b; e += blockDim.x) {
+    const int i = e / b, c = e % b;
+    it.G[e] = i < c ? (dinv[i] != 0.0 ? S[e] : 0.0) : i == c ? diag[i] : 0.0;
+    if (i == c) dinv_all[(int64_t)blockIdx.x * CH_SMALL + i] = dinv[i];
+  }
+}
+
+// X = R^{-1}, columns c0 .. c0 + CHI_COLS - 1: row i of X is final once every row below it has been
+// eliminated, and is then subtracted from the rows above it.  Rows are scaled by 1/R_ii on the way
+// out (0 for a dropped one).
+__global__ void __launch_bounds__(256) chol_small_inv_kernel(CholBatchP bp, const double *__restrict__ dinv_all) {
+  const CholItem it = bp.it[blockIdx.y];
+  const int b = it.b, c0 = blockIdx.x * CHI_COLS, tid = threadIdx.x;
+  if (c0 >= b) return;
+  extern __shared__ double sm[];
+  const int m = min(b, c0 + CHI_COLS);  // rows that can be nonzero
+  double *R = sm, *X = sm + b * b;
+  __shared__ double dinv[CH_SMALL];
+  for (int e = tid; e < m * b; e += blockDim.x) R[e] = it.G[e];
+  for (int e = tid; e < m; e += blockDim.x) dinv[e] = dinv_all[(int64_t)blockIdx.y * CH_SMALL + e];
+  const int c = tid % CHI_COLS, rg = tid / CHI_COLS;
+  constexpr int RG = 256 / CHI_COLS;
+  for (int r = rg; r < m; r += RG) X[r * CHI_COLS + c] = r == c0 + c ? 1.0 : 0.0;
+  __syncthreads();
+  for (int i = m - 1; i > 0; --i) {
+    const double xi = X[i * CHI_COLS + c] * dinv[i];
+    for (int r = rg; r < i; r += RG) X[r * CHI_COLS + c] = fma(-R[r * b + i], xi, X[r * CHI_COLS + c]);
+    __syncthreads();
+  }
+  if (c0 + c < b)
+    for (int r = rg; r < b; r += RG)
+      it.Rinv[(int64_t)r * b + c0 + c] = r < m ? X[r * CHI_COLS + c] * dinv[r] : 0.0;
+}
+
 void chol_inv_batched(cudaStream_t st, const std::vector<CholItem> &items, double tol) {
   for (size_t s = 0; s < items.size(); s += CH_MAXB) {
     CholBatchP b;
     memset(&b, 0, sizeof(b));
     const int cnt = (int)std::min<size_t>(CH_MAXB, items.size() - s);
-    for (int i = 0; i < cnt; ++i) b.it[i] = items[s + i];
-    chol_inv_kernel<<<cnt, 512, 0, st>>>(b, tol);
+    int bmax = 0;
+    for (int i = 0; i < cnt; ++i) {
+      b.it[i] = items[s + i];
+      bmax = std::max(bmax, b.it[i].b);
+    }
+    if (bmax > CH_SMALL) {
+      chol_inv_kernel<<<cnt, 512, 0, st>>>(b, tol);
+      RFDD_CHECK_LAUNCH();
+      continue;
+    }
+    const int sm1 = bmax * bmax * (int)sizeof(double), sm2 = sm1 + bmax * CHI_COLS * (int)sizeof(double);
+    RFDD_CUDA(cudaFuncSetAttribute(chol_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1));
+    RFDD_CUDA(cudaFuncSetAttribute(chol_small_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2));
+    double *dinv = nullptr;
+    RFDD_CUDA(cudaMallocAsync((void **)&dinv, (size_t)cnt * CH_SMALL * sizeof(double), st));
+    chol_small_kernel<<<cnt, 512, sm1, st>>>(b, tol, dinv);
     RFDD_CHECK_LAUNCH();
+    chol_small_inv_kernel<<<dim3(ceil_div(bmax, CHI_COLS), cnt), 256, sm2, st>>>(b, dinv);
+    RFDD_CHECK_LAUNCH();
+    RFDD_CUDA(cudaFreeAsync(dinv, st));
   }
 }
 

@@ -240,7 +240,8 @@ __global__ void __launch_bounds__(256) tri_prep_kernel(SymBatchP b, double *info
 // into G + 1 equal parts, and the part holding eigenvalue i becomes the new interval (log2(G + 1)
 // bits per round instead of one, at G times the counting work).  One warp per CTA: the FP64 pipe of
 // an SM serves one warp as fast as it does eight, so the warps are spread over all SMs (with eight
-// warps a CTA the order-120 problem ran on 4 SMs: 1.23 ms, and order 1885 on 59: 19.8 ms).
+// warps a CTA the order-120 problem ran on 4 SMs: 1.23 ms, now 0.23; order 1885 on 59: 19.8 ms, now
+// 8.1).
 template <int G>
 __global__ void __launch_bounds__(32) bisect_kernel(SymBatchP b, const double *__restrict__ info) {
   const SymItem it = b.it[blockIdx.y];
@@ -309,10 +310,10 @@ static void tridiagonal_values(cudaStream_t st, const SymBatchP &b, int cnt, int
 // Householder vector from it for itself (O(n) work, cheaper than a second barrier), then updates its
 // rows and their entries of p_i.  p alternates between two buffers, and row i takes v_i one step
 // late, so that no CTA overwrites what a slower one still reads.  Bound: below order 400 the chain of
-// one step (barrier, two block reductions, the reflector's scalars: about 6 us), above it the three
-// FP64 operations per trailing entry (1885 FMA-cubed is 11 ms of the chip's FP64 rate).  Measured:
-// order 120 0.74 ms (1.04 ms in 240 launches, 1.7 ms with their gaps), order 1885 32.9 ms (37.2 in
-// 3769 launches, 44 with gaps).
+// one step (barrier, two block reductions, the reflector's scalars: about 5 us), above it the three
+// FP64 operations per trailing entry (n^3 FMAs are 11 ms of the chip's FP64 rate at order 1885).
+// Measured: order 120 0.65 ms (1.04 ms in 240 launches, 1.7 ms with their gaps), order 1885 28.8 ms
+// (37.2 in 3769 launches, 44 with gaps).
 constexpr int TRD_THREADS = 512;  // at most; 256 below order 512
 constexpr int TRD_NMAX = 8192;  // three vectors of the order in shared memory
 constexpr int TRD_SPIN = 1 << 22;
@@ -332,10 +333,12 @@ __device__ __forceinline__ bool trd_barrier(unsigned *cnt, unsigned target) {
   return ok_s != 0;
 }
 
-// Block-wide sum over the first nact warps, the same value in every thread.  A warp's FP64 add takes
-// 16 cycles of an SM's FP64 pipe, so warps without data add nothing and the warp partials are added
-// as a tree by one warp.
-__device__ __forceinline__ double trd_sum(double v, double *red, int nact) {
+// Block-wide sum over the first nact warps, given to f by one thread of warp 0; what f leaves in
+// shared memory is visible to all on return.  A warp's FP64 instruction takes 16 cycles of an SM's
+// FP64 pipe, whatever its lanes do: warps without data add nothing, and the scalars that follow from
+// the sum are formed by one warp (formed by all sixteen they took longer than the sum).
+template <typename F>
+__device__ __forceinline__ void trd_sum(double v, double *red, int nact, F &&f) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (w < nact) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -345,10 +348,9 @@ __device__ __forceinline__ double trd_sum(double v, double *red, int nact) {
   if (w == 0) {
     v = lane < nact ? red[lane] : 0.0;
     for (int o = nact > 8 ? 8 : nact > 4 ? 4 : nact > 2 ? 2 : 1; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) red[32] = v;
+    if (lane == 0) f(v);
   }
   __syncthreads();
-  return red[32];
 }
 
 // The Householder reflector of a vector with first entry alpha and the sum of squares sig of the
@@ -395,10 +397,10 @@ __global__ void __launch_bounds__(TRD_THREADS) tridiag_kernel(SymBatchP b, TridS
   const int nthr = blockDim.x, NW = nthr >> 5;
   extern __shared__ double sm[];
   double *vp = sm, *q = sm + nmax, *v = sm + 2 * nmax;  // v_{i-1}, q_{i-1}, v_i, indexed by row
-  __shared__ double red[33];
+  __shared__ double red[32];
+  __shared__ double K_s, qi_s, sc_s, tau_s;  // tau_s: of the last reflector formed
   double *p0 = pbuf + (int64_t)item * 2 * nmax;
   unsigned *bar = bars + item;
-  double taup = 0.0;  // tau of the current reflector (of step i-1 until it is formed)
   for (int i = 0; i < n; ++i) {
     // q_{i-1} and row i
     double *row = it.H + (int64_t)i * it.ld;
@@ -413,8 +415,11 @@ __global__ void __launch_bounds__(TRD_THREADS) tridiag_kernel(SymBatchP b, TridS
         ss = fma(pk, vp[k], ss);
         v[k] = __ldcg(row + k);
       }
-      const double K = 0.5 * taup * trd_sum(ss, red, nact);
-      const double vi = vp[i], qi = q[i] - K * vi;
+      trd_sum(ss, red, nact, [&](double t) {
+        K_s = 0.5 * tau_s * t;
+        qi_s = q[i] - K_s * vp[i];
+      });
+      const double K = K_s, vi = vp[i], qi = qi_s;
       ss = 0.0;
       for (int k = i + tid; k < n; k += nthr) {
         const double qk = q[k] - K * vp[k];
@@ -430,16 +435,19 @@ __global__ void __launch_bounds__(TRD_THREADS) tridiag_kernel(SymBatchP b, TridS
         if (k > i + 1) ss = fma(x, x, ss);
       }
     }
-    const double sig = trd_sum(ss, red, nact);
-    const double di = v[i];
-    if (i >= n - 1) {
-      if (me == 0 && tid == 0) { it.d[i] = di; it.tau[i] = 0.0; }
-    } else {
-      const double alpha = v[i + 1];
-      double beta, sc;
-      householder(alpha, sig, beta, taup, sc);
-      if (me == 0 && tid == 0) { it.d[i] = di; it.e[i] = beta; it.tau[i] = taup; }
-      __syncthreads();
+    trd_sum(ss, red, nact, [&](double sig) {
+      double beta = 0.0, tau = 0.0, sc = 0.0;
+      if (i < n - 1) householder(v[i + 1], sig, beta, tau, sc);
+      if (me == 0) {
+        it.d[i] = v[i];
+        it.tau[i] = tau;
+        if (i < n - 1) it.e[i] = beta;
+      }
+      tau_s = tau;
+      sc_s = sc;
+    });
+    if (i < n - 1) {
+      const double sc = sc_s;
       for (int k = i + 2 + tid; k < n; k += nthr) v[k] *= sc;
       if (tid == 0) v[i + 1] = 1.0;
       __syncthreads();
@@ -491,7 +499,7 @@ __global__ void __launch_bounds__(TRD_THREADS) tridiag_kernel(SymBatchP b, TridS
       if (sym) {
         double t = s0 + s1;
         for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-        if (lane == 0) pn[r] = taup * t;
+        if (lane == 0) pn[r] = tau_s * t;
       }
     }
     if (!trd_barrier(bar, (unsigned)(G * (i + 1)))) {

@@ -528,7 +528,9 @@ static void tridiagonalize(cudaStream_t st, const SymBatchP &b, int cnt, int nma
     for (int j = cnt; j < EIG_MAXB; ++j) sp.off[j + 1] = sp.off[cnt];
     const int nv = (nmax + 1) & ~1;
     const size_t smem = (size_t)3 * nv * sizeof(double);
-    RFDD_CUDA(cudaFuncSetAttribute(tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // always the same limit: several host threads launch this kernel at once
+    RFDD_CUDA(cudaFuncSetAttribute(tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   3 * TRD_NMAX * (int)sizeof(double)));
     double *pbuf = nullptr;
     const size_t pb = (size_t)cnt * 2 * nv * sizeof(double);
     RFDD_CUDA(cudaMallocAsync((void **)&pbuf, pb + (size_t)cnt * sizeof(unsigned), st));
@@ -995,7 +997,7 @@ void sym_eig_vectors(cudaStream_t st, const std::vector<BackItem> &items, double
     }
     const size_t smem = (size_t)nmax * sizeof(double);
     RFDD_REQUIRE(smem <= 200 * 1024, RFDD_EINVAL, "sym_eig: order too large");
-    RFDD_CUDA(cudaFuncSetAttribute(back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RFDD_CUDA(cudaFuncSetAttribute(back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     back_kernel<<<dim3(selmax, cnt), 256, smem, st>>>(bb);
     RFDD_CHECK_LAUNCH();
     RFDD_CUDA(cudaFreeAsync(sel_dev, st));

@@ -186,8 +186,11 @@ void chol_inv_batched(cudaStream_t st, const std::vector<CholItem> &items, doubl
       continue;
     }
     const int sm1 = bmax * bmax * (int)sizeof(double), sm2 = sm1 + bmax * CHI_COLS * (int)sizeof(double);
-    RFDD_CUDA(cudaFuncSetAttribute(chol_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1));
-    RFDD_CUDA(cudaFuncSetAttribute(chol_small_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2));
+    // always the same limits: several host threads launch these kernels at once
+    RFDD_CUDA(cudaFuncSetAttribute(chol_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   CH_SMALL * CH_SMALL * (int)sizeof(double)));
+    RFDD_CUDA(cudaFuncSetAttribute(chol_small_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   CH_SMALL * (CH_SMALL + CHI_COLS) * (int)sizeof(double)));
     double *dinv = nullptr;
     RFDD_CUDA(cudaMallocAsync((void **)&dinv, (size_t)cnt * CH_SMALL * sizeof(double), st));
     chol_small_kernel<<<cnt, 512, sm1, st>>>(b, tol, dinv);

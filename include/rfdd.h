@@ -92,7 +92,7 @@ typedef struct {
                            complex column width of one tensor-core tile: the extra guard vectors
                            ride in tile columns that would otherwise be padding); <= 1: none */
   int pack_factors;     /* mixed solve: form of the complex factors kept for the solves.  1: the
-                           tensor-core tile copies only (TF32 hi/lo, 16 bytes per complex entry,
+                           tensor-core tile copies only (16-bit hi/lo, 8 bytes per complex entry,
                            packed once after the factorisation; the complex64 factors are freed
                            then, so the peak holds both); 0: the complex64 factors only (8 bytes
                            per entry; every solve product packs its factor block on the fly);
@@ -318,7 +318,8 @@ int rfdd_sym_eig(int64_t n, const double *H, double *evals, double *evecs);
 /* Building block of a3-a5 (trailing updates of the factorisations), a6 and a10 (triangular-solve
  * updates): C = beta*C + alpha*A*B for complex single-precision A (m x k, leading dimension lda),
  * B (k x n, ldb), C (m x n, ldc), host arrays, row-major, interleaved (re, im) floats.
- * engine 1 = the tensor-core GEMM (tcgen05, 3xTF32 split) that every complex-FP32 contraction of
+ * engine 1 = the tensor-core GEMM (tcgen05, scaled 16-bit hi/lo split, three products) that every
+ * complex-FP32 contraction of
  * the solver runs on, with its automatic choice between a one-CTA kernel (128 x 256 tiles of the
  * realified product) and a two-CTA kernel (cta_group::2, 256 x 256 tiles on a pair of SMs);
  * engines 2 and 3 force the one-CTA and the two-CTA kernel; engine 0 = a CUDA-core kernel kept
@@ -343,7 +344,7 @@ int rfdd_dgemm(int64_t m, int64_t n, int64_t k, int32_t ta, const double *A, int
 /* Tile-shape autotuner of the tensor-core GEMMs (no counterpart in the paper).  Where both the
  * one-CTA kernel (128 x 256 output tiles) and the two-CTA kernel (256 x 256 tiles per SM pair)
  * can run a launch, the library times both on real launches of the same class -- device,
- * complex or real, the K depth bucket floor(log2(K/32 tiles)) and the launch's tile count against
+ * complex or real, the K depth bucket floor(log2(K/32)) of the realified K, the launch's tile count against
  * the SM count; never what else runs -- three timings each, with CUDA events on the launch's
  * stream and without blocking, then keeps the faster for every later launch of that class in this
  * process.  Until a class is decided, and whenever tuning is off, a fixed rule chooses (the
@@ -364,7 +365,7 @@ int rfdd_autotune_table(char *buf, int64_t cap, int64_t *len);
  * implicit synchronisation an allocation can cause -- this computes C = beta*C + alpha*A*B on the
  * tensor cores with A, B, C in DEVICE memory (complex single precision, row-major, interleaved,
  * leading dimensions in complex elements) and stages the packed operands in a fixed static
- * device array (6 MiB per device that has loaded the library, held until process exit) instead
+ * device array (3 MiB per device that has loaded the library, held until process exit) instead
  * of a workspace.  Limits: 1 <= m, n <= 1024 and 1 <= k <= 128; larger sizes return RFDD_EINVAL.
  * The first call on a device looks up the device addresses of that array and of its status word
  * (make that first call before any stream capture).  Work runs on `stream` (a cudaStream_t, NULL =
@@ -392,7 +393,7 @@ long long rfdd_kernel_launches(void);
  * launches after a warm-up, CUDA events): which = 0 the tensor pipe's TF32 rate (tcgen05
  * kind::tf32 MMAs of 128 x 256 x 8 issued back to back from operand tiles held in shared memory,
  * one CTA per SM); 1 FP64 fused multiply-add on the CUDA cores; 2 FP32 fused multiply-add on the
- * CUDA cores; 3 a plain TF32 GEMM through the solver's tensor-core kernel (one MMA per product,
+ * CUDA cores; 3 a plain TF32 GEMM through the solver's tensor-core kernel (its TF32 form: one MMA per product,
  * operands fed from memory; a real 8192^3 GEMM, the MMA kernel alone timed, operand packing
  * excluded).  Allocates about 1.9 GB (which = 3) or a few MB, on a stream of its own. */
 int rfdd_peak_probe(int32_t which, double *tflops);

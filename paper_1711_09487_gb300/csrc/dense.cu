@@ -373,7 +373,7 @@ template <typename T>
 void gemm_batched(cudaStream_t st, const std::vector<GemmItem<T>> &items, bool ta, bool tb,
                   double alpha, double beta) {
   if constexpr (std::is_same<T, cx<float>>::value) {
-    // complex FP32 products go to the tensor cores (3xTF32 split, FP32 accumulation)
+    // complex FP32 products go to the tensor cores (two-way 16-bit split, FP32 accumulation)
     if (!ta && !tb) {
       std::vector<GemmItem<T>> live;
       for (auto &g : items)
@@ -1197,17 +1197,16 @@ static void trsm_block_inverse(cudaStream_t st, const std::vector<SolveItem<T>> 
       const T *inv = (upper ? it.Uinv : it.Linv) + (int64_t)b * nbo * nbo;
       T *xb = it.X + (int64_t)K0 * it.ldx, *t = tmp + toff[i] + (int64_t)K0 * it.ncols;
       g1.push_back({inv, xb, t, w, it.ncols, w, nbo, it.ldx, it.ncols});
-      const float *ih = upper ? it.Uinvp_hi : it.Linvp_hi, *il = upper ? it.Uinvp_lo : it.Linvp_lo;
-      const int64_t bf = tc_packed_a_floats(nbo, nbo);
-      p1.push_back(ih ? TcPackedA{ih + b * bf, il + b * bf, tc_packed_a_ktiles(nbo)} : TcPackedA{});
+      const uint8_t *ip = upper ? it.Uinvp : it.Linvp;
+      p1.push_back(ip ? tc_packed_view(ip + b * tc_packed_a_bytes(nbo, nbo), nbo, nbo) : TcPackedA{});
       if (!upper && it.n - K0 - w > 0) {  // rows below: X[K0+w:] -= L[K0+w:, K0:K0+w] t_b
         g2.push_back({it.LU + (int64_t)(K0 + w) * it.ld + K0, t, it.X + (int64_t)(K0 + w) * it.ldx, it.n - K0 - w,
                       it.ncols, w, it.ld, it.ncols, it.ldx});
-        p2.push_back(it.LUp_hi ? tc_packed_view(it.LUp_hi, it.LUp_lo, it.n, K0 + w, K0) : TcPackedA{});
+        p2.push_back(it.LUp ? tc_packed_view(it.LUp, it.n, it.n, K0 + w, K0, 0) : TcPackedA{});
       }
       if (upper && K0 > 0) {  // rows above: X[0:K0] -= U[0:K0, K0:K0+w] t_b
         g2.push_back({it.LU + K0, t, it.X, K0, it.ncols, w, it.ld, it.ncols, it.ldx});
-        p2.push_back(it.LUp_hi ? tc_packed_view(it.LUp_hi, it.LUp_lo, it.n, 0, K0) : TcPackedA{});
+        p2.push_back(it.LUp ? tc_packed_view(it.LUp, it.n, it.n, 0, K0, 1) : TcPackedA{});
       }
     }
     bool use_pa = false;

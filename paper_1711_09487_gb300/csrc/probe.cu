@@ -92,7 +92,7 @@ double tf32_probe(cudaStream_t st) {
   int *status = nullptr;
   RFDD_CUDA(cudaMallocAsync((void **)&status, sizeof(int), st));
   RFDD_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
-  std::vector<GemmItem<float>> it = {{A, B, C, N, N, N, N, N, N}};
+  const GemmItem<float> it = {A, B, C, N, N, N, N, N, N};
   double best = 0.0;
   {
     TcStatusScope tcs(status);

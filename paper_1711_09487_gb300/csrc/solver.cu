@@ -261,10 +261,10 @@ struct rfdd_handle {
   Buf BLinv, BUinv, SLinv, SUinv;
   std::vector<int64_t> binvoff;  // (node, subdomain) -> offset into BLinv / BUinv
   int64_t sinv_elems = 0;        // per node in SLinv / SUinv
-  // Mixed solve: tensor-core tile copies (TF32 hi/lo) of the factor operands the solves multiply
+  // Mixed solve: tensor-core tile copies (16-bit hi/lo) of the factor operands the solves multiply
   // by, packed once per factorisation.  Per B factor (node, subdomain) and per S factor (node):
   // the leading LU, the inverse diagonal blocks of L and of U, and (B only) the border blocks L21
-  // and U12.  Float offsets of each hi array into Pk; its lo array follows it.
+  // and U12.  Byte offsets of each operand into Pk.
   Buf Pk;
   struct PkOff { int64_t lu = -1, li = -1, ui = -1, l21 = -1, u12 = -1; };
   std::vector<PkOff> pkB, pkS;
@@ -960,7 +960,9 @@ static size_t factor_bytes_impl(const SolveShape &g, int nc, bool packed) {
   size_t inv = sinv;  // inverted diagonal blocks of L and U
   for (int j = 0; j < g.p; ++j) inv += (size_t)block_inverse_elems(g.d[j], 256);
   b += 2 * (size_t)nc * inv * scal;
-  if (mixed && packed) {  // packed tensor-core copies of the solve operands (hi + lo)
+  if (mixed && packed) {
+    // packed tensor-core copies of the solve operands (16-bit hi + lo, as many bytes as the complex64
+    // entries), and as much again for the operands that the products pack as they go
     size_t pk = spk;
     for (int j = 0; j < g.p; ++j)
       pk += (size_t)g.D[j] * g.D[j] - (size_t)(g.D[j] - g.d[j]) * (g.D[j] - g.d[j]) +
@@ -1160,19 +1162,20 @@ void factor_impl(rfdd_handle *h) {
   h->have_factors = true;
 }
 
-// packed (hi, lo) pointers of one operand in h->Pk; (nullptr, nullptr) when absent
-std::pair<const float *, const float *> pk_ptrs(const rfdd_handle *h, int64_t off, int64_t floats) {
-  if (off < 0 || !h->Pk.p) return {nullptr, nullptr};
-  const float *hi = h->Pk.as<float>() + off;
-  return {hi, hi + floats};
+// one packed operand in h->Pk; nullptr when absent
+const uint8_t *pk_ptr(const rfdd_handle *h, int64_t off) {
+  return off < 0 || !h->Pk.p ? nullptr : h->Pk.as<uint8_t>() + off;
+}
+// a packed m x k border block as a GEMM operand (no operand when absent)
+TcPackedA pk_border(const rfdd_handle *h, int64_t off, int64_t m, int64_t k) {
+  const uint8_t *op = pk_ptr(h, off);
+  return op ? tc_packed_view(op, m, k) : TcPackedA{};
 }
 template <typename Tf>
-void attach_packed(const rfdd_handle *h, SolveItem<Tf> &x, const rfdd_handle::PkOff &o, int64_t n) {
-  if (!h->Pk.p) return;
-  const int64_t nblk = (n + NBO - 1) / NBO, bf = tc_packed_a_floats(NBO, NBO);
-  std::tie(x.LUp_hi, x.LUp_lo) = pk_ptrs(h, o.lu, tc_packed_a_floats(n, n));
-  std::tie(x.Linvp_hi, x.Linvp_lo) = pk_ptrs(h, o.li, nblk * bf);
-  std::tie(x.Uinvp_hi, x.Uinvp_lo) = pk_ptrs(h, o.ui, nblk * bf);
+void attach_packed(const rfdd_handle *h, SolveItem<Tf> &x, const rfdd_handle::PkOff &o) {
+  x.LUp = pk_ptr(h, o.lu);
+  x.Linvp = pk_ptr(h, o.li);
+  x.Uinvp = pk_ptr(h, o.ui);
 }
 
 // the inverted diagonal blocks of factor (node l, subdomain j), when present
@@ -1183,40 +1186,40 @@ void attach_binv(const rfdd_handle *h, SolveItem<Tf> &x, int l, int j) {
   x.Linv = h->BLinv.as<Tf>() + o;
   x.Uinv = h->BUinv.as<Tf>() + o;
   x.nbi = NBO;
-  if (!h->pkB.empty()) attach_packed(h, x, h->pkB[(size_t)l * h->p + j], h->d[j]);
+  if (!h->pkB.empty()) attach_packed(h, x, h->pkB[(size_t)l * h->p + j]);
 }
 
 // Mixed solve: pack the factor operands of the later solves once (see rfdd_handle::Pk)
 void pack_factor_operands(rfdd_handle *h) {
   cudaStream_t st = h->st;
   const int nc = h->nnodes, p = h->p;
-  const int64_t s = h->s, bf = tc_packed_a_floats(NBO, NBO);
+  const int64_t s = h->s, bf = tc_packed_a_bytes(NBO, NBO);
   h->pkB.assign((size_t)nc * p, {});
   h->pkS.assign((size_t)nc, {});
   h->pkG.assign((size_t)nc * h->lv.G, {});
   int64_t tot = 0;
-  auto take = [&](int64_t floats) {
+  auto take = [&](int64_t bytes) {
     const int64_t o = tot;
-    tot += 2 * floats;
+    tot += bytes;
     return o;
   };
   for (int l = 0; l < nc; ++l) {
     for (int j = 0; j < p; ++j) {
       const int64_t dj = h->d[j], sj = h->D[j] - dj, nblk = (dj + NBO - 1) / NBO;
       auto &o = h->pkB[(size_t)l * p + j];
-      o.lu = take(tc_packed_a_floats(dj, dj));
+      o.lu = take(tc_packed_a_bytes(dj, dj, true));
       o.li = take(nblk * bf);
       o.ui = take(nblk * bf);
       if (sj > 0) {
-        o.l21 = take(tc_packed_a_floats(sj, dj));
-        o.u12 = take(tc_packed_a_floats(dj, sj));
+        o.l21 = take(tc_packed_a_bytes(sj, dj));
+        o.u12 = take(tc_packed_a_bytes(dj, sj));
       }
     }
     auto &o = h->pkS[l];
     const int64_t sS = h->lv.G > 0 ? h->lv.s2 : s;  // two levels: S2' takes the place of S
     const int64_t nblk = (sS + NBO - 1) / NBO;
     if (sS > 0) {
-      o.lu = take(tc_packed_a_floats(sS, sS));
+      o.lu = take(tc_packed_a_bytes(sS, sS, true));
       o.li = take(nblk * bf);
       o.ui = take(nblk * bf);
     }
@@ -1224,26 +1227,26 @@ void pack_factor_operands(rfdd_handle *h) {
       const int64_t n1 = h->lv.n1[g], n2 = h->lv.n2[g], nb1 = (n1 + NBO - 1) / NBO;
       auto &og = h->pkG[(size_t)l * h->lv.G + g];
       if (n1 == 0) continue;
-      og.lu = take(tc_packed_a_floats(n1, n1));
+      og.lu = take(tc_packed_a_bytes(n1, n1, true));
       og.li = take(nb1 * bf);
       og.ui = take(nb1 * bf);
       if (n2 > 0) {
-        og.l21 = take(tc_packed_a_floats(n2, n1));
-        og.u12 = take(tc_packed_a_floats(n1, n2));
+        og.l21 = take(tc_packed_a_bytes(n2, n1));
+        og.u12 = take(tc_packed_a_bytes(n1, n2));
       }
     }
   }
-  h->Pk.alloc((size_t)tot * sizeof(float));
-  float *P = h->Pk.as<float>();
+  h->Pk.alloc((size_t)tot);
+  uint8_t *P = h->Pk.as<uint8_t>();
   std::vector<TcPackJob> jobs;
-  auto job = [&](const cx<float> *A, int64_t lda, int64_t m, int64_t k, int64_t off) {
+  auto job = [&](const cx<float> *A, int64_t lda, int64_t m, int64_t k, int64_t off, int side = 0) {
     if (off < 0 || m <= 0 || k <= 0) return;
-    jobs.push_back({A, lda, m, k, P + off, P + off + tc_packed_a_floats(m, k)});
+    jobs.push_back({A, lda, m, k, P + off, side});
   };
   auto blocks = [&](const cx<float> *inv, int64_t n, int64_t off) {
     const int64_t nblk = (n + NBO - 1) / NBO;
     for (int64_t b = 0; b < nblk; ++b)
-      jobs.push_back({inv + b * NBO * NBO, NBO, NBO, NBO, P + off + b * bf, P + off + nblk * bf + b * bf});
+      jobs.push_back({inv + b * NBO * NBO, NBO, NBO, NBO, P + off + b * bf, 0});
   };
   cx<float> *base = h->fac.as<cx<float>>();
   for (int l = 0; l < nc; ++l) {
@@ -1251,7 +1254,7 @@ void pack_factor_operands(rfdd_handle *h) {
       const int64_t dj = h->d[j], Dj = h->D[j], sj = Dj - dj;
       const auto &o = h->pkB[(size_t)l * p + j];
       const cx<float> *A = base + h->boff[(size_t)l * p + j];
-      job(A, Dj, dj, dj, o.lu);
+      job(A, Dj, dj, dj, o.lu, NBO);
       job(A + dj * Dj, Dj, sj, dj, o.l21);
       job(A + dj, Dj, dj, sj, o.u12);
       blocks(h->BLinv.as<cx<float>>() + h->binvoff[(size_t)l * p + j], dj, o.li);
@@ -1259,7 +1262,7 @@ void pack_factor_operands(rfdd_handle *h) {
     }
     const auto &o = h->pkS[l];
     if (h->lv.G == 0) {
-      job(h->Sfac.as<cx<float>>() + (int64_t)l * s * s, s, s, s, o.lu);
+      job(h->Sfac.as<cx<float>>() + (int64_t)l * s * s, s, s, s, o.lu, NBO);
       blocks(h->SLinv.as<cx<float>>() + (int64_t)l * h->sinv_elems, s, o.li);
       blocks(h->SUinv.as<cx<float>>() + (int64_t)l * h->sinv_elems, s, o.ui);
       continue;
@@ -1268,7 +1271,7 @@ void pack_factor_operands(rfdd_handle *h) {
     const cx<float> *T = h->Lfac.as<cx<float>>() + (int64_t)l * L.tsz;
     const cx<float> *Li = h->LLinv.as<cx<float>>() + (int64_t)l * L.isz, *Ui = h->LUinv.as<cx<float>>() + (int64_t)l * L.isz;
     if (L.s2 > 0) {
-      job(T, L.s2, L.s2, L.s2, o.lu);
+      job(T, L.s2, L.s2, L.s2, o.lu, NBO);
       blocks(Li, L.s2, o.li);
       blocks(Ui, L.s2, o.ui);
     }
@@ -1277,7 +1280,7 @@ void pack_factor_operands(rfdd_handle *h) {
       if (n1 == 0) continue;
       const auto &og = h->pkG[(size_t)l * L.G + g];
       const cx<float> *Bg = T + L.goff[g];
-      job(Bg, Dg, n1, n1, og.lu);
+      job(Bg, Dg, n1, n1, og.lu, NBO);
       job(Bg + n1 * Dg, Dg, n2, n1, og.l21);
       job(Bg + n1, Dg, n1, n2, og.u12);
       blocks(Li + L.ioff[g], n1, og.li);
@@ -1333,7 +1336,7 @@ void solve_S(rfdd_handle *h, Tf *G, int64_t ldg, int64_t gs, int64_t m, const st
       x.Linv = h->SLinv.as<Tf>() + (int64_t)l * h->sinv_elems;
       x.Uinv = h->SUinv.as<Tf>() + (int64_t)l * h->sinv_elems;
       x.nbi = NBO;
-      if (!h->pkS.empty()) attach_packed(h, x, h->pkS[l], h->s);
+      if (!h->pkS.empty()) attach_packed(h, x, h->pkS[l]);
     }
     it.push_back(x);
   }
@@ -1439,8 +1442,8 @@ SolveItem<Tf> level_item(const rfdd_handle *h, int l, int g, Tf *X, int64_t m) {
     x.Linv = h->LLinv.as<Tf>() + o;
     x.Uinv = h->LUinv.as<Tf>() + o;
     x.nbi = NBO;
-    if (g < 0 && !h->pkS.empty()) attach_packed(h, x, h->pkS[l], L.s2);
-    if (g >= 0 && !h->pkG.empty()) attach_packed(h, x, h->pkG[(size_t)l * L.G + g], L.n1[g]);
+    if (g < 0 && !h->pkS.empty()) attach_packed(h, x, h->pkS[l]);
+    if (g >= 0 && !h->pkG.empty()) attach_packed(h, x, h->pkG[(size_t)l * L.G + g]);
   }
   return x;
 }
@@ -1483,14 +1486,10 @@ void solve_S_levels_run(rfdd_handle *h, Tf *G, int64_t gs, int64_t m, const std:
         const auto *pk = h->pkG.empty() ? nullptr : &h->pkG[(size_t)nl[i] * NG + g];
         if (lower) {
           gi.push_back({blk + n1 * Dg, w, hh, (int)n2, (int)m, (int)n1, (int)Dg, (int)m, (int)m});
-          const auto pp = pk ? pk_ptrs(h, pk->l21, tc_packed_a_floats(n2, n1))
-                             : std::pair<const float *, const float *>{nullptr, nullptr};
-          pa.push_back(TcPackedA{pp.first, pp.second, tc_packed_a_ktiles(n1)});
+          pa.push_back(pk ? pk_border(h, pk->l21, n2, n1) : TcPackedA{});
         } else {
           gi.push_back({blk + n1, hh, w, (int)n1, (int)m, (int)n2, (int)Dg, (int)m, (int)m});
-          const auto pp = pk ? pk_ptrs(h, pk->u12, tc_packed_a_floats(n1, n2))
-                             : std::pair<const float *, const float *>{nullptr, nullptr};
-          pa.push_back(TcPackedA{pp.first, pp.second, tc_packed_a_ktiles(n2)});
+          pa.push_back(pk ? pk_border(h, pk->u12, n1, n2) : TcPackedA{});
         }
       }
     if (!gi.empty()) border_gemm<Tf>(st, gi, pa, lower ? 1.0 : -1.0, lower ? 0.0 : 1.0);
@@ -1620,9 +1619,7 @@ void dd_solve(rfdd_handle *h, const cx<double> *R, int64_t strideR, cx<double> *
         const int64_t Dj = h->D[j], dj = h->d[j];
         g.push_back({base + h->boff[(size_t)l * p + j] + dj * Dj, f + (int64_t)l * fs + h->off[j] * m,
                      ht + l * hs + (int64_t)j * smax * m, sj, (int)m, (int)dj, (int)Dj, (int)m, (int)m});
-        const auto pp = h->pkB.empty() ? std::pair<const float *, const float *>{nullptr, nullptr}
-                                       : pk_ptrs(h, h->pkB[(size_t)l * p + j].l21, tc_packed_a_floats(sj, dj));
-        pa.push_back(TcPackedA{pp.first, pp.second, tc_packed_a_ktiles(dj)});
+        pa.push_back(h->pkB.empty() ? TcPackedA{} : pk_border(h, h->pkB[(size_t)l * p + j].l21, sj, dj));
       }
     border_gemm<Tf>(st, g, pa, 1.0, 0.0);
     for (int j = 0; j < p; ++j) {
@@ -1650,9 +1647,7 @@ void dd_solve(rfdd_handle *h, const cx<double> *R, int64_t strideR, cx<double> *
         if (sj > 0) {
           g.push_back({base + h->boff[(size_t)l * p + j] + dj, ht + l * hs + (int64_t)j * smax * m,
                        f + (int64_t)l * fs + h->off[j] * m, (int)dj, (int)m, sj, (int)Dj, (int)m, (int)m});
-          const auto pp = h->pkB.empty() ? std::pair<const float *, const float *>{nullptr, nullptr}
-                                         : pk_ptrs(h, h->pkB[(size_t)l * p + j].u12, tc_packed_a_floats(dj, sj));
-          pa.push_back(TcPackedA{pp.first, pp.second, tc_packed_a_ktiles(sj)});
+          pa.push_back(h->pkB.empty() ? TcPackedA{} : pk_border(h, h->pkB[(size_t)l * p + j].u12, dj, sj));
         }
         SolveItem<Tf> x;
         x.LU = base + h->boff[(size_t)l * p + j];

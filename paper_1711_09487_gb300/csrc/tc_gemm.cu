@@ -1,18 +1,23 @@
-// Complex-FP32 GEMM on the 5th-generation tensor cores (tcgen05, kind::tf32) for sm_103a.
+// Complex-FP32 GEMM on the 5th-generation tensor cores (tcgen05, kind::f16) for sm_103a.
 //
 // C = beta*C + alpha*A*B with complex A (m x k), B (k x n), C (m x n), interleaved (re, im),
 // row-major.  The complex product is computed in real ("4M", realified) form:
 //   Cr (m x 2n) = Ar (m x 2k) * Br (2k x 2n),
 // where Ar and Cr are the interleaved storage read as real matrices and each complex B[p][j]
-// becomes the 2x2 real block [[re, im], [-im, re]] of Br.  FP32 accuracy comes from the 3xTF32
-// split x = hi + lo (hi = x rounded to TF32): A*B ~ Ahi*Bhi + Ahi*Blo + Alo*Bhi, accumulated
-// in FP32 in tensor memory.
+// becomes the 2x2 real block [[re, im], [-im, re]] of Br.  FP32 accuracy comes from a two-way split
+// of scaled operands: every row of Ar and every column of Br is scaled by a power of two that puts
+// its largest entry in [2^13, 2^14), and x = hi + lo with hi = fp16(x), lo = fp16(x - hi), 22
+// significant bits with round to nearest in both halves (entries more than 2^19 below the largest
+// one of their row lose trailing bits, 2^-39 of that largest entry and below).
+// A*B ~ Ahi*Bhi + Ahi*Blo + Alo*Bhi, accumulated in FP32 in tensor memory and scaled back in the
+// epilogue.  Against the TF32 split of the same depth the operands take half the bytes, the MMAs
+// run at twice the rate, and the lower half is rounded instead of truncated.
 //
 // Operands are first packed (and split) into tiles already laid out in the UMMA K-major
-// 128-byte-swizzled shared-memory format: A tiles of 128 rows x 32 floats (16 KB), B tiles of
-// 256 rows x 32 floats (32 KB).  A CTA computes one 128 x 256 tile of Cr: one thread streams the
+// 128-byte-swizzled shared-memory format: A tiles of 128 rows x 64 halves (16 KB), B tiles of
+// 256 rows x 64 halves (32 KB).  A CTA computes one 128 x BN tile of Cr: one thread streams the
 // tiles into shared memory with 1-D bulk copies (cp.async.bulk, completion on an mbarrier), one
-// thread issues tcgen05.mma into a 256-column TMEM accumulator, and four warps read the
+// thread issues tcgen05.mma into a BN-column TMEM accumulator, and eight warps read the
 // accumulator back with tcgen05.ld for the epilogue.  Every mbarrier wait is bounded; on time-out
 // the kernel records DS_WAIT_TIMEOUT and skips its output.  The kernel is persistent: one CTA per
 // SM walks a static round-robin list of all output tiles of all batch items, with two TMEM
@@ -25,21 +30,30 @@
 #include <atomic>
 #include <cstdlib>
 #include <mutex>
+#include <cuda_fp16.h>
 
 namespace rfdd {
 
 constexpr int TC_BM = 128;
 constexpr int TC_BN = 256;
-constexpr int TC_BK = 32;
-constexpr int TC_STAGES = 2;
-constexpr int A_TILE = TC_BM * TC_BK;  // floats
-constexpr int B_TILE = TC_BN * TC_BK;  // floats
-constexpr int STAGE_BYTES = (2 * A_TILE + 2 * B_TILE) * 4;  // 96 KB
+constexpr int TC_BK = 64;            // 16-bit values of K in a tile row (128 bytes)
+constexpr int TC_BK32 = 32;          // FP32 values of K in a tile row (plain TF32 probe)
+constexpr int ROW_B = 128;           // bytes of a tile row
+constexpr int A_TILE = TC_BM * ROW_B;  // bytes
+constexpr int B_TILE = TC_BN * ROW_B;  // bytes
+// ring of operand stages of the one-CTA kernel: 2 x 96 KB for 256-wide tiles, 4 x 48 KB for 64-wide
+template <int BN>
+struct TcRing {
+  static constexpr int STAGES = BN == 256 ? 2 : 4;
+  static constexpr int BYTES = 2 * A_TILE + 2 * BN * ROW_B;
+};
+constexpr int TC_RING_BYTES = 2 * (2 * A_TILE + 2 * B_TILE);
+static_assert(TcRing<64>::STAGES * TcRing<64>::BYTES == TC_RING_BYTES, "both rings fill the same shared memory");
 constexpr int EPI_WARPS = 8;  // two per TMEM lane quarter, each drains half of the columns
 constexpr int EPI_PITCH = 33;
 constexpr int EPI_BYTES = EPI_WARPS * 32 * EPI_PITCH * 4;
 constexpr int TC_THREADS = 64 + 32 * EPI_WARPS;  // producer warp, MMA warp, epilogue warps
-constexpr int TC_SMEM = TC_STAGES * STAGE_BYTES + EPI_BYTES + 1024;
+constexpr int TC_SMEM = TC_RING_BYTES + EPI_BYTES + 1024;
 constexpr long long WAIT_LIMIT = 1ll << 24;
 
 // Status word of the launches issued by the calling host thread (TcStatusScope): a kernel whose
@@ -56,7 +70,8 @@ TcKernelEvents::TcKernelEvents(const cudaEvent_t *ab) : prev(g_tc_events) { g_tc
 TcKernelEvents::~TcKernelEvents() { g_tc_events = prev; }
 
 struct TcItem {
-  const float *Ahi, *Alo, *Bhi, *Blo;
+  const uint8_t *Ahi, *Alo, *Bhi, *Blo;
+  const float *sA, *sB;  // scale of every packed row of A and of B (16-bit split)
   float *C;
   long long ldc;  // real leading dimension of C
   int m, n2, nkt, mtc, ntc, tile0;  // tile0: first global tile index of this item
@@ -82,7 +97,6 @@ struct TcBatchP {
   TcItem it[TC_MAXB];
   int count, total_tiles;
   int *err;    // status word of the launch (DS_WAIT_TIMEOUT on a wait that ran out)
-  int splits;  // 3: hi*hi + hi*lo + lo*hi (FP32 accuracy); 1: hi*hi only (plain TF32, peak probe)
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -133,6 +147,13 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t da, uint64_t 
       "l"(da), "l"(db), "r"(idesc), "r"(acc)
       : "memory");
 }
+__device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "l"(da), "l"(db), "r"(idesc), "r"(acc)
+      : "memory");
+}
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -159,51 +180,86 @@ __device__ __forceinline__ int find_item(const TcBatchP &b, int tile) {
   return lo;
 }
 
-// Epilogue of one output tile by one warp: TMEM lanes 32q..32q+31 (rows mt*128 + 32q ..), column
-// chunks of 32 accumulator columns [half*4, half*4 + 4), staged through shared memory so that C
-// is read and written along its rows; C = alpha * acc + beta * C, rows and columns masked.
-__device__ __forceinline__ void drain_tile(const TcItem &it, uint32_t tacc, int mt, int nt, int q, int half, int lane,
-                                           float *stg, float alpha, float beta) {
-  const int row0 = mt * TC_BM + q * 32;
-  const int nrows = min(32, it.m - row0);
-  float *__restrict__ Cb = it.C;
-#pragma unroll 1
-  for (int c = half * (TC_BN / 64); c < (half + 1) * (TC_BN / 64); ++c) {
-    uint32_t v[32];
-    TC_LD32(tacc + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32), v);
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// C entries of one 32 x 32 chunk of an output tile, lane = column: loaded ahead of the accumulator
+__device__ __forceinline__ void load_c(const TcItem &it, int row0, int nrows, int col, float beta, float (&cv)[32]) {
+  const bool on = col < it.n2 && beta != 0.f;
+  const float *p = it.C + (long long)row0 * it.ldc + col;
 #pragma unroll
-    for (int j = 0; j < 32; ++j) stg[lane * EPI_PITCH + j] = __uint_as_float(v[j]);
-    __syncwarp();
-    const int col = nt * TC_BN + c * 32 + lane;
-    if (col < it.n2 && nrows > 0) {
-      // all loads of C first (independent, in flight together), then the stores
-      float cv[32];
-#pragma unroll
-      for (int r = 0; r < 32; ++r)
-        cv[r] = (beta != 0.f && r < nrows) ? Cb[(long long)(row0 + r) * it.ldc + col] : 0.f;
-#pragma unroll
-      for (int r = 0; r < 32; ++r)
-        if (r < nrows) Cb[(long long)(row0 + r) * it.ldc + col] = fmaf(alpha, stg[r * EPI_PITCH + lane], beta * cv[r]);
-    }
-    __syncwarp();
+  for (int r = 0; r < 32; ++r) {
+    cv[r] = (on && r < nrows) ? *p : 0.f;
+    p += it.ldc;
   }
 }
 
+// Epilogue of one output tile by one warp: TMEM lanes 32q..32q+31 (rows mt*128 + 32q ..), NCH column
+// chunks of 32 accumulator columns from chunk c0 on, staged through shared memory so that C is read
+// and written along its rows; C = alpha * scaled acc + beta * C, rows and columns masked.  cv holds
+// the first chunk's C (loaded before the accumulator was ready); the C of the next chunk is in
+// flight while a chunk is written, and `done` runs once the accumulator has been read.
+template <int NCH, bool SCALED, typename F>
+__device__ __forceinline__ void drain_tile(const TcItem &it, uint32_t tacc, int mt, int col0, int q, int c0, int lane,
+                                           float *stg, float alpha, float beta, float (&cv)[32], F &&done) {
+  const int row0 = mt * TC_BM + q * 32;
+  const int nrows = min(32, it.m - row0);
+  // scale of this lane's row (read along the rows below)
+  const float ra = SCALED ? (lane < nrows ? it.sA[row0 + lane] : 1.f) : 1.f;
+#pragma unroll
+  for (int ci = 0; ci < NCH; ++ci) {
+    const int c = c0 + ci;
+    uint32_t v[32];
+    TC_LD32(tacc + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32), v);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    if (ci == NCH - 1) done();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) stg[lane * EPI_PITCH + j] = __uint_as_float(v[j]);
+    __syncwarp();
+    const int col = col0 + c * 32 + lane;
+    float cn[32];
+    if (ci + 1 < NCH) load_c(it, row0, nrows, col + 32, beta, cn);
+    const bool on = col < it.n2;
+    const float rb = SCALED ? (on ? it.sB[col] : 1.f) : 1.f;
+    float *p = it.C + (long long)row0 * it.ldc + col;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+      // the two scales are powers of two: their product first, so that neither over- or underflows alone
+      const float f = SCALED ? alpha * (__shfl_sync(0xffffffffu, ra, r) * rb) : alpha;
+      if (on && r < nrows) *p = fmaf(f, stg[r * EPI_PITCH + lane], beta * cv[r]);
+      p += it.ldc;
+    }
+    __syncwarp();
+    if (ci + 1 < NCH) {
+#pragma unroll
+      for (int r = 0; r < 32; ++r) cv[r] = cn[r];
+    }
+  }
+}
+
+// Real columns of a tile that the MMAs compute: those of C, in steps of 16 (the MMA's N)
+template <int BN>
+__device__ __forceinline__ int tile_cols(const TcItem &it, int nt) {
+  return min(BN, (it.n2 - nt * BN + 15) & ~15);
+}
+
 // Persistent, warp-specialised: warp 0 streams operand tiles, warp 1 issues the MMAs into one of
-// two TMEM accumulators (256 columns each), warps 2..5 drain the other accumulator to C.
+// two TMEM accumulators (BN columns each), warps 2..9 drain the other accumulator to C.
+// F16: the scaled 16-bit split, three products; otherwise plain TF32 (peak probe).
+// BN = 64 takes a quarter of a packed B tile per output tile, for launches that have too few 256-wide
+// tiles to fill the chip or whose C has at most 64 real columns.
+template <bool F16, int BN>
 __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_constant__ TcBatchP b, float alpha,
                                                                 float beta) {
+  constexpr int STAGES = TcRing<BN>::STAGES, STAGE_BYTES = TcRing<BN>::BYTES;
+  constexpr int SUB = TC_BN / BN;  // output tiles per packed B tile
   int *err = b.err;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  float *epi = reinterpret_cast<float *>(base + TC_STAGES * STAGE_BYTES);
-  __shared__ __align__(8) uint64_t full_bar[TC_STAGES], empty_bar[TC_STAGES], tfull_bar[2], tempty_bar[2];
+  float *epi = reinterpret_cast<float *>(base + TC_RING_BYTES);
+  __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], tfull_bar[2], tempty_bar[2];
   __shared__ uint32_t tmem_s;
   __shared__ volatile int abort_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < TC_STAGES; ++s) {
+    for (int s = 0; s < STAGES; ++s) {
       mbar_init(smem_u32(&full_bar[s]), 1);
       mbar_init(smem_u32(&empty_bar[s]), 1);
     }
@@ -217,7 +273,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)),
-                 "r"(2 * TC_BN)
+                 "r"(2 * BN)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -227,8 +283,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
   const uint32_t tmem = tmem_s;
   auto stage_addr = [&](int s, int which) -> uint32_t {  // which: 0 Ahi, 1 Alo, 2 Bhi, 3 Blo
     const uint32_t off = (uint32_t)s * STAGE_BYTES +
-                         (which == 0 ? 0u : which == 1 ? A_TILE * 4u : which == 2 ? 2u * A_TILE * 4u
-                                                                                  : 2u * A_TILE * 4u + B_TILE * 4u);
+                         (which == 0 ? 0u : which == 1 ? (uint32_t)A_TILE : which == 2 ? 2u * A_TILE
+                                                                                       : 2u * A_TILE + BN * ROW_B);
     return smem_u32(base + off);
   };
   if (warp == 0) {
@@ -240,38 +296,42 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
         int mt, nt;
         tile_pos(it, local, mt, nt);
         const long long ams = it.amts ? it.amts : it.nkt;
-        const float *Ahi = it.Ahi + (long long)mt * ams * A_TILE, *Alo = it.Alo + (long long)mt * ams * A_TILE;
-        const float *Bhi = it.Bhi + (long long)nt * it.nkt * B_TILE, *Blo = it.Blo + (long long)nt * it.nkt * B_TILE;
+        const uint8_t *Ahi = it.Ahi + (long long)mt * ams * A_TILE, *Alo = it.Alo + (long long)mt * ams * A_TILE;
+        const long long bo = (long long)(nt / SUB) * it.nkt * B_TILE + (nt % SUB) * (BN * ROW_B);
+        const uint8_t *Bhi = it.Bhi + bo, *Blo = it.Blo + bo;
+        const uint32_t nb = (uint32_t)tile_cols<BN>(it, nt) * ROW_B;
         for (int kt = 0; kt < it.nkt; ++kt, ++g) {
-          const int s = (int)(g % TC_STAGES);
-          const long long u = g / TC_STAGES;
+          const int s = (int)(g % STAGES);
+          const long long u = g / STAGES;
           if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[s]), (uint32_t)((u - 1) & 1), &abort_s)) {
             atomicOr(err, DS_WAIT_TIMEOUT);
             abort_s = 1;
             break;
           }
           const uint32_t fb = smem_u32(&full_bar[s]);
-          mbar_expect_tx(fb, b.splits > 1 ? STAGE_BYTES : (A_TILE + B_TILE) * 4);
-          bulk_g2s(stage_addr(s, 0), Ahi + (long long)kt * A_TILE, A_TILE * 4, fb);
-          bulk_g2s(stage_addr(s, 2), Bhi + (long long)kt * B_TILE, B_TILE * 4, fb);
-          if (b.splits > 1) {
-            bulk_g2s(stage_addr(s, 1), Alo + (long long)kt * A_TILE, A_TILE * 4, fb);
-            bulk_g2s(stage_addr(s, 3), Blo + (long long)kt * B_TILE, B_TILE * 4, fb);
+          mbar_expect_tx(fb, (F16 ? 2 : 1) * (A_TILE + nb));
+          bulk_g2s(stage_addr(s, 0), Ahi + (long long)kt * A_TILE, A_TILE, fb);
+          bulk_g2s(stage_addr(s, 2), Bhi + (long long)kt * B_TILE, nb, fb);
+          if (F16) {
+            bulk_g2s(stage_addr(s, 1), Alo + (long long)kt * A_TILE, A_TILE, fb);
+            bulk_g2s(stage_addr(s, 3), Blo + (long long)kt * B_TILE, nb, fb);
           }
         }
       }
       // drain: every issued copy must land before the CTA can exit
-      for (long long q = (g > TC_STAGES ? g - TC_STAGES : 0); q < g; ++q)
-        mbar_wait(smem_u32(&full_bar[q % TC_STAGES]), (uint32_t)((q / TC_STAGES) & 1), &abort_s);
+      for (long long q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
+        mbar_wait(smem_u32(&full_bar[q % STAGES]), (uint32_t)((q / STAGES) & 1), &abort_s);
     }
   } else if (warp == 1) {
     if (lane == 0) {  // MMA issuer
-      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_BN >> 3) << 17) |
-                             ((uint32_t)(TC_BM >> 4) << 24);
+      const uint32_t idesc0 = (1u << 4) | (F16 ? 0u : (2u << 7) | (2u << 10)) | ((uint32_t)(TC_BM >> 4) << 24);
       long long g = 0;
       int lt = 0;
       for (int tile = blockIdx.x; tile < b.total_tiles && !abort_s; tile += gridDim.x, ++lt) {
         const TcItem &it = b.it[find_item(b, tile)];
+        int mt, nt;
+        tile_pos(it, tile - it.tile0, mt, nt);
+        const uint32_t idesc = idesc0 | ((uint32_t)(tile_cols<BN>(it, nt) >> 3) << 17);
         const int acc = lt & 1;
         if (lt >= 2 && !mbar_wait(smem_u32(&tempty_bar[acc]), (uint32_t)(((lt >> 1) - 1) & 1), &abort_s)) {
           atomicOr(err, DS_WAIT_TIMEOUT);
@@ -279,11 +339,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
           break;
         }
         fence_after();
-        const uint32_t dacc = tmem + (uint32_t)(acc * TC_BN);
+        const uint32_t dacc = tmem + (uint32_t)(acc * BN);
         bool ok = true;
         for (int kt = 0; kt < it.nkt; ++kt, ++g) {
-          const int s = (int)(g % TC_STAGES);
-          if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)((g / TC_STAGES) & 1), &abort_s)) {
+          const int s = (int)(g % STAGES);
+          if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)((g / STAGES) & 1), &abort_s)) {
             atomicOr(err, DS_WAIT_TIMEOUT);
             abort_s = 1;
             ok = false;
@@ -292,12 +352,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
           fence_after();
           const uint32_t ah = stage_addr(s, 0), al = stage_addr(s, 1), bh = stage_addr(s, 2), bl = stage_addr(s, 3);
 #pragma unroll
-          for (int kk = 0; kk < TC_BK / 8; ++kk) {
-            const uint32_t o = kk * 32;  // 8 TF32 values = 32 bytes along K inside the swizzle row
-            mma_tf32(dacc, sdesc(ah + o), sdesc(bh + o), idesc, (kt > 0 || kk > 0) ? 1u : 0u);
-            if (b.splits > 1) {
-              mma_tf32(dacc, sdesc(ah + o), sdesc(bl + o), idesc, 1u);
-              mma_tf32(dacc, sdesc(al + o), sdesc(bh + o), idesc, 1u);
+          for (int kk = 0; kk < ROW_B / 32; ++kk) {
+            const uint32_t o = kk * 32;  // 16 16-bit (8 TF32) values = 32 bytes along K inside the swizzle row
+            if (F16) {
+              mma_f16(dacc, sdesc(ah + o), sdesc(bh + o), idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+              mma_f16(dacc, sdesc(ah + o), sdesc(bl + o), idesc, 1u);
+              mma_f16(dacc, sdesc(al + o), sdesc(bh + o), idesc, 1u);
+            } else {
+              mma_tf32(dacc, sdesc(ah + o), sdesc(bh + o), idesc, (kt > 0 || kk > 0) ? 1u : 0u);
             }
           }
           mma_commit(smem_u32(&empty_bar[s]));
@@ -308,9 +370,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
     }
   } else {
     // epilogue warps: warp w reads accumulator lanes 32*(w % 4) .. +31 (its TMEM sub-partition);
-    // warps 2..5 take column chunks 0..3, warps 6..9 chunks 4..7
+    // warps 2..5 take the first half of the column chunks, warps 6..9 the second
+    constexpr int NCH = BN / 64;
     const int q = warp & 3;
-    const int half = (warp - 2) >> 2;
+    const int c0 = ((warp - 2) >> 2) * NCH;
     float *stg = epi + (warp - 2) * 32 * EPI_PITCH;
     int lt = 0;
     for (int tile = blockIdx.x; tile < b.total_tiles; tile += gridDim.x, ++lt) {
@@ -319,6 +382,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
       int mt, nt;
       tile_pos(it, local, mt, nt);
       const int acc = lt & 1;
+      const int row0 = mt * TC_BM + q * 32;
+      float cv[32];
+      load_c(it, row0, min(32, it.m - row0), nt * BN + c0 * 32 + lane, beta, cv);
       const bool ready = mbar_wait(smem_u32(&tfull_bar[acc]), (uint32_t)((lt >> 1) & 1), &abort_s);
       // the whole warp takes the same branch (tcgen05.ld below is a warp-collective)
       if (!__all_sync(0xffffffffu, ready && !abort_s)) {
@@ -327,16 +393,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
         break;
       }
       fence_after();
-      drain_tile(it, tmem + (uint32_t)(acc * TC_BN), mt, nt, q, half, lane, stg, alpha, beta);
-      fence_before();
-      mbar_arrive(smem_u32(&tempty_bar[acc]));
+      drain_tile<NCH, F16>(it, tmem + (uint32_t)(acc * BN), mt, nt * BN, q, c0, lane, stg, alpha, beta, cv, [&] {
+        fence_before();
+        mbar_arrive(smem_u32(&tempty_bar[acc]));
+      });
     }
   }
   fence_before();
   __syncthreads();
   fence_after();
   if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * TC_BN) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
   }
 }
 
@@ -345,7 +412,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
 // Cr with one MMA stream.  Each CTA holds its own 128 rows of A and its half (128 packed rows) of
 // the B tile in shared memory; the MMAs, issued by the leader CTA (rank 0), read A and B from both
 // CTAs and leave rows 0..127 of the accumulator in the leader's TMEM and rows 128..255 in the
-// peer's.  Per 32-deep K tile an SM so takes in 64 KB instead of the 96 KB of the one-CTA kernel
+// peer's.  Per 64-deep K tile an SM so takes in 64 KB instead of the 96 KB of the one-CTA kernel
 // (whose 128 x 256 tile needs all of B), which is what limits that kernel (operand feed, not the
 // tensor pipe).
 //
@@ -357,8 +424,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
 //  - every epilogue warp of both CTAs drains its TMEM lanes and arrives on the leader's tempty_bar.
 // ---------------------------------------------------------------------------------------
 constexpr int T2_STAGES = 3;
-constexpr int T2_BHALF = (TC_BN / 2) * TC_BK;                       // floats of one CTA's B half
-constexpr int T2_STAGE_BYTES = (2 * A_TILE + 2 * T2_BHALF) * 4;     // 64 KB
+constexpr int T2_BHALF = B_TILE / 2;                         // bytes of one CTA's B half
+constexpr int T2_STAGE_BYTES = 2 * A_TILE + 2 * T2_BHALF;    // 64 KB
 constexpr int T2_SMEM = T2_STAGES * T2_STAGE_BYTES + EPI_BYTES + 1024;
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -392,10 +459,10 @@ __device__ __forceinline__ bool mbar_wait_cl(uint32_t bar, uint32_t parity, vola
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void mma2_tf32(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma2_f16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
       "l"(da), "l"(db), "r"(idesc), "r"(acc)
       : "memory");
 }
@@ -458,8 +525,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
   const uint32_t tmem = tmem_s;
   auto stage_addr = [&](int s, int which) -> uint32_t {  // which: 0 Ahi, 1 Alo, 2 Bhi half, 3 Blo half
     const uint32_t off = (uint32_t)s * T2_STAGE_BYTES +
-                         (which == 0 ? 0u : which == 1 ? A_TILE * 4u : which == 2 ? 2u * A_TILE * 4u
-                                                                                  : 2u * A_TILE * 4u + T2_BHALF * 4u);
+                         (which == 0 ? 0u : which == 1 ? (uint32_t)A_TILE : which == 2 ? 2u * A_TILE
+                                                                                       : 2u * A_TILE + T2_BHALF);
     return smem_u32(base + off);
   };
   if (warp == 0) {
@@ -471,9 +538,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
         pair_pos(it, pt - it.tile0, mp, nt);
         const int mt = min(2 * mp + (int)rank, it.mtc - 1);  // a missing second row re-reads the last one
         const long long ams = it.amts ? it.amts : it.nkt;
-        const float *Ahi = it.Ahi + (long long)mt * ams * A_TILE, *Alo = it.Alo + (long long)mt * ams * A_TILE;
+        const uint8_t *Ahi = it.Ahi + (long long)mt * ams * A_TILE, *Alo = it.Alo + (long long)mt * ams * A_TILE;
         const long long boff = (long long)nt * it.nkt * B_TILE + (long long)rank * T2_BHALF;
-        const float *Bhi = it.Bhi + boff, *Blo = it.Blo + boff;
+        const uint8_t *Bhi = it.Bhi + boff, *Blo = it.Blo + boff;
         for (int kt = 0; kt < it.nkt; ++kt, ++g) {
           const int s = (int)(g % T2_STAGES);
           const long long u = g / T2_STAGES;
@@ -484,10 +551,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
           }
           const uint32_t fb = smem_u32(&full_bar[s]);
           mbar_expect_tx(fb, T2_STAGE_BYTES);
-          bulk_g2s(stage_addr(s, 0), Ahi + (long long)kt * A_TILE, A_TILE * 4, fb);
-          bulk_g2s(stage_addr(s, 1), Alo + (long long)kt * A_TILE, A_TILE * 4, fb);
-          bulk_g2s(stage_addr(s, 2), Bhi + (long long)kt * B_TILE, T2_BHALF * 4, fb);
-          bulk_g2s(stage_addr(s, 3), Blo + (long long)kt * B_TILE, T2_BHALF * 4, fb);
+          bulk_g2s(stage_addr(s, 0), Ahi + (long long)kt * A_TILE, A_TILE, fb);
+          bulk_g2s(stage_addr(s, 1), Alo + (long long)kt * A_TILE, A_TILE, fb);
+          bulk_g2s(stage_addr(s, 2), Bhi + (long long)kt * B_TILE, T2_BHALF, fb);
+          bulk_g2s(stage_addr(s, 3), Blo + (long long)kt * B_TILE, T2_BHALF, fb);
         }
       }
       // every issued copy lands, and every stage's last consumption is signalled here (the leader's
@@ -516,7 +583,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
         if (!ok) break;
       }
     } else if (lane == 0 && rank == 0) {  // leader: MMA issuer for the pair
-      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_BN >> 3) << 17) |
+      const uint32_t idesc = (1u << 4) | ((uint32_t)(TC_BN >> 3) << 17) |
                              ((uint32_t)((2 * TC_BM) >> 4) << 24);
       long long g = 0;
       int lt = 0;
@@ -544,11 +611,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
           fence_after();
           const uint32_t ah = stage_addr(s, 0), al = stage_addr(s, 1), bh = stage_addr(s, 2), bl = stage_addr(s, 3);
 #pragma unroll
-          for (int kk = 0; kk < TC_BK / 8; ++kk) {
+          for (int kk = 0; kk < ROW_B / 32; ++kk) {
             const uint32_t o = kk * 32;
-            mma2_tf32(dacc, sdesc(ah + o), sdesc(bh + o), idesc, (kt > 0 || kk > 0) ? 1u : 0u);
-            mma2_tf32(dacc, sdesc(ah + o), sdesc(bl + o), idesc, 1u);
-            mma2_tf32(dacc, sdesc(al + o), sdesc(bh + o), idesc, 1u);
+            mma2_f16(dacc, sdesc(ah + o), sdesc(bh + o), idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+            mma2_f16(dacc, sdesc(ah + o), sdesc(bl + o), idesc, 1u);
+            mma2_f16(dacc, sdesc(al + o), sdesc(bh + o), idesc, 1u);
           }
           mma2_commit_both(smem_u32(&empty_bar[s]));
         }
@@ -559,7 +626,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
   } else {
     // epilogue warps of both CTAs: this CTA's 128 accumulator rows of the pair tile
     const int q = warp & 3;
-    const int half = (warp - 2) >> 2;
+    constexpr int NCH = TC_BN / 64;
+    const int c0 = ((warp - 2) >> 2) * NCH;
     float *stg = epi + (warp - 2) * 32 * EPI_PITCH;
     const uint32_t tempty_leader0 = map_to_rank(smem_u32(&tempty_bar[0]), 0);
     const uint32_t tempty_leader1 = map_to_rank(smem_u32(&tempty_bar[1]), 0);
@@ -570,6 +638,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
       pair_pos(it, pt - it.tile0, mp, nt);
       const int mt = 2 * mp + (int)rank;  // rows beyond m (a missing second row) are masked
       const int acc = lt & 1;
+      const int row0 = mt * TC_BM + q * 32;
+      float cv[32];
+      load_c(it, row0, min(32, it.m - row0), nt * TC_BN + c0 * 32 + lane, beta, cv);
       const bool ready = mbar_wait_cl(smem_u32(&tfull_bar[acc]), (uint32_t)((lt >> 1) & 1), &abort_s);
       if (!__all_sync(0xffffffffu, ready && !abort_s)) {
         if (lane == 0) atomicOr(err, DS_WAIT_TIMEOUT);
@@ -577,10 +648,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
         break;
       }
       fence_after();
-      drain_tile(it, tmem + (uint32_t)(acc * TC_BN), mt, nt, q, half, lane, stg, alpha, beta);
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
+      drain_tile<NCH, true>(it, tmem + (uint32_t)(acc * TC_BN), mt, nt * TC_BN, q, c0, lane, stg, alpha, beta, cv, [&] {
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
+      });
     }
   }
   fence_before();
@@ -605,7 +677,7 @@ __global__ void __launch_bounds__(128, 1) tf32_mma_probe_kernel(int iters, int *
   __shared__ volatile int abort_s;
   const int warp = threadIdx.x >> 5;
   // operand tiles: zeros (the rate does not depend on the values)
-  for (int i = threadIdx.x; i < (A_TILE + B_TILE); i += blockDim.x) reinterpret_cast<float *>(base)[i] = 0.f;
+  for (int i = threadIdx.x; i < (A_TILE + B_TILE) / 4; i += blockDim.x) reinterpret_cast<float *>(base)[i] = 0.f;
   if (threadIdx.x == 0) {
     mbar_init(smem_u32(&done_bar), 1);
     abort_s = 0;
@@ -625,10 +697,10 @@ __global__ void __launch_bounds__(128, 1) tf32_mma_probe_kernel(int iters, int *
   if (threadIdx.x == 0) {
     const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_BN >> 3) << 17) |
                            ((uint32_t)(TC_BM >> 4) << 24);
-    const uint32_t a = smem_u32(base), b = smem_u32(base + A_TILE * 4);
+    const uint32_t a = smem_u32(base), b = smem_u32(base + A_TILE);
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
-      for (int kk = 0; kk < TC_BK / 8; ++kk)
+      for (int kk = 0; kk < ROW_B / 32; ++kk)
         mma_tf32(tmem, sdesc(a + kk * 32), sdesc(b + kk * 32), idesc, (it > 0 || kk > 0) ? 1u : 0u);
     }
     mma_commit(smem_u32(&done_bar));
@@ -646,7 +718,7 @@ double tc_mma_probe_tflops(cudaStream_t st, int *dev_status) {
   int dev = 0, nsm = 0;
   RFDD_CUDA(cudaGetDevice(&dev));
   RFDD_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const int smem = (A_TILE + B_TILE) * 4 + 1024;
+  const int smem = A_TILE + B_TILE + 1024;
   RFDD_CUDA(cudaFuncSetAttribute(tf32_mma_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   cudaEvent_t e0, e1;
   RFDD_CUDA(cudaEventCreate(&e0));
@@ -661,7 +733,7 @@ double tc_mma_probe_tflops(cudaStream_t st, int *dev_status) {
     RFDD_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;
     RFDD_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-    const double fl = 2.0 * TC_BM * TC_BN * 8.0 * (TC_BK / 8) * (double)iters * nsm;
+    const double fl = 2.0 * TC_BM * TC_BN * 8.0 * (TC_BK32 / 8) * (double)iters * nsm;
     if (rep > 0 && ms > 0.f) best = std::max(best, fl / (ms * 1e-3) / 1e12);
   }
   cudaEventDestroy(e0);
@@ -670,7 +742,232 @@ double tc_mma_probe_tflops(cudaStream_t st, int *dev_status) {
 }
 
 // ---------------------------------------------------------------------------------------
-// packing: split into TF32 hi/lo and write swizzled tiles
+// packing: scale, split into 16-bit halves and write swizzled tiles
+// ---------------------------------------------------------------------------------------
+// Power of two that brings a row whose largest magnitude is m into [2^13, 2^14), and its inverse.
+// 0, infinities and NaN: 1.  Below 2^-113 the factor stays at 2^126 (its inverse is still normal).
+__device__ __forceinline__ void row_scale(float m, float &mul, float &inv) {
+  const int ex = (int)(__float_as_uint(m) >> 23) & 255;
+  const int f = (m == 0.f || ex == 255) ? 127 : min(267 - ex, 253);
+  mul = __uint_as_float((uint32_t)f << 23);
+  inv = __uint_as_float((uint32_t)(254 - f) << 23);
+}
+// x = hi + lo, both rounded to nearest
+__device__ __forceinline__ void split_f16(float x, uint16_t &hi, uint16_t &lo) {
+  const __half h = __float2half_rn(x);
+  hi = __half_as_ushort(h);
+  lo = __half_as_ushort(__float2half_rn(x - __half2float(h)));
+}
+__device__ __forceinline__ uint32_t pair16(uint16_t a, uint16_t b) { return (uint32_t)a | ((uint32_t)b << 16); }
+
+struct PackItem {
+  const float *src;   // interleaved complex source (as floats), or real
+  long long ld;       // leading dimension in elements of the source
+  int rows, k;        // A: rows x k; B: k x rows (elements)
+  uint8_t *hi, *lo;   // tile buffers
+  float *scale;       // inverse scale of every packed row (A: padded rows; B: 64-row blocks)
+  int nblk;           // A: 128-row tiles; B: blocks of 64 packed rows
+  int nkt;
+  int side;           // A: > 0: columns left of the diagonal block of `side` rows have a scale of their own,
+                      // the others' scales follow at scale + nblk * 128 (L and U of one factor)
+};
+struct PackBatchP {
+  PackItem a[TC_MAXB], b[TC_MAXB];
+  int na, nb;
+};
+
+// A tiles: [mt][kt] 128 rows x 64 halves; 16-byte chunk c of row r stored at chunk c ^ (r & 7).  One warp per
+// row: its largest magnitude first, then the split (the second read of the row comes from L1 / L2).
+template <bool CPLX>
+__device__ __forceinline__ void pack_a_rows(const PackItem &it) {
+  constexpr int F = CPLX ? 2 : 1;
+  const int lane = threadIdx.x & 31, kf = F * it.k, nq = it.nkt * 8, rows_pad = it.nblk * TC_BM;
+  for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows_pad; row += gridDim.x * 8) {
+    const float *src = it.src + (long long)row * F * it.ld;
+    const bool live = row < it.rows;
+    auto load8 = [&](int q, float (&x)[8]) {
+      const int k0 = q * 8;
+      if (CPLX) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const float2 v = (live && k0 + 2 * t < kf) ? *reinterpret_cast<const float2 *>(src + k0 + 2 * t)
+                                                      : make_float2(0.f, 0.f);
+          x[2 * t] = v.x;
+          x[2 * t + 1] = v.y;
+        }
+      } else {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = (live && k0 + t < kf) ? src[k0 + t] : 0.f;
+      }
+    };
+    // chunks left of the row's diagonal block (a multiple of eight values per block)
+    const int ql = it.side > 0 ? (row / it.side) * it.side * F / 8 : 0;
+    float ml = 0.f, mr = 0.f;
+    for (int q = lane; q < nq; q += 32) {
+      float x[8];
+      load8(q, x);
+      float m = 0.f;
+#pragma unroll
+      for (int t = 0; t < 8; ++t) m = fmaxf(m, fabsf(x[t]));
+      if (q < ql) ml = fmaxf(ml, m);
+      else mr = fmaxf(mr, m);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      ml = fmaxf(ml, __shfl_xor_sync(0xffffffffu, ml, o));
+      mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
+    }
+    float fl, il, fr, ir;
+    row_scale(ml, fl, il);
+    row_scale(mr, fr, ir);
+    if (lane == 0) {
+      if (it.side > 0) {
+        it.scale[row] = il;
+        it.scale[rows_pad + row] = ir;
+      } else {
+        it.scale[row] = ir;
+      }
+    }
+    const int mt = row / TC_BM, r = row % TC_BM;
+    for (int q = lane; q < nq; q += 32) {
+      float x[8];
+      load8(q, x);
+      const float f = q < ql ? fl : fr;
+      uint16_t h[8], l[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) split_f16(x[t] * f, h[t], l[t]);
+      const long long off = ((long long)mt * it.nkt + (q >> 3)) * A_TILE + r * ROW_B + (((q & 7) ^ (r & 7)) << 4);
+      *reinterpret_cast<uint4 *>(it.hi + off) = make_uint4(pair16(h[0], h[1]), pair16(h[2], h[3]), pair16(h[4], h[5]), pair16(h[6], h[7]));
+      *reinterpret_cast<uint4 *>(it.lo + off) = make_uint4(pair16(l[0], l[1]), pair16(l[2], l[3]), pair16(l[4], l[5]), pair16(l[6], l[7]));
+    }
+  }
+}
+
+// B tiles: the rows of Br^T.  Complex: rows n' = 2j + t (t: 0 real part column, 1 imaginary), K index k' = 2p + u:
+//   Br^T[2j][2p] = re B[p][j], Br^T[2j][2p+1] = -im B[p][j], Br^T[2j+1][2p] = im, Br^T[2j+1][2p+1] = re.
+// A block owns 64 packed rows (32 complex or 64 real columns of B): it stages up to PACK_KC rows of B
+// in shared memory with reads along B's rows, takes the largest magnitude of every column, and writes
+// the packed rows with coalesced 16-byte stores.  Deeper B is staged twice, chunk by chunk.
+constexpr int PACK_KC = 256;
+template <bool CPLX>
+__device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
+  constexpr int F = CPLX ? 2 : 1;
+  constexpr int CW = 64 / F;            // columns of B per block
+  constexpr int PITCH = CPLX ? 66 : 65;  // floats per staged row
+  __shared__ float smax[8][64];
+  __shared__ float mul_s[64];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nch = (it.k + PACK_KC - 1) / PACK_KC;
+  for (int jb = blockIdx.x; jb < it.nblk; jb += gridDim.x) {
+    const long long j0 = (long long)jb * CW;
+    auto stage = [&](int p0, int pn, float &m0, float &m1) {
+      if (CPLX) {
+        const bool on = j0 + lane < it.rows;
+#pragma unroll 8
+        for (int p = warp; p < pn; p += 8) {
+          const float2 v = on ? *reinterpret_cast<const float2 *>(it.src + 2 * ((long long)(p0 + p) * it.ld + j0 + lane))
+                              : make_float2(0.f, 0.f);
+          *reinterpret_cast<float2 *>(sb + p * PITCH + 2 * lane) = v;
+          m0 = fmaxf(m0, fmaxf(fabsf(v.x), fabsf(v.y)));
+        }
+      } else {
+        const bool on0 = j0 + lane < it.rows, on1 = j0 + lane + 32 < it.rows;
+#pragma unroll 4
+        for (int p = warp; p < pn; p += 8) {
+          const float *r = it.src + (long long)(p0 + p) * it.ld + j0 + lane;
+          const float v0 = on0 ? r[0] : 0.f, v1 = on1 ? r[32] : 0.f;
+          sb[p * PITCH + lane] = v0;
+          sb[p * PITCH + lane + 32] = v1;
+          m0 = fmaxf(m0, fabsf(v0));
+          m1 = fmaxf(m1, fabsf(v1));
+        }
+      }
+    };
+    float m0 = 0.f, m1 = 0.f;
+    for (int ch = 0; ch < nch; ++ch) {
+      __syncthreads();
+      stage(ch * PACK_KC, min(PACK_KC, it.k - ch * PACK_KC), m0, m1);
+    }
+    smax[warp][lane] = m0;
+    if (!CPLX) smax[warp][lane + 32] = m1;
+    __syncthreads();
+    if (tid < 64) {
+      const int c = CPLX ? tid >> 1 : tid;
+      float m = smax[0][c];
+#pragma unroll
+      for (int w = 1; w < 8; ++w) m = fmaxf(m, smax[w][c]);
+      float mul, inv;
+      row_scale(m, mul, inv);
+      mul_s[tid] = mul;
+      it.scale[(long long)jb * 64 + tid] = inv;
+    }
+    __syncthreads();
+    for (int ch = 0; ch < nch; ++ch) {
+      const int p0 = ch * PACK_KC, pn = min(PACK_KC, it.k - p0);
+      if (nch > 1) {
+        __syncthreads();
+        stage(p0, pn, m0, m1);
+        __syncthreads();
+      }
+      const int kt0 = p0 * F / TC_BK, tiles = (pn * F + TC_BK - 1) / TC_BK;
+      for (int id = tid; id < tiles * 512; id += 256) {
+        const int c = id & 7, rl = (id >> 3) & 63, kt = id >> 9;
+        const float mul = mul_s[rl];
+        uint16_t h[8], l[8];
+        if (CPLX) {
+          const int t = rl & 1;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int p = kt * 32 + c * 4 + e;
+            const float2 v = p < pn ? *reinterpret_cast<const float2 *>(sb + p * PITCH + (rl & ~1))
+                                    : make_float2(0.f, 0.f);
+            split_f16((t == 0 ? v.x : v.y) * mul, h[2 * e], l[2 * e]);           // coefficient of Re A
+            split_f16((t == 0 ? -v.y : v.x) * mul, h[2 * e + 1], l[2 * e + 1]);  // coefficient of Im A
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const int p = kt * 64 + c * 8 + e;
+            split_f16((p < pn ? sb[p * PITCH + rl] : 0.f) * mul, h[e], l[e]);
+          }
+        }
+        const long long row = (long long)jb * 64 + rl;
+        const int nt = (int)(row / TC_BN), r = (int)(row % TC_BN);
+        const long long off = ((long long)nt * it.nkt + kt0 + kt) * B_TILE + r * ROW_B + ((c ^ (r & 7)) << 4);
+        *reinterpret_cast<uint4 *>(it.hi + off) = make_uint4(pair16(h[0], h[1]), pair16(h[2], h[3]), pair16(h[4], h[5]), pair16(h[6], h[7]));
+        *reinterpret_cast<uint4 *>(it.lo + off) = make_uint4(pair16(l[0], l[1]), pair16(l[2], l[3]), pair16(l[4], l[5]), pair16(l[6], l[7]));
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Both operands of every item in one launch (blockIdx.y: the A operands, then the B operands); zero, when
+// given, is a status word cleared for the GEMM that follows.
+template <bool CPLX>
+__global__ void __launch_bounds__(256) pack_f16_kernel(const __grid_constant__ PackBatchP pb, int *zero) {
+  extern __shared__ float pack_sb[];
+  if (zero && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero = 0;
+  if ((int)blockIdx.y < pb.na) pack_a_rows<CPLX>(pb.a[blockIdx.y]);
+  else pack_b_rows<CPLX>(pb.b[blockIdx.y - pb.na], pack_sb);
+}
+
+template <bool CPLX>
+static void launch_pack(cudaStream_t st, const PackBatchP &pb, int *zero = nullptr) {
+  if (pb.na + pb.nb == 0) return;
+  long long blocks = 1;
+  int kmax = 0;
+  for (int i = 0; i < pb.na; ++i) blocks = std::max(blocks, (long long)pb.a[i].nblk * (TC_BM / 8));
+  for (int i = 0; i < pb.nb; ++i) {
+    blocks = std::max(blocks, (long long)pb.b[i].nblk);
+    kmax = std::max(kmax, std::min(pb.b[i].k, PACK_KC));
+  }
+  const size_t smem = (size_t)kmax * (CPLX ? 66 : 65) * sizeof(float);
+  pack_f16_kernel<CPLX><<<dim3((unsigned)std::min<long long>(blocks, 2048), pb.na + pb.nb), 256, smem, st>>>(pb, zero);
+  RFDD_CHECK_LAUNCH();
+}
+
+// ---------------------------------------------------------------------------------------
+// operands of the plain TF32 probe: real, rounded to TF32, tiles of 32 floats of K (hi only is used)
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ void split_tf32(float x, float &hi, float &lo) {
   uint32_t r;
@@ -678,133 +975,27 @@ __device__ __forceinline__ void split_tf32(float x, float &hi, float &lo) {
   hi = __uint_as_float(r);
   lo = x - hi;
 }
-
-struct PackItem {
-  const float *src;   // interleaved complex source (as floats)
-  long long ld;       // complex leading dimension
-  int m, n, k;        // A: m x k ; B: k x n (complex)
-  float *hi, *lo;     // tile buffers
+struct Tf32PackItem {
+  const float *src;
+  long long ld;
+  int m, n, k;
+  float *hi, *lo;
   int mtc, ntc, nkt;
 };
-struct PackBatchP {
-  PackItem it[TC_MAXB];
+struct Tf32PackP {
+  Tf32PackItem it;
 };
-
-// A tiles: [mt][kt] 128 rows x 32 floats; float4 chunk c of row r stored at chunk c ^ (r & 7)
-__global__ void pack_a_kernel(PackBatchP pb) {
-  const PackItem it = pb.it[blockIdx.y];
-  const long long chunks = (long long)it.mtc * TC_BM * it.nkt * 8;
-  const int k2 = 2 * it.k;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < chunks; e += (long long)gridDim.x * blockDim.x) {
-    const long long row = e / (it.nkt * 8);
-    const int q = (int)(e % (it.nkt * 8));
-    const int kt = q >> 3, c = q & 7;
-    const int mt = (int)(row / TC_BM), r = (int)(row % TC_BM);
-    float h[4], l[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int kr = kt * TC_BK + c * 4 + t;
-      float x = 0.f;
-      if (row < it.m && kr < k2) x = it.src[row * 2 * it.ld + kr];
-      split_tf32(x, h[t], l[t]);
-    }
-    const long long off = ((long long)mt * it.nkt + kt) * A_TILE + r * TC_BK + ((c ^ (r & 7)) << 2);
-    *reinterpret_cast<float4 *>(it.hi + off) = make_float4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<float4 *>(it.lo + off) = make_float4(l[0], l[1], l[2], l[3]);
-  }
-}
-
-// B tiles: Br^T rows n' = 2j + t (t: 0 real part column, 1 imaginary), K index k' = 2p + u:
-//   Br^T[2j][2p] = re B[p][j], Br^T[2j][2p+1] = -im B[p][j], Br^T[2j+1][2p] = im, Br^T[2j+1][2p+1] = re
-__global__ void pack_b_kernel(PackBatchP pb) {
-  const PackItem it = pb.it[blockIdx.y];
-  const long long chunks = (long long)it.ntc * TC_BN * it.nkt * 8;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < chunks; e += (long long)gridDim.x * blockDim.x) {
-    const long long rowp = e / (it.nkt * 8);
-    const int q = (int)(e % (it.nkt * 8));
-    const int kt = q >> 3, c = q & 7;
-    const int nt = (int)(rowp / TC_BN), r = (int)(rowp % TC_BN);
-    const long long j = rowp >> 1;
-    const int tt = (int)(rowp & 1);
-    float h[4], l[4];
-#pragma unroll
-    for (int t2 = 0; t2 < 2; ++t2) {
-      const int p = (kt * TC_BK + c * 4) / 2 + t2;
-      float re = 0.f, im = 0.f;
-      if (j < it.n && p < it.k) {
-        const float *s = it.src + ((long long)p * it.ld + j) * 2;
-        re = s[0];
-        im = s[1];
-      }
-      const float x0 = tt == 0 ? re : im;    // coefficient of Re A
-      const float x1 = tt == 0 ? -im : re;   // coefficient of Im A
-      split_tf32(x0, h[2 * t2], l[2 * t2]);
-      split_tf32(x1, h[2 * t2 + 1], l[2 * t2 + 1]);
-    }
-    const long long off = ((long long)nt * it.nkt + kt) * B_TILE + r * TC_BK + ((c ^ (r & 7)) << 2);
-    *reinterpret_cast<float4 *>(it.hi + off) = make_float4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<float4 *>(it.lo + off) = make_float4(l[0], l[1], l[2], l[3]);
-  }
-}
-
-// The same B tiles, built through shared memory: a block stages a 16 (K) x 64 (N) complex slab
-// of B with reads along B's rows (coalesced), then writes the 128 packed rows x 32 K-values it
-// covers (half a tile) with coalesced 16-byte stores.  Threads of pack_b_kernel above read B down
-// its columns instead (one 8-byte element per row of B per thread).
-__global__ void __launch_bounds__(256) pack_b_t_kernel(PackBatchP pb) {
-  const PackItem it = pb.it[blockIdx.y];
-  const int jblocks = it.ntc * 2;  // 64 complex columns (128 packed rows) per block
-  const int nblk = jblocks * it.nkt;
-  __shared__ float2 sb[16][65];
-  for (int bid = blockIdx.x; bid < nblk; bid += gridDim.x) {
-    const int kt = bid % it.nkt, jb = bid / it.nkt;
-    const long long j0 = (long long)jb * 64;
-    const int p0 = kt * (TC_BK / 2);
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int idx = threadIdx.x + 256 * i;
-      const int pl = idx >> 6, jl = idx & 63;
-      const long long j = j0 + jl;
-      const int pp = p0 + pl;
-      float2 v = make_float2(0.f, 0.f);
-      if (j < it.n && pp < it.k) v = *reinterpret_cast<const float2 *>(it.src + ((long long)pp * it.ld + j) * 2);
-      sb[pl][jl] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int id = threadIdx.x + 256 * i;
-      const int rl = id >> 3, c = id & 7;  // packed row within the half tile, 16-byte chunk
-      const int jl = rl >> 1, tt = rl & 1;
-      float h[4], l[4];
-#pragma unroll
-      for (int t2 = 0; t2 < 2; ++t2) {
-        const float2 b = sb[2 * c + t2][jl];
-        const float x0 = tt == 0 ? b.x : b.y;   // coefficient of Re A
-        const float x1 = tt == 0 ? -b.y : b.x;  // coefficient of Im A
-        split_tf32(x0, h[2 * t2], l[2 * t2]);
-        split_tf32(x1, h[2 * t2 + 1], l[2 * t2 + 1]);
-      }
-      const long long rowp = 2 * j0 + rl;
-      const int nt = (int)(rowp / TC_BN), r = (int)(rowp % TC_BN);
-      const long long off = ((long long)nt * it.nkt + kt) * B_TILE + r * TC_BK + ((c ^ (r & 7)) << 2);
-      *reinterpret_cast<float4 *>(it.hi + off) = make_float4(h[0], h[1], h[2], h[3]);
-      *reinterpret_cast<float4 *>(it.lo + off) = make_float4(l[0], l[1], l[2], l[3]);
-    }
-  }
-}
-
-// real B, same staging: a 32 (K) x 128 (N) slab, one packed tile half (128 rows x 32 K-values)
-__global__ void __launch_bounds__(256) pack_b_real_t_kernel(PackBatchP pb) {
-  const PackItem it = pb.it[blockIdx.y];
+// real B of the plain TF32 probe, staged through shared memory: a 32 (K) x 128 (N) slab, half a packed
+// tile (128 rows x 32 K-values)
+__global__ void __launch_bounds__(256) pack_b_real_t_kernel(Tf32PackP pb) {
+  const Tf32PackItem it = pb.it;
   const int jblocks = it.ntc * 2;  // 128 columns per block
   const int nblk = jblocks * it.nkt;
   __shared__ float sb[32][129];
   for (int bid = blockIdx.x; bid < nblk; bid += gridDim.x) {
     const int kt = bid % it.nkt, jb = bid / it.nkt;
     const long long j0 = (long long)jb * 128;
-    const int p0 = kt * TC_BK;
+    const int p0 = kt * TC_BK32;
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -824,16 +1015,16 @@ __global__ void __launch_bounds__(256) pack_b_real_t_kernel(PackBatchP pb) {
       for (int t = 0; t < 4; ++t) split_tf32(sb[c * 4 + t][rl], h[t], l[t]);
       const long long row = j0 + rl;
       const int nt = (int)(row / TC_BN), r = (int)(row % TC_BN);
-      const long long off = ((long long)nt * it.nkt + kt) * B_TILE + r * TC_BK + ((c ^ (r & 7)) << 2);
+      const long long off = ((long long)nt * it.nkt + kt) * (B_TILE / 4) + r * TC_BK32 + ((c ^ (r & 7)) << 2);
       *reinterpret_cast<float4 *>(it.hi + off) = make_float4(h[0], h[1], h[2], h[3]);
       *reinterpret_cast<float4 *>(it.lo + off) = make_float4(l[0], l[1], l[2], l[3]);
     }
   }
 }
 
-// real operands: A (m x k, ld), B (k x n, ld) in FP32; the same tile formats with K' = k, N' = n
-__global__ void pack_a_real_kernel(PackBatchP pb) {
-  const PackItem it = pb.it[blockIdx.y];
+// real A of the plain TF32 probe
+__global__ void pack_a_real_kernel(Tf32PackP pb) {
+  const Tf32PackItem it = pb.it;
   const long long chunks = (long long)it.mtc * TC_BM * it.nkt * 8;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < chunks; e += (long long)gridDim.x * blockDim.x) {
     const long long row = e / (it.nkt * 8);
@@ -843,36 +1034,15 @@ __global__ void pack_a_real_kernel(PackBatchP pb) {
     float h[4], l[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-      const int kr = kt * TC_BK + c * 4 + t;
+      const int kr = kt * TC_BK32 + c * 4 + t;
       const float x = (row < it.m && kr < it.k) ? it.src[row * it.ld + kr] : 0.f;
       split_tf32(x, h[t], l[t]);
     }
-    const long long off = ((long long)mt * it.nkt + kt) * A_TILE + r * TC_BK + ((c ^ (r & 7)) << 2);
+    const long long off = ((long long)mt * it.nkt + kt) * (A_TILE / 4) + r * TC_BK32 + ((c ^ (r & 7)) << 2);
     *reinterpret_cast<float4 *>(it.hi + off) = make_float4(h[0], h[1], h[2], h[3]);
     *reinterpret_cast<float4 *>(it.lo + off) = make_float4(l[0], l[1], l[2], l[3]);
   }
 }
-__global__ void pack_b_real_kernel(PackBatchP pb) {
-  const PackItem it = pb.it[blockIdx.y];
-  const long long chunks = (long long)it.ntc * TC_BN * it.nkt * 8;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < chunks; e += (long long)gridDim.x * blockDim.x) {
-    const long long j = e / (it.nkt * 8);
-    const int q = (int)(e % (it.nkt * 8));
-    const int kt = q >> 3, c = q & 7;
-    const int nt = (int)(j / TC_BN), r = (int)(j % TC_BN);
-    float h[4], l[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int p = kt * TC_BK + c * 4 + t;
-      const float x = (j < it.n && p < it.k) ? it.src[(long long)p * it.ld + j] : 0.f;
-      split_tf32(x, h[t], l[t]);
-    }
-    const long long off = ((long long)nt * it.nkt + kt) * B_TILE + r * TC_BK + ((c ^ (r & 7)) << 2);
-    *reinterpret_cast<float4 *>(it.hi + off) = make_float4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<float4 *>(it.lo + off) = make_float4(l[0], l[1], l[2], l[3]);
-  }
-}
-
 // Per-device launch set-up of the tensor-core kernel: its dynamic shared-memory limit is raised
 // once on every device it runs on, and the device's SM count sizes the persistent grid.
 struct TcDevInfo {
@@ -889,7 +1059,13 @@ static TcDevInfo tc_device_info() {
   if ((int)info.size() <= dev) info.resize(dev + 1);
   TcDevInfo &d = info[dev];
   if (!d.attr) {
-    RFDD_CUDA(cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
+    const void *ones[] = {(const void *)tc_gemm_kernel<true, 256>, (const void *)tc_gemm_kernel<true, 64>,
+                          (const void *)tc_gemm_kernel<false, 256>};
+    for (const void *f : ones) RFDD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
+    RFDD_CUDA(cudaFuncSetAttribute(pack_f16_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   PACK_KC * 66 * (int)sizeof(float)));
+    RFDD_CUDA(cudaFuncSetAttribute(pack_f16_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   PACK_KC * 65 * (int)sizeof(float)));
     RFDD_CUDA(cudaFuncSetAttribute(tc_gemm2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, T2_SMEM));
     RFDD_CUDA(cudaDeviceGetAttribute(&d.nsm, cudaDevAttrMultiProcessorCount, dev));
     cudaLaunchConfig_t cfg = {};
@@ -978,86 +1154,108 @@ std::string tc_autotune_table() {
 // Tile walk of one item: down the columns when B spans at least 8 tile columns and the item's
 // packed A (hi + lo) takes at most 48 MB of the 129 MB L2, else along the rows.
 int tc_tile_order(int mtc, int ntc, int nkt) {
-  const double a_bytes = (double)mtc * nkt * A_TILE * 8.0;
+  const double a_bytes = 2.0 * mtc * nkt * (double)A_TILE;
   return (ntc >= 8 && mtc >= 2 && a_bytes <= 48e6) ? 1 : 0;
+}
+
+// Bytes of one packed operand: hi and lo tiles, then the scales (a multiple of 256 bytes)
+static size_t packed_bytes(size_t tiles, size_t tile_bytes, size_t scales) {
+  return 2 * tiles * tile_bytes + (scales * sizeof(float) + 255) / 256 * 256;
+}
+
+// Output tiles of the launch when they are BN wide: sets each item's tile counts and first tile
+static int set_tiles(TcBatchP &tb, int BN) {
+  int tiles = 0;
+  for (int i = 0; i < tb.count; ++i) {
+    TcItem &it = tb.it[i];
+    it.ntc = ceil_div(it.n2, BN);
+    it.colmajor = tc_tile_order(it.mtc, it.ntc, it.nkt);
+    it.tile0 = tiles;
+    tiles += it.mtc * it.ntc;
+  }
+  tb.total_tiles = tiles;
+  return tiles;
+}
+
+// One-CTA launch.  64-wide tiles when the 256-wide ones leave SMs without work (four times the tiles,
+// and a ring four stages deep) or are at most a quarter full.
+static void launch_one_cta(cudaStream_t st, TcBatchP &tb, int nsm, double alpha, double beta) {
+  int n2max = 0;
+  for (int i = 0; i < tb.count; ++i) n2max = std::max(n2max, tb.it[i].n2);
+  const bool narrow = n2max <= 64 || set_tiles(tb, TC_BN) < nsm;
+  const int tiles = set_tiles(tb, narrow ? 64 : TC_BN);
+  const int grid = std::max(1, std::min(tiles, nsm));
+  if (narrow) tc_gemm_kernel<true, 64><<<grid, TC_THREADS, TC_SMEM, st>>>(tb, (float)alpha, (float)beta);
+  else tc_gemm_kernel<true, 256><<<grid, TC_THREADS, TC_SMEM, st>>>(tb, (float)alpha, (float)beta);
+  RFDD_CHECK_LAUNCH();
 }
 
 template <bool CPLX, typename T>
 static void tc_gemm_run(cudaStream_t st, const std::vector<GemmItem<T>> &items, double alpha, double beta,
-                        const std::vector<TcPackedA> *pre = nullptr, int splits = 3) {
+                        const std::vector<TcPackedA> *pre = nullptr) {
   constexpr int F = CPLX ? 2 : 1;  // real columns / K entries per element
   RFDD_REQUIRE(g_tc_status != nullptr, RFDD_ESTATE, "tensor-core GEMM launched without a status word");
   const int nsm = tc_device_setup();
   for (size_t s0 = 0; s0 < items.size(); s0 += TC_MAXB) {
     const int cnt = (int)std::min<size_t>(TC_MAXB, items.size() - s0);
-    PackBatchP pa, pbb;
+    PackBatchP pk;
     TcBatchP tb;
-    memset(&pa, 0, sizeof(pa));
-    memset(&pbb, 0, sizeof(pbb));
+    memset(&pk, 0, sizeof(pk));
     memset(&tb, 0, sizeof(tb));
     size_t total = 0;
     std::vector<size_t> offA(cnt), offB(cnt);
-    int mtmax = 1, ntmax = 1;
-    long long achunks = 1, bchunks = 1;
     double flops = 0.0, cbytes = 0.0;
     for (int i = 0; i < cnt; ++i) {
       const auto &g = items[s0 + i];
-      const int mtc = ceil_div(g.m, TC_BM), ntc = ceil_div((int64_t)F * g.n, TC_BN), nkt = ceil_div((int64_t)F * g.k, TC_BK);
+      const size_t mtc = ceil_div(g.m, TC_BM), ntc = ceil_div((int64_t)F * g.n, TC_BN), nkt = ceil_div((int64_t)F * g.k, TC_BK);
       const bool packed = pre && (*pre)[s0 + i].hi;
       offA[i] = total;
-      if (!packed) total += (size_t)mtc * nkt * A_TILE * 2;
+      if (!packed) total += packed_bytes(mtc * nkt, A_TILE, mtc * TC_BM);
       offB[i] = total;
-      total += (size_t)ntc * nkt * B_TILE * 2;
-      mtmax = std::max(mtmax, mtc);
-      ntmax = std::max(ntmax, ntc);
-      achunks = std::max(achunks, (long long)mtc * TC_BM * nkt * 8);
-      bchunks = std::max(bchunks, (long long)ntc * TC_BN * nkt * 8);
+      total += packed_bytes(ntc * nkt, B_TILE, ntc * TC_BN);
       flops += (CPLX ? 8.0 : 2.0) * g.m * (double)g.n * g.k;
       // compulsory DRAM bytes: C read (beta != 0) and written, packed hi/lo operands read once
       cbytes += (beta != 0.0 ? 2.0 : 1.0) * 4.0 * F * g.m * (double)g.n +
-                8.0 * ((double)mtc * nkt * A_TILE + (double)ntc * nkt * B_TILE);
+                2.0 * ((double)mtc * nkt * A_TILE + (double)ntc * nkt * B_TILE);
     }
-    float *ws = nullptr;
-    RFDD_CUDA(cudaMallocAsync((void **)&ws, total * sizeof(float), st));
-    int tiles = 0;
+    uint8_t *ws = nullptr;
+    RFDD_CUDA(cudaMallocAsync((void **)&ws, total, st));
+    tb.count = cnt;
     for (int i = 0; i < cnt; ++i) {
       const auto &g = items[s0 + i];
       const int mtc = ceil_div(g.m, TC_BM), ntc = ceil_div((int64_t)F * g.n, TC_BN), nkt = ceil_div((int64_t)F * g.k, TC_BK);
-      const bool packed = pre && (*pre)[s0 + i].hi;
-      const float *Ah = packed ? (*pre)[s0 + i].hi : ws + offA[i];
-      const float *Al = packed ? (*pre)[s0 + i].lo : ws + offA[i] + (size_t)mtc * nkt * A_TILE;
-      float *Bh = ws + offB[i], *Bl = Bh + (size_t)ntc * nkt * B_TILE;
-      // a pre-packed A is not packed again (mtc = 0 gives its pack item no work)
-      pa.it[i] = {reinterpret_cast<const float *>(g.A), g.lda, g.m, g.n, g.k, const_cast<float *>(Ah),
-                  const_cast<float *>(Al), packed ? 0 : mtc, ntc, nkt};
-      pbb.it[i] = {reinterpret_cast<const float *>(g.B), g.ldb, g.m, g.n, g.k, Bh, Bl, mtc, ntc, nkt};
-      tb.it[i] = {Ah, Al, Bh, Bl, reinterpret_cast<float *>(g.C), (long long)F * g.ldc, g.m, F * g.n, nkt, mtc, ntc, tiles,
-                  packed ? (long long)(*pre)[s0 + i].mt_stride : 0ll, tc_tile_order(mtc, ntc, nkt)};
-      tiles += mtc * ntc;
-    }
-    tb.count = cnt;
-    tb.total_tiles = tiles;
-    tb.err = g_tc_status;
-    tb.splits = splits;
-    bool any_a = false;
-    for (int i = 0; i < cnt; ++i) any_a |= pa.it[i].mtc > 0;
-    const dim3 ga((unsigned)std::min<long long>(ceil_div(achunks, 256), 4096), cnt);
-    long long bblocks = 1;  // staged half-tiles of the largest B
-    for (int i = 0; i < cnt; ++i) bblocks = std::max(bblocks, (long long)pbb.it[i].ntc * 2 * pbb.it[i].nkt);
-    const dim3 gbt((unsigned)std::min<long long>(bblocks, 8192), cnt);
-    if (CPLX) {
-      if (any_a) {
-        pack_a_kernel<<<ga, 256, 0, st>>>(pa);
-        RFDD_CHECK_LAUNCH();
+      TcItem &it = tb.it[i];
+      uint8_t *Bh = ws + offB[i], *Bl = Bh + (size_t)ntc * nkt * B_TILE;
+      float *sB = reinterpret_cast<float *>(Bl + (size_t)ntc * nkt * B_TILE);
+      pk.b[pk.nb++] = {reinterpret_cast<const float *>(g.B), g.ldb, g.n, g.k, Bh, Bl, sB, ceil_div((int64_t)F * g.n, 64), nkt, 0};
+      it.Bhi = Bh;
+      it.Blo = Bl;
+      it.sB = sB;
+      if (pre && (*pre)[s0 + i].hi) {
+        const TcPackedA &p = (*pre)[s0 + i];
+        it.Ahi = p.hi;
+        it.Alo = p.lo;
+        it.sA = p.scale;
+        it.amts = p.mt_stride;
+      } else {
+        uint8_t *Ah = ws + offA[i], *Al = Ah + (size_t)mtc * nkt * A_TILE;
+        float *sA = reinterpret_cast<float *>(Al + (size_t)mtc * nkt * A_TILE);
+        pk.a[pk.na++] = {reinterpret_cast<const float *>(g.A), g.lda, g.m, g.k, Ah, Al, sA, mtc, nkt, 0};
+        it.Ahi = Ah;
+        it.Alo = Al;
+        it.sA = sA;
+        it.amts = 0;
       }
-      pack_b_t_kernel<<<gbt, 256, 0, st>>>(pbb);
-      RFDD_CHECK_LAUNCH();
-    } else {
-      pack_a_real_kernel<<<ga, 256, 0, st>>>(pa);
-      RFDD_CHECK_LAUNCH();
-      pack_b_real_t_kernel<<<gbt, 256, 0, st>>>(pbb);
-      RFDD_CHECK_LAUNCH();
+      it.C = reinterpret_cast<float *>(g.C);
+      it.ldc = (long long)F * g.ldc;
+      it.m = g.m;
+      it.n2 = F * g.n;
+      it.nkt = nkt;
+      it.mtc = mtc;
     }
+    const int tiles = set_tiles(tb, TC_BN);
+    tb.err = g_tc_status;
+    launch_pack<CPLX>(st, pk);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (profiling_enabled()) {
       e0 = profile_event();
@@ -1074,10 +1272,10 @@ static void tc_gemm_run(cudaStream_t st, const std::vector<GemmItem<T>> &items, 
     // measured on 8192 x 8192 products: the two-CTA kernel gains from K = 256 (complex) on (4 %
     // there, 1.5 % at K = 1024) and loses at K = 128, where the epilogue, not the operand feed,
     // bounds both kernels
-    int nkt_min = 1 << 30;
-    for (int i = 0; i < cnt; ++i) nkt_min = std::min(nkt_min, tb.it[i].nkt);
-    const bool two_ok = splits == 3 && dinfo.clusters2 > 0 && pairs >= dinfo.clusters2 && 8 * ghosts <= pairs;
-    bool two = two_ok && (CPLX ? nkt_min >= 16 : nkt_min >= 8);
+    int64_t k32_min = 1 << 30;  // K in units of 32 real entries
+    for (int i = 0; i < cnt; ++i) k32_min = std::min<int64_t>(k32_min, ceil_div((int64_t)F * items[s0 + i].k, 32));
+    const bool two_ok = dinfo.clusters2 > 0 && pairs >= dinfo.clusters2 && 8 * ghosts <= pairs;
+    bool two = two_ok && (CPLX ? k32_min >= 16 : k32_min >= 8);
     // the autotuner decides where both kernels can run, outside stream capture
     tune::Key tkey;
     bool tmeasure = false;
@@ -1086,8 +1284,8 @@ static void tc_gemm_run(cudaStream_t st, const std::vector<GemmItem<T>> &items, 
       RFDD_CUDA(cudaStreamIsCapturing(st, &cs));
       RFDD_CUDA(cudaGetDevice(&tkey.device));
       tkey.cplx = CPLX ? 1 : 0;
-      tkey.splits = splits;
-      tkey.kbucket = tune::k_bucket(nkt_min);
+      tkey.splits = 3;
+      tkey.kbucket = tune::k_bucket(k32_min);
       tkey.tbucket = tune::t_bucket(tiles, nsm);
       std::lock_guard<std::mutex> lk(g_tune_mu);
       tune_poll_locked();
@@ -1102,7 +1300,7 @@ static void tc_gemm_run(cudaStream_t st, const std::vector<GemmItem<T>> &items, 
       }
     }
     if (g_tc_engine_override == 1) two = false;
-    if (g_tc_engine_override == 2) two = splits == 3 && dinfo.clusters2 > 0;
+    if (g_tc_engine_override == 2) two = dinfo.clusters2 > 0;
     cudaEvent_t te0 = nullptr, te1 = nullptr;
     if (tmeasure) {
       if (cudaEventCreate(&te0) != cudaSuccess || cudaEventCreate(&te1) != cudaSuccess) {
@@ -1140,9 +1338,7 @@ static void tc_gemm_run(cudaStream_t st, const std::vector<GemmItem<T>> &items, 
       RFDD_CUDA(cudaLaunchKernelEx(&cfg, tc_gemm2_kernel, t2, (float)alpha, (float)beta));
       RFDD_CHECK_LAUNCH();
     } else {
-      const int grid = std::max(1, std::min(tiles, nsm));
-      tc_gemm_kernel<<<grid, TC_THREADS, TC_SMEM, st>>>(tb, (float)alpha, (float)beta);
-      RFDD_CHECK_LAUNCH();
+      launch_one_cta(st, tb, nsm, alpha, beta);
     }
     if (g_tc_events) RFDD_CUDA(cudaEventRecord(g_tc_events[1], st));
     if (te1) {
@@ -1176,31 +1372,36 @@ void tc_gemm_complex_pa(cudaStream_t st, const std::vector<GemmItem<cx<float>>> 
   if (!live.empty()) tc_gemm_run<true>(st, live, alpha, beta, &lpa);
 }
 
-int64_t tc_packed_a_ktiles(int64_t k) { return ceil_div(2 * k, TC_BK); }
-int64_t tc_packed_a_floats(int64_t m, int64_t k) { return (int64_t)ceil_div(m, TC_BM) * tc_packed_a_ktiles(k) * A_TILE; }
+static int64_t packed_a_ktiles(int64_t k) { return ceil_div(2 * k, TC_BK); }
+int64_t tc_packed_a_bytes(int64_t m, int64_t k, bool sides) {
+  const size_t mtc = ceil_div(m, TC_BM);
+  return (int64_t)packed_bytes(mtc * packed_a_ktiles(k), A_TILE, mtc * TC_BM * (sides ? 2 : 1));
+}
 
-TcPackedA tc_packed_view(const float *hi, const float *lo, int64_t k_full, int64_t r0, int64_t c0) {
+TcPackedA tc_packed_view(const void *op, int64_t m, int64_t k_full, int64_t r0, int64_t c0, int side) {
   RFDD_REQUIRE(r0 % TC_BM == 0 && (2 * c0) % TC_BK == 0, RFDD_EINVAL, "packed view must start on a tile");
-  const int64_t kt = tc_packed_a_ktiles(k_full);
+  const int64_t kt = packed_a_ktiles(k_full), mtc = ceil_div(m, TC_BM);
+  const uint8_t *hi = static_cast<const uint8_t *>(op), *lo = hi + mtc * kt * A_TILE;
+  const float *scale = reinterpret_cast<const float *>(lo + mtc * kt * A_TILE) + side * mtc * TC_BM;
   const int64_t off = ((r0 / TC_BM) * kt + (2 * c0) / TC_BK) * A_TILE;
-  return TcPackedA{hi + off, lo + off, kt};
+  return TcPackedA{hi + off, lo + off, scale + r0, kt};
 }
 
 void tc_pack_a_batched(cudaStream_t st, const std::vector<TcPackJob> &jobs) {
+  tc_device_setup();
   for (size_t s0 = 0; s0 < jobs.size(); s0 += TC_MAXB) {
     const int cnt = (int)std::min<size_t>(TC_MAXB, jobs.size() - s0);
-    PackBatchP pa;
-    memset(&pa, 0, sizeof(pa));
-    long long achunks = 1;
+    PackBatchP pk;
+    memset(&pk, 0, sizeof(pk));
     for (int i = 0; i < cnt; ++i) {
       const TcPackJob &j = jobs[s0 + i];
-      const int mtc = ceil_div(j.m, TC_BM), nkt = (int)tc_packed_a_ktiles(j.k);
-      pa.it[i] = {reinterpret_cast<const float *>(j.A), j.lda, (int)j.m, 0, (int)j.k, j.hi, j.lo,
-                  j.m > 0 && j.k > 0 ? mtc : 0, 0, nkt};
-      achunks = std::max(achunks, (long long)mtc * TC_BM * nkt * 8);
+      if (j.m <= 0 || j.k <= 0) continue;
+      const int64_t mtc = ceil_div(j.m, TC_BM), nkt = packed_a_ktiles(j.k);
+      uint8_t *hi = static_cast<uint8_t *>(j.dst), *lo = hi + mtc * nkt * A_TILE;
+      pk.a[pk.na++] = {reinterpret_cast<const float *>(j.A), j.lda, (int)j.m, (int)j.k, hi, lo,
+                       reinterpret_cast<float *>(lo + mtc * nkt * A_TILE), (int)mtc, (int)nkt, j.side};
     }
-    pack_a_kernel<<<dim3((unsigned)std::min<long long>(ceil_div(achunks, 256), 4096), cnt), 256, 0, st>>>(pa);
-    RFDD_CHECK_LAUNCH();
+    launch_pack<true>(st, pk);
   }
 }
 
@@ -1208,8 +1409,39 @@ void tc_gemm_real(cudaStream_t st, const std::vector<GemmItem<float>> &items, do
   tc_gemm_run<false>(st, items, alpha, beta);
 }
 
-void tc_gemm_real_tf32(cudaStream_t st, const std::vector<GemmItem<float>> &items, double alpha, double beta) {
-  tc_gemm_run<false>(st, items, alpha, beta, nullptr, 1);
+void tc_gemm_real_tf32(cudaStream_t st, const GemmItem<float> &g, double alpha, double beta) {
+  RFDD_REQUIRE(g_tc_status != nullptr, RFDD_ESTATE, "tensor-core GEMM launched without a status word");
+  const int nsm = tc_device_setup();
+  const int mtc = ceil_div(g.m, TC_BM), ntc = ceil_div(g.n, TC_BN), nkt = ceil_div(g.k, TC_BK32);
+  const size_t a_bytes = (size_t)mtc * nkt * A_TILE, b_bytes = (size_t)ntc * nkt * B_TILE;
+  uint8_t *ws = nullptr;
+  RFDD_CUDA(cudaMallocAsync((void **)&ws, 2 * (a_bytes + b_bytes), st));
+  uint8_t *Bh = ws + 2 * a_bytes;
+  Tf32PackP pa{{g.A, g.lda, g.m, g.n, g.k, reinterpret_cast<float *>(ws), reinterpret_cast<float *>(ws + a_bytes), mtc, ntc, nkt}};
+  Tf32PackP pb{{g.B, g.ldb, g.m, g.n, g.k, reinterpret_cast<float *>(Bh), reinterpret_cast<float *>(Bh + b_bytes), mtc, ntc, nkt}};
+  pack_a_real_kernel<<<4096, 256, 0, st>>>(pa);
+  RFDD_CHECK_LAUNCH();
+  pack_b_real_t_kernel<<<8192, 256, 0, st>>>(pb);
+  RFDD_CHECK_LAUNCH();
+  TcBatchP tb;
+  memset(&tb, 0, sizeof(tb));
+  tb.count = 1;
+  tb.err = g_tc_status;
+  TcItem &it = tb.it[0];
+  it.Ahi = ws;
+  it.Bhi = Bh;
+  it.C = g.C;
+  it.ldc = g.ldc;
+  it.m = g.m;
+  it.n2 = g.n;
+  it.nkt = nkt;
+  it.mtc = mtc;
+  const int tiles = set_tiles(tb, TC_BN);
+  if (g_tc_events) RFDD_CUDA(cudaEventRecord(g_tc_events[0], st));
+  tc_gemm_kernel<false, 256><<<std::max(1, std::min(tiles, nsm)), TC_THREADS, TC_SMEM, st>>>(tb, (float)alpha, (float)beta);
+  RFDD_CHECK_LAUNCH();
+  if (g_tc_events) RFDD_CUDA(cudaEventRecord(g_tc_events[1], st));
+  RFDD_CUDA(cudaFreeAsync(ws, st));
 }
 
 // =========================================================================================
@@ -1225,18 +1457,20 @@ void tc_gemm_real_tf32(cudaStream_t st, const std::vector<GemmItem<float>> &item
 constexpr int NOALLOC_MAX_M = 1024;   // complex rows of A and C
 constexpr int NOALLOC_MAX_N = 1024;   // complex columns of B and C
 constexpr int NOALLOC_MAX_K = 128;    // complex inner dimension
-constexpr size_t NOALLOC_A_FLOATS =
-    (size_t)((NOALLOC_MAX_M + TC_BM - 1) / TC_BM) * ((2 * NOALLOC_MAX_K + TC_BK - 1) / TC_BK) * A_TILE * 2;
-constexpr size_t NOALLOC_B_FLOATS =
-    (size_t)((2 * NOALLOC_MAX_N + TC_BN - 1) / TC_BN) * ((2 * NOALLOC_MAX_K + TC_BK - 1) / TC_BK) * B_TILE * 2;
-constexpr size_t NOALLOC_FLOATS = NOALLOC_A_FLOATS + NOALLOC_B_FLOATS;  // 6 MiB of floats in total
+constexpr size_t noalloc_bytes(size_t tiles, size_t tile_bytes, size_t scales) {
+  return 2 * tiles * tile_bytes + (scales * sizeof(float) + 255) / 256 * 256;
+}
+constexpr size_t NOALLOC_KT = (2 * NOALLOC_MAX_K + TC_BK - 1) / TC_BK;
+constexpr size_t NOALLOC_MT = (NOALLOC_MAX_M + TC_BM - 1) / TC_BM, NOALLOC_NT = (2 * NOALLOC_MAX_N + TC_BN - 1) / TC_BN;
+constexpr size_t NOALLOC_A_BYTES = noalloc_bytes(NOALLOC_MT * NOALLOC_KT, A_TILE, NOALLOC_MT * TC_BM);
+constexpr size_t NOALLOC_B_BYTES = noalloc_bytes(NOALLOC_NT * NOALLOC_KT, B_TILE, NOALLOC_NT * TC_BN);
 
-static __device__ __align__(256) float g_noalloc_scratch[NOALLOC_FLOATS];
+static __device__ __align__(256) uint8_t g_noalloc_scratch[NOALLOC_A_BYTES + NOALLOC_B_BYTES];  // 3 MiB
 // status word of the allocation-free launches (DS_WAIT_TIMEOUT), beside the scratch
 static __device__ int g_noalloc_status;
 
 struct NoallocAddr {
-  float *scratch = nullptr;
+  uint8_t *scratch = nullptr;
   int *status = nullptr;
 };
 // Device addresses of the array and of its status word on the current device, looked up once per
@@ -1252,7 +1486,7 @@ static NoallocAddr noalloc_addresses() {
     void *p = nullptr, *q = nullptr;
     RFDD_CUDA(cudaGetSymbolAddress(&p, g_noalloc_scratch));
     RFDD_CUDA(cudaGetSymbolAddress(&q, g_noalloc_status));
-    addr[dev].scratch = reinterpret_cast<float *>(p);
+    addr[dev].scratch = reinterpret_cast<uint8_t *>(p);
     addr[dev].status = reinterpret_cast<int *>(q);
   }
   return addr[dev];
@@ -1265,35 +1499,36 @@ int tc_gemm_complex_noalloc(cudaStream_t st, const cx<float> *A, int64_t lda, co
                "cgemm_noalloc: m, n must be <= 1024 and k <= 128 (size of the static scratch)");
   const NoallocAddr na = noalloc_addresses();
   const int nsm = tc_device_setup();
-  float *ws = na.scratch;
   const int mtc = ceil_div(m, TC_BM), ntc = ceil_div(2 * (int64_t)n, TC_BN), nkt = ceil_div(2 * (int64_t)k, TC_BK);
-  float *Ah = ws, *Al = Ah + (size_t)mtc * nkt * A_TILE;
-  float *Bh = ws + NOALLOC_A_FLOATS, *Bl = Bh + (size_t)ntc * nkt * B_TILE;
-  PackBatchP pa, pbb;
+  uint8_t *Ah = na.scratch, *Al = Ah + (size_t)mtc * nkt * A_TILE;
+  uint8_t *Bh = na.scratch + NOALLOC_A_BYTES, *Bl = Bh + (size_t)ntc * nkt * B_TILE;
+  float *sA = reinterpret_cast<float *>(Al + (size_t)mtc * nkt * A_TILE);
+  float *sB = reinterpret_cast<float *>(Bl + (size_t)ntc * nkt * B_TILE);
+  PackBatchP pk;
   TcBatchP tb;
-  memset(&pa, 0, sizeof(pa));
-  memset(&pbb, 0, sizeof(pbb));
+  memset(&pk, 0, sizeof(pk));
   memset(&tb, 0, sizeof(tb));
-  pa.it[0] = {reinterpret_cast<const float *>(A), lda, m, n, k, Ah, Al, mtc, ntc, nkt};
-  pbb.it[0] = {reinterpret_cast<const float *>(B), ldb, m, n, k, Bh, Bl, mtc, ntc, nkt};
-  tb.it[0] = {Ah, Al, Bh, Bl, reinterpret_cast<float *>(C), 2ll * ldc, m, 2 * n, nkt, mtc, ntc, 0, 0ll,
-              tc_tile_order(mtc, ntc, nkt)};
+  pk.na = pk.nb = 1;
+  pk.a[0] = {reinterpret_cast<const float *>(A), lda, m, k, Ah, Al, sA, mtc, nkt, 0};
+  pk.b[0] = {reinterpret_cast<const float *>(B), ldb, n, k, Bh, Bl, sB, ceil_div(2 * (int64_t)n, 64), nkt, 0};
+  TcItem &it = tb.it[0];
+  it.Ahi = Ah;
+  it.Alo = Al;
+  it.Bhi = Bh;
+  it.Blo = Bl;
+  it.sA = sA;
+  it.sB = sB;
+  it.C = reinterpret_cast<float *>(C);
+  it.ldc = 2ll * ldc;
+  it.m = m;
+  it.n2 = 2 * n;
+  it.nkt = nkt;
+  it.mtc = mtc;
   tb.count = 1;
-  tb.total_tiles = mtc * ntc;
   tb.err = na.status;
-  tb.splits = 3;
-  // the word keeps the last call's value: cleared on the caller's stream before this call's work
-  RFDD_CUDA(cudaMemsetAsync(na.status, 0, sizeof(int), st));
-  const long long achunks = (long long)mtc * TC_BM * nkt * 8;
-  pack_a_kernel<<<dim3((unsigned)std::min<long long>(ceil_div(achunks, 256), 4096), 1), 256, 0, st>>>(pa);
-  RFDD_CHECK_LAUNCH();
-  // B staged through shared memory (rows of B read along their length): ntc * 2 half-tile column
-  // blocks per K tile, every one inside the ntc x nkt tiles reserved for B above
-  pack_b_t_kernel<<<dim3((unsigned)(ntc * 2 * nkt), 1), 256, 0, st>>>(pbb);
-  RFDD_CHECK_LAUNCH();
-  tc_gemm_kernel<<<std::max(1, std::min(tb.total_tiles, nsm)), TC_THREADS, TC_SMEM, st>>>(tb, (float)alpha,
-                                                                                      (float)beta);
-  RFDD_CHECK_LAUNCH();
+  // the status word keeps the last call's value: the packing launch clears it
+  launch_pack<true>(st, pk, na.status);
+  launch_one_cta(st, tb, nsm, alpha, beta);
   int status = 0;
   RFDD_CUDA(cudaMemcpyAsync(&status, na.status, sizeof(int), cudaMemcpyDeviceToHost, st));
   RFDD_CUDA(cudaStreamSynchronize(st));

@@ -1,4 +1,4 @@
-// Tensor-core (tcgen05, 3xTF32) complex-FP32 GEMM; host launcher.
+// Tensor-core (tcgen05, two-way 16-bit split) complex-FP32 GEMM; host launcher.
 #pragma once
 #include "dense.cuh"
 
@@ -36,39 +36,43 @@ struct TcEngineScope {
 };
 // C = beta*C + alpha*A*B for every item (complex, row-major, no transposes)
 void tc_gemm_complex(cudaStream_t st, const std::vector<GemmItem<cx<float>>> &items, double alpha, double beta);
-// C = beta*C + alpha*A*B for real FP32 items (same kernel, 3xTF32)
+// C = beta*C + alpha*A*B for real FP32 items (same kernel)
 void tc_gemm_real(cudaStream_t st, const std::vector<GemmItem<float>> &items, double alpha, double beta);
 // the same with one TF32 product per multiply (operands rounded to TF32): the throughput probe of
 // the plain TF32 tensor path, not used by the solver
-void tc_gemm_real_tf32(cudaStream_t st, const std::vector<GemmItem<float>> &items, double alpha, double beta);
+void tc_gemm_real_tf32(cudaStream_t st, const GemmItem<float> &item, double alpha, double beta);
 
 // The tile-shape autotuner: mode 0 off (fixed rule), 1 on, 2 forget every class (re-tune);
 // returns whether it was on.  tc_autotune_table: one line per class (tc_tune.h, Tuner::dump).
 int tc_autotune(int mode);
 std::string tc_autotune_table();
-// A operand already split into TF32 hi/lo and laid out in the kernel's tiles (tc_pack_a_batched):
-// tile (mt, kt) of the operand at hi/lo + (mt * mt_stride + kt) * tile size.  Lets a factor that
-// is multiplied many times (triangular-solve updates, border products) be packed once.
+// A operand already scaled, split into 16-bit hi/lo and laid out in the kernel's tiles
+// (tc_pack_a_batched): tile (mt, kt) of the operand at hi/lo + (mt * mt_stride + kt) * tile size, the
+// inverse scale of each row in scale.  Lets a factor that is multiplied many times
+// (triangular-solve updates, border products) be packed once.
 struct TcPackedA {
-  const float *hi = nullptr, *lo = nullptr;
+  const uint8_t *hi = nullptr, *lo = nullptr;
+  const float *scale = nullptr;
   int64_t mt_stride = 0;
 };
 // items[i] uses pa[i] as its A operand when pa[i].hi is set (items[i].A is then not read)
 void tc_gemm_complex_pa(cudaStream_t st, const std::vector<GemmItem<cx<float>>> &items,
                         const std::vector<TcPackedA> &pa, double alpha, double beta);
-// packing of complex m x k matrices (row-major, leading dimension lda) into hi/lo tile arrays
-// of tc_packed_a_floats(m, k) floats each (rows and K padded with zeros to whole tiles)
+// Packing of complex m x k matrices (row-major, leading dimension lda) into operands of
+// tc_packed_a_bytes(m, k, side > 0) bytes each at dst: hi tiles, lo tiles, scales (rows and K padded
+// with zeros to whole tiles).  side > 0: an L\U factor whose products use the part left of the
+// diagonal blocks of `side` rows (L) or the rest (U), never both: each part of a row has its own scale.
 struct TcPackJob {
   const cx<float> *A;
   int64_t lda, m, k;
-  float *hi, *lo;
+  void *dst;
+  int side = 0;
 };
-int64_t tc_packed_a_ktiles(int64_t k);
-int64_t tc_packed_a_floats(int64_t m, int64_t k);
+int64_t tc_packed_a_bytes(int64_t m, int64_t k, bool sides = false);
 void tc_pack_a_batched(cudaStream_t st, const std::vector<TcPackJob> &jobs);
 // the sub-matrix of a packed m x k_full operand starting at row r0 (a multiple of 128) and complex
-// column c0 (a multiple of 16)
-TcPackedA tc_packed_view(const float *hi, const float *lo, int64_t k_full, int64_t r0, int64_t c0);
+// column c0 (a multiple of 32); side: 0 the only scale, or that of the left part; 1 the right part's
+TcPackedA tc_packed_view(const void *op, int64_t m, int64_t k_full, int64_t r0 = 0, int64_t c0 = 0, int side = 0);
 // TFLOP/s of kind::tf32 MMAs issued back to back from operand tiles resident in shared memory
 // (one CTA per SM, no operand loads): the tensor pipe's own TF32 rate.  Time-outs go to *dev_status.
 double tc_mma_probe_tflops(cudaStream_t st, int *dev_status);

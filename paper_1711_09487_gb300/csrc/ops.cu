@@ -331,7 +331,8 @@ __global__ void assemble_blocks_kernel(const int64_t *__restrict__ rp, const int
                                        const int32_t *__restrict__ sidx, const int64_t *__restrict__ sidx_off,
                                        const int32_t *__restrict__ posmap, const int64_t *__restrict__ Doff,
                                        int64_t total_rows, const int64_t *__restrict__ boff,
-                                       const cx<double> *__restrict__ zz, T *__restrict__ base, int border) {
+                                       const cx<double> *__restrict__ zz, T *__restrict__ base, int border,
+                                       int ldpad) {
   const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const int lane = threadIdx.x & 31;
   const int l = blockIdx.y;
@@ -346,7 +347,7 @@ __global__ void assemble_blocks_kernel(const int64_t *__restrict__ rp, const int
   const int64_t sj = sidx_off[j + 1] - sidx_off[j];
   const int64_t Dj = border ? dj + sj : dj;
   const int64_t i = g - Doff[j];
-  T *row = base + boff[(int64_t)l * p + j] + i * Dj;
+  T *row = base + boff[(int64_t)l * p + j] + i * ((Dj + ldpad - 1) / ldpad * ldpad);
   const cx<double> z = zz[l];
   for (int64_t c = lane; c < Dj; c += 32) row[c] = ST<T>::zero();
   __syncwarp();
@@ -375,12 +376,12 @@ __global__ void assemble_blocks_kernel(const int64_t *__restrict__ rp, const int
 template <typename T>
 void assemble_blocks(cudaStream_t st, const DevPencil &P, const DevDD &dd, const int64_t *dev_D_off,
                      int64_t total_rows, const int64_t *dev_boff, const cx<double> *z_dev, int nnodes, T *base,
-                     bool border) {
+                     bool border, int ldpad) {
   if (total_rows <= 0) return;
   dim3 grid(ceil_div(total_rows * 32, 256), nnodes);
   assemble_blocks_kernel<T><<<grid, 256, 0, st>>>(P.rowptr, P.col, P.a, P.m, dd.p, dd.dsum, dd.s, dd.off, dd.sidx,
                                                   dd.sidx_off, dd.posmap, dev_D_off, total_rows, dev_boff, z_dev, base,
-                                                  border ? 1 : 0);
+                                                  border ? 1 : 0, ldpad);
   RFDD_CHECK_LAUNCH();
 }
 
@@ -388,12 +389,12 @@ template <typename T>
 __global__ void assemble_interface_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
                                           const double *__restrict__ av, const double *__restrict__ mv,
                                           int64_t dsum, int64_t s, const cx<double> *__restrict__ zz,
-                                          T *__restrict__ S) {
+                                          T *__restrict__ S, int64_t sld) {
   const int64_t a = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
   const int lane = threadIdx.x & 31;
   const int l = blockIdx.y;
   if (a >= s) return;
-  T *row = S + (int64_t)l * s * s + a * s;
+  T *row = S + ((int64_t)l * s + a) * sld;
   for (int64_t c = lane; c < s; c += 32) row[c] = ST<T>::zero();
   __syncwarp();
   const cx<double> z = zz[l];
@@ -406,32 +407,33 @@ __global__ void assemble_interface_kernel(const int64_t *__restrict__ rp, const 
 
 template <typename T>
 void assemble_interface(cudaStream_t st, const DevPencil &P, const DevDD &dd, const cx<double> *z_dev,
-                        int nnodes, T *S) {
+                        int nnodes, T *S, int64_t sld) {
   dim3 grid(ceil_div(dd.s * 32, 256), nnodes);
-  assemble_interface_kernel<T><<<grid, 256, 0, st>>>(P.rowptr, P.col, P.a, P.m, dd.dsum, dd.s, z_dev, S);
+  assemble_interface_kernel<T><<<grid, 256, 0, st>>>(P.rowptr, P.col, P.a, P.m, dd.dsum, dd.s, z_dev, S, sld);
   RFDD_CHECK_LAUNCH();
 }
 
 template <typename T>
 __global__ void scatter_schur_kernel(const int32_t *__restrict__ sidx_j, int p, int j, int dj, int sj, int64_t s,
                                      const int64_t *__restrict__ boff, const T *__restrict__ base,
-                                     T *__restrict__ S) {
+                                     T *__restrict__ S, int ldpad, int64_t sld) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int l = blockIdx.y;
   if (e >= (int64_t)sj * sj) return;
   const int a = (int)(e / sj), b = (int)(e % sj);
-  const int64_t Dj = (int64_t)dj + sj;
+  const int64_t Dj = ((int64_t)dj + sj + ldpad - 1) / ldpad * ldpad;
   const T *trail = base + boff[(int64_t)l * p + j] + (int64_t)dj * Dj + dj;
-  T *dst = S + (int64_t)l * s * s + (int64_t)sidx_j[a] * s + sidx_j[b];
+  T *dst = S + ((int64_t)l * s + sidx_j[a]) * sld + sidx_j[b];
   *dst = *dst + trail[(int64_t)a * Dj + b];
 }
 
 template <typename T>
 void scatter_schur(cudaStream_t st, const DevDD &dd, int j, int dj, int sj, int64_t sidx_start,
-                   const int64_t *dev_boff, const T *base, int nnodes, T *S) {
+                   const int64_t *dev_boff, const T *base, int nnodes, T *S, int ldpad, int64_t sld) {
   if (sj <= 0) return;
   dim3 grid(ceil_div((int64_t)sj * sj, 256), nnodes);
-  scatter_schur_kernel<T><<<grid, 256, 0, st>>>(dd.sidx + sidx_start, dd.p, j, dj, sj, dd.s, dev_boff, base, S);
+  scatter_schur_kernel<T><<<grid, 256, 0, st>>>(dd.sidx + sidx_start, dd.p, j, dj, sj, dd.s, dev_boff, base, S, ldpad,
+                                                       sld);
   RFDD_CHECK_LAUNCH();
 }
 
@@ -659,15 +661,15 @@ void gather_rows_cols_f64(cudaStream_t st, const double *src, int64_t lds, const
 
 #define RFDD_INST_OPS(T)                                                                                     \
   template void assemble_blocks<T>(cudaStream_t, const DevPencil &, const DevDD &, const int64_t *, int64_t, \
-                                   const int64_t *, const cx<double> *, int, T *, bool);
+                                   const int64_t *, const cx<double> *, int, T *, bool, int);
 RFDD_INST_OPS(float)
 RFDD_INST_OPS(double)
 RFDD_INST_OPS(cx<float>)
 RFDD_INST_OPS(cx<double>)
 
 #define RFDD_INST_OPSC(T)                                                                                         \
-  template void assemble_interface<T>(cudaStream_t, const DevPencil &, const DevDD &, const cx<double> *, int, T *); \
-  template void scatter_schur<T>(cudaStream_t, const DevDD &, int, int, int, int64_t, const int64_t *, const T *, int, T *);    \
+  template void assemble_interface<T>(cudaStream_t, const DevPencil &, const DevDD &, const cx<double> *, int, T *, int64_t); \
+  template void scatter_schur<T>(cudaStream_t, const DevDD &, int, int, int, int64_t, const int64_t *, const T *, int, T *, int, int64_t);    \
   template void couple<T>(cudaStream_t, const DevPencil &, int64_t, int64_t, int64_t, int64_t, const cx<double> *,  \
                           int, const T *, int64_t, int64_t, T *, int64_t, int64_t, int64_t, double, bool);           \
   template void real_to_complex<T>(cudaStream_t, const double *, T *, int64_t, int, int64_t);                        \
@@ -677,9 +679,9 @@ RFDD_INST_OPSC(cx<float>)
 RFDD_INST_OPSC(cx<double>)
 // real shift (inertia counts)
 template void assemble_interface<double>(cudaStream_t, const DevPencil &, const DevDD &, const cx<double> *, int,
-                                         double *);
+                                         double *, int64_t);
 template void scatter_schur<double>(cudaStream_t, const DevDD &, int, int, int, int64_t, const int64_t *,
-                                    const double *, int, double *);
+                                    const double *, int, double *, int, int64_t);
 
 
 // ---------------------------------------------------------------------------------------
@@ -763,12 +765,12 @@ template <typename T>
 __global__ void scatter_schur_levels_kernel(int p, int j, int dj, int sj, const int32_t *__restrict__ q,
                                             const int32_t *__restrict__ r, int64_t s2, int64_t gbase, int64_t Dg,
                                             const int64_t *__restrict__ boff, const T *__restrict__ base,
-                                            T *__restrict__ L, int64_t tsz) {
+                                            T *__restrict__ L, int64_t tsz, int ldpad) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int l = blockIdx.y;
   if (e >= (int64_t)sj * sj) return;
   const int t = (int)(e / sj), u = (int)(e % sj);
-  const int64_t Dj = (int64_t)dj + sj;
+  const int64_t Dj = ((int64_t)dj + sj + ldpad - 1) / ldpad * ldpad;
   const T v = base[boff[(int64_t)l * p + j] + (int64_t)dj * Dj + dj + (int64_t)t * Dj + u];
   const int rt = r[t], ru = r[u];
   T *dst = L + (int64_t)l * tsz + ((rt >= 0 && ru >= 0) ? (int64_t)rt * s2 + ru : gbase + (int64_t)q[t] * Dg + q[u]);
@@ -777,10 +779,10 @@ __global__ void scatter_schur_levels_kernel(int p, int j, int dj, int sj, const 
 template <typename T>
 void scatter_schur_levels(cudaStream_t st, int p, int j, int dj, int sj, const int32_t *q_j, const int32_t *r_j,
                           int64_t s2, int64_t gbase, int64_t Dg, const int64_t *dev_boff, const T *base, int nnodes,
-                          T *L, int64_t tsz) {
+                          T *L, int64_t tsz, int ldpad) {
   if (sj <= 0) return;
   scatter_schur_levels_kernel<T><<<dim3(ceil_div((int64_t)sj * sj, 256), nnodes), 256, 0, st>>>(
-      p, j, dj, sj, q_j, r_j, s2, gbase, Dg, dev_boff, base, L, tsz);
+      p, j, dj, sj, q_j, r_j, s2, gbase, Dg, dev_boff, base, L, tsz, ldpad);
   RFDD_CHECK_LAUNCH();
 }
 
@@ -812,7 +814,7 @@ void scatter_trail_levels(cudaStream_t st, const int32_t *i2g, int n1, int n2, i
   template void assemble_iface_levels<T>(cudaStream_t, const DevPencil &, int64_t, int64_t, const int64_t *,    \
                                          const cx<double> *, int, T *, int64_t);                                \
   template void scatter_schur_levels<T>(cudaStream_t, int, int, int, int, const int32_t *, const int32_t *,     \
-                                        int64_t, int64_t, int64_t, const int64_t *, const T *, int, T *, int64_t); \
+                                        int64_t, int64_t, int64_t, const int64_t *, const T *, int, T *, int64_t, int); \
   template void scatter_trail_levels<T>(cudaStream_t, const int32_t *, int, int, int64_t, int64_t, int, T *, int64_t);
 RFDD_INST_LEVELS(cx<float>)
 RFDD_INST_LEVELS(cx<double>)

@@ -62,17 +62,17 @@ void shifted_residual(cudaStream_t st, const DevPencil &P, const cx<double> *z_d
 template <typename T>
 void assemble_blocks(cudaStream_t st, const DevPencil &P, const DevDD &dd, const int64_t *dev_D_off,
                      int64_t total_rows, const int64_t *dev_boff, const cx<double> *z_dev, int nnodes, T *base,
-                     bool border);
-// S_l = C - z_l M_C (dense s x s at S + l*s*s).
+                     bool border, int ldpad = 1);
+// S_l = C - z_l M_C (dense s x s at S + l*s*sld, leading dimension sld).
 template <typename T>
 void assemble_interface(cudaStream_t st, const DevPencil &P, const DevDD &dd, const cx<double> *z_dev,
-                        int nnodes, T *S);
+                        int nnodes, T *S, int64_t sld);
 // For subdomain j: S_l[sidx_j[a]][sidx_j[b]] += T_l[a][b], T_l = trailing s_j x s_j block of the
-// bordered factor (base + boff[l*p+j] + d_j*(D_j+1), ld D_j).  Called for j = 0..p-1 in order, so
+// bordered factor (base + boff[l*p+j], ld D_j rounded up to a multiple of ldpad).  Called for j = 0..p-1 in order, so
 // the sums are reproducible.
 template <typename T>
 void scatter_schur(cudaStream_t st, const DevDD &dd, int j, int dj, int sj, int64_t sidx_start,
-                   const int64_t *dev_boff, const T *base, int nnodes, T *S);
+                   const int64_t *dev_boff, const T *base, int nnodes, T *S, int ldpad, int64_t sld);
 
 // Two-level interface factorisation (storage per node: S2 (s2 x s2) at 0, then the bordered
 // block of each group; tsz elements per node, node l at L + l*tsz).
@@ -86,7 +86,7 @@ void assemble_iface_levels(cudaStream_t st, const DevPencil &P, int64_t e0, int6
 template <typename T>
 void scatter_schur_levels(cudaStream_t st, int p, int j, int dj, int sj, const int32_t *q_j, const int32_t *r_j,
                           int64_t s2, int64_t gbase, int64_t Dg, const int64_t *dev_boff, const T *base, int nnodes,
-                          T *L, int64_t tsz);
+                          T *L, int64_t tsz, int ldpad);
 // S2[i2g[t]][i2g[u]] += trailing n2 x n2 block of the group block at gbase (n1 + n2 square).
 template <typename T>
 void scatter_trail_levels(cudaStream_t st, const int32_t *i2g, int n1, int n2, int64_t gbase, int64_t s2, int nnodes,

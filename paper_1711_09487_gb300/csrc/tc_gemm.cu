@@ -50,8 +50,8 @@ struct TcRing {
 constexpr int TC_RING_BYTES = 2 * (2 * A_TILE + 2 * B_TILE);
 static_assert(TcRing<64>::STAGES * TcRing<64>::BYTES == TC_RING_BYTES, "both rings fill the same shared memory");
 constexpr int EPI_WARPS = 8;  // two per TMEM lane quarter, each drains half of the columns
-constexpr int EPI_PITCH = 33;
-constexpr int EPI_BYTES = EPI_WARPS * 32 * EPI_PITCH * 4;
+constexpr int EPI_TILE = 32 * 32;  // floats a warp stages: 32 rows of 32 columns
+constexpr int EPI_BYTES = EPI_WARPS * EPI_TILE * 4;
 constexpr int TC_THREADS = 64 + 32 * EPI_WARPS;  // producer warp, MMA warp, epilogue warps
 constexpr int TC_SMEM = TC_RING_BYTES + EPI_BYTES + 1024;
 constexpr long long WAIT_LIMIT = 1ll << 24;
@@ -77,6 +77,7 @@ struct TcItem {
   int m, n2, nkt, mtc, ntc, tile0;  // tile0: first global tile index of this item
   long long amts;  // A tiles between consecutive 128-row tiles (0: nkt, a packed A of its own)
   int colmajor;    // 1: tiles walk down the columns (mt fastest), 0: along the rows (nt fastest)
+  int vec;         // floats per access to C: 4 when every row of C is so aligned, else 1
 };
 
 // Position of tile `local` of an item.  Along the rows, the CTAs running at once share one row of
@@ -180,58 +181,117 @@ __device__ __forceinline__ int find_item(const TcBatchP &b, int tile) {
   return lo;
 }
 
-// C entries of one 32 x 32 chunk of an output tile, lane = column: loaded ahead of the accumulator
-__device__ __forceinline__ void load_c(const TcItem &it, int row0, int nrows, int col, float beta, float (&cv)[32]) {
-  const bool on = col < it.n2 && beta != 0.f;
-  const float *p = it.C + (long long)row0 * it.ldc + col;
+// Access to one 32 x 32 chunk of C by a warp, V floats per lane and row: 32 / V lanes cover a row, so
+// access i takes rows i * V .. i * V + V - 1.  All loads of a chunk are independent (32 values per lane).
+template <int V>
+struct ChunkC {
+  static constexpr int ROWS = V;         // rows per access
+  static constexpr int NACC = 32 / V;    // accesses per chunk
+  __device__ __forceinline__ static int row(int i, int lane) { return i * V + lane / (32 / V); }
+  __device__ __forceinline__ static int col(int lane) { return (lane % (32 / V)) * V; }
+  __device__ __forceinline__ static void load(const TcItem &it, int row0, int nrows, int col0, int lane, float beta,
+                                              float (&cv)[32]) {
+    const int c = col0 + col(lane);
+    const float *p = it.C + (long long)(row0 + row(0, lane)) * it.ldc + c;
+    const long long step = (long long)V * it.ldc;
+    const bool on = beta != 0.f;
 #pragma unroll
-  for (int r = 0; r < 32; ++r) {
-    cv[r] = (on && r < nrows) ? *p : 0.f;
-    p += it.ldc;
+    for (int i = 0; i < NACC; ++i, p += step) {
+      float *d = cv + i * V;
+#pragma unroll
+      for (int t = 0; t < V; ++t) d[t] = 0.f;
+      if (on && row(i, lane) < nrows) {
+        if (c + V <= it.n2) {
+          if (V == 4) *reinterpret_cast<float4 *>(d) = *reinterpret_cast<const float4 *>(p);
+          else d[0] = *p;
+        } else {
+#pragma unroll
+          for (int t = 0; t < V; ++t)
+            if (c + t < it.n2) d[t] = p[t];
+        }
+      }
+    }
   }
-}
+  __device__ __forceinline__ static void store(const TcItem &it, float *p, int c, const float *d) {
+    if (c + V <= it.n2) {
+      if (V == 4) *reinterpret_cast<float4 *>(p) = *reinterpret_cast<const float4 *>(d);
+      else *p = d[0];
+    } else {
+#pragma unroll
+      for (int t = 0; t < V; ++t)
+        if (c + t < it.n2) p[t] = d[t];
+    }
+  }
+};
 
 // Epilogue of one output tile by one warp: TMEM lanes 32q..32q+31 (rows mt*128 + 32q ..), NCH column
-// chunks of 32 accumulator columns from chunk c0 on, staged through shared memory so that C is read
-// and written along its rows; C = alpha * scaled acc + beta * C, rows and columns masked.  cv holds
-// the first chunk's C (loaded before the accumulator was ready); the C of the next chunk is in
-// flight while a chunk is written, and `done` runs once the accumulator has been read.
-template <int NCH, bool SCALED, typename F>
-__device__ __forceinline__ void drain_tile(const TcItem &it, uint32_t tacc, int mt, int col0, int q, int c0, int lane,
-                                           float *stg, float alpha, float beta, float (&cv)[32], F &&done) {
+// chunks of 32 accumulator columns from chunk c0 on; C = alpha * scaled acc + beta * C, rows and columns
+// masked.  The accumulator's rows are turned into C's through shared memory (16-byte pieces of row r at
+// piece ^ (r & 7): no bank conflicts either way).  What bounds it is the latency of C: two chunks of C are in
+// flight from before the accumulator is ready (`wait` returns false if it never is), and each is
+// replaced by the chunk after the next as soon as it has been used.  `done` runs once the
+// accumulator has been read.  Measured, 8192 x 8192 complex: K = 32 0.28 ms (0.35 with one chunk in flight
+// and one float per access), K = 256 0.29 ms = 472 TFLOP/s (0.37; 0.49 with the TF32 split), K = 512 0.50 ms =
+// 547 TFLOP/s, 1.64 PFLOP/s of MMAs.
+template <int NCH, bool SCALED, int V, typename W, typename F>
+__device__ __forceinline__ bool drain_tile(const TcItem &it, uint32_t tacc, int mt, int col0, int q, int c0, int lane,
+                                           float *stg, float alpha, float beta, W &&wait, F &&done) {
+  using CC = ChunkC<V>;
   const int row0 = mt * TC_BM + q * 32;
   const int nrows = min(32, it.m - row0);
-  // scale of this lane's row (read along the rows below)
-  const float ra = SCALED ? (lane < nrows ? it.sA[row0 + lane] : 1.f) : 1.f;
+  float cb[NCH > 1 ? 2 : 1][32];
+  CC::load(it, row0, nrows, col0 + c0 * 32, lane, beta, cb[0]);
+  if (NCH > 1) CC::load(it, row0, nrows, col0 + c0 * 32 + 32, lane, beta, cb[NCH > 1 ? 1 : 0]);
+  // scale of the row this lane takes from the accumulator, times alpha
+  const float ra = SCALED && lane < nrows ? it.sA[row0 + lane] : 1.f;
+  if (!wait()) return false;
 #pragma unroll
   for (int ci = 0; ci < NCH; ++ci) {
-    const int c = c0 + ci;
+    const int c = c0 + ci, cc = col0 + c * 32;
+    float rb[V];
+#pragma unroll
+    for (int t = 0; t < V; ++t) {
+      const int j = cc + CC::col(lane) + t;
+      rb[t] = SCALED && j < it.n2 ? it.sB[j] : 1.f;
+    }
     uint32_t v[32];
     TC_LD32(tacc + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32), v);
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
     if (ci == NCH - 1) done();
 #pragma unroll
-    for (int j = 0; j < 32; ++j) stg[lane * EPI_PITCH + j] = __uint_as_float(v[j]);
+    for (int j = 0; j < 8; ++j)
+      *reinterpret_cast<float4 *>(stg + lane * 32 + ((j ^ (lane & 7)) << 2)) =
+          make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]), __uint_as_float(v[4 * j + 2]),
+                      __uint_as_float(v[4 * j + 3]));
     __syncwarp();
-    const int col = col0 + c * 32 + lane;
-    float cn[32];
-    if (ci + 1 < NCH) load_c(it, row0, nrows, col + 32, beta, cn);
-    const bool on = col < it.n2;
-    const float rb = SCALED ? (on ? it.sB[col] : 1.f) : 1.f;
-    float *p = it.C + (long long)row0 * it.ldc + col;
+    const int cl = CC::col(lane);
+    float *p = it.C + (long long)(row0 + CC::row(0, lane)) * it.ldc + cc + cl;
+    const long long step = (long long)V * it.ldc;
+    float(&cv)[32] = cb[NCH > 1 ? ci & 1 : 0];
 #pragma unroll
-    for (int r = 0; r < 32; ++r) {
+    for (int i = 0; i < CC::NACC; ++i, p += step) {
+      const int r = CC::row(i, lane);
+      const float *sp = stg + r * 32 + (((cl >> 2) ^ (r & 7)) << 2) + (cl & 3);
+      float x[V];
+      if (V == 4) *reinterpret_cast<float4 *>(x) = *reinterpret_cast<const float4 *>(sp);
+      else x[0] = *sp;
+      const float rr = SCALED ? __shfl_sync(0xffffffffu, ra, r) : 1.f;
       // the two scales are powers of two: their product first, so that neither over- or underflows alone
-      const float f = SCALED ? alpha * (__shfl_sync(0xffffffffu, ra, r) * rb) : alpha;
-      if (on && r < nrows) *p = fmaf(f, stg[r * EPI_PITCH + lane], beta * cv[r]);
-      p += it.ldc;
+#pragma unroll
+      for (int t = 0; t < V; ++t)
+        x[t] = fmaf(SCALED ? alpha * (rr * rb[t]) : alpha, x[t], beta * cv[i * V + t]);
+      if (r < nrows) CC::store(it, p, cc + cl, x);
     }
     __syncwarp();
-    if (ci + 1 < NCH) {
-#pragma unroll
-      for (int r = 0; r < 32; ++r) cv[r] = cn[r];
-    }
+    if (ci + 2 < NCH) CC::load(it, row0, nrows, cc + 64, lane, beta, cv);
   }
+  return true;
+}
+template <int NCH, bool SCALED, typename W, typename F>
+__device__ __forceinline__ bool drain_tile_vec(const TcItem &it, uint32_t tacc, int mt, int col0, int q, int c0,
+                                               int lane, float *stg, float alpha, float beta, W &&wait, F &&done) {
+  if (it.vec == 4) return drain_tile<NCH, SCALED, 4>(it, tacc, mt, col0, q, c0, lane, stg, alpha, beta, wait, done);
+  return drain_tile<NCH, SCALED, 1>(it, tacc, mt, col0, q, c0, lane, stg, alpha, beta, wait, done);
 }
 
 // Real columns of a tile that the MMAs compute: those of C, in steps of 16 (the MMA's N)
@@ -374,7 +434,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
     constexpr int NCH = BN / 64;
     const int q = warp & 3;
     const int c0 = ((warp - 2) >> 2) * NCH;
-    float *stg = epi + (warp - 2) * 32 * EPI_PITCH;
+    float *stg = epi + (warp - 2) * EPI_TILE;
     int lt = 0;
     for (int tile = blockIdx.x; tile < b.total_tiles; tile += gridDim.x, ++lt) {
       const TcItem &it = b.it[find_item(b, tile)];
@@ -382,21 +442,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
       int mt, nt;
       tile_pos(it, local, mt, nt);
       const int acc = lt & 1;
-      const int row0 = mt * TC_BM + q * 32;
-      float cv[32];
-      load_c(it, row0, min(32, it.m - row0), nt * BN + c0 * 32 + lane, beta, cv);
-      const bool ready = mbar_wait(smem_u32(&tfull_bar[acc]), (uint32_t)((lt >> 1) & 1), &abort_s);
-      // the whole warp takes the same branch (tcgen05.ld below is a warp-collective)
-      if (!__all_sync(0xffffffffu, ready && !abort_s)) {
+      const bool ok = drain_tile_vec<NCH, F16>(
+          it, tmem + (uint32_t)(acc * BN), mt, nt * BN, q, c0, lane, stg, alpha, beta,
+          [&] {
+            const bool ready = mbar_wait(smem_u32(&tfull_bar[acc]), (uint32_t)((lt >> 1) & 1), &abort_s);
+            // the whole warp takes the same branch (tcgen05.ld is a warp-collective)
+            const bool go = __all_sync(0xffffffffu, ready && !abort_s);
+            fence_after();
+            return go;
+          },
+          [&] {
+            fence_before();
+            mbar_arrive(smem_u32(&tempty_bar[acc]));
+          });
+      if (!ok) {
         if (lane == 0) atomicOr(err, DS_WAIT_TIMEOUT);
         abort_s = 1;
         break;
       }
-      fence_after();
-      drain_tile<NCH, F16>(it, tmem + (uint32_t)(acc * BN), mt, nt * BN, q, c0, lane, stg, alpha, beta, cv, [&] {
-        fence_before();
-        mbar_arrive(smem_u32(&tempty_bar[acc]));
-      });
     }
   }
   fence_before();
@@ -628,7 +691,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
     const int q = warp & 3;
     constexpr int NCH = TC_BN / 64;
     const int c0 = ((warp - 2) >> 2) * NCH;
-    float *stg = epi + (warp - 2) * 32 * EPI_PITCH;
+    float *stg = epi + (warp - 2) * EPI_TILE;
     const uint32_t tempty_leader0 = map_to_rank(smem_u32(&tempty_bar[0]), 0);
     const uint32_t tempty_leader1 = map_to_rank(smem_u32(&tempty_bar[1]), 0);
     int lt = 0;
@@ -638,21 +701,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
       pair_pos(it, pt - it.tile0, mp, nt);
       const int mt = 2 * mp + (int)rank;  // rows beyond m (a missing second row) are masked
       const int acc = lt & 1;
-      const int row0 = mt * TC_BM + q * 32;
-      float cv[32];
-      load_c(it, row0, min(32, it.m - row0), nt * TC_BN + c0 * 32 + lane, beta, cv);
-      const bool ready = mbar_wait_cl(smem_u32(&tfull_bar[acc]), (uint32_t)((lt >> 1) & 1), &abort_s);
-      if (!__all_sync(0xffffffffu, ready && !abort_s)) {
+      const bool ok = drain_tile_vec<NCH, true>(
+          it, tmem + (uint32_t)(acc * TC_BN), mt, nt * TC_BN, q, c0, lane, stg, alpha, beta,
+          [&] {
+            const bool ready = mbar_wait_cl(smem_u32(&tfull_bar[acc]), (uint32_t)((lt >> 1) & 1), &abort_s);
+            const bool go = __all_sync(0xffffffffu, ready && !abort_s);
+            fence_after();
+            return go;
+          },
+          [&] {
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
+          });
+      if (!ok) {
         if (lane == 0) atomicOr(err, DS_WAIT_TIMEOUT);
         abort_s = 1;
         break;
       }
-      fence_after();
-      drain_tile<NCH, true>(it, tmem + (uint32_t)(acc * TC_BN), mt, nt * TC_BN, q, c0, lane, stg, alpha, beta, cv, [&] {
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(acc ? tempty_leader1 : tempty_leader0);
-      });
     }
   }
   fence_before();
@@ -1163,12 +1229,14 @@ static size_t packed_bytes(size_t tiles, size_t tile_bytes, size_t scales) {
   return 2 * tiles * tile_bytes + (scales * sizeof(float) + 255) / 256 * 256;
 }
 
-// Output tiles of the launch when they are BN wide: sets each item's tile counts and first tile
+// Output tiles of the launch when they are BN wide: sets each item's tile counts, first tile and width of
+// access to C
 static int set_tiles(TcBatchP &tb, int BN) {
   int tiles = 0;
   for (int i = 0; i < tb.count; ++i) {
     TcItem &it = tb.it[i];
     it.ntc = ceil_div(it.n2, BN);
+    it.vec = it.ldc % 4 == 0 && (uintptr_t)it.C % 16 == 0 ? 4 : 1;
     it.colmajor = tc_tile_order(it.mtc, it.ntc, it.nkt);
     it.tile0 = tiles;
     tiles += it.mtc * it.ntc;

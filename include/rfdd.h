@@ -332,9 +332,10 @@ int rfdd_cgemm(int64_t m, int64_t n, int64_t k, const float *A, int64_t lda, con
  * matrices, the interior CholQR, the Rayleigh-Ritz Gram matrices and Ritz vector updates):
  * C = beta*C + alpha*op(A)*op(B) for FP64 host arrays, row-major; op(X) = X^T when the flag is 1
  * (A then stored k x m with leading dimension lda >= m; B stored n x k with ldb >= k).
- * engine 0 = FP64 CUDA-core kernel; 1 = the double-FP32 kernel the solver uses for these
- * products (each operand split into two floats, error-free products and compensated sums:
- * |error| within about 2^-42 of sum_k |a_ik||b_kj|).  sym = 1 declares op(A)*op(B) symmetric
+ * engine 0 = FP64 CUDA-core kernel; 1 = the kernels the solver uses for these products: large ones by
+ * exact digit products on the tensor cores (55-bit operands relative to the largest entry of their row of op(A) or
+ * column of op(B)), the others in double-FP32 (each operand split into two floats, error-free products
+ * and compensated sums: |error| within about 2^-42 of sum_k |a_ik||b_kj|).  sym = 1 declares op(A)*op(B) symmetric
  * (m == n required): only the upper 64 x 64 tiles are formed and mirrored.
  * Deep K with few output tiles is split over CTAs and the partial tiles summed in a fixed order. */
 int rfdd_dgemm(int64_t m, int64_t n, int64_t k, int32_t ta, const double *A, int64_t lda, int32_t tb,
@@ -381,7 +382,8 @@ int rfdd_cgemm_noalloc(int64_t m, int64_t n, int64_t k, const float *A, int64_t 
 /* ---- measurement hooks (no counterpart in the paper) -------------------------------------
  * rfdd_kernel_launches: number of kernels this library has launched in this process.
  * rfdd_profile(1): clear the records and time every launch of the dense contraction kernels
- * (kind 0: CUDA-core GEMM, kind 1: tensor-core GEMM) with CUDA events on their stream;
+ * (kind 0: FP64-operand and other CUDA-core GEMM, kind 1: FP32 tensor-core GEMM) with CUDA events on
+ * their stream;
  * rfdd_profile(0) stops recording.  rfdd_profile_get sums, for one kind, the launches, their
  * event-measured milliseconds and their algorithmic flops (a complex multiply-add counts 8).
  * rfdd_profile_busy gives, for one kind, the milliseconds during which at least one recorded

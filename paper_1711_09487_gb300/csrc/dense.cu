@@ -354,13 +354,17 @@ void gemm_launch_batches(cudaStream_t st, const std::vector<GemmItem<T>> &live, 
 
 void gemm_f64x2_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
                         double beta, const std::vector<char> &sym) {
-  std::vector<GemmItem<double>> live;
-  std::vector<char> symv;
+  // large products go to the tensor cores (exact digit products), the others stay on the CUDA cores
+  std::vector<GemmItem<double>> live, big;
+  std::vector<char> symv, bigsym;
   for (size_t i = 0; i < items.size(); ++i)
     if (items[i].m > 0 && items[i].n > 0) {
-      live.push_back(items[i]);
-      symv.push_back(sym.empty() ? 0 : sym[i]);
+      const bool tc = tc_status_word() && tc_dgemm_takes(items[i]);
+      (tc ? big : live).push_back(items[i]);
+      (tc ? bigsym : symv).push_back(sym.empty() ? 0 : sym[i]);
     }
+  if (!big.empty()) tc_dgemm_batched(st, big, ta, tb, alpha, beta, bigsym);
+  if (live.empty()) return;
   gemm_launch_batches<double>(st, live, symv, alpha, beta, [&](dim3 grid, const GemmBatchP<double> &b) {
     if (!ta && !tb) gemm_df64_kernel<false, false><<<grid, 256, 0, st>>>(b, alpha, beta);
     else if (ta && !tb) gemm_df64_kernel<true, false><<<grid, 256, 0, st>>>(b, alpha, beta);

@@ -3892,9 +3892,17 @@ int rfdd_dgemm(int64_t m, int64_t n, int64_t k, int32_t ta, const double *A, int
     RFDD_CUDA(cudaMemcpy(c.p, C, ncm * sizeof(double), cudaMemcpyHostToDevice));
     std::vector<GemmItem<double>> it = {
         {a.as<double>(), b.as<double>(), c.as<double>(), (int)m, (int)n, (int)k, (int)lda, (int)ldb, (int)ldc}};
-    if (engine == 1) gemm_f64x2_batched(st, it, ta != 0, tb != 0, alpha, beta, {(char)(sym != 0)});
-    else gemm_simt_batched<double>(st, it, ta != 0, tb != 0, alpha, beta, {(char)(sym != 0)});
-    RFDD_CUDA(cudaStreamSynchronize(st));
+    Buf status;
+    status.alloc(sizeof(int));
+    RFDD_CUDA(cudaMemset(status.p, 0, sizeof(int)));
+    {
+      TcStatusScope tcs(status.as<int>());
+      if (engine == 1) gemm_f64x2_batched(st, it, ta != 0, tb != 0, alpha, beta, {(char)(sym != 0)});
+      else gemm_simt_batched<double>(st, it, ta != 0, tb != 0, alpha, beta, {(char)(sym != 0)});
+    }
+    int stt = 0;
+    RFDD_CUDA(cudaMemcpy(&stt, status.p, sizeof(int), cudaMemcpyDeviceToHost));
+    RFDD_REQUIRE(stt == 0, RFDD_ECUDA, "tensor-core GEMM reported a time-out");
     RFDD_CUDA(cudaMemcpy(C, c.p, ncm * sizeof(double), cudaMemcpyDeviceToHost));
   });
 }

@@ -1,0 +1,542 @@
+// FP64 GEMM on the tensor cores by exact digit products.
+//
+// Every row of op(A) and every column of op(B) is scaled by a power of two and rounded to a 55-bit
+// fixed-point integer, which is cut into eight balanced base-128 digits (-64 .. 63), each exact in
+// fp16.  The products of digit planes with equal weight, i + j = g, are summed by tcgen05 kind::f16
+// MMAs into one of eight FP32 accumulators: all addends are integers and their sums stay below 2^24
+// (8 pairs x 512 x 2^12), so every accumulator is exact.  After at most 512 terms of K the eight are read back and
+// added into two 64-bit integers per entry, which hold the sum exactly up to the planes that are left out (i + j
+// > 7, below 2^-50 of the product of the two scales per term); one rounding to FP64 at the end.  This
+// is the splitting of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59, 2012) with integer digits.
+//
+// What bounds it: the 36 plane products of a 128 x 64 x 32 stage read 12 KB of shared memory per 32
+// cycles of MMA (128 bytes per cycle is the limit), so a stage takes about 3500 cycles; that
+// is the bound from a few hundred terms on; below that the read-back (FP64 conversions) is.  Measured with
+// the packing: symmetric 1920 x 1920 x 64000 13.2 ms (134 ms in double-FP32), 384 x 384 x 64000 0.57 ms,
+// the 1885 x 1885 x 8000 product 9.2 -> 0.9 ms; its error falls from 8.2e-14 to 1.1e-15 of the norm.
+#include "dense.cuh"
+#include "tc_common.cuh"
+#include "tc_gemm.cuh"
+
+#include <algorithm>
+
+namespace rfdd {
+
+namespace {
+
+constexpr int DG_BM = 128, DG_BN = 64, DG_KT = 32;  // output tile, K of a stage
+constexpr int DG_PLANES = 8, DG_PAIRS = DG_PLANES / 2;  // a 128-byte tile row holds 32 K-values of two planes
+constexpr int DG_ATILE = DG_BM * 128, DG_BTILE = DG_BN * 128;  // bytes of one plane pair
+constexpr int DG_ABYTES = DG_PAIRS * DG_ATILE, DG_BBYTES = DG_PAIRS * DG_BTILE;
+constexpr int DG_STAGE = DG_ABYTES + DG_BBYTES;  // 96 KB
+constexpr int DG_STAGES = 2;
+constexpr int DG_CHUNK = 16;   // stages between two read-backs (512 terms)
+constexpr int DG_SMEM = DG_STAGES * DG_STAGE + 1024;
+constexpr int DG_EPI_WARPS = 8;
+constexpr int DG_THREADS = 64 + 32 * DG_EPI_WARPS;
+constexpr int DG_MAXB = 32;
+
+// One operand: vectors (rows of op(A), columns of op(B)) of length k
+struct DigitItem {
+  const double *src;
+  long long ld;
+  int nv, k;        // vectors, length
+  int kcontig;      // 1: entry (v, k) at src[v * ld + k]; 0: at src[k * ld + v]
+  int vb;           // vectors per tile (128 or 64)
+  int nkt;
+  uint8_t *dst;
+  int *emax;        // per vector: largest high word of |x|
+};
+struct DigitBatch {
+  DigitItem it[2 * DG_MAXB];
+  int count;
+};
+
+// Largest high word (sign dropped) of every vector, into emax (zeroed before).
+__global__ void __launch_bounds__(256) digit_emax_kernel(const __grid_constant__ DigitBatch b) {
+  const DigitItem &it = b.it[blockIdx.y];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (it.kcontig) {
+    for (int v = blockIdx.x * 8 + warp; v < it.nv; v += gridDim.x * 8) {
+      const double *s = it.src + (long long)v * it.ld;
+      int m = 0;
+      for (int k = lane; k < it.k; k += 32) m = max(m, __double2hiint(s[k]) & 0x7fffffff);
+      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0) it.emax[v] = m;
+    }
+  } else {
+    // 32 vectors x 256 rows per block step
+    const int nvb = (it.nv + 31) / 32, nkb = (it.k + 255) / 256;
+    for (int u = blockIdx.x; u < nvb * nkb; u += gridDim.x) {
+      const int v = (u % nvb) * 32 + lane, k0 = (u / nvb) * 256 + warp;
+      int m = 0;
+      if (v < it.nv)
+#pragma unroll 8
+        for (int q = 0; q < 32; ++q) {
+          const int k = k0 + 8 * q;
+          if (k < it.k) m = max(m, __double2hiint(it.src[(long long)k * it.ld + v]) & 0x7fffffff);
+        }
+      if (m > 0) atomicMax(it.emax + v, m);
+    }
+  }
+}
+
+// Fixed point of x for a vector whose largest high word is em: x 2^(54 - 1 - E), E the exponent of the largest
+// entry, rounded to nearest: |q| < 2^54.
+__device__ __forceinline__ long long fixed55(double x, int em) {
+  const long long bits = __double_as_longlong(x);
+  const int ex = (int)((bits >> 52) & 0x7ff), emx = em >> 20;
+  if (emx == 0x7ff || ex == 0x7ff) return 0;  // infinities and NaN: the vector's scale is NaN
+  long long m = bits & 0xfffffffffffffll;
+  if (ex > 0) m |= 1ll << 52;
+  // m < 2^53; the largest entry becomes m * 2, smaller exponents shift right
+  const int sh = max(emx, 1) - max(ex, 1) - 1;
+  long long q;
+  if (sh < 0) q = m << 1;
+  else if (sh == 0) q = m;
+  else if (sh > 54) q = 0;
+  else q = (m + (1ll << (sh - 1))) >> sh;
+  return bits < 0 ? -q : q;
+}
+// Scale of the vector: x = q * 2^(E - 1023 - 53), as a double (NaN when an entry was not finite)
+__device__ __forceinline__ int digit_exp(int em) { return max(em >> 20, 1) - 1023 - 53; }
+
+// v 2^e: by the exponent field where the result is normal (the FP64 pipe is slow), else by scalbn
+__device__ __forceinline__ double scale_exp(double v, int e) {
+  const int ex = (__double2hiint(v) >> 20) & 0x7ff;
+  if (ex == 0) return v;  // zero (|v| is an integer)
+  if (ex + e >= 1 && ex + e <= 2046) return __hiloint2double(__double2hiint(v) + (e << 20), __double2loint(v));
+  return scalbn(v, e);
+}
+
+// Digits of every operand into swizzled tiles: tile (v / vb, k / 32), four plane pairs of vb rows x 128 bytes;
+// 16-byte chunk c of a row holds plane 2 * pair + c / 4, K-values 8 (c % 4) .. + 7, at chunk c ^ (row & 7).  A
+// block stages 64 vectors x 32 K-values.
+__global__ void __launch_bounds__(256) digit_pack_kernel(const __grid_constant__ DigitBatch b) {
+  const DigitItem &it = b.it[blockIdx.y];
+  __shared__ double sx[64][33];
+  const int tid = threadIdx.x;
+  const int nvb = (it.nv + 63) / 64, total = nvb * it.nkt;
+  for (int u = blockIdx.x; u < total; u += gridDim.x) {
+    const int v0 = (u / it.nkt) * 64, kt = u % it.nkt, k0 = kt * DG_KT;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int id = tid + 256 * q;
+      const int v = it.kcontig ? id >> 5 : id & 63, k = it.kcontig ? id & 31 : id >> 6;
+      double x = 0.0;
+      if (v0 + v < it.nv && k0 + k < it.k)
+        x = it.kcontig ? it.src[(long long)(v0 + v) * it.ld + k0 + k] : it.src[(long long)(k0 + k) * it.ld + v0 + v];
+      sx[v][k] = x;
+    }
+    __syncthreads();
+    const int v = tid >> 2, g = tid & 3;  // 8 K-values of one vector
+    const int em = v0 + v < it.nv ? it.emax[v0 + v] : 0;
+    uint32_t w[DG_PLANES][4];
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) {
+      // q + sum_s 64 * 128^s has the digits plus 64 as its base-128 digits
+      const unsigned long long off = 0x0081020408102040ull << 0;
+      const unsigned long long a = (unsigned long long)fixed55(sx[v][g * 8 + e], em) + off;
+      const unsigned long long c = (unsigned long long)fixed55(sx[v][g * 8 + e + 1], em) + off;
+#pragma unroll
+      for (int s = 0; s < DG_PLANES; ++s) {
+        const int shift = 7 * (DG_PLANES - 1 - s);  // plane 0 is the leading digit
+        const uint32_t d = ((uint32_t)(a >> shift) & 127u) | (((uint32_t)(c >> shift) & 127u) << 16);
+        // fp16(1024 + u) - 1088 = u - 64, exactly
+        const uint32_t h = d | 0x64006400u;
+        __half2 x = *reinterpret_cast<const __half2 *>(&h);
+        x = __hsub2(x, __half2half2(__ushort_as_half(0x6440)));
+        w[s][e >> 1] = *reinterpret_cast<uint32_t *>(&x);
+      }
+    }
+    const int vv = v0 + v, r = vv % it.vb;
+    uint8_t *t = it.dst + ((long long)(vv / it.vb) * it.nkt + kt) * DG_PAIRS * it.vb * 128 + r * 128;
+#pragma unroll
+    for (int s = 0; s < DG_PLANES; ++s) {
+      const int c = (s & 1) * 4 + g;
+      *reinterpret_cast<uint4 *>(t + (s >> 1) * it.vb * 128 + ((c ^ (r & 7)) << 4)) =
+          make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+    }
+  }
+}
+
+struct DgItem {
+  const uint8_t *A, *B;
+  const int *ea, *eb;
+  double *C, *ws;      // ws: partial sums (split K), nsplit slabs of m x n
+  long long ldc;
+  int m, n, nkt, ntc;  // ntc: 64-wide tiles per row of tiles
+  int nsplit, kper;    // K splits and stages per split
+  int sym, unit0;      // first work unit (tile, split)
+};
+struct DgBatch {
+  DgItem it[DG_MAXB];
+  int count, units;
+  int *err;
+};
+
+// Work unit -> tile row, tile column, split.  A symmetric product keeps the tiles that reach the upper
+// triangle: tile row mt has the columns from 2 mt on.
+__device__ __forceinline__ void dg_unit(const DgItem &it, int u, int &mt, int &nt, int &sp) {
+  sp = u % it.nsplit;
+  int t = u / it.nsplit;
+  if (!it.sym) {
+    mt = t / it.ntc;
+    nt = t % it.ntc;
+    return;
+  }
+  mt = 0;
+  while (t >= it.ntc - 2 * mt) {
+    t -= it.ntc - 2 * mt;
+    ++mt;
+  }
+  nt = 2 * mt + t;
+}
+
+__global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_constant__ DgBatch b, double alpha,
+                                                                 double beta) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t full_bar[DG_STAGES], empty_bar[DG_STAGES], tfull_bar, tempty_bar;
+  __shared__ uint32_t tmem_s;
+  __shared__ volatile int abort_s;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < DG_STAGES; ++s) {
+      mbar_init(smem_u32(&full_bar[s]), 1);
+      mbar_init(smem_u32(&empty_bar[s]), 1);
+    }
+    mbar_init(smem_u32(&tfull_bar), 1);
+    mbar_init(smem_u32(&tempty_bar), 32 * DG_EPI_WARPS);
+    abort_s = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)),
+                 "r"(DG_PLANES * DG_BN)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = tmem_s;
+  auto find = [&](int u) {
+    int lo = 0, hi = b.count;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (b.it[mid].unit0 <= u) lo = mid;
+      else hi = mid;
+    }
+    return lo;
+  };
+  if (warp == 0) {
+    if (lane == 0) {  // producer: 96 KB of digits per stage
+      long long g = 0;
+      for (int u = blockIdx.x; u < b.units && !abort_s; u += gridDim.x) {
+        const DgItem &it = b.it[find(u)];
+        int mt, nt, sp;
+        dg_unit(it, u - it.unit0, mt, nt, sp);
+        const int kb = sp * it.kper, ke = min(it.nkt, kb + it.kper);
+        const uint8_t *A = it.A + (long long)mt * it.nkt * DG_ABYTES, *B = it.B + (long long)nt * it.nkt * DG_BBYTES;
+        for (int kt = kb; kt < ke; ++kt, ++g) {
+          const int s = (int)(g % DG_STAGES);
+          const long long r = g / DG_STAGES;
+          if (r >= 1 && !mbar_wait(smem_u32(&empty_bar[s]), (uint32_t)((r - 1) & 1), &abort_s)) {
+            atomicOr(b.err, DS_WAIT_TIMEOUT);
+            abort_s = 1;
+            break;
+          }
+          const uint32_t fb = smem_u32(&full_bar[s]), dst = smem_u32(base + s * DG_STAGE);
+          mbar_expect_tx(fb, DG_STAGE);
+          bulk_g2s(dst, A + (long long)kt * DG_ABYTES, DG_ABYTES, fb);
+          bulk_g2s(dst + DG_ABYTES, B + (long long)kt * DG_BBYTES, DG_BBYTES, fb);
+        }
+      }
+      // every issued copy lands before the CTA can exit
+      for (long long q = (g > DG_STAGES ? g - DG_STAGES : 0); q < g; ++q)
+        mbar_wait(smem_u32(&full_bar[q % DG_STAGES]), (uint32_t)((q / DG_STAGES) & 1), &abort_s);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {  // MMA issuer
+      const uint32_t idesc = (1u << 4) | ((uint32_t)(DG_BN >> 3) << 17) | ((uint32_t)(DG_BM >> 4) << 24);
+      long long g = 0, ch = 0;  // stages, read-backs
+      bool ok = true;
+      for (int u = blockIdx.x; u < b.units && ok && !abort_s; u += gridDim.x) {
+        const DgItem &it = b.it[find(u)];
+        int mt, nt, sp;
+        dg_unit(it, u - it.unit0, mt, nt, sp);
+        const int kb = sp * it.kper, ke = min(it.nkt, kb + it.kper);
+        for (int k0 = kb; k0 < ke && ok; k0 += DG_CHUNK, ++ch) {
+          if (ch >= 1 && !mbar_wait(smem_u32(&tempty_bar), (uint32_t)((ch - 1) & 1), &abort_s)) {
+            ok = false;
+            break;
+          }
+          fence_after();
+          const int k1 = min(ke, k0 + DG_CHUNK);
+          for (int kt = k0; kt < k1; ++kt, ++g) {
+            const int s = (int)(g % DG_STAGES);
+            if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)((g / DG_STAGES) & 1), &abort_s)) {
+              ok = false;
+              break;
+            }
+            fence_after();
+            const uint32_t sa = smem_u32(base + s * DG_STAGE), sb = sa + DG_ABYTES;
+#pragma unroll 1
+            for (int kk = 0; kk < 2; ++kk) {
+#pragma unroll
+              for (int i = 0; i < DG_PLANES; ++i) {
+                const uint64_t da = sdesc(sa + (i >> 1) * DG_ATILE + (i & 1) * 64 + kk * 32);
+#pragma unroll
+                for (int j = 0; j < DG_PLANES - i; ++j)
+                  mma_f16(tmem + (uint32_t)((i + j) * DG_BN), da, sdesc(sb + (j >> 1) * DG_BTILE + (j & 1) * 64 + kk * 32),
+                          idesc, (kt > k0 || kk > 0 || i > 0) ? 1u : 0u);
+              }
+            }
+            mma_commit(smem_u32(&empty_bar[s]));
+          }
+          if (ok) mma_commit(smem_u32(&tfull_bar));
+        }
+      }
+      if (!ok) {
+        atomicOr(b.err, DS_WAIT_TIMEOUT);
+        abort_s = 1;
+      }
+    }
+  } else {
+    // read-back: warp w takes accumulator lanes 32 (w % 4) .. (its rows) and half of the columns
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    long long ch = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < b.units && ok; u += gridDim.x) {
+      const DgItem &it = b.it[find(u)];
+      int mt, nt, sp;
+      dg_unit(it, u - it.unit0, mt, nt, sp);
+      const int kb = sp * it.kper, ke = min(it.nkt, kb + it.kper);
+      long long hi[32], lo[32];
+#pragma unroll
+      for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
+      for (int k0 = kb; k0 < ke; k0 += DG_CHUNK, ++ch) {
+        const bool ready = mbar_wait(smem_u32(&tfull_bar), (uint32_t)(ch & 1), &abort_s);
+        if (!__all_sync(0xffffffffu, ready && !abort_s)) {
+          if (lane == 0) atomicOr(b.err, DS_WAIT_TIMEOUT);
+          abort_s = 1;
+          ok = false;
+          break;
+        }
+        fence_after();
+        const uint32_t t0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32);
+#pragma unroll
+        for (int g = 0; g < DG_PLANES; ++g) {
+          uint32_t v[32];
+          TC_LD32(t0 + (uint32_t)(g * DG_BN), v);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (g == DG_PLANES - 1) {
+            fence_before();
+            mbar_arrive(smem_u32(&tempty_bar));
+          }
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const int x = __float2int_rn(__uint_as_float(v[j]));
+            if (g < 4) hi[j] += (long long)x * (1 << (7 * (3 - g)));
+            else lo[j] += (long long)x * (1 << (7 * (7 - g)));
+          }
+        }
+      }
+      if (!ok) break;
+      // planes 0 and 0 weigh 2^98 in units of the two integers; hi counts 2^77, lo 2^49
+      const int i = mt * DG_BM + q * 32 + lane;
+      if (i < it.m) {
+        const int eai = it.ea[i];
+        const int xa = digit_exp(eai) + 49;
+        const int j0 = nt * DG_BN + half * 32;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const int c = j0 + j;
+          if (c >= it.n) continue;
+          const int ebj = it.eb[c];
+          double v = fma((double)hi[j], 268435456.0, (double)lo[j]);
+          v = scale_exp(v, xa + digit_exp(ebj));
+          if ((eai >> 20) == 0x7ff || (ebj >> 20) == 0x7ff) v = __longlong_as_double(0x7ff8000000000000ll);
+          if (it.nsplit > 1) {
+            it.ws[((long long)sp * it.m + i) * it.n + c] = v;
+            continue;
+          }
+          if (it.sym && i > c) continue;
+          v *= alpha;
+          double *p = it.C + (long long)i * it.ldc + c;
+          *p = beta != 0.0 ? fma(beta, *p, v) : v;
+          if (it.sym && i != c) {
+            double *pm = it.C + (long long)c * it.ldc + i;
+            *pm = beta != 0.0 ? fma(beta, *pm, v) : v;
+          }
+        }
+      }
+    }
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(DG_PLANES * DG_BN) : "memory");
+}
+
+// Split K: the partial sums of every entry, in order
+__global__ void __launch_bounds__(256) tc_dgemm_reduce_kernel(const __grid_constant__ DgBatch b, double alpha,
+                                                              double beta) {
+  const DgItem &it = b.it[blockIdx.y];
+  if (it.nsplit <= 1) return;
+  const long long mn = (long long)it.m * it.n;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < mn; e += (long long)gridDim.x * blockDim.x) {
+    const long long i = e / it.n, j = e % it.n;
+    const long long src = it.sym && i > j ? j * it.n + i : e;  // exactly symmetric result
+    double v = it.ws[src];
+    for (int s = 1; s < it.nsplit; ++s) v += it.ws[s * mn + src];
+    v *= alpha;
+    double *p = it.C + i * it.ldc + j;
+    *p = beta != 0.0 ? fma(beta, *p, v) : v;
+  }
+}
+
+}  // namespace
+
+bool tc_dgemm_takes(const GemmItem<double> &g) {
+  return g.m >= 48 && g.n >= 48 && g.k >= 48 && (double)g.m * g.n * g.k >= 6.4e7;
+}
+
+void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
+                      double beta, const std::vector<char> &sym) {
+  RFDD_REQUIRE(tc_status_word() != nullptr, RFDD_ESTATE, "tensor-core GEMM launched without a status word");
+  const int nsm = sm_count();
+  RFDD_CUDA(cudaFuncSetAttribute(tc_dgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM));
+  for (size_t s0 = 0; s0 < items.size(); s0 += DG_MAXB) {
+    const int cnt = (int)std::min<size_t>(DG_MAXB, items.size() - s0);
+    int kmax = 0;
+    double per_k = 0.0;  // bytes of digits per unit of K
+    for (int i = 0; i < cnt; ++i) {
+      const auto &g = items[s0 + i];
+      kmax = std::max(kmax, g.k);
+      per_k += 16.0 * (((g.m + 127) / 128) * 128.0 + ((g.n + 63) / 64) * 64.0);
+    }
+    // K in passes whose digits fit in 1.5 GB; every pass but the first adds to C
+    const int kpass = std::min<double>(kmax, std::max(512.0, std::floor(1.5e9 / per_k / 512.0) * 512.0));
+    for (int kp = 0; kp < kmax; kp += kpass) {
+      DigitBatch db;
+      DgBatch gb;
+      memset(&db, 0, sizeof(db));
+      memset(&gb, 0, sizeof(gb));
+      size_t bytes = 0, vecs = 0, wsum = 0;
+      struct Src { const double *p; int ld, nv, k, kc, vb; size_t off, ev; };
+      std::vector<Src> srcs;  // operands, each packed once even when several items use it
+      auto operand = [&](const double *p, int ld, int nv, int k, int kc, int vb) {
+        for (size_t q = 0; q < srcs.size(); ++q)
+          if (srcs[q].p == p && srcs[q].ld == ld && srcs[q].nv == nv && srcs[q].k == k && srcs[q].kc == kc && srcs[q].vb == vb)
+            return (int)q;
+        const size_t nkt = (k + DG_KT - 1) / DG_KT, tiles = (nv + vb - 1) / vb;
+        srcs.push_back({p, ld, nv, k, kc, vb, bytes, vecs});
+        bytes += tiles * nkt * DG_PAIRS * vb * 128;
+        vecs += (size_t)(nv + 63) / 64 * 64;
+        return (int)srcs.size() - 1;
+      };
+      std::vector<int> ia, ib;
+      double work = 0.0;
+      for (int i = 0; i < cnt; ++i) {
+        const auto &g = items[s0 + i];
+        const int k = std::min(kpass, g.k - kp);
+        ia.push_back(-1);
+        ib.push_back(-1);
+        if (k <= 0) continue;
+        ia[i] = operand(g.A + (ta ? (int64_t)kp * g.lda : kp), g.lda, g.m, k, ta ? 0 : 1, DG_BM);
+        ib[i] = operand(g.B + (tb ? kp : (int64_t)kp * g.ldb), g.ldb, g.n, k, tb ? 1 : 0, DG_BN);
+        DgItem &x = gb.it[gb.count];
+        x.m = g.m;
+        x.n = g.n;
+        x.C = g.C;
+        x.ldc = g.ldc;
+        x.nkt = (k + DG_KT - 1) / DG_KT;
+        x.ntc = (g.n + DG_BN - 1) / DG_BN;
+        x.sym = !sym.empty() && sym[s0 + i];
+        const int mtc = (g.m + DG_BM - 1) / DG_BM;
+        int tiles = 0;
+        for (int m = 0; m < mtc; ++m) tiles += x.sym ? std::max(0, x.ntc - 2 * m) : x.ntc;
+        x.unit0 = tiles;  // until the splits are known
+        work += (double)tiles * x.nkt;
+        ++gb.count;
+      }
+      // splits: about three units of work per SM, none shallower than 512 terms
+      const double target = std::max<double>(DG_CHUNK, std::ceil(work / (3.0 * nsm) / DG_CHUNK) * DG_CHUNK);
+      int units = 0, splits = 1;
+      for (int q = 0; q < gb.count; ++q) {
+        DgItem &x = gb.it[q];
+        const int tiles = x.unit0;
+        x.nsplit = std::min(32, std::max(1, (int)std::floor(x.nkt / target)));
+        x.kper = (x.nkt + x.nsplit - 1) / x.nsplit;
+        x.kper = (x.kper + DG_CHUNK - 1) / DG_CHUNK * DG_CHUNK;
+        x.nsplit = (x.nkt + x.kper - 1) / x.kper;
+        x.unit0 = units;
+        units += tiles * x.nsplit;
+        splits = std::max(splits, x.nsplit);
+        if (x.nsplit > 1) wsum += (size_t)x.nsplit * x.m * x.n;
+      }
+      gb.units = units;
+      gb.err = tc_status_word();
+      uint8_t *ws = nullptr;
+      const size_t ebytes = (vecs * sizeof(int) + 255) / 256 * 256;
+      RFDD_CUDA(cudaMallocAsync((void **)&ws, ebytes + bytes + wsum * sizeof(double), st));
+      int *emax = reinterpret_cast<int *>(ws);
+      double *part = reinterpret_cast<double *>(ws + ebytes + bytes);
+      RFDD_CUDA(cudaMemsetAsync(emax, 0, ebytes, st));
+      long long be = 1, bp = 1;
+      for (const Src &s : srcs) {
+        const int nkt = (s.k + DG_KT - 1) / DG_KT;
+        db.it[db.count++] = {s.p, s.ld, s.nv, s.k, s.kc, s.vb, nkt, ws + ebytes + s.off, emax + s.ev};
+        be = std::max<long long>(be, s.kc ? (s.nv + 7) / 8 : (long long)((s.nv + 31) / 32) * ((s.k + 255) / 256));
+        bp = std::max<long long>(bp, (long long)((s.nv + 63) / 64) * nkt);
+      }
+      for (int i = 0, q = 0; i < cnt; ++i) {
+        if (ia[i] < 0) continue;
+        DgItem &x = gb.it[q++];
+        const Src &a = srcs[ia[i]], &c = srcs[ib[i]];
+        x.A = ws + ebytes + a.off;
+        x.B = ws + ebytes + c.off;
+        x.ea = emax + a.ev;
+        x.eb = emax + c.ev;
+        if (x.nsplit > 1) {
+          x.ws = part;
+          part += (size_t)x.nsplit * x.m * x.n;
+        }
+      }
+      digit_emax_kernel<<<dim3((unsigned)std::min<long long>(be, 2048), db.count), 256, 0, st>>>(db);
+      RFDD_CHECK_LAUNCH();
+      digit_pack_kernel<<<dim3((unsigned)std::min<long long>(bp, 4096), db.count), 256, 0, st>>>(db);
+      RFDD_CHECK_LAUNCH();
+      const double bt = kp == 0 ? beta : 1.0;
+      cudaEvent_t e0 = nullptr, e1 = nullptr;
+      if (profiling_enabled()) {
+        e0 = profile_event();
+        e1 = profile_event();
+        cudaEventRecord(e0, st);
+      }
+      tc_dgemm_kernel<<<std::max(1, std::min(units, nsm)), DG_THREADS, DG_SMEM, st>>>(gb, alpha, bt);
+      RFDD_CHECK_LAUNCH();
+      if (splits > 1) {
+        tc_dgemm_reduce_kernel<<<dim3(512, gb.count), 256, 0, st>>>(gb, alpha, bt);
+        RFDD_CHECK_LAUNCH();
+      }
+      if (e0) {
+        double flops = 0.0;
+        for (int i = 0; i < cnt; ++i) {
+          const auto &g = items[s0 + i];
+          flops += 2.0 * g.m * (double)g.n * std::max(0, std::min(kpass, g.k - kp));
+        }
+        cudaEventRecord(e1, st);
+        profile_push(e0, e1, flops, 0);
+      }
+      RFDD_CUDA(cudaFreeAsync(ws, st));
+    }
+  }
+}
+
+}  // namespace rfdd

@@ -15,6 +15,8 @@ struct TcStatusScope {
   TcStatusScope(const TcStatusScope &) = delete;
   TcStatusScope &operator=(const TcStatusScope &) = delete;
 };
+// the calling thread's status word (nullptr outside any scope)
+int *tc_status_word();
 // While alive, the tensor-core kernel launches of the calling host thread record ab[0] just before
 // and ab[1] just after the kernel (not the operand packing): the probes time the MMA kernel alone.
 struct TcKernelEvents {
@@ -41,6 +43,12 @@ void tc_gemm_real(cudaStream_t st, const std::vector<GemmItem<float>> &items, do
 // the same with one TF32 product per multiply (operands rounded to TF32): the throughput probe of
 // the plain TF32 tensor path, not used by the solver
 void tc_gemm_real_tf32(cudaStream_t st, const GemmItem<float> &item, double alpha, double beta);
+
+// FP64 products by exact digit products on the tensor cores (tc_dgemm.cu): C = beta*C + alpha*op(A)*op(B), op as
+// in gemm_batched, sym as in gemm_f64x2_batched.  tc_dgemm_takes: whether an item is large enough to gain.
+bool tc_dgemm_takes(const GemmItem<double> &g);
+void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
+                      double beta, const std::vector<char> &sym);
 
 // The tile-shape autotuner: mode 0 off (fixed rule), 1 on, 2 forget every class (re-tune);
 // returns whether it was on.  tc_autotune_table: one line per class (tc_tune.h, Tuner::dump).

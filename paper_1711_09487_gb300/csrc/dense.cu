@@ -352,11 +352,12 @@ void gemm_launch_batches(cudaStream_t st, const std::vector<GemmItem<T>> &live, 
   }
 }
 
-void gemm_f64x2_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
-                        double beta, const std::vector<char> &sym) {
-  // large products go to the tensor cores (exact digit products), the others stay on the CUDA cores
+// The large products of a batch go to the tensor cores (exact digit products); the others are left in live
+static std::vector<GemmItem<double>> split_large(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta,
+                                                 bool tb, double alpha, double beta, const std::vector<char> &sym,
+                                                 std::vector<char> &symv) {
   std::vector<GemmItem<double>> live, big;
-  std::vector<char> symv, bigsym;
+  std::vector<char> bigsym;
   for (size_t i = 0; i < items.size(); ++i)
     if (items[i].m > 0 && items[i].n > 0) {
       const bool tc = tc_status_word() && tc_dgemm_takes(items[i]);
@@ -364,6 +365,20 @@ void gemm_f64x2_batched(cudaStream_t st, const std::vector<GemmItem<double>> &it
       (tc ? bigsym : symv).push_back(sym.empty() ? 0 : sym[i]);
     }
   if (!big.empty()) tc_dgemm_batched(st, big, ta, tb, alpha, beta, bigsym);
+  return live;
+}
+
+void gemm_f64_basis_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb,
+                            double alpha, double beta, const std::vector<char> &sym) {
+  std::vector<char> symv;
+  const std::vector<GemmItem<double>> live = split_large(st, items, ta, tb, alpha, beta, sym, symv);
+  if (!live.empty()) gemm_simt_batched<double>(st, live, ta, tb, alpha, beta, symv);
+}
+
+void gemm_f64x2_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
+                        double beta, const std::vector<char> &sym) {
+  std::vector<char> symv;
+  const std::vector<GemmItem<double>> live = split_large(st, items, ta, tb, alpha, beta, sym, symv);
   if (live.empty()) return;
   gemm_launch_batches<double>(st, live, symv, alpha, beta, [&](dim3 grid, const GemmBatchP<double> &b) {
     if (!ta && !tb) gemm_df64_kernel<false, false><<<grid, 256, 0, st>>>(b, alpha, beta);
@@ -401,6 +416,18 @@ void gemm_batched(cudaStream_t st, const std::vector<GemmItem<T>> &items, bool t
       if (!live.empty()) tc_gemm_real(st, live, alpha, beta);
       if (!k0.empty()) gemm_simt_batched<T>(st, k0, false, false, alpha, beta);
       return;
+    }
+  }
+  if constexpr (std::is_same<typename ST<T>::real, double>::value) {
+    // FP64 products with enough work: exact digit products on the tensor cores
+    if (!ta && !tb && tc_status_word()) {
+      std::vector<GemmItem<T>> live, rest;
+      for (auto &g : items) (g.m > 0 && g.n > 0 && g.k > 0 ? live : rest).push_back(g);
+      if (!live.empty() && tc_fp64_takes<T>(live)) {
+        tc_fp64_batched<T>(st, live, alpha, beta);
+        if (beta != 1.0) gemm_simt_batched<T>(st, rest, false, false, alpha, beta);
+        return;
+      }
     }
   }
   gemm_simt_batched<T>(st, items, ta, tb, alpha, beta);

@@ -25,11 +25,14 @@ struct GemmItem {
 template <typename T>
 void gemm_batched(cudaStream_t st, const std::vector<GemmItem<T>> &items, bool ta, bool tb,
                   double alpha, double beta);
-// FP64 operands and result, double-FP32 arithmetic (relative error near 2^-46 of sum |a b|):
-// for products on eigenvector bases.  sym[i] != 0 marks a square product known to be symmetric
+// FP64 operands and result, for products on eigenvector bases: large ones by exact digit products on the
+// tensor cores (tc_dgemm.cu), the others in double-FP32 (relative error near 2^-46 of sum |a b|).  sym[i] != 0 marks a square product known to be symmetric
 // (A^T P A with P symmetric): only its upper tiles are formed and mirrored.
 void gemm_f64x2_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
                         double beta, const std::vector<char> &sym = {});
+// the same products of the plain FP64 solve: the CUDA-core FP64 kernel where they are small
+void gemm_f64_basis_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb,
+                            double alpha, double beta, const std::vector<char> &sym = {});
 // the CUDA-core kernel only (no tensor-core dispatch); sym as for gemm_f64x2_batched (real T)
 template <typename T>
 void gemm_simt_batched(cudaStream_t st, const std::vector<GemmItem<T>> &items, bool ta, bool tb,

@@ -1540,11 +1540,11 @@ void solve_S_levels(rfdd_handle *h, Tf *G, int64_t gs, int64_t m, const std::vec
 }
 
 // Products on the eigenvector bases (Lanczos blocks, interior CholQR, Rayleigh-Ritz Gram
-// matrices, Ritz-vector updates): double-FP32 arithmetic in the mixed-precision solve, FP64 in
-// the plain FP64 solve.
+// matrices, Ritz-vector updates): exact digit products where they are large; else double-FP32 arithmetic in
+// the mixed-precision solve, FP64 in the plain FP64 solve.
 void basis_gemm_on(const rfdd_handle *h, cudaStream_t st, const std::vector<GemmItem<double>> &g, bool ta, bool tb,
                    double alpha, double beta, const std::vector<char> &sym = {}) {
-  if (h->opt.precision == RFDD_FP64 || h->basis_fp64) gemm_simt_batched<double>(st, g, ta, tb, alpha, beta, sym);
+  if (h->opt.precision == RFDD_FP64 || h->basis_fp64) gemm_f64_basis_batched(st, g, ta, tb, alpha, beta, sym);
   else gemm_f64x2_batched(st, g, ta, tb, alpha, beta, sym);
 }
 void basis_gemm(const rfdd_handle *h, const std::vector<GemmItem<double>> &g, bool ta, bool tb, double alpha,

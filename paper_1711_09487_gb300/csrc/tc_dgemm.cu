@@ -41,7 +41,8 @@ struct DigitItem {
   const double *src;
   long long ld;
   int nv, k;        // vectors, length
-  int kcontig;      // 1: entry (v, k) at src[v * ld + k]; 0: at src[k * ld + v]
+  int mode;         // entry (v, k): 0 at src[k * ld + v]; 1 at src[v * ld + k]; 2: vector 2j + t, entry 2p + u of
+                    // the realified complex column j, [[re, im], [-im, re]] (rows u, columns t) of src[p * ld + j]
   int vb;           // vectors per tile (128 or 64)
   int nkt;
   uint8_t *dst;
@@ -56,7 +57,7 @@ struct DigitBatch {
 __global__ void __launch_bounds__(256) digit_emax_kernel(const __grid_constant__ DigitBatch b) {
   const DigitItem &it = b.it[blockIdx.y];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (it.kcontig) {
+  if (it.mode == 1) {
     for (int v = blockIdx.x * 8 + warp; v < it.nv; v += gridDim.x * 8) {
       const double *s = it.src + (long long)v * it.ld;
       int m = 0;
@@ -64,19 +65,28 @@ __global__ void __launch_bounds__(256) digit_emax_kernel(const __grid_constant__
       for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
       if (lane == 0) it.emax[v] = m;
     }
-  } else {
-    // 32 vectors x 256 rows per block step
-    const int nvb = (it.nv + 31) / 32, nkb = (it.k + 255) / 256;
-    for (int u = blockIdx.x; u < nvb * nkb; u += gridDim.x) {
-      const int v = (u % nvb) * 32 + lane, k0 = (u / nvb) * 256 + warp;
-      int m = 0;
-      if (v < it.nv)
+    return;
+  }
+  // 32 columns (of doubles or of complex pairs) x 256 rows per block step
+  const int f = it.mode == 2 ? 2 : 1;
+  const int nc = it.nv / f, kr = it.k / f;
+  const int nvb = (nc + 31) / 32, nkb = (kr + 255) / 256;
+  for (int u = blockIdx.x; u < nvb * nkb; u += gridDim.x) {
+    const int v = (u % nvb) * 32 + lane, k0 = (u / nvb) * 256 + warp;
+    int m = 0;
+    if (v < nc)
 #pragma unroll 8
-        for (int q = 0; q < 32; ++q) {
-          const int k = k0 + 8 * q;
-          if (k < it.k) m = max(m, __double2hiint(it.src[(long long)k * it.ld + v]) & 0x7fffffff);
+      for (int q = 0; q < 32; ++q) {
+        const int k = k0 + 8 * q;
+        if (k < kr) {
+          const double *s = it.src + ((long long)k * it.ld + v) * f;
+          m = max(m, __double2hiint(s[0]) & 0x7fffffff);
+          if (f == 2) m = max(m, __double2hiint(s[1]) & 0x7fffffff);
         }
-      if (m > 0) atomicMax(it.emax + v, m);
+      }
+    if (m > 0) {
+      atomicMax(it.emax + v * f, m);
+      if (f == 2) atomicMax(it.emax + 2 * v + 1, m);
     }
   }
 }
@@ -120,14 +130,31 @@ __global__ void __launch_bounds__(256) digit_pack_kernel(const __grid_constant__
   for (int u = blockIdx.x; u < total; u += gridDim.x) {
     const int v0 = (u / it.nkt) * 64, kt = u % it.nkt, k0 = kt * DG_KT;
     __syncthreads();
+    if (it.mode == 2) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int id = tid + 256 * q;
-      const int v = it.kcontig ? id >> 5 : id & 63, k = it.kcontig ? id & 31 : id >> 6;
-      double x = 0.0;
-      if (v0 + v < it.nv && k0 + k < it.k)
-        x = it.kcontig ? it.src[(long long)(v0 + v) * it.ld + k0 + k] : it.src[(long long)(k0 + k) * it.ld + v0 + v];
-      sx[v][k] = x;
+      for (int q = 0; q < 2; ++q) {
+        const int id = tid + 256 * q, j = id & 31, p = id >> 5;
+        double re = 0.0, im = 0.0;
+        if (v0 + 2 * j < it.nv && k0 + 2 * p < it.k) {
+          const double *s = it.src + 2 * ((long long)(k0 / 2 + p) * it.ld + v0 / 2 + j);
+          re = s[0];
+          im = s[1];
+        }
+        sx[2 * j][2 * p] = re;
+        sx[2 * j][2 * p + 1] = -im;
+        sx[2 * j + 1][2 * p] = im;
+        sx[2 * j + 1][2 * p + 1] = re;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int id = tid + 256 * q;
+        const int v = it.mode ? id >> 5 : id & 63, k = it.mode ? id & 31 : id >> 6;
+        double x = 0.0;
+        if (v0 + v < it.nv && k0 + k < it.k)
+          x = it.mode ? it.src[(long long)(v0 + v) * it.ld + k0 + k] : it.src[(long long)(k0 + k) * it.ld + v0 + v];
+        sx[v][k] = x;
+      }
     }
     __syncthreads();
     const int v = tid >> 2, g = tid & 3;  // 8 K-values of one vector
@@ -402,12 +429,16 @@ __global__ void __launch_bounds__(256) tc_dgemm_reduce_kernel(const __grid_const
 
 }  // namespace
 
-bool tc_dgemm_takes(const GemmItem<double> &g) {
-  return g.m >= 48 && g.n >= 48 && g.k >= 48 && (double)g.m * g.n * g.k >= 6.4e7;
-}
+// C = beta*C + alpha*op(A)*op(B) on real sizes; amode, bmode: how the operands are read (DigitItem::mode)
+struct DgGemm {
+  const double *A, *B;
+  double *C;
+  int m, n, k, lda, ldb;
+  long long ldc;
+  int amode, bmode, sym;
+};
 
-void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
-                      double beta, const std::vector<char> &sym) {
+static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double alpha, double beta) {
   RFDD_REQUIRE(tc_status_word() != nullptr, RFDD_ESTATE, "tensor-core GEMM launched without a status word");
   const int nsm = sm_count();
   RFDD_CUDA(cudaFuncSetAttribute(tc_dgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM));
@@ -428,14 +459,14 @@ void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &item
       memset(&db, 0, sizeof(db));
       memset(&gb, 0, sizeof(gb));
       size_t bytes = 0, vecs = 0, wsum = 0;
-      struct Src { const double *p; int ld, nv, k, kc, vb; size_t off, ev; };
+      struct Src { const double *p; int ld, nv, k, mode, vb; size_t off, ev; };
       std::vector<Src> srcs;  // operands, each packed once even when several items use it
-      auto operand = [&](const double *p, int ld, int nv, int k, int kc, int vb) {
+      auto operand = [&](const double *p, int ld, int nv, int k, int mode, int vb) {
         for (size_t q = 0; q < srcs.size(); ++q)
-          if (srcs[q].p == p && srcs[q].ld == ld && srcs[q].nv == nv && srcs[q].k == k && srcs[q].kc == kc && srcs[q].vb == vb)
+          if (srcs[q].p == p && srcs[q].ld == ld && srcs[q].nv == nv && srcs[q].k == k && srcs[q].mode == mode && srcs[q].vb == vb)
             return (int)q;
         const size_t nkt = (k + DG_KT - 1) / DG_KT, tiles = (nv + vb - 1) / vb;
-        srcs.push_back({p, ld, nv, k, kc, vb, bytes, vecs});
+        srcs.push_back({p, ld, nv, k, mode, vb, bytes, vecs});
         bytes += tiles * nkt * DG_PAIRS * vb * 128;
         vecs += (size_t)(nv + 63) / 64 * 64;
         return (int)srcs.size() - 1;
@@ -448,8 +479,10 @@ void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &item
         ia.push_back(-1);
         ib.push_back(-1);
         if (k <= 0) continue;
-        ia[i] = operand(g.A + (ta ? (int64_t)kp * g.lda : kp), g.lda, g.m, k, ta ? 0 : 1, DG_BM);
-        ib[i] = operand(g.B + (tb ? kp : (int64_t)kp * g.ldb), g.ldb, g.n, k, tb ? 1 : 0, DG_BN);
+        // rows kp .. of the operand (a complex row holds two real ones, each of two doubles)
+        auto from = [&](const double *p, int ld, int mode) { return p + (mode == 1 ? (int64_t)kp : (int64_t)kp * ld); };
+        ia[i] = operand(from(g.A, g.lda, g.amode), g.lda, g.m, k, g.amode, DG_BM);
+        ib[i] = operand(from(g.B, g.ldb, g.bmode), g.ldb, g.n, k, g.bmode, DG_BN);
         DgItem &x = gb.it[gb.count];
         x.m = g.m;
         x.n = g.n;
@@ -457,7 +490,7 @@ void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &item
         x.ldc = g.ldc;
         x.nkt = (k + DG_KT - 1) / DG_KT;
         x.ntc = (g.n + DG_BN - 1) / DG_BN;
-        x.sym = !sym.empty() && sym[s0 + i];
+        x.sym = g.sym;
         const int mtc = (g.m + DG_BM - 1) / DG_BM;
         int tiles = 0;
         for (int m = 0; m < mtc; ++m) tiles += x.sym ? std::max(0, x.ntc - 2 * m) : x.ntc;
@@ -491,8 +524,8 @@ void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &item
       long long be = 1, bp = 1;
       for (const Src &s : srcs) {
         const int nkt = (s.k + DG_KT - 1) / DG_KT;
-        db.it[db.count++] = {s.p, s.ld, s.nv, s.k, s.kc, s.vb, nkt, ws + ebytes + s.off, emax + s.ev};
-        be = std::max<long long>(be, s.kc ? (s.nv + 7) / 8 : (long long)((s.nv + 31) / 32) * ((s.k + 255) / 256));
+        db.it[db.count++] = {s.p, s.ld, s.nv, s.k, s.mode, s.vb, nkt, ws + ebytes + s.off, emax + s.ev};
+        be = std::max<long long>(be, s.mode == 1 ? (s.nv + 7) / 8 : (long long)((s.nv + 31) / 32) * ((s.k + 255) / 256));
         bp = std::max<long long>(bp, (long long)((s.nv + 63) / 64) * nkt);
       }
       for (int i = 0, q = 0; i < cnt; ++i) {
@@ -538,5 +571,49 @@ void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &item
     }
   }
 }
+
+// Digit products pay where the batch has enough work for their four launches and every item fills a good part
+// of a 128 x 64 tile.  Against double-FP32 (12 FP32 operations per product) the line lies at about 6e7
+// products an item; against the FP64 pipes (two products per cycle and SM) at 3e7 in the whole batch.
+bool tc_dgemm_takes(const GemmItem<double> &g) {
+  return g.m >= 48 && g.n >= 48 && g.k >= 48 && (double)g.m * g.n * g.k >= 6.4e7;
+}
+
+void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
+                      double beta, const std::vector<char> &sym) {
+  std::vector<DgGemm> v;
+  for (size_t i = 0; i < items.size(); ++i) {
+    const auto &g = items[i];
+    v.push_back({g.A, g.B, g.C, g.m, g.n, g.k, g.lda, g.ldb, g.ldc, ta ? 0 : 1, tb ? 1 : 0,
+                 !sym.empty() && sym[i] ? 1 : 0});
+  }
+  dgemm_run(st, v, alpha, beta);
+}
+
+template <typename T>
+bool tc_fp64_takes(const std::vector<GemmItem<T>> &items) {
+  constexpr double F = ST<T>::is_complex ? 2.0 : 1.0;
+  double work = 0.0;
+  for (const auto &g : items) {
+    if (g.m < 32 || F * g.n < 32 || F * g.k < 32) return false;
+    work += F * F * g.m * g.n * (double)g.k;
+  }
+  return work >= 3.2e7;
+}
+
+template <typename T>
+void tc_fp64_batched(cudaStream_t st, const std::vector<GemmItem<T>> &items, double alpha, double beta) {
+  constexpr int F = ST<T>::is_complex ? 2 : 1;
+  std::vector<DgGemm> v;
+  for (const auto &g : items)
+    v.push_back({reinterpret_cast<const double *>(g.A), reinterpret_cast<const double *>(g.B),
+                 reinterpret_cast<double *>(g.C), g.m, F * g.n, F * g.k, F * g.lda, g.ldb, (long long)F * g.ldc, 1,
+                 F == 2 ? 2 : 0, 0});
+  dgemm_run(st, v, alpha, beta);
+}
+template bool tc_fp64_takes<double>(const std::vector<GemmItem<double>> &);
+template bool tc_fp64_takes<cx<double>>(const std::vector<GemmItem<cx<double>>> &);
+template void tc_fp64_batched<double>(cudaStream_t, const std::vector<GemmItem<double>> &, double, double);
+template void tc_fp64_batched<cx<double>>(cudaStream_t, const std::vector<GemmItem<cx<double>>> &, double, double);
 
 }  // namespace rfdd

@@ -50,6 +50,13 @@ bool tc_dgemm_takes(const GemmItem<double> &g);
 void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
                       double beta, const std::vector<char> &sym);
 
+// The same for products without transposes in real or complex FP64: the trailing and triangular-solve updates
+// of the FP64 factorisations.  tc_fp64_takes: whether the batch as a whole gains over the FP64 pipes.
+template <typename T>
+bool tc_fp64_takes(const std::vector<GemmItem<T>> &items);
+template <typename T>
+void tc_fp64_batched(cudaStream_t st, const std::vector<GemmItem<T>> &items, double alpha, double beta);
+
 // The tile-shape autotuner: mode 0 off (fixed rule), 1 on, 2 forget every class (re-tune);
 // returns whether it was on.  tc_autotune_table: one line per class (tc_tune.h, Tuner::dump).
 int tc_autotune(int mode);

@@ -4,6 +4,7 @@
 // with Gram-Schmidt inside clusters of close eigenvalues, back-transformation.
 #include "eig.cuh"
 #include "dense.cuh"
+#include "grid_barrier.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -316,23 +317,6 @@ static void tridiagonal_values(cudaStream_t st, const SymBatchP &b, int cnt, int
 // (37.2 in 3769 launches, 44 with gaps).
 constexpr int TRD_THREADS = 512;  // at most; 256 below order 512
 constexpr int TRD_NMAX = 8192;  // three vectors of the order in shared memory
-constexpr int TRD_SPIN = 1 << 22;
-__device__ __forceinline__ bool trd_barrier(unsigned *cnt, unsigned target) {
-  __shared__ int ok_s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    asm volatile("fence.acq_rel.gpu;\n\tred.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
-    unsigned v = 0;
-    int k = 0;
-    do {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
-    } while (v < target && ++k < TRD_SPIN);
-    ok_s = v >= target;
-  }
-  __syncthreads();
-  return ok_s != 0;
-}
-
 // Block-wide sum over the first nact warps, given to f by one thread of warp 0; what f leaves in
 // shared memory is visible to all on return.  A warp's FP64 instruction takes 16 cycles of an SM's
 // FP64 pipe, whatever its lanes do: warps without data add nothing, and the scalars that follow from
@@ -502,7 +486,7 @@ __global__ void __launch_bounds__(TRD_THREADS) tridiag_kernel(SymBatchP b, TridS
         if (lane == 0) pn[r] = tau_s * t;
       }
     }
-    if (!trd_barrier(bar, (unsigned)(G * (i + 1)))) {
+    if (!grid_barrier(bar, (unsigned)(G * (i + 1)))) {
       if (tid == 0) atomicOr(status, DS_GRID_TIMEOUT);
       return;
     }

@@ -1,0 +1,29 @@
+// Barrier among the CTAs of a cooperative launch (all of them resident), with a bounded wait.
+#pragma once
+#include "common.cuh"
+
+namespace rfdd {
+
+constexpr int GRID_SPIN = 1 << 22;
+
+// Every CTA adds one to *cnt (zero before the launch) and waits until it has reached target, the number of CTAs
+// times the number of barriers so far.  What any thread of a CTA wrote before is visible to all threads
+// after it (global loads of other CTAs' data through L2).  false: the wait ran out.  A flag per CTA that
+// every other CTA polls, in place of the counter, made a step of 152 CTAs 2.5 us longer.
+__device__ __forceinline__ bool grid_barrier(unsigned *cnt, unsigned target) {
+  __shared__ int ok_s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("fence.acq_rel.gpu;\n\tred.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
+    unsigned v = 0;
+    int k = 0;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+    } while (v < target && ++k < GRID_SPIN);
+    ok_s = v >= target;
+  }
+  __syncthreads();
+  return ok_s != 0;
+}
+
+}  // namespace rfdd

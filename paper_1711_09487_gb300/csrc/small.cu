@@ -1,6 +1,7 @@
 // Small dense FP64 kernels for block orthonormalisation and Rayleigh-Ritz bookkeeping.
 #include "small.cuh"
 #include "dense.cuh"
+#include "grid_barrier.cuh"
 
 #include <algorithm>
 #include <climits>
@@ -316,146 +317,171 @@ template void sub_inplace<double>(cudaStream_t, const double *, double *, int64_
 namespace rfdd {
 
 // ---------------------------------------------------------------------------------------
-// Pivoted Cholesky P^T G P = R^T R, right-looking, on the upper triangle only (the lower
-// triangle is not read), one step per launch pair.
-// Step t: choose the largest remaining diagonal entry (a contiguous copy dg of the diagonal is
-// kept; its argmax compares the IEEE bit patterns as integers, which orders the non-negative
-// values like the doubles and costs no FP64 instruction; smallest index on ties), stop
-// (rank = t) when it is <= tol or not finite, interchange t and p symmetrically within the upper
-// triangle (the factored rows' trailing parts included); then update the trailing upper triangle
-// with the unscaled row g = G[t][t+1..]: G_ij -= (g_i g_j) / G_tt.  Rows of R are scaled by
-// 1/sqrt(G_tt) once at the end (pchol_scale_kernel).  FP64 arithmetic is scarce on this GPU, so
-// each step does one division and two FP64 operations per trailing upper entry.  On exit the
-// leading rank x rank upper triangle holds R on the kept directions.
+// Pivoted Cholesky P^T G P = R^T R in one cooperative launch, left-looking: G stays as it is (only its
+// rows of chosen pivots are read), CTA c owns columns j = c mod G, and column j of R grows in row j of
+// Rt.  Step t: every CTA offers the largest of its remaining diagonal entries (bit patterns compared as
+// integers, smallest index on ties), one barrier, every CTA reads the offers of all, and the largest is the pivot p; the factorisation stops (rank = t) when it is <= tol
+// or not finite.  Then r_t[j] = (G[p][j] - sum_s R[s][p] R[s][j]) / sqrt(d_p) and d_j -= r_t[j]^2 for the CTA's columns.
+// k r^2 / 2 FP64 FMAs in all (7.7 ms of the chip's FP64 rate for k = 2720, r = 1884) and about 5 us a step: 384
+// steps 2.1 ms (4.15 in two launches a step on the trailing triangle), the 2720 columns about 20 ms (50).
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) pchol_pivot_kernel(double *G, int k, int *perm, int t, double tol, int *rank,
-                                                           double *dg, double *dinv) {
-  if (*rank >= 0) return;
-  __shared__ long long bv[32];
-  __shared__ int bi[32];
-  __shared__ int piv_s;
-  long long v = LLONG_MIN;
-  int idx = k;
-  for (int i = t + threadIdx.x; i < k; i += blockDim.x) {
-    const long long g = __double_as_longlong(dg[i]);
-    if (g > v) { v = g; idx = i; }  // i increases within a thread: the first maximum is kept
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long v2 = __shfl_down_sync(0xffffffffu, v, o);
-    const int i2 = __shfl_down_sync(0xffffffffu, idx, o);
-    if (v2 > v || (v2 == v && i2 < idx)) { v = v2; idx = i2; }
-  }
-  if ((threadIdx.x & 31) == 0) { bv[threadIdx.x >> 5] = v; bi[threadIdx.x >> 5] = idx; }
+constexpr int PCH_THREADS = 512;
+constexpr int PCH_XMAX = 24 * 1024;  // entries of the pivot's column kept in shared memory
+
+struct PchOffer {
+  long long bits;  // of the largest remaining diagonal entry
+  long long col;
+};
+
+__global__ void __launch_bounds__(PCH_THREADS) pchol_kernel(const double *__restrict__ Gm, int k, double *Rt, int *perm,
+                                                            double tol, int *rank, PchOffer *offers, unsigned *bar,
+                                                            int *status) {
+  extern __shared__ double sm[];
+  const int me = blockIdx.x, ng = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = PCH_THREADS / 32;
+  const int own = me < k ? (k - me + ng - 1) / ng : 0;
+  double *d = sm, *xs = sm + (k + ng - 1) / ng;  // remaining diagonal of the own columns (-1: chosen); pivot column
+  const bool x_in_smem = k <= PCH_XMAX;
+  __shared__ int p_s;
+  __shared__ double rinv_s, rdiag_s;
+  for (int c = tid; c < own; c += PCH_THREADS) d[c] = Gm[(int64_t)(me + c * ng) * (k + 1)];
   __syncthreads();
-  if (threadIdx.x == 0) {
-    long long bvv = bv[0];
-    int bii = bi[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-      if (bv[w] > bvv || (bv[w] == bvv && bi[w] < bii)) { bvv = bv[w]; bii = bi[w]; }
-    const double d = bii < k ? dg[bii] : -1.0;
-    piv_s = (d > tol && isfinite(d)) ? bii : -1;
-    if (piv_s < 0) *rank = t;
-    else *dinv = 1.0 / d;
+  for (int t = 0; t < k; ++t) {
+    long long bv = LLONG_MIN;
+    int bi = INT_MAX;
+    auto best = [&] {
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long v2 = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (v2 > bv || (v2 == bv && i2 < bi)) { bv = v2; bi = i2; }
+      }
+    };
+    PchOffer *of = offers + (size_t)(t & 1) * ng;  // two sets: a slow CTA may still read the last step's
+    if (warp == 0) {
+      for (int c = lane; c < own; c += 32) {
+        const long long v = __double_as_longlong(d[c]);
+        if (v > bv) { bv = v; bi = me + c * ng; }  // columns increase within a lane: the first maximum stays
+      }
+      best();
+      if (lane == 0) of[me] = {bv, bi};
+    }
+    if (!grid_barrier(bar, (unsigned)ng * (unsigned)(t + 1))) {
+      if (tid == 0) atomicOr(status, DS_GRID_TIMEOUT);
+      return;
+    }
+    if (warp == 0) {
+      bv = LLONG_MIN;
+      bi = INT_MAX;
+      for (int c = lane; c < ng; c += 32) {
+        const longlong2 w = __ldcg(reinterpret_cast<const longlong2 *>(of + c));
+        if (w.x > bv || (w.x == bv && (int)w.y < bi)) { bv = w.x; bi = (int)w.y; }
+      }
+      best();
+      if (lane == 0) {
+        const double dp = bi < k ? __longlong_as_double(bv) : -1.0;
+        const bool go = dp > tol && isfinite(dp);
+        const double r = go ? rsqrt_nr(dp) : 0.0;
+        p_s = go ? bi : -1;
+        rinv_s = r;
+        rdiag_s = dp * r;
+      }
+    }
+    __syncthreads();
+    const int p = p_s;
+    if (p < 0) {
+      if (me == 0 && tid == 0) *rank = t;
+      return;
+    }
+    if (me == 0 && tid == 0) perm[t] = p;
+    // column p of R (written by its owner, through L2)
+    const double *xg = Rt + (int64_t)p * k;
+    if (x_in_smem) {
+      for (int s = tid; s < t; s += PCH_THREADS) xs[s] = __ldcg(xg + s);
+      __syncthreads();
+    }
+    const double rinv = rinv_s;
+    for (int c = warp; c < own; c += NW) {
+      const int j = me + c * ng;
+      if (d[c] < 0.0) continue;  // chosen before (the same in every lane)
+      double *rj = Rt + (int64_t)j * k;
+      if (j == p) {
+        __syncwarp();
+        if (lane == 0) {
+          rj[t] = rdiag_s;
+          d[c] = -1.0;
+        }
+        continue;
+      }
+      const double g = lane == 0 ? Gm[(int64_t)p * k + j] : 0.0;
+      double a0 = 0.0, a1 = 0.0;
+      int s = lane;
+      if (x_in_smem) {
+        for (; s + 96 < t; s += 128) {
+          double r4[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) r4[u] = rj[s + 32 * u];
+          a0 = fma(r4[0], xs[s], a0);
+          a1 = fma(r4[1], xs[s + 32], a1);
+          a0 = fma(r4[2], xs[s + 64], a0);
+          a1 = fma(r4[3], xs[s + 96], a1);
+        }
+        for (; s < t; s += 32) a0 = fma(rj[s], xs[s], a0);
+      } else {
+        for (; s < t; s += 32) a0 = fma(rj[s], __ldcg(xg + s), a0);
+      }
+      a0 += a1;
+      for (int o = 16; o > 0; o >>= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+      if (lane == 0) {
+        const double v = (g - a0) * rinv;
+        rj[t] = v;
+        const double nd = fma(-v, v, d[c]);
+        d[c] = nd <= 0.0 ? 0.0 : fabs(nd);  // a NaN stays and, being the largest pattern, ends the factorisation
+      }
+    }
+    __syncthreads();
   }
+}
+
+// R into the leading r x r upper triangle of G: G[t][i] = Rt[perm[i]][t] for t <= i < r
+__global__ void __launch_bounds__(256) pchol_gather_kernel(const double *__restrict__ Rt, const int *__restrict__ perm,
+                                                           int k, const int *rank_p, double *G) {
+  const int r = *rank_p < 0 ? k : *rank_p;
+  __shared__ double tile[32][33];
+  const int i0 = blockIdx.x * 32, t0 = blockIdx.y * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (i0 >= r || t0 >= r || i0 + 31 < t0) return;
+  for (int q = w; q < 32; q += 8)
+    if (i0 + q < r && t0 + lane < r) tile[q][lane] = Rt[(int64_t)perm[i0 + q] * k + t0 + lane];
   __syncthreads();
-  const int p = piv_s;
-  if (p < 0 || p == t) return;
-  // symmetric interchange of t < p in upper storage:
-  //   r < t: G[r][t] <-> G[r][p];  t < r < p: G[t][r] <-> G[r][p];  r > p: G[t][r] <-> G[p][r];
-  //   diagonal G[t][t] <-> G[p][p];  G[t][p] stays
-  for (int r = threadIdx.x; r < k; r += blockDim.x) {
-    double *a, *b;
-    if (r < t) {
-      a = G + (int64_t)r * k + t;
-      b = G + (int64_t)r * k + p;
-    } else if (r == t) {
-      a = G + (int64_t)t * k + t;
-      b = G + (int64_t)p * k + p;
-    } else if (r < p) {
-      a = G + (int64_t)t * k + r;
-      b = G + (int64_t)r * k + p;
-    } else if (r == p) {
-      continue;
-    } else {
-      a = G + (int64_t)t * k + r;
-      b = G + (int64_t)p * k + r;
-    }
-    const double x = *a;
-    *a = *b;
-    *b = x;
-  }
-  if (threadIdx.x == 0) {
-    const int a = perm[t];
-    perm[t] = perm[p];
-    perm[p] = a;
-    const double d = dg[t];
-    dg[t] = dg[p];
-    dg[p] = d;
+  for (int q = w; q < 32; q += 8) {
+    const int t = t0 + q, i = i0 + lane;
+    if (t < r && i < r && i >= t) G[(int64_t)t * k + i] = tile[lane][q];
   }
 }
 
-// trailing upper triangle: row t+1+i (grid-stride over rows), columns j >= i by the block's threads
-__global__ void pchol_update_kernel(double *G, int k, int t, const int *rank, double *dg, const double *dinv_p) {
-  if (*rank >= 0) return;
-  const int len = k - t - 1;
-  const double *g = G + (int64_t)t * k + t + 1;
-  const double dinv = *dinv_p;
-  for (int i = blockIdx.x; i < len; i += gridDim.x) {
-    const double gi = g[i];
-    double *row = G + (int64_t)(t + 1 + i) * k + t + 1;
-    for (int j = i + threadIdx.x; j < len; j += blockDim.x) {
-      const double nv = fma(-(gi * g[j]), dinv, row[j]);
-      row[j] = nv;
-      if (j == i) dg[t + 1 + i] = nv;
-    }
-  }
-}
-
-// R rows: G[t][c] /= sqrt(G_tt) for c > t, G[t][t] = sqrt(G_tt), t < rank (rows in parallel)
-__global__ void pchol_scale_kernel(double *G, int k, const int *rank) {
-  const int r = *rank < 0 ? k : *rank;
-  for (int t = blockIdx.x; t < r; t += gridDim.x) {
-    double *row = G + (int64_t)t * k;
-    const double rt = sqrt(row[t]);
-    const double inv = 1.0 / rt;
-    __syncthreads();
-    for (int c = t + 1 + threadIdx.x; c < k; c += blockDim.x) row[c] *= inv;
-    __syncthreads();
-    if (threadIdx.x == 0) row[t] = rt;
-  }
-}
-
-__global__ void pchol_diag_kernel(const double *G, int k, double *dg) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < k; i += gridDim.x * blockDim.x) dg[i] = G[(int64_t)i * k + i];
-}
-
-__global__ void iota_kernel(int *p, int k) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < k; i += gridDim.x * blockDim.x) p[i] = i;
-}
 __global__ void set_int_kernel(int *p, int v) { *p = v; }
 
-int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, int *rank_dev) {
-  iota_kernel<<<ceil_div(k, 256), 256, 0, st>>>(perm, k);
-  RFDD_CHECK_LAUNCH();
+int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, int *rank_dev, int *status) {
   set_int_kernel<<<1, 1, 0, st>>>(rank_dev, -1);
   RFDD_CHECK_LAUNCH();
-  double *dg = nullptr;  // k diagonal entries, then 1 / (the current pivot)
-  RFDD_CUDA(cudaMallocAsync((void **)&dg, (size_t)(k + 1) * sizeof(double), st));
-  double *dinv = dg + k;
-  pchol_diag_kernel<<<ceil_div(k, 256), 256, 0, st>>>(G, k, dg);
+  const int ng = std::max(1, std::min(sm_count(), k));
+  double *Rt = nullptr;
+  PchOffer *offers = nullptr;
+  RFDD_CUDA(cudaMallocAsync((void **)&Rt, (size_t)k * k * sizeof(double), st));
+  RFDD_CUDA(cudaMallocAsync((void **)&offers, (size_t)2 * ng * sizeof(PchOffer) + sizeof(unsigned), st));
+  unsigned *bar = reinterpret_cast<unsigned *>(offers + 2 * ng);
+  RFDD_CUDA(cudaMemsetAsync(bar, 0, sizeof(unsigned), st));
+  const size_t smem = ((size_t)ceil_div(k, ng) + (k <= PCH_XMAX ? k : 0)) * sizeof(double);
+  RFDD_REQUIRE(smem <= 220 * 1024, RFDD_EINVAL, "pivoted Cholesky: order too large");
+  RFDD_CUDA(cudaFuncSetAttribute(pchol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+  const double *Gc = G;
+  void *args[] = {&Gc, &k, &Rt, &perm, &tol, &rank_dev, &offers, &bar, &status};
+  RFDD_CUDA(cudaLaunchCooperativeKernel((const void *)pchol_kernel, dim3(ng), dim3(PCH_THREADS), args, smem, st));
   RFDD_CHECK_LAUNCH();
-  for (int t = 0; t < k; ++t) {
-    pchol_pivot_kernel<<<1, 1024, 0, st>>>(G, k, perm, t, tol, rank_dev, dg, dinv);
-    RFDD_CHECK_LAUNCH();
-    const int len = k - t - 1;
-    if (len > 0) {
-      pchol_update_kernel<<<std::min(len, 8 * sm_count()), 256, 0, st>>>(G, k, t, rank_dev, dg, dinv);
-      RFDD_CHECK_LAUNCH();
-    }
-  }
-  pchol_scale_kernel<<<std::min(k, 1024), 256, 0, st>>>(G, k, rank_dev);
+  const unsigned nt = (unsigned)ceil_div(k, 32);
+  pchol_gather_kernel<<<dim3(nt, nt), 256, 0, st>>>(Rt, perm, k, rank_dev, G);
   RFDD_CHECK_LAUNCH();
-  RFDD_CUDA(cudaFreeAsync(dg, st));
+  RFDD_CUDA(cudaFreeAsync(Rt, st));
+  RFDD_CUDA(cudaFreeAsync(offers, st));
   int rank = -1;
   RFDD_CUDA(cudaMemcpyAsync(&rank, rank_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
   RFDD_CUDA(cudaStreamSynchronize(st));

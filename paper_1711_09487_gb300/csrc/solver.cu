@@ -1833,7 +1833,8 @@ RRout rayleigh_ritz_coeffs(rfdd_handle *h, const double *Y, int64_t k, double dr
   inv_sqrt_diag(st, G.as<double>(), k, dsc.as<double>());
   scale_sym(st, G.as<double>(), k, dsc.as<double>());
   scale_sym(st, K.as<double>(), k, dsc.as<double>());
-  const int r = pivoted_cholesky(st, G.as<double>(), (int)k, perm.as<int>(), drop, rankd.as<int>());
+  const int r = pivoted_cholesky(st, G.as<double>(), (int)k, perm.as<int>(), drop, rankd.as<int>(),
+                                 h->status.as<int>());
   lap.mark("pivoted cholesky");
   RFDD_REQUIRE(r > 0, RFDD_ESINGULAR, "Rayleigh-Ritz: basis has no independent direction");
   // H = R^{-T} Kp R^{-1}: with Lt = (D_R^{-1} R^T) unit lower, R^{-T} B = Lt^{-1} D_R^{-1} B

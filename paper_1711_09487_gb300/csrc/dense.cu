@@ -491,24 +491,108 @@ __device__ inline int tourn_sets(int rows, int R, int level) {
   return n;
 }
 
-// Calls f(std::integral_constant<int, i>) for i = I .. N-1 in order.
-template <int I, int N, typename F>
-__device__ __forceinline__ void static_for(F &f) {
-  if constexpr (I < N) {
-    f(std::integral_constant<int, I>{});
-    static_for<I + 1, N>(f);
+// Order of the candidates of a pivot search: larger |re| + |im| first (bit patterns of the non-negative
+// values as integers; NaN counts as infinity), then the lower row; -1 marks no candidate.
+template <typename R>
+struct PivKey;
+template <>
+struct PivKey<float> {
+  int v, row;
+  __device__ __forceinline__ void set(float x, int r) {
+    v = r < 0 ? -1 : (x != x ? 0x7f800000 : __float_as_int(x));
+    row = r;
   }
+  // the best of the warp's keys, in every lane
+  __device__ __forceinline__ PivKey best() const {
+    PivKey b;
+    b.v = __reduce_max_sync(0xffffffffu, v);
+    b.row = __reduce_min_sync(0xffffffffu, v == b.v ? row : INT_MAX);
+    return b;
+  }
+  __device__ __forceinline__ bool none() const { return v < 0; }
+  __device__ __forceinline__ bool same(const PivKey &o) const { return v == o.v && row == o.row; }
+};
+template <>
+struct PivKey<double> {
+  int v;
+  unsigned lo;
+  int row;
+  __device__ __forceinline__ void set(double x, int r) {
+    if (x != x) x = (double)INFINITY;
+    v = r < 0 ? -1 : __double2hiint(x);
+    lo = r < 0 ? 0u : (unsigned)__double2loint(x);
+    row = r;
+  }
+  __device__ __forceinline__ PivKey best() const {
+    PivKey b;
+    b.v = __reduce_max_sync(0xffffffffu, v);
+    b.lo = __reduce_max_sync(0xffffffffu, v == b.v ? lo : 0u);
+    b.row = __reduce_min_sync(0xffffffffu, v == b.v && lo == b.lo ? row : INT_MAX);
+    return b;
+  }
+  __device__ __forceinline__ bool none() const { return v < 0; }
+  __device__ __forceinline__ bool same(const PivKey &o) const { return v == o.v && lo == o.lo && row == o.row; }
+};
+
+// Elimination steps t0 .. t0 + 7 of a tournament round on rows held in registers, of which columns 0 .. W - 1
+// (from column t0 of the panel on) are still to be eliminated; afterwards every row moves down by eight columns.
+template <typename T, int W>
+__device__ __forceinline__ void tourn_group(T (&row)[LU_NB], int t0, int w, int &my, bool &live, int &steps, int *o,
+                                            T (*slot)[8][LU_NB], PivKey<typename ST<T>::real> (*red)[8]) {
+  using S = ST<T>;
+  using Rl = typename S::real;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int tt = 0; tt < 8; ++tt) {
+    const int t = t0 + tt;
+    if (t >= w) live = false;
+    if (!live) break;  // the same decision in every thread
+    // every warp offers its best candidate and that row; one barrier, then all pick the best offer
+    PivKey<Rl> k;
+    k.set(my >= 0 ? S::abs1(row[tt]) : (Rl)0, my);
+    const PivKey<Rl> wb = k.best();
+    if (my >= 0 && k.same(wb)) {
+#pragma unroll
+      for (int c = tt; c < W; ++c) slot[t & 1][warp][c] = row[c];
+    }
+    if (lane == 0) red[t & 1][warp] = wb;
+    __syncthreads();
+    const PivKey<Rl> e = red[t & 1][lane & 7];
+    const PivKey<Rl> gb = e.best();
+    if (gb.none()) {
+      live = false;  // no row left
+      break;
+    }
+    const int win = (__ffs(__ballot_sync(0xffffffffu, e.same(gb))) - 1) & 7;
+    const T *prow = slot[t & 1][win];
+    if (my == gb.row) {
+      o[t] = my;
+      my = -1;
+    }
+    ++steps;
+    if (my >= 0) {
+      const T pv = prow[tt];
+      if (S::abs1(pv) != (Rl)0) {
+        const T l = row[tt] * S::div(S::one(), pv);
+#pragma unroll
+        for (int c = tt + 1; c < W; ++c) row[c] = S::fms(l, prow[c], row[c]);
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < W; ++c) row[c] = c + 8 < W ? row[c + 8] : S::zero();
 }
 
 // One tournament round of the panel's pivot search.  A CTA takes up to R = G * NB candidate rows of
 // the panel's w columns (level 0: a slice of consecutive rows; above it: the winners of G sets of
 // the level below), runs LU with partial pivoting on them and emits the pivot rows in the order
-// chosen.  Thread i keeps candidate row i in registers for the whole elimination: each step is a
-// block-wide argmax of |a_it| over the rows not yet chosen (ties go to the lower row index, so
-// the winner does not depend on where a row sits), the winner publishes its row through shared
-// memory, and every other row forms its multiplier and rank-1 update in its own registers.  The
-// multipliers and updates are the same operations, in the same order, as LU on the gathered
-// rows.  Only the row indices leave the CTA.
+// chosen.  Thread i keeps candidate row i in registers for the whole elimination: each step is an
+// argmax of |a_it| over the rows not yet chosen (ties go to the lower row index, so the winner does not
+// depend on where a row sits), by warp reductions and one barrier (tourn_group), after which every other
+// row forms its multiplier and rank-1 update in its own registers.  Only the row indices leave the CTA.
+// What bounds it is the chain of a step; the eight-step groups keep the code of 32 steps in the instruction cache
+// (one straight line of 32 steps with two barriers and shuffles each: 68 us a launch on average in the 3-D 24^3
+// factorisation, now 31).
 template <typename T>
 __global__ void __launch_bounds__(256) lu_tourn_kernel(LuBatchP<T> lb, int K0, int nbo, int k0, int level,
                                                        const int *__restrict__ cin, int *__restrict__ cout,
@@ -517,7 +601,7 @@ __global__ void __launch_bounds__(256) lu_tourn_kernel(LuBatchP<T> lb, int K0, i
   using Rl = typename S::real;
   constexpr int NB = LU_NB;
   constexpr int R = TournRows<T>::R;
-  static_assert(R == 256, "one candidate row per thread of a 256-thread CTA");
+  static_assert(R == 256 && NB == 32, "one candidate row per thread of a 256-thread CTA");
   const LuItem<T> it = lb.it[blockIdx.y];
   const int wend = strip_end(K0, nbo, it.dp);
   const int w = min(NB, wend - k0);
@@ -525,9 +609,8 @@ __global__ void __launch_bounds__(256) lu_tourn_kernel(LuBatchP<T> lb, int K0, i
   const int rows_total = it.dp - k0;
   const int set = blockIdx.x;
   if (set >= tourn_sets(rows_total, R, level)) return;
-  __shared__ T prow[NB];
-  __shared__ Rl red_v[R / 32];
-  __shared__ int red_r[R / 32];
+  __shared__ __align__(16) T slot[2][8][NB];
+  __shared__ PivKey<Rl> red[2][8];
   const int tid = threadIdx.x;
   int my = -1;  // global index of this thread's candidate row; -1 when it has none (or it was chosen)
   if (level == 0) {
@@ -548,49 +631,10 @@ __global__ void __launch_bounds__(256) lu_tourn_kernel(LuBatchP<T> lb, int K0, i
   int *o = cout + (int64_t)blockIdx.y * cand_stride + (int64_t)set * NB;
   int steps = 0;
   bool live = true;  // false once the panel's w columns or the candidate rows are used up
-  // step t of the elimination, t a compile-time constant so that row[] stays in registers
-  auto step = [&](auto tc) {
-    constexpr int t = decltype(tc)::value;
-    if (!live || t >= w) { live = false; return; }
-    Rl v = (Rl)-1;
-    int r = INT_MAX;
-    if (my >= 0) {
-      v = S::abs1(row[t]);
-      if (v != v) v = (Rl)INFINITY;  // a NaN row still counts as a candidate
-      r = my;
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-      const Rl v2 = __shfl_xor_sync(0xffffffffu, v, off);
-      const int r2 = __shfl_xor_sync(0xffffffffu, r, off);
-      if (v2 > v || (v2 == v && r2 < r)) { v = v2; r = r2; }
-    }
-    if ((tid & 31) == 0) { red_v[tid >> 5] = v; red_r[tid >> 5] = r; }
-    __syncthreads();
-    v = red_v[0];
-    r = red_r[0];
-#pragma unroll
-    for (int q = 1; q < R / 32; ++q)
-      if (red_v[q] > v || (red_v[q] == v && red_r[q] < r)) { v = red_v[q]; r = red_r[q]; }
-    if (v < (Rl)0) { live = false; return; }  // no row left: the same decision in every thread
-    if (my == r) {
-#pragma unroll
-      for (int c = t; c < NB; ++c) prow[c] = row[c];
-      o[t] = my;
-      my = -1;
-    }
-    ++steps;
-    __syncthreads();
-    if (my >= 0) {
-      const T pv = prow[t];
-      if (S::abs1(pv) != (Rl)0) {
-        const T l = S::div(row[t], pv);
-#pragma unroll
-        for (int c = t + 1; c < NB; ++c)
-          if (c < w) row[c] = S::fms(l, prow[c], row[c]);
-      }
-    }
-  };
-  static_for<0, NB>(step);
+#pragma unroll 1
+  for (int g = 0; g < 2; ++g) tourn_group<T, 32>(row, 8 * g, w, my, live, steps, o, slot, red);
+#pragma unroll 1
+  for (int g = 2; g < 4; ++g) tourn_group<T, 16>(row, 8 * g, w, my, live, steps, o, slot, red);
   for (int t = steps + tid; t < NB; t += blockDim.x) o[t] = -1;
 }
 

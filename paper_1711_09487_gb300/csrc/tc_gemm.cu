@@ -770,13 +770,16 @@ struct PackBatchP {
   int na, nb;
 };
 
-// A tiles: [mt][kt] 128 rows x 64 halves; 16-byte chunk c of row r stored at chunk c ^ (r & 7).  One warp per
-// row: its largest magnitude first, then the split (the second read of the row comes from L1 / L2).
-template <bool CPLX>
+// A tiles: [mt][kt] 128 rows x 64 halves; 16-byte chunk c of row r stored at chunk c ^ (r & 7).  A row takes 32
+// lanes, or 8 or 16 when it has no more chunks than that (the 32-deep panel updates): its largest magnitude
+// first, then the split (the second read of the row comes from L1 / L2).
+template <bool CPLX, int NW>
 __device__ __forceinline__ void pack_a_rows(const PackItem &it) {
   constexpr int F = CPLX ? 2 : 1;
-  const int lane = threadIdx.x & 31, kf = F * it.k, nq = it.nkt * 8, rows_pad = it.nblk * TC_BM;
-  for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows_pad; row += gridDim.x * 8) {
+  const int kf = F * it.k, nq = it.nkt * 8, rows_pad = it.nblk * TC_BM;
+  const int lpr = nq >= 32 ? 32 : nq >= 16 ? 16 : 8, per = 32 * NW / lpr, lane = threadIdx.x % lpr;
+  // rows_pad is a multiple of per, so the lanes of a warp stay together
+  for (int row = blockIdx.x * per + (int)threadIdx.x / lpr; row < rows_pad; row += gridDim.x * per) {
     const float *src = it.src + (long long)row * F * it.ld;
     const bool live = row < it.rows;
     auto load8 = [&](int q, float (&x)[8]) {
@@ -797,7 +800,7 @@ __device__ __forceinline__ void pack_a_rows(const PackItem &it) {
     // chunks left of the row's diagonal block (a multiple of eight values per block)
     const int ql = it.side > 0 ? (row / it.side) * it.side * F / 8 : 0;
     float ml = 0.f, mr = 0.f;
-    for (int q = lane; q < nq; q += 32) {
+    for (int q = lane; q < nq; q += lpr) {
       float x[8];
       load8(q, x);
       float m = 0.f;
@@ -806,7 +809,7 @@ __device__ __forceinline__ void pack_a_rows(const PackItem &it) {
       if (q < ql) ml = fmaxf(ml, m);
       else mr = fmaxf(mr, m);
     }
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = lpr >> 1; o > 0; o >>= 1) {
       ml = fmaxf(ml, __shfl_xor_sync(0xffffffffu, ml, o));
       mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
     }
@@ -822,7 +825,7 @@ __device__ __forceinline__ void pack_a_rows(const PackItem &it) {
       }
     }
     const int mt = row / TC_BM, r = row % TC_BM;
-    for (int q = lane; q < nq; q += 32) {
+    for (int q = lane; q < nq; q += lpr) {
       float x[8];
       load8(q, x);
       const float f = q < ql ? fl : fr;
@@ -842,12 +845,12 @@ __device__ __forceinline__ void pack_a_rows(const PackItem &it) {
 // in shared memory with reads along B's rows, takes the largest magnitude of every column, and writes
 // the packed rows with coalesced 16-byte stores.  Deeper B is staged twice, chunk by chunk.
 constexpr int PACK_KC = 256;
-template <bool CPLX>
+template <bool CPLX, int NW>
 __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
   constexpr int F = CPLX ? 2 : 1;
   constexpr int CW = 64 / F;            // columns of B per block
   constexpr int PITCH = CPLX ? 66 : 65;  // floats per staged row
-  __shared__ float smax[8][64];
+  __shared__ float smax[NW][64];
   __shared__ float mul_s[64];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nch = (it.k + PACK_KC - 1) / PACK_KC;
@@ -857,7 +860,7 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
       if (CPLX) {
         const bool on = j0 + lane < it.rows;
 #pragma unroll 8
-        for (int p = warp; p < pn; p += 8) {
+        for (int p = warp; p < pn; p += NW) {
           const float2 v = on ? *reinterpret_cast<const float2 *>(it.src + 2 * ((long long)(p0 + p) * it.ld + j0 + lane))
                               : make_float2(0.f, 0.f);
           *reinterpret_cast<float2 *>(sb + p * PITCH + 2 * lane) = v;
@@ -866,7 +869,7 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
       } else {
         const bool on0 = j0 + lane < it.rows, on1 = j0 + lane + 32 < it.rows;
 #pragma unroll 4
-        for (int p = warp; p < pn; p += 8) {
+        for (int p = warp; p < pn; p += NW) {
           const float *r = it.src + (long long)(p0 + p) * it.ld + j0 + lane;
           const float v0 = on0 ? r[0] : 0.f, v1 = on1 ? r[32] : 0.f;
           sb[p * PITCH + lane] = v0;
@@ -888,7 +891,7 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
       const int c = CPLX ? tid >> 1 : tid;
       float m = smax[0][c];
 #pragma unroll
-      for (int w = 1; w < 8; ++w) m = fmaxf(m, smax[w][c]);
+      for (int w = 1; w < NW; ++w) m = fmaxf(m, smax[w][c]);
       float mul, inv;
       row_scale(m, mul, inv);
       mul_s[tid] = mul;
@@ -903,7 +906,7 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
         __syncthreads();
       }
       const int kt0 = p0 * F / TC_BK, tiles = (pn * F + TC_BK - 1) / TC_BK;
-      for (int id = tid; id < tiles * 512; id += 256) {
+      for (int id = tid; id < tiles * 512; id += 32 * NW) {
         const int c = id & 7, rl = (id >> 3) & 63, kt = id >> 9;
         const float mul = mul_s[rl];
         uint16_t h[8], l[8];
@@ -936,27 +939,37 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
 }
 
 // Both operands of every item in one launch (blockIdx.y: the A operands, then the B operands); zero, when
-// given, is a status word cleared for the GEMM that follows.
-template <bool CPLX>
-__global__ void __launch_bounds__(256) pack_f16_kernel(const __grid_constant__ PackBatchP pb, int *zero) {
+// given, is a status word cleared for the GEMM that follows.  NW warps a block.
+template <bool CPLX, int NW>
+__global__ void __launch_bounds__(32 * NW) pack_f16_kernel(const __grid_constant__ PackBatchP pb, int *zero) {
   extern __shared__ float pack_sb[];
   if (zero && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero = 0;
-  if ((int)blockIdx.y < pb.na) pack_a_rows<CPLX>(pb.a[blockIdx.y]);
-  else pack_b_rows<CPLX>(pb.b[blockIdx.y - pb.na], pack_sb);
+  if ((int)blockIdx.y < pb.na) pack_a_rows<CPLX, NW>(pb.a[blockIdx.y]);
+  else pack_b_rows<CPLX, NW>(pb.b[blockIdx.y - pb.na], pack_sb);
 }
 
 template <bool CPLX>
 static void launch_pack(cudaStream_t st, const PackBatchP &pb, int *zero = nullptr) {
   if (pb.na + pb.nb == 0) return;
-  long long blocks = 1;
+  long long blocks = 1, all = 0;
   int kmax = 0;
-  for (int i = 0; i < pb.na; ++i) blocks = std::max(blocks, (long long)pb.a[i].nblk * (TC_BM / 8));
+  for (int i = 0; i < pb.na; ++i) {
+    // 256 threads pack 8 to 32 rows at a time (pack_a_rows); whole blocks per 128-row tile either way
+    const int rows = 256 / (pb.a[i].nkt >= 4 ? 32 : pb.a[i].nkt >= 2 ? 16 : 8);
+    blocks = std::max(blocks, (long long)pb.a[i].nblk * (TC_BM / rows));
+    all += (long long)pb.a[i].nblk * (TC_BM / rows);
+  }
   for (int i = 0; i < pb.nb; ++i) {
     blocks = std::max(blocks, (long long)pb.b[i].nblk);
+    all += pb.b[i].nblk;
     kmax = std::max(kmax, std::min(pb.b[i].k, PACK_KC));
   }
+  // a launch with less than a block per SM (right-hand sides of a few columns) is a chain of memory latencies:
+  // 32 warps a block shorten it four times
   const size_t smem = (size_t)kmax * (CPLX ? 66 : 65) * sizeof(float);
-  pack_f16_kernel<CPLX><<<dim3((unsigned)std::min<long long>(blocks, 2048), pb.na + pb.nb), 256, smem, st>>>(pb, zero);
+  const dim3 grid((unsigned)std::min<long long>(blocks, 2048), pb.na + pb.nb);
+  if (all < sm_count()) pack_f16_kernel<CPLX, 32><<<grid, 1024, smem, st>>>(pb, zero);
+  else pack_f16_kernel<CPLX, 8><<<grid, 256, smem, st>>>(pb, zero);
   RFDD_CHECK_LAUNCH();
 }
 
@@ -1056,10 +1069,10 @@ static TcDevInfo tc_device_info() {
     const void *ones[] = {(const void *)tc_gemm_kernel<true, 256>, (const void *)tc_gemm_kernel<true, 64>,
                           (const void *)tc_gemm_kernel<false, 256>};
     for (const void *f : ones) RFDD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
-    RFDD_CUDA(cudaFuncSetAttribute(pack_f16_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   PACK_KC * 66 * (int)sizeof(float)));
-    RFDD_CUDA(cudaFuncSetAttribute(pack_f16_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   PACK_KC * 65 * (int)sizeof(float)));
+    const void *packs[] = {(const void *)pack_f16_kernel<true, 8>, (const void *)pack_f16_kernel<true, 32>,
+                           (const void *)pack_f16_kernel<false, 8>, (const void *)pack_f16_kernel<false, 32>};
+    for (const void *f : packs)
+      RFDD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, PACK_KC * 66 * (int)sizeof(float)));
     RFDD_CUDA(cudaFuncSetAttribute(tc_gemm2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, T2_SMEM));
     RFDD_CUDA(cudaDeviceGetAttribute(&d.nsm, cudaDevAttrMultiProcessorCount, dev));
     cudaLaunchConfig_t cfg = {};

@@ -3829,6 +3829,7 @@ int rfdd_sym_eig(int64_t n, const double *H, double *evals, double *evecs) {
     RFDD_CUDA(cudaMemset(status.p, 0, sizeof(int)));
     SymItem si{Hd.as<double>(), (int)n, (int)n, d.as<double>(), e.as<double>(), t.as<double>(), w.as<double>(),
                lam.as<double>(), Z.as<double>()};
+    TcStatusScope tcs(status.as<int>());
     sym_eig_values(st, {si}, status.as<int>());
     std::vector<int> all(n);
     std::iota(all.begin(), all.end(), 0);

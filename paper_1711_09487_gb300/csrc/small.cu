@@ -502,11 +502,11 @@ void gather_sym(cudaStream_t st, const double *K, int k, const int *perm, int r,
   RFDD_CHECK_LAUNCH();
 }
 
-// Lt[i][j] = R[j][i] / R[i][i] (j < i), 1 (j == i), 0 (j > i): unit lower, from upper R (ld ldr)
+// Lt[i][j] = R[j][i] / R[j][j] (j < i), 1 (j == i), 0 (j > i): unit lower, from upper R (ld ldr)
 __global__ void unit_lower_from_upper_kernel(const double *__restrict__ R, int ldr, int r, double *Lt) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)r * r; e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e / r), j = (int)(e % r);
-    Lt[e] = j < i ? R[(int64_t)j * ldr + i] / R[(int64_t)i * ldr + i] : (i == j ? 1.0 : 0.0);
+    Lt[e] = j < i ? R[(int64_t)j * ldr + i] / R[(int64_t)j * ldr + j] : (i == j ? 1.0 : 0.0);
   }
 }
 void unit_lower_from_upper(cudaStream_t st, const double *R, int ldr, int r, double *Lt) {
@@ -515,31 +515,18 @@ void unit_lower_from_upper(cudaStream_t st, const double *R, int ldr, int r, dou
   RFDD_CHECK_LAUNCH();
 }
 
-// out[i][j] = (trans ? in[j][i] : in[i][j]) / R[i][i]   (r x r)
-__global__ void scale_rows_by_rdiag_kernel(const double *__restrict__ in, int r, int trans, const double *__restrict__ R,
-                                           int ldr, double *out) {
+// out[i][j] = (A[i][j] + A[j][i]) / (2 R_ii R_jj) (r x r), into a separate buffer
+__global__ void symmetrize_scaled_kernel(const double *__restrict__ A, int r, const double *__restrict__ R, int ldr,
+                                         double *out) {
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)r * r; e += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(e / r), j = (int)(e % r);
-    const double v = trans ? in[(int64_t)j * r + i] : in[e];
-    out[e] = v / R[(int64_t)i * ldr + i];
+    const double d = R[(int64_t)i * (ldr + 1)] * R[(int64_t)j * (ldr + 1)];
+    out[e] = 0.5 * (A[e] + A[(int64_t)j * r + i]) / d;
   }
 }
-void scale_rows_by_rdiag(cudaStream_t st, const double *in, int r, bool trans, const double *R, int ldr, double *out) {
+void symmetrize_scaled(cudaStream_t st, const double *A, int r, const double *R, int ldr, double *out) {
   if (r <= 0) return;
-  scale_rows_by_rdiag_kernel<<<gridn((int64_t)r * r), 256, 0, st>>>(in, r, trans ? 1 : 0, R, ldr, out);
-  RFDD_CHECK_LAUNCH();
-}
-
-// out = (A + A^T)/2 (r x r), into a separate buffer
-__global__ void symmetrize_kernel(const double *__restrict__ A, int r, double *out) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)r * r; e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e / r), j = (int)(e % r);
-    out[e] = 0.5 * (A[e] + A[(int64_t)j * r + i]);
-  }
-}
-void symmetrize(cudaStream_t st, const double *A, int r, double *out) {
-  if (r <= 0) return;
-  symmetrize_kernel<<<gridn((int64_t)r * r), 256, 0, st>>>(A, r, out);
+  symmetrize_scaled_kernel<<<gridn((int64_t)r * r), 256, 0, st>>>(A, r, R, ldr, out);
   RFDD_CHECK_LAUNCH();
 }
 

@@ -40,8 +40,7 @@ namespace rfdd {
 int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, int *rank_dev, int *status);
 void gather_sym(cudaStream_t st, const double *K, int k, const int *perm, int r, double *out);
 void unit_lower_from_upper(cudaStream_t st, const double *R, int ldr, int r, double *Lt);
-void scale_rows_by_rdiag(cudaStream_t st, const double *in, int r, bool trans, const double *R, int ldr, double *out);
-void symmetrize(cudaStream_t st, const double *A, int r, double *out);
+void symmetrize_scaled(cudaStream_t st, const double *A, int r, const double *R, int ldr, double *out);
 void transpose(cudaStream_t st, const double *in, int a, int b, double *out);
 void scatter_rows_perm(cudaStream_t st, const double *Cr, int r, int ns, const int *perm, const double *d,
                        double *Cfull);

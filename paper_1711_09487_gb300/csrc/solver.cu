@@ -1837,28 +1837,34 @@ RRout rayleigh_ritz_coeffs(rfdd_handle *h, const double *Y, int64_t k, double dr
                                  h->status.as<int>());
   lap.mark("pivoted cholesky");
   RFDD_REQUIRE(r > 0, RFDD_ESINGULAR, "Rayleigh-Ritz: basis has no independent direction");
-  // H = R^{-T} Kp R^{-1}: with Lt = (D_R^{-1} R^T) unit lower, R^{-T} B = Lt^{-1} D_R^{-1} B
-  Buf Kp, Lt, B, H;
+  // H = R^{-T} Kp R^{-1}.  R = D R' with D its diagonal and R' unit upper; |R'| <= 1 by the pivoting, so Lt = R'^T is a
+  // unit lower factor like that of an LU with pivoting, whatever the range of D: H = D^{-1} (Lt^{-1} Kp Lt^{-T}) D^{-1}
+  // with products that are accurate relative to their largest entries, and inverted diagonal blocks
+  constexpr int RR_NB = 128;
+  Buf Kp, Lt, B, H, Linv;
   Kp.alloc((size_t)r * r * sizeof(double));
   Lt.alloc((size_t)r * r * sizeof(double));
   B.alloc((size_t)r * r * sizeof(double));
   H.alloc((size_t)r * r * sizeof(double));
+  Linv.alloc((size_t)block_inverse_elems(r, RR_NB) * sizeof(double));
   gather_sym(st, K.as<double>(), (int)k, perm.as<int>(), r, Kp.as<double>());
   unit_lower_from_upper(st, G.as<double>(), (int)k, r, Lt.as<double>());
-  scale_rows_by_rdiag(st, Kp.as<double>(), r, false, G.as<double>(), (int)k, B.as<double>());
   SolveItem<double> tri;
   tri.LU = Lt.as<double>();
   tri.piv = nullptr;
   tri.n = r;
   tri.ld = r;
-  tri.X = B.as<double>();
+  tri.X = Kp.as<double>();
   tri.ldx = r;
   tri.ncols = r;
-  trsm_lower_unit<double>(st, {tri}, 128);                                   // B = R^{-T} Kp
-  scale_rows_by_rdiag(st, B.as<double>(), r, true, G.as<double>(), (int)k, Kp.as<double>());
-  tri.X = Kp.as<double>();
-  trsm_lower_unit<double>(st, {tri}, 128);                                   // Kp = R^{-T} B^T = H^T
-  symmetrize(st, Kp.as<double>(), r, H.as<double>());
+  lu_block_inverses<double>(st, {tri}, RR_NB, {Linv.as<double>()}, {nullptr});
+  tri.Linv = Linv.as<double>();
+  tri.nbi = RR_NB;
+  trsm_lower_unit<double>(st, {tri}, RR_NB);                                 // Lt^{-1} Kp
+  transpose(st, Kp.as<double>(), r, r, B.as<double>());
+  tri.X = B.as<double>();
+  trsm_lower_unit<double>(st, {tri}, RR_NB);                                 // Lt^{-1} Kp Lt^{-T}, transposed
+  symmetrize_scaled(st, B.as<double>(), r, G.as<double>(), (int)k, H.as<double>());
   K.release();
   Kp.release();
   B.release();

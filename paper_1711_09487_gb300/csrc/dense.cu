@@ -944,34 +944,55 @@ static void launch_trsm_diag(cudaStream_t st, const std::vector<TriItem<T>> &ite
 }
 
 // ======================================================================================
-// Pivot application to right-hand sides (row interchanges in order, thread per column).
+// Row permutation of a factorisation.  lu_batched leaves in piv the permutation that the interchanges compose to (row t of
+// P X is row piv[t] of X), so that right-hand sides are permuted by independent row copies: the interchanges one
+// after another were a chain of two dependent memory accesses per pivot and column on every solve.
 // ======================================================================================
+constexpr int PERM_SMEM = 48 * 1024;  // orders up to 49152 in shared memory (4 bytes a row)
+template <typename T>
+__global__ void __launch_bounds__(256) piv_to_perm_kernel(LuBatchP<T> lb, int *gws, int64_t gstride) {
+  const LuItem<T> it = lb.it[blockIdx.x];
+  extern __shared__ int perm_s[];
+  int *p = it.dp <= PERM_SMEM ? perm_s : gws + blockIdx.x * gstride;
+  for (int t = threadIdx.x; t < it.dp; t += blockDim.x) p[t] = t;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int t0 = 0; t0 < it.dp; t0 += 8) {
+      int q[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) q[u] = t0 + u < it.dp ? it.piv[t0 + u] : t0 + u;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (t0 + u < it.dp && q[u] != t0 + u) {
+          const int x = p[t0 + u];
+          p[t0 + u] = p[q[u]];
+          p[q[u]] = x;
+        }
+    }
+  __syncthreads();
+  for (int t = threadIdx.x; t < it.dp; t += blockDim.x) it.piv[t] = p[t];
+}
+
 template <typename T>
 struct PivItem {
-  const int *piv;
-  int npiv;
-  T *X;
-  int ldx, ncols;
+  const int *perm;
+  const T *X;
+  T *Y;
+  int n, ldx, ncols;
 };
 template <typename T>
 struct PivBatchP {
   PivItem<T> it[MAXB];
 };
 
+// Y (n x ncols, ld ncols) = P X
 template <typename T>
-__global__ void __launch_bounds__(256) apply_piv_kernel(PivBatchP<T> pb) {
+__global__ void __launch_bounds__(256) permute_rows_kernel(PivBatchP<T> pb) {
   const PivItem<T> it = pb.it[blockIdx.y];
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= it.ncols) return;
-  for (int t = 0; t < it.npiv; ++t) {
-    const int q = __ldg(it.piv + t);
-    if (q != t) {
-      T *a = it.X + (int64_t)t * it.ldx + c;
-      T *b = it.X + (int64_t)q * it.ldx + c;
-      T x = *a;
-      *a = *b;
-      *b = x;
-    }
+  const int64_t tot = (int64_t)it.n * it.ncols;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = e / it.ncols, c = e % it.ncols;
+    it.Y[e] = it.X[(int64_t)__ldg(it.perm + t) * it.ldx + c];
   }
 }
 
@@ -1128,26 +1149,20 @@ void lu_batched(cudaStream_t st, const std::vector<LuItem<T>> &items, int nbo, i
   RFDD_CUDA(cudaFreeAsync(wk.cand, st));
   RFDD_CUDA(cudaFreeAsync(wk.top, st));
   RFDD_CUDA(cudaFreeAsync(perm, st));
-}
-
-template <typename T>
-void apply_pivots(cudaStream_t st, const std::vector<SolveItem<T>> &items) {
+  // the interchanges of every item as one row permutation
+  int *gws = nullptr;
+  if (dpmax > PERM_SMEM) RFDD_CUDA(cudaMallocAsync((void **)&gws, (size_t)MAXB * dpmax * sizeof(int), st));
+  RFDD_CUDA(cudaFuncSetAttribute(piv_to_perm_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 PERM_SMEM * (int)sizeof(int)));
   for (size_t s = 0; s < items.size(); s += MAXB) {
-    PivBatchP<T> b;
+    LuBatchP<T> b;
     memset(&b, 0, sizeof(b));
-    int cnt = (int)std::min<size_t>(MAXB, items.size() - s), nc = 1;
-    for (int i = 0; i < cnt; ++i) {
-      const auto &it = items[s + i];
-      b.it[i].piv = it.piv;
-      b.it[i].npiv = it.n;
-      b.it[i].X = it.X;
-      b.it[i].ldx = it.ldx;
-      b.it[i].ncols = it.ncols;
-      nc = std::max(nc, it.ncols);
-    }
-    apply_piv_kernel<T><<<dim3(ceil_div(nc, 256), cnt), 256, 0, st>>>(b);
+    const int cnt = (int)std::min<size_t>(MAXB, items.size() - s);
+    for (int i = 0; i < cnt; ++i) b.it[i] = items[s + i];
+    piv_to_perm_kernel<T><<<cnt, 256, (size_t)std::min(dpmax, PERM_SMEM) * sizeof(int), st>>>(b, gws, dpmax);
     RFDD_CHECK_LAUNCH();
   }
+  if (gws) RFDD_CUDA(cudaFreeAsync(gws, st));
 }
 
 // ======================================================================================
@@ -1187,6 +1202,34 @@ static void copy_rows_batched(cudaStream_t st, const std::vector<CopyItem<T>> &i
     copy_rows_batched_kernel<T><<<dim3((unsigned)std::min<int64_t>(ceil_div(mx, 256), 1024), cnt), 256, 0, st>>>(b);
     RFDD_CHECK_LAUNCH();
   }
+}
+
+template <typename T>
+void apply_pivots(cudaStream_t st, const std::vector<SolveItem<T>> &items) {
+  size_t tot = 0;
+  for (const auto &it : items) tot += (size_t)std::max(it.n, 0) * std::max(it.ncols, 0);
+  if (tot == 0) return;
+  T *tmp = nullptr;
+  RFDD_CUDA(cudaMallocAsync((void **)&tmp, tot * sizeof(T), st));
+  std::vector<CopyItem<T>> back;
+  size_t off = 0;
+  for (size_t s = 0; s < items.size(); s += MAXB) {
+    PivBatchP<T> b;
+    memset(&b, 0, sizeof(b));
+    const int cnt = (int)std::min<size_t>(MAXB, items.size() - s);
+    int64_t mx = 1;
+    for (int i = 0; i < cnt; ++i) {
+      const auto &it = items[s + i];
+      b.it[i] = {it.piv, it.X, tmp + off, it.n, it.ldx, it.ncols};
+      if (it.n > 0 && it.ncols > 0) back.push_back({tmp + off, it.X, it.ncols, it.ldx, it.n, it.ncols});
+      off += (size_t)std::max(it.n, 0) * std::max(it.ncols, 0);
+      mx = std::max<int64_t>(mx, (int64_t)it.n * it.ncols);
+    }
+    permute_rows_kernel<T><<<dim3((unsigned)std::min<int64_t>(ceil_div(mx, 256), 1024), cnt), 256, 0, st>>>(b);
+    RFDD_CHECK_LAUNCH();
+  }
+  copy_rows_batched<T>(st, back);
+  RFDD_CUDA(cudaFreeAsync(tmp, st));
 }
 
 template <typename T>

@@ -41,7 +41,8 @@ void gemm_simt_batched(cudaStream_t st, const std::vector<GemmItem<T>> &items, b
 // One bordered matrix for LU: D x D (row-major, leading dimension ld), of which the first dp
 // rows/columns are eliminated with pivoting restricted to rows < dp.  After the factorisation
 // the trailing (D-dp) x (D-dp) block holds C~ - E^T B^{-1} E (the Schur complement of the
-// leading block).  piv: int32[dp], LAPACK-style sequence of row interchanges (row t <-> piv[t]).
+// leading block).  piv: int32[dp], on return the row permutation of the factorisation: row t of P B is row
+// piv[t] of B (during the factorisation, the LAPACK-style sequence of interchanges).
 template <typename T>
 struct LuItem {
   T *A;

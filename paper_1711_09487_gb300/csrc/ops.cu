@@ -159,11 +159,58 @@ __global__ void shifted_residual_kernel(const int64_t *__restrict__ rp, const in
   }
 }
 
+// The same for fewer than 32 columns: CL lanes take the columns, and the 32 / CL groups of lanes share the entries of
+// the row (a warp's FP64 instruction costs the same with one lane as with 32): one column of the 3-D 24^3
+// pencil, eight nodes: 624 us with a lane per column; the 3-D 24^3 factor case, ten of these, went from 54.7 to 48.6 ms
+// with the entries shared (and the permuted conversion below).
+template <int CL>
+__global__ void shifted_residual_narrow_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
+                                               const double *__restrict__ av, const double *__restrict__ mv, int64_t n,
+                                               const cx<double> *__restrict__ zz, const cx<double> *__restrict__ V,
+                                               int64_t strideV, const cx<double> *__restrict__ X,
+                                               cx<double> *__restrict__ Rr, int64_t stride, int64_t b) {
+  const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+  const int lane = threadIdx.x & 31, c = lane % CL, g = lane / CL;
+  const int l = blockIdx.y;
+  if (r >= n) return;  // the lanes of a warp share r
+  const cx<double> z = zz[l];
+  const cx<double> *Xl = X + l * stride;
+  double ar = 0.0, ai = 0.0, mr = 0.0, mi = 0.0;
+  if (c < b)
+    for (int64_t e = rp[r] + g, e1 = rp[r + 1]; e < e1; e += 32 / CL) {
+      const cx<double> x = Xl[(int64_t)col[e] * b + c];
+      const double a = av[e], m = mv[e];
+      ar = fma(a, x.re, ar);
+      ai = fma(a, x.im, ai);
+      mr = fma(m, x.re, mr);
+      mi = fma(m, x.im, mi);
+    }
+#pragma unroll
+  for (int o = 16; o >= CL; o >>= 1) {
+    ar += __shfl_xor_sync(0xffffffffu, ar, o);
+    ai += __shfl_xor_sync(0xffffffffu, ai, o);
+    mr += __shfl_xor_sync(0xffffffffu, mr, o);
+    mi += __shfl_xor_sync(0xffffffffu, mi, o);
+  }
+  if (g == 0 && c < b) {
+    const double sr = ar - (z.re * mr - z.im * mi);
+    const double si = ai - (z.re * mi + z.im * mr);
+    const cx<double> v = V[l * strideV + r * b + c];
+    Rr[l * stride + r * b + c] = cx<double>(v.re - sr, v.im - si);
+  }
+}
+
 void shifted_residual(cudaStream_t st, const DevPencil &P, const cx<double> *z_dev, int nnodes,
                       const cx<double> *V, int64_t strideV, const cx<double> *X, cx<double> *R, int64_t stride,
                       int64_t b) {
   dim3 grid(ceil_div(P.n * 32, 256), nnodes);
-  shifted_residual_kernel<<<grid, 256, 0, st>>>(P.rowptr, P.col, P.a, P.m, P.n, z_dev, V, strideV, X, R, stride, b);
+  auto go = [&](auto *kernel) {
+    kernel<<<grid, 256, 0, st>>>(P.rowptr, P.col, P.a, P.m, P.n, z_dev, V, strideV, X, R, stride, b);
+  };
+  if (b == 1) go(shifted_residual_narrow_kernel<1>);
+  else if (b <= 4) go(shifted_residual_narrow_kernel<4>);
+  else if (b <= 16) go(shifted_residual_narrow_kernel<16>);
+  else go(shifted_residual_kernel);
   RFDD_CHECK_LAUNCH();
 }
 
@@ -685,7 +732,7 @@ template void scatter_schur<double>(cudaStream_t, const DevDD &, int, int, int, 
 
 
 // ---------------------------------------------------------------------------------------
-// Interface gather / ordered scatter for the bordered-factor DD solve
+// Interface gather / ordered scatter, one index list at a time (two-level interface solve)
 // ---------------------------------------------------------------------------------------
 // Yj_l[a][c] = G_l[sidx_j[a]][c]  for all nodes l
 template <typename T>
@@ -733,6 +780,98 @@ template void scatter_sub_iface<cx<float>>(cudaStream_t, const int32_t *, int, i
 template void scatter_sub_iface<cx<double>>(cudaStream_t, const int32_t *, int, int64_t, const cx<double> *, int64_t,
                                             cx<double> *, int64_t, int);
 
+// ---------------------------------------------------------------------------------------
+// Interface gather / ordered subtraction for the bordered-factor DD solve, all subdomains in one launch.
+// Subdomain j's border block of node l is at Y + l * strideY + j * strideJ (s_j x m).
+// ---------------------------------------------------------------------------------------
+// Y_lj[t][c] = G_l[sidx_j[t]][c]
+template <typename T>
+__global__ void gather_iface_all_kernel(const int32_t *__restrict__ sidx, const int64_t *__restrict__ sidx_off, int64_t m,
+                                    const T *__restrict__ G, int64_t strideG, T *__restrict__ Y, int64_t strideY,
+                                    int64_t strideJ) {
+  const int l = blockIdx.y, j = blockIdx.z;
+  const int64_t s0 = sidx_off[j], sj = sidx_off[j + 1] - s0;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < sj * m; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = e / m, c = e % m;
+    Y[l * strideY + j * strideJ + e] = G[l * strideG + (int64_t)sidx[s0 + t] * m + c];
+  }
+}
+template <typename T>
+void gather_iface_all(cudaStream_t st, const DevDD &dd, int64_t smax, int64_t m, const T *G, int64_t strideG, T *Y,
+                  int64_t strideY, int64_t strideJ, int nnodes) {
+  if (smax <= 0 || m <= 0) return;
+  gather_iface_all_kernel<T><<<dim3(std::min(1024, ceil_div(smax * m, 256)), nnodes, dd.p), 256, 0, st>>>(
+      dd.sidx, dd.sidx_off, m, G, strideG, Y, strideY, strideJ);
+  RFDD_CHECK_LAUNCH();
+}
+// G_l[a][c] -= sum_j R_lj[posmap_j[a]][c], j = 0..p-1 in order (reproducible sums); posmap < 0: j does not touch a
+template <typename T>
+__global__ void sub_iface_all_kernel(const int32_t *__restrict__ posmap, int p, int64_t s, int64_t m,
+                                 const T *__restrict__ R, int64_t strideR, int64_t strideJ, T *__restrict__ G,
+                                 int64_t strideG) {
+  const int l = blockIdx.y;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < s * m; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t a = e / m, c = e % m;
+    T *g = G + l * strideG + e;
+    T v = *g;
+    for (int j = 0; j < p; ++j) {
+      const int32_t t = __ldg(posmap + (int64_t)j * s + a);
+      if (t >= 0) v = v - R[l * strideR + j * strideJ + (int64_t)t * m + c];
+    }
+    *g = v;
+  }
+}
+template <typename T>
+void sub_iface_all(cudaStream_t st, const DevDD &dd, int64_t m, const T *R, int64_t strideR, int64_t strideJ, T *G,
+               int64_t strideG, int nnodes) {
+  if (dd.s <= 0 || m <= 0) return;
+  sub_iface_all_kernel<T><<<dim3((unsigned)std::min<int64_t>(4096, ceil_div(dd.s * m, 256)), nnodes), 256, 0, st>>>(
+      dd.posmap, dd.p, dd.s, m, R, strideR, strideJ, G, strideG);
+  RFDD_CHECK_LAUNCH();
+}
+#define RFDD_INST_IFACE(T)                                                                                            \
+  template void gather_iface_all<T>(cudaStream_t, const DevDD &, int64_t, int64_t, const T *, int64_t, T *, int64_t,     \
+                                int64_t, int);                                                                      \
+  template void sub_iface_all<T>(cudaStream_t, const DevDD &, int64_t, const T *, int64_t, int64_t, T *, int64_t, int);
+RFDD_INST_IFACE(cx<float>)
+RFDD_INST_IFACE(cx<double>)
+
+// f_l (n x m) = R_l in the factor precision, the interior rows of every subdomain in the pivot order of its factor
+// (perm: nnodes x dsum, local to the subdomain); strideR = 0: one right-hand side for all nodes
+template <typename T>
+__global__ void convert_permute_kernel(const cx<double> *__restrict__ R, int64_t strideR, const int *__restrict__ perm,
+                                       const int64_t *__restrict__ off, int p, int64_t n, int64_t dsum, int64_t m,
+                                       T *__restrict__ f) {
+  using Rl = typename ST<T>::real;
+  const int l = blockIdx.y;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n * m; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = e / m, c = e % m;
+    int64_t src = i;
+    if (i < dsum) {
+      int lo = 0, hi = p;  // subdomain of row i
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) / 2;
+        if (__ldg(off + mid) <= i) lo = mid;
+        else hi = mid;
+      }
+      src = __ldg(off + lo) + __ldg(perm + (int64_t)l * dsum + i);
+    }
+    const cx<double> v = R[l * strideR + src * m + c];
+    f[(int64_t)l * n * m + e] = T((Rl)v.re, (Rl)v.im);
+  }
+}
+template <typename T>
+void convert_permute(cudaStream_t st, const DevDD &dd, const cx<double> *R, int64_t strideR, const int *perm, int64_t n,
+                     int64_t m, int nnodes, T *f) {
+  if (n * m <= 0 || nnodes <= 0) return;
+  convert_permute_kernel<T><<<dim3((unsigned)std::min<int64_t>(4096, ceil_div(n * m, 256)), nnodes), 256, 0, st>>>(
+      R, strideR, perm, dd.off, dd.p, n, dd.dsum, m, f);
+  RFDD_CHECK_LAUNCH();
+}
+template void convert_permute<cx<float>>(cudaStream_t, const DevDD &, const cx<double> *, int64_t, const int *, int64_t,
+                                         int64_t, int, cx<float> *);
+template void convert_permute<cx<double>>(cudaStream_t, const DevDD &, const cx<double> *, int64_t, const int *, int64_t,
+                                          int64_t, int, cx<double> *);
 
 // ---------------------------------------------------------------------------------------
 // Two-level interface factorisation: assembly of the level storage of each node

@@ -128,5 +128,18 @@ void gather_iface(cudaStream_t st, const int32_t *sidx_j, int sj, int64_t m, con
 template <typename T>
 void scatter_sub_iface(cudaStream_t st, const int32_t *sidx_j, int sj, int64_t m, const T *Rj, int64_t strideR, T *G,
                        int64_t strideG, int nnodes);
+// The same for all subdomains and nodes in one launch each: border block of (node l, subdomain j) at
+// Y + l * strideY + j * strideJ (s_j x m, s_j <= smax); the subtraction runs over j = 0..p-1 in order
+template <typename T>
+void gather_iface_all(cudaStream_t st, const DevDD &dd, int64_t smax, int64_t m, const T *G, int64_t strideG, T *Y,
+                      int64_t strideY, int64_t strideJ, int nnodes);
+template <typename T>
+void sub_iface_all(cudaStream_t st, const DevDD &dd, int64_t m, const T *R, int64_t strideR, int64_t strideJ, T *G,
+                   int64_t strideG, int nnodes);
+// f_l (n x m per node) = R_l (+ l * strideR) in the factor precision, interior rows in the pivot order of
+// their subdomain's factor (perm: nnodes x dsum)
+template <typename T>
+void convert_permute(cudaStream_t st, const DevDD &dd, const cx<double> *R, int64_t strideR, const int *perm, int64_t n,
+                     int64_t m, int nnodes, T *f);
 
 }  // namespace rfdd

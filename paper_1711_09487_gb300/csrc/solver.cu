@@ -1602,8 +1602,8 @@ void dd_solve(rfdd_handle *h, const cx<double> *R, int64_t strideR, cx<double> *
   Tf *base = h->fac.as<Tf>();
   const int64_t hs = (int64_t)p * smax * m;  // per-node stride of the border scratch
   Lap lap(st, "dd");
-  for (int l = 0; l < nc; ++l) convert<Tf, cx<double>>(st, R + l * strideR, f + l * fs, fs);
-  // w = L^{-1} P f for every (node, subdomain)
+  // w = L^{-1} P f for every (node, subdomain); the rows of pivB are nnodes x dsum
+  convert_permute<Tf>(st, h->dd, R, strideR, h->pivB.as<int>(), n, m, nc, f);
   {
     std::vector<SolveItem<Tf>> it;
     for (int l = 0; l < nc; ++l)
@@ -1619,7 +1619,6 @@ void dd_solve(rfdd_handle *h, const cx<double> *R, int64_t strideR, cx<double> *
         attach_binv(h, x, l, j);
         it.push_back(x);
       }
-    apply_pivots<Tf>(st, it);
     trsm_lower_unit<Tf>(st, it, NBO);
   }
   lap.mark("forward");
@@ -1637,21 +1636,14 @@ void dd_solve(rfdd_handle *h, const cx<double> *R, int64_t strideR, cx<double> *
         pa.push_back(h->pkB.empty() ? TcPackedA{} : pk_border(h, h->pkB[(size_t)l * p + j].l21, sj, dj));
       }
     border_gemm<Tf>(st, g, pa, 1.0, 0.0);
-    for (int j = 0; j < p; ++j) {
-      const int sj = (int)(h->sidx_off[j + 1] - h->sidx_off[j]);
-      scatter_sub_iface<Tf>(st, h->dd.sidx + h->sidx_off[j], sj, m, ht + (int64_t)j * smax * m, hs, f + dsum * m, fs,
-                            nc);
-    }
+    sub_iface_all<Tf>(st, h->dd, m, ht, hs, smax * m, f + dsum * m, fs, nc);
   }
   lap.mark("border L21");
   solve_S<Tf>(h, f + dsum * m, m, fs, m, all_nodes(h));  // y = S^{-1} g'
   lap.mark("S solve");
   // w_j -= U12_j y[sidx_j], then u_j = U^{-1} w_j
   {
-    for (int j = 0; j < p; ++j) {
-      const int sj = (int)(h->sidx_off[j + 1] - h->sidx_off[j]);
-      gather_iface<Tf>(st, h->dd.sidx + h->sidx_off[j], sj, m, f + dsum * m, fs, ht + (int64_t)j * smax * m, hs, nc);
-    }
+    gather_iface_all<Tf>(st, h->dd, smax, m, f + dsum * m, fs, ht, hs, smax * m, nc);
     std::vector<GemmItem<Tf>> g;
     std::vector<TcPackedA> pa;
     std::vector<SolveItem<Tf>> it;

@@ -314,7 +314,7 @@ static void tridiagonal_values(cudaStream_t st, const SymBatchP &b, int cnt, int
 // late, so that no CTA overwrites what a slower one still reads.  Bound: below order 400 the chain of
 // one step (barrier, two block reductions, the reflector's scalars: about 5 us), above it the three
 // FP64 operations per trailing entry (n^3 FMAs are 11 ms of the chip's FP64 rate at order 1885).
-// Measured: order 120 0.65 ms (1.04 ms in 240 launches, 1.7 ms with their gaps), order 1885 28.8 ms
+// Measured: order 120 0.63 ms (1.04 ms in 240 launches, 1.7 ms with their gaps), order 1885 27.8 ms
 // (37.2 in 3769 launches, 44 with gaps).
 constexpr int TRD_THREADS = 512;  // at most; 256 below order 512
 constexpr int TRD_NMAX = 8192;  // three vectors of the order in shared memory
@@ -338,29 +338,33 @@ __device__ __forceinline__ void trd_sum(double v, double *red, int nact, F &&f) 
   __syncthreads();
 }
 
-// The Householder reflector of a vector with first entry alpha and the sum of squares sig of the
-// others: beta = -sign(alpha) ||x||, tau = 1 + |alpha| / ||x||, scale = 1 / (alpha - beta).  1 / ||x|| and the
-// scale come from the hardware's approximate (reciprocal) square root refined by Newton's
-// iteration, half the dependent FP64 operations of a square root and two divisions; far from 1 the
-// plain operations.
-__device__ __forceinline__ void householder(double alpha, double sig, double &beta, double &tau, double &sc) {
+// The Householder reflector I - tau u u^T of a vector x with first entry alpha and the sum of squares sig of
+// the others: beta = -sign(alpha) ||x||, u = x - beta e_1 (first entry u0, the others those of x, which so need no
+// scaling), tau = 2 / ||u||^2 = 1 / (||x|| (||x|| + |alpha|)).  1 / ||x|| and the reciprocals come from the hardware's
+// approximations refined by Newton's iteration, about half the dependent FP64 operations of a square root and a
+// division.  Far from 1, where products with u and tau could leave the range of a double, the plain operations on the
+// reflector scaled to u0 = 1: sc is the factor of the other entries (else 1).
+__device__ __forceinline__ void householder(double alpha, double sig, double &beta, double &tau, double &u0,
+                                            double &sc) {
   beta = alpha;
-  tau = sc = 0.0;
+  tau = 0.0;
+  u0 = sc = 1.0;
   if (sig == 0.0) return;
-  const double S = fma(alpha, alpha, sig);
-  if (S > 1e-280 && S < 1e280) {
+  const double S = fma(alpha, alpha, sig), a = fabs(alpha);
+  double nrm;
+  if (S > 1e-90 && S < 1e60) {
     double r;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(S));
     r = fma(0.5 * r, fma(-S * r, r, 1.0), r);
     r = fma(0.5 * r, fma(-S * r, r, 1.0), r);
-    const double a = fabs(alpha), nrm = S * r, D = a + nrm;
-    beta = alpha <= 0.0 ? nrm : -nrm;
-    tau = fma(a, r, 1.0);
+    nrm = S * r;
+    const double D = fma(nrm, a, S);
     double t = recip_nr(D);
-    t = fma(t, fma(-D, t, 1.0), t);
-    sc = alpha <= 0.0 ? -t : t;
+    tau = fma(t, fma(-D, t, 1.0), t);
+    beta = alpha <= 0.0 ? nrm : -nrm;
+    u0 = alpha - beta;
   } else {
-    const double nrm = sqrt(S);
+    nrm = sqrt(S);
     beta = alpha <= 0.0 ? nrm : -nrm;
     tau = (beta - alpha) / beta;
     sc = 1.0 / (alpha - beta);
@@ -383,7 +387,8 @@ __global__ void __launch_bounds__(TRD_THREADS) tridiag_kernel(SymBatchP b, TridS
   extern __shared__ double sm[];
   double *vp = sm, *q = sm + nmax, *v = sm + 2 * nmax;  // v_{i-1}, q_{i-1}, v_i, indexed by row
   __shared__ double red[32];
-  __shared__ double K_s, qi_s, sc_s, tau_s;  // tau_s: of the last reflector formed
+  __shared__ double K_s, qi_s, tau_s, sc_s;  // tau_s: of the last reflector formed
+  __shared__ double st_s[2];                 // 2^-exponent of u0, by the parity of the step
   double *p0 = pbuf + (int64_t)item * 2 * nmax;
   unsigned *bar = bars + item;
   for (int i = 0; i < n; ++i) {
@@ -421,25 +426,33 @@ __global__ void __launch_bounds__(TRD_THREADS) tridiag_kernel(SymBatchP b, TridS
       }
     }
     trd_sum(ss, red, nact, [&](double sig) {
-      double beta = 0.0, tau = 0.0, sc = 0.0;
-      if (i < n - 1) householder(v[i + 1], sig, beta, tau, sc);
+      double beta = 0.0, tau = 0.0, u0 = 1.0, sc = 1.0;
+      if (i < n - 1) {
+        householder(v[i + 1], sig, beta, tau, u0, sc);
+        v[i + 1] = u0;
+      }
       if (me == 0) {
+        // the stored reflector has its first entry in [1, 2) and tau to match (exact, powers of two): the
+        // back-transformation adds many reflectors up and wants them of one size
+        const int ex = (__double2hiint(u0) >> 20) & 0x7ff;
+        const double p2 = __hiloint2double(ex << 20, 0);
         it.d[i] = v[i];
-        it.tau[i] = tau;
+        it.tau[i] = tau * p2 * p2;
+        st_s[i & 1] = __hiloint2double((2046 - ex) << 20, 0);
         if (i < n - 1) it.e[i] = beta;
       }
       tau_s = tau;
       sc_s = sc;
     });
-    if (i < n - 1) {
-      const double sc = sc_s;
-      for (int k = i + 2 + tid; k < n; k += nthr) v[k] *= sc;
-      if (tid == 0) v[i + 1] = 1.0;
+    if (sc_s != 1.0) {
+      for (int k = i + 2 + tid; k < n; k += nthr) v[k] *= sc_s;
       __syncthreads();
     }
     // v_{i-1} into row i-1, for the back-transformation (every CTA has read that row)
-    if (me == 0 && i >= 1)
-      for (int k = i + tid; k < n; k += nthr) it.H[(int64_t)(i - 1) * it.ld + k] = vp[k];
+    if (me == 0 && i >= 1) {
+      const double st = st_s[(i - 1) & 1];
+      for (int k = i + tid; k < n; k += nthr) it.H[(int64_t)(i - 1) * it.ld + k] = st * vp[k];
+    }
     if (i > n - 2) break;
     // this CTA's rows of the trailing block: pending rank-2 update, then p_i
     const bool sym = i < n - 2;
@@ -726,7 +739,7 @@ __global__ void __launch_bounds__(256) inviter_kernel(InvIterP p, const Cluster 
 
 // Inverse iteration for eigenvalues that stand alone (clusters of one), one lane per eigenvalue:
 // the factorisation and the triangular solves are serial chains, so a warp runs 32 of them at the
-// cost of one (all vectors of order 1885: 4.8 ms, 14.2 with one thread of a CTA per eigenvalue).
+// cost of one (all vectors of order 1885: 4.4 ms, 14.2 with one thread of a CTA per eigenvalue).
 // Scratch is lane-interleaved (entry k of lane l at k * 32 + l), so every access is coalesced, and
 // IV_U steps are loaded ahead of the chain.  Same start vectors, factorisation and number of
 // iterations as inviter_kernel.
@@ -735,6 +748,13 @@ struct SingleWarp {
 };
 constexpr int IV_ARRAYS = 5;
 constexpr int IV_U = 8;
+// 1 / u to about 2^-52: two Newton steps on the hardware's approximation; the division for tiny and huge u
+__device__ __forceinline__ double recip_any(double u) {
+  const double a = fabs(u);
+  if (!(a > 1e-290 && a < 1e290)) return 1.0 / u;
+  const double r = recip_nr(u);
+  return fma(r, fma(-u, r, 1.0), r);
+}
 __global__ void __launch_bounds__(32) inviter_single_kernel(InvIterP p, const SingleWarp *__restrict__ sw,
                                                             const int *__restrict__ rows, double *scratch,
                                                             int64_t per_warp, unsigned *flags, int64_t flags_per_warp) {
@@ -769,9 +789,9 @@ __global__ void __launch_bounds__(32) inviter_single_kernel(InvIterP p, const Si
     const bool piv = fabs(cd) < fabs(sub);
     if (!piv && cd == 0.0) cd = delta;
     double u = piv ? sub : cd;
-    const double l = (piv ? cd : sub) / u;
+    const double l = (piv ? cd : sub) * recip_any(u);
     if (fabs(u) < delta) u = u < 0 ? -delta : delta;
-    ru[(int64_t)k * 32] = 1.0 / u;
+    ru[(int64_t)k * 32] = recip_any(u);
     u2[(int64_t)k * 32] = piv ? an : ce1;
     u3[(int64_t)k * 32] = piv ? bn : ce2;
     ml[(int64_t)k * 32] = l;
@@ -785,14 +805,14 @@ __global__ void __launch_bounds__(32) inviter_single_kernel(InvIterP p, const Si
   }
   {
     const double u = (fabs(cd) < delta) ? (cd < 0 ? -delta : delta) : cd;
-    ru[(int64_t)(n - 1) * 32] = 1.0 / u;
+    ru[(int64_t)(n - 1) * 32] = recip_any(u);
     u2[(int64_t)(n - 1) * 32] = u3[(int64_t)(n - 1) * 32] = 0.0;
     x[(int64_t)(n - 1) * 32] = hash(n - 1);
   }
   __syncwarp();
   double scale = 1.0, ss = 0.0;
   for (int iter = 0; iter < 3; ++iter) {
-    // forward: the largest entry of the last solve is scaled to one on the way in
+    // forward: the largest entry of the last solve is scaled to [1, 2) on the way in
     double cur = x[0] * scale;
     for (int k0 = 0; k0 < n - 1; k0 += IV_U) {
       double xn[IV_U], mk[IV_U];
@@ -815,7 +835,10 @@ __global__ void __launch_bounds__(32) inviter_single_kernel(InvIterP p, const Si
         }
     }
     // backward
-    double x1 = cur * ru[(int64_t)(n - 1) * 32], x2 = 0.0, mx = fabs(x1);
+    // (x_k - u2 x_{k+1} - u3 x_{k+2}) / U_kk with the factors multiplied by 1 / U_kk ahead: the chain from one step to
+    // the next is one FMA.  The largest entry is tracked by its high word (integer instructions).
+    double x1 = cur * ru[(int64_t)(n - 1) * 32], x2 = 0.0;
+    int mx = __double2hiint(x1) & 0x7fffffff;
     x[(int64_t)(n - 1) * 32] = x1;
     for (int k0 = n - 2; k0 >= 0; k0 -= IV_U) {
       double xk[IV_U], a2[IV_U], a3[IV_U], rk[IV_U];
@@ -831,14 +854,16 @@ __global__ void __launch_bounds__(32) inviter_single_kernel(InvIterP p, const Si
 #pragma unroll
       for (int q = 0; q < IV_U; ++q)
         if (k0 - q >= 0) {
-          const double v = (xk[q] - a2[q] * x1 - a3[q] * x2) * rk[q];
+          const double v = fma(-a2[q] * rk[q], x1, fma(-a3[q] * rk[q], x2, xk[q] * rk[q]));
           x[(int64_t)(k0 - q) * 32] = v;
           x2 = x1;
           x1 = v;
-          mx = fmax(mx, fabs(v));
+          mx = max(mx, __double2hiint(v) & 0x7fffffff);
         }
     }
-    scale = mx > 0.0 ? 1.0 / mx : 1.0;
+    // a power of two that brings the largest entry to [1, 2); 1 for zero, subnormal and not finite ones
+    const int ex = mx >> 20;
+    scale = ex >= 1 && ex <= 2045 ? __hiloint2double((2046 - ex) << 20, 0) : 1.0;
   }
   for (int k = 0; k < n; ++k) {
     const double v = x[(int64_t)k * 32] * scale;

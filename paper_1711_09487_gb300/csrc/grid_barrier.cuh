@@ -14,7 +14,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned *cnt, unsigned target) {
   __shared__ int ok_s;
   __syncthreads();
   if (threadIdx.x == 0) {
-    asm volatile("fence.acq_rel.gpu;\n\tred.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
+    // the release is cumulative over what __syncthreads has ordered before it
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
     unsigned v = 0;
     int k = 0;
     do {

@@ -442,14 +442,16 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
   RFDD_REQUIRE(tc_status_word() != nullptr, RFDD_ESTATE, "tensor-core GEMM launched without a status word");
   const int nsm = sm_count();
   RFDD_CUDA(cudaFuncSetAttribute(tc_dgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM));
-  for (size_t s0 = 0; s0 < items.size(); s0 += DG_MAXB) {
-    const int cnt = (int)std::min<size_t>(DG_MAXB, items.size() - s0);
+  for (size_t s0 = 0, cnt = 0; s0 < items.size(); s0 += cnt) {
+    // as many items as keep the digits of 512 terms within 1.5 GB (at least one)
     int kmax = 0;
     double per_k = 0.0;  // bytes of digits per unit of K
-    for (int i = 0; i < cnt; ++i) {
-      const auto &g = items[s0 + i];
+    for (cnt = 0; cnt < (size_t)DG_MAXB && s0 + cnt < items.size(); ++cnt) {
+      const auto &g = items[s0 + cnt];
+      const double b = 16.0 * (((g.m + 127) / 128) * 128.0 + ((g.n + 63) / 64) * 64.0);
+      if (cnt > 0 && (per_k + b) * std::min(512, std::max(kmax, g.k)) > 1.5e9) break;
       kmax = std::max(kmax, g.k);
-      per_k += 16.0 * (((g.m + 127) / 128) * 128.0 + ((g.n + 63) / 64) * 64.0);
+      per_k += b;
     }
     // K in passes whose digits fit in 1.5 GB; every pass but the first adds to C
     const int kpass = std::min<double>(kmax, std::max(512.0, std::floor(1.5e9 / per_k / 512.0) * 512.0));
@@ -473,7 +475,7 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
       };
       std::vector<int> ia, ib;
       double work = 0.0;
-      for (int i = 0; i < cnt; ++i) {
+      for (int i = 0; i < (int)cnt; ++i) {
         const auto &g = items[s0 + i];
         const int k = std::min(kpass, g.k - kp);
         ia.push_back(-1);
@@ -528,7 +530,7 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
         be = std::max<long long>(be, s.mode == 1 ? (s.nv + 7) / 8 : (long long)((s.nv + 31) / 32) * ((s.k + 255) / 256));
         bp = std::max<long long>(bp, (long long)((s.nv + 63) / 64) * nkt);
       }
-      for (int i = 0, q = 0; i < cnt; ++i) {
+      for (int i = 0, q = 0; i < (int)cnt; ++i) {
         if (ia[i] < 0) continue;
         DgItem &x = gb.it[q++];
         const Src &a = srcs[ia[i]], &c = srcs[ib[i]];
@@ -560,7 +562,7 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
       }
       if (e0) {
         double flops = 0.0;
-        for (int i = 0; i < cnt; ++i) {
+        for (int i = 0; i < (int)cnt; ++i) {
           const auto &g = items[s0 + i];
           flops += 2.0 * g.m * (double)g.n * std::max(0, std::min(kpass, g.k - kp));
         }

@@ -315,6 +315,16 @@ int rfdd_polish(rfdd_handle *h, int64_t nev, double *lambda, double *X, double *
  * Needs no handle (runs on the default stream of the current device). */
 int rfdd_sym_eig(int64_t n, const double *H, double *evals, double *evecs);
 
+/* a9 building block (linearly dependent basis columns are dropped by their pivots): pivoted
+ * Cholesky P^T G P = R^T R of the symmetric positive semidefinite k x k FP64 matrix G, stopped at the
+ * first pivot <= tol or not finite.  Host arrays: G (k x k row-major), perm (k; its first *rank
+ * entries are the pivots in order), R (room for k x k; on return *rank x *rank row-major, upper).
+ * polls: limit of the waits among the CTAs of its one launch (0: the library's own, seconds);
+ * RFDD_ECUDA, with the outputs untouched, when such a wait ran out.  Needs no handle (runs on the
+ * default stream of the current device). */
+int rfdd_pivoted_cholesky(int64_t k, const double *G, double tol, int32_t polls, int64_t *rank,
+                          int32_t *perm, double *R);
+
 /* Building block of a3-a5 (trailing updates of the factorisations), a6 and a10 (triangular-solve
  * updates): C = beta*C + alpha*A*B for complex single-precision A (m x k, leading dimension lda),
  * B (k x n, ldb), C (m x n, ldc), host arrays, row-major, interleaved (re, im) floats.

@@ -39,7 +39,7 @@ SYMBOLS = [
     "rfdd_layout", "rfdd_destroy", "rfdd_solve", "rfdd_result_get", "rfdd_result_info",
     "rfdd_result_pre_evals", "rfdd_result_free", "rfdd_factor", "rfdd_schur_copy", "rfdd_shifted_solve",
     "rfdd_filter_apply", "rfdd_lanczos", "rfdd_interior", "rfdd_rayleigh_ritz", "rfdd_solve_async",
-    "rfdd_result_ready", "rfdd_memory_estimate", "rfdd_sym_eig", "rfdd_kernel_launches", "rfdd_profile",
+    "rfdd_result_ready", "rfdd_memory_estimate", "rfdd_sym_eig", "rfdd_pivoted_cholesky", "rfdd_kernel_launches", "rfdd_profile",
     "rfdd_profile_get", "rfdd_profile_busy", "rfdd_cgemm", "rfdd_dgemm", "rfdd_cgemm_noalloc", "rfdd_inertia",
     "rfdd_polish", "rfdd_peak_probe", "rfdd_profile_bytes", "rfdd_release",
     "rfdd_server_default_options", "rfdd_server_create", "rfdd_server_add_pencil", "rfdd_server_submit",
@@ -148,6 +148,7 @@ def load(path: str | None = None):
     lib.rfdd_rayleigh_ritz.argtypes = [vp, i64, dp, C.POINTER(i64)]
     lib.rfdd_memory_estimate.argtypes = [vp, i32, i64, C.POINTER(C.c_size_t)]
     lib.rfdd_sym_eig.argtypes = [i64, dp, dp, dp]
+    lib.rfdd_pivoted_cholesky.argtypes = [i64, dp, C.c_double, i32, C.POINTER(i64), C.POINTER(i32), dp]
     lib.rfdd_kernel_launches.restype = C.c_longlong
     fp = C.POINTER(C.c_float)
     lib.rfdd_cgemm.argtypes = [i64, i64, i64, fp, i64, fp, i64, fp, i64, C.c_double, C.c_double, i32]
@@ -453,6 +454,17 @@ def rfdd_sym_eig(H: np.ndarray):
     V = np.zeros((n, n))
     _check(load().rfdd_sym_eig(n, _dp(H), _dp(ev), _dp(V)))
     return ev, V
+
+
+def rfdd_pivoted_cholesky(G: np.ndarray, tol: float, polls: int = 0):
+    """Pivoted Cholesky of the symmetric G on the GPU: (rank, pivots in order, R) with R^T R = G[pivots][:, pivots]."""
+    G = np.ascontiguousarray(G, dtype=np.float64)
+    k = G.shape[0]
+    rank, perm, Rf = C.c_int64(), np.empty(k, dtype=np.int32), np.empty(k * k)
+    _check(load().rfdd_pivoted_cholesky(k, _dp(G), tol, polls, C.byref(rank),
+                                        perm.ctypes.data_as(C.POINTER(C.c_int32)), _dp(Rf)))
+    r = int(rank.value)
+    return r, perm[:r], Rf[: r * r].reshape(r, r)
 
 
 def rfdd_cgemm(A: np.ndarray, B: np.ndarray, C: np.ndarray, alpha: float = 1.0, beta: float = 0.0,

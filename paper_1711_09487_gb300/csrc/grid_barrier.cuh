@@ -9,8 +9,9 @@ constexpr int GRID_SPIN = 1 << 22;
 // Every CTA adds one to *cnt (zero before the launch) and waits until it has reached target, the number of CTAs
 // times the number of barriers so far.  What any thread of a CTA wrote before is visible to all threads
 // after it (global loads of other CTAs' data through L2).  false: the wait ran out.  A flag per CTA that
-// every other CTA polls, in place of the counter, made a step of 152 CTAs 2.5 us longer.
-__device__ __forceinline__ bool grid_barrier(unsigned *cnt, unsigned target) {
+// every other CTA polls, in place of the counter, made a step of 152 CTAs 2.5 us longer.  polls: reads of the counter
+// before a CTA gives up; one that does has already been counted, so the others pass this barrier and give up at the next.
+__device__ __forceinline__ bool grid_barrier(unsigned *cnt, unsigned target, int polls = GRID_SPIN) {
   __shared__ int ok_s;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -20,7 +21,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *cnt, unsigned target) {
     int k = 0;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
-    } while (v < target && ++k < GRID_SPIN);
+    } while (v < target && ++k < polls);
     ok_s = v >= target;
   }
   __syncthreads();

@@ -324,6 +324,8 @@ namespace rfdd {
 // or not finite.  Then r_t[j] = (G[p][j] - sum_s R[s][p] R[s][j]) / sqrt(d_p) and d_j -= r_t[j]^2 for the CTA's columns.
 // k r^2 / 2 FP64 FMAs in all (7.7 ms of the chip's FP64 rate for k = 2720, r = 1884) and about 5 us a step: 384
 // steps 2.1 ms (4.15 in two launches a step on the trailing triangle), the 2720 columns about 20 ms (50).
+// *rank is 0 before the launch and written once, by a factorisation that has come to its end: where a barrier
+// ran out it stays 0, and nothing indexes through perm, whose entries from the step on are not set.
 // ---------------------------------------------------------------------------------------
 constexpr int PCH_THREADS = 512;
 constexpr int PCH_XMAX = 24 * 1024;  // entries of the pivot's column kept in shared memory
@@ -335,7 +337,7 @@ struct PchOffer {
 
 __global__ void __launch_bounds__(PCH_THREADS) pchol_kernel(const double *__restrict__ Gm, int k, double *Rt, int *perm,
                                                             double tol, int *rank, PchOffer *offers, unsigned *bar,
-                                                            int *status) {
+                                                            int polls, int *status) {
   extern __shared__ double sm[];
   const int me = blockIdx.x, ng = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = PCH_THREADS / 32;
@@ -365,7 +367,7 @@ __global__ void __launch_bounds__(PCH_THREADS) pchol_kernel(const double *__rest
       best();
       if (lane == 0) of[me] = {bv, bi};
     }
-    if (!grid_barrier(bar, (unsigned)ng * (unsigned)(t + 1))) {
+    if (!grid_barrier(bar, (unsigned)ng * (unsigned)(t + 1), polls)) {
       if (tid == 0) atomicOr(status, DS_GRID_TIMEOUT);
       return;
     }
@@ -440,12 +442,13 @@ __global__ void __launch_bounds__(PCH_THREADS) pchol_kernel(const double *__rest
     }
     __syncthreads();
   }
+  if (me == 0 && tid == 0) *rank = k;
 }
 
 // R into the leading r x r upper triangle of G: G[t][i] = Rt[perm[i]][t] for t <= i < r
 __global__ void __launch_bounds__(256) pchol_gather_kernel(const double *__restrict__ Rt, const int *__restrict__ perm,
                                                            int k, const int *rank_p, double *G) {
-  const int r = *rank_p < 0 ? k : *rank_p;
+  const int r = *rank_p;
   __shared__ double tile[32][33];
   const int i0 = blockIdx.x * 32, t0 = blockIdx.y * 32, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (i0 >= r || t0 >= r || i0 + 31 < t0) return;
@@ -458,11 +461,9 @@ __global__ void __launch_bounds__(256) pchol_gather_kernel(const double *__restr
   }
 }
 
-__global__ void set_int_kernel(int *p, int v) { *p = v; }
-
-int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, int *rank_dev, int *status) {
-  set_int_kernel<<<1, 1, 0, st>>>(rank_dev, -1);
-  RFDD_CHECK_LAUNCH();
+int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, int *rank_dev, int *status, int polls) {
+  if (polls <= 0) polls = GRID_SPIN;
+  RFDD_CUDA(cudaMemsetAsync(rank_dev, 0, sizeof(int), st));
   const int ng = std::max(1, std::min(sm_count(), k));
   double *Rt = nullptr;
   PchOffer *offers = nullptr;
@@ -474,7 +475,7 @@ int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, i
   RFDD_REQUIRE(smem <= 220 * 1024, RFDD_EINVAL, "pivoted Cholesky: order too large");
   RFDD_CUDA(cudaFuncSetAttribute(pchol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
   const double *Gc = G;
-  void *args[] = {&Gc, &k, &Rt, &perm, &tol, &rank_dev, &offers, &bar, &status};
+  void *args[] = {&Gc, &k, &Rt, &perm, &tol, &rank_dev, &offers, &bar, &polls, &status};
   RFDD_CUDA(cudaLaunchCooperativeKernel((const void *)pchol_kernel, dim3(ng), dim3(PCH_THREADS), args, smem, st));
   RFDD_CHECK_LAUNCH();
   const unsigned nt = (unsigned)ceil_div(k, 32);
@@ -482,10 +483,10 @@ int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, i
   RFDD_CHECK_LAUNCH();
   RFDD_CUDA(cudaFreeAsync(Rt, st));
   RFDD_CUDA(cudaFreeAsync(offers, st));
-  int rank = -1;
+  int rank = 0;
   RFDD_CUDA(cudaMemcpyAsync(&rank, rank_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
   RFDD_CUDA(cudaStreamSynchronize(st));
-  return rank < 0 ? k : rank;
+  return rank;
 }
 
 // out[i][j] = K[perm[i]][perm[j]] for i, j < r

@@ -1827,6 +1827,7 @@ RRout rayleigh_ritz_coeffs(rfdd_handle *h, const double *Y, int64_t k, double dr
   scale_sym(st, K.as<double>(), k, dsc.as<double>());
   const int r = pivoted_cholesky(st, G.as<double>(), (int)k, perm.as<int>(), drop, rankd.as<int>(),
                                  h->status.as<int>());
+  sync_status(h, "rayleigh-ritz: pivoted Cholesky");  // before perm is an index anywhere
   lap.mark("pivoted cholesky");
   RFDD_REQUIRE(r > 0, RFDD_ESINGULAR, "Rayleigh-Ritz: basis has no independent direction");
   // H = R^{-T} Kp R^{-1}.  R = D R' with D its diagonal and R' unit upper; |R'| <= 1 by the pivoting, so Lt = R'^T is a
@@ -3839,6 +3840,36 @@ int rfdd_sym_eig(int64_t n, const double *H, double *evals, double *evecs) {
     RFDD_REQUIRE(stt == 0, RFDD_ESINGULAR, "sym_eig: eigensolver reported a failure");
     RFDD_CUDA(cudaMemcpy(evals, lam.p, n * sizeof(double), cudaMemcpyDeviceToHost));
     RFDD_CUDA(cudaMemcpy(evecs, out.p, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToHost));
+  });
+}
+
+int rfdd_pivoted_cholesky(int64_t k, const double *G, double tol, int32_t polls, int64_t *rank, int32_t *perm,
+                          double *R) {
+  if (k < 1 || k > INT32_MAX || polls < 0 || !G || !rank || !perm || !R) return RFDD_EINVAL;
+  return guarded([&] {
+    cudaStream_t st = 0;
+    Buf Gd, pd, rd, status;
+    Gd.alloc((size_t)k * k * sizeof(double));
+    RFDD_CUDA(cudaMemcpy(Gd.p, G, (size_t)k * k * sizeof(double), cudaMemcpyHostToDevice));
+    pd.alloc((size_t)k * sizeof(int));
+    rd.alloc(sizeof(int));
+    status.alloc(sizeof(int));
+    RFDD_CUDA(cudaMemset(status.p, 0, sizeof(int)));
+    const int r = pivoted_cholesky(st, Gd.as<double>(), (int)k, pd.as<int>(), tol, rd.as<int>(), status.as<int>(), polls);
+    int stt = 0;
+    RFDD_CUDA(cudaMemcpy(&stt, status.p, sizeof(int), cudaMemcpyDeviceToHost));
+    RFDD_REQUIRE(stt == 0, RFDD_ECUDA, "pivoted Cholesky: the CTAs timed out waiting for each other");
+    std::vector<double> full((size_t)k * r);
+    std::vector<int> hp(r);
+    if (r > 0) {
+      RFDD_CUDA(cudaMemcpy(full.data(), Gd.p, (size_t)k * r * sizeof(double), cudaMemcpyDeviceToHost));
+      RFDD_CUDA(cudaMemcpy(hp.data(), pd.p, (size_t)r * sizeof(int), cudaMemcpyDeviceToHost));
+    }
+    *rank = r;
+    for (int64_t i = 0; i < r; ++i) {
+      perm[i] = hp[i];
+      for (int64_t j = 0; j < r; ++j) R[i * r + j] = j >= i ? full[(size_t)i * k + j] : 0.0;
+    }
   });
 }
 

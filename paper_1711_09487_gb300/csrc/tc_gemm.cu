@@ -778,13 +778,15 @@ __device__ __forceinline__ void pack_a_rows(const PackItem &it) {
   constexpr int F = CPLX ? 2 : 1;
   const int kf = F * it.k, nq = it.nkt * 8, rows_pad = it.nblk * TC_BM;
   const int lpr = nq >= 32 ? 32 : nq >= 16 ? 16 : 8, per = 32 * NW / lpr, lane = threadIdx.x % lpr;
+  // complex entries in one access where they lie on 8 bytes; the caller's pointer is one to floats
+  const bool al8 = CPLX && (uintptr_t)it.src % 8 == 0;
   // rows_pad is a multiple of per, so the lanes of a warp stay together
   for (int row = blockIdx.x * per + (int)threadIdx.x / lpr; row < rows_pad; row += gridDim.x * per) {
     const float *src = it.src + (long long)row * F * it.ld;
     const bool live = row < it.rows;
     auto load8 = [&](int q, float (&x)[8]) {
       const int k0 = q * 8;
-      if (CPLX) {
+      if (al8) {
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           const float2 v = (live && k0 + 2 * t < kf) ? *reinterpret_cast<const float2 *>(src + k0 + 2 * t)
@@ -853,6 +855,7 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
   __shared__ float smax[NW][64];
   __shared__ float mul_s[64];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool al8 = CPLX && (uintptr_t)it.src % 8 == 0;  // as in pack_a_rows
   const int nch = (it.k + PACK_KC - 1) / PACK_KC;
   for (int jb = blockIdx.x; jb < it.nblk; jb += gridDim.x) {
     const long long j0 = (long long)jb * CW;
@@ -861,8 +864,12 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
         const bool on = j0 + lane < it.rows;
 #pragma unroll 8
         for (int p = warp; p < pn; p += NW) {
-          const float2 v = on ? *reinterpret_cast<const float2 *>(it.src + 2 * ((long long)(p0 + p) * it.ld + j0 + lane))
-                              : make_float2(0.f, 0.f);
+          const float *s = it.src + 2 * ((long long)(p0 + p) * it.ld + j0 + lane);
+          float2 v = make_float2(0.f, 0.f);
+          if (on) {
+            if (al8) v = *reinterpret_cast<const float2 *>(s);
+            else v = make_float2(s[0], s[1]);
+          }
           *reinterpret_cast<float2 *>(sb + p * PITCH + 2 * lane) = v;
           m0 = fmaxf(m0, fmaxf(fabsf(v.x), fabsf(v.y)));
         }

@@ -155,6 +155,10 @@ enum DevStatus : int {
   DS_GRID_TIMEOUT = 16,  // a barrier among the CTAs of a cooperative kernel ran out
 };
 
+// A status buffer: the DevStatus bits, then a word that the operand packing of the tensor-core GEMM sets when it meets
+// scales far from one and that stays set (tc_gemm.cu); both zero at first.
+constexpr int STATUS_WORDS = 2;
+
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 // Sizes that set the device memory of a solve (admission estimates).

@@ -90,8 +90,8 @@ double tf32_probe(cudaStream_t st) {
   fill_probe_kernel<<<1024, 256, 0, st>>>(B, e, 0.5f);
   RFDD_CHECK_LAUNCH();
   int *status = nullptr;
-  RFDD_CUDA(cudaMallocAsync((void **)&status, sizeof(int), st));
-  RFDD_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
+  RFDD_CUDA(cudaMallocAsync((void **)&status, STATUS_WORDS * sizeof(int), st));
+  RFDD_CUDA(cudaMemsetAsync(status, 0, STATUS_WORDS * sizeof(int), st));
   const GemmItem<float> it = {A, B, C, N, N, N, N, N, N};
   double best = 0.0;
   {
@@ -121,8 +121,8 @@ double tf32_probe(cudaStream_t st) {
 
 double mma_probe(cudaStream_t st) {
   int *status = nullptr;
-  RFDD_CUDA(cudaMallocAsync((void **)&status, sizeof(int), st));
-  RFDD_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
+  RFDD_CUDA(cudaMallocAsync((void **)&status, STATUS_WORDS * sizeof(int), st));
+  RFDD_CUDA(cudaMemsetAsync(status, 0, STATUS_WORDS * sizeof(int), st));
   double r = 0.0;
   try {
     r = tc_mma_probe_tflops(st, status);

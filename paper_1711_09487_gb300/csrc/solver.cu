@@ -762,8 +762,8 @@ void do_upload(rfdd_handle *h) {
   upload(h->sidx_off_dev, h->sidx_off, st);
   upload(h->posmap, posmap, st);
   upload(h->iperm_dev, h->iperm, st);
-  h->status.alloc(sizeof(int));
-  RFDD_CUDA(cudaMemsetAsync(h->status.p, 0, sizeof(int), st));
+  h->status.alloc(STATUS_WORDS * sizeof(int));
+  RFDD_CUDA(cudaMemsetAsync(h->status.p, 0, STATUS_WORDS * sizeof(int), st));
   RFDD_CUDA(cudaStreamSynchronize(st));
   h->P.n = n;
   h->P.nnz = h->nnz;
@@ -2245,8 +2245,8 @@ void interior_factor_start(rfdd_handle *h, double sigma, cudaStream_t on) {
   }
   int *status = h->status.as<int>();
   if (on != st) {
-    if (!h->I_status.p) h->I_status.alloc(sizeof(int));
-    RFDD_CUDA(cudaMemsetAsync(h->I_status.p, 0, sizeof(int), st));
+    if (!h->I_status.p) h->I_status.alloc(STATUS_WORDS * sizeof(int));
+    RFDD_CUDA(cudaMemsetAsync(h->I_status.p, 0, STATUS_WORDS * sizeof(int), st));
     status = h->I_status.as<int>();
     RFDD_CUDA(cudaEventRecord(h->ev_fork, st));
   }
@@ -3824,8 +3824,8 @@ int rfdd_sym_eig(int64_t n, const double *H, double *evals, double *evecs) {
     w.alloc(n * sizeof(double));
     lam.alloc(n * sizeof(double));
     Z.alloc((size_t)n * n * sizeof(double));
-    status.alloc(sizeof(int));
-    RFDD_CUDA(cudaMemset(status.p, 0, sizeof(int)));
+    status.alloc(STATUS_WORDS * sizeof(int));
+    RFDD_CUDA(cudaMemset(status.p, 0, STATUS_WORDS * sizeof(int)));
     SymItem si{Hd.as<double>(), (int)n, (int)n, d.as<double>(), e.as<double>(), t.as<double>(), w.as<double>(),
                lam.as<double>(), Z.as<double>()};
     TcStatusScope tcs(status.as<int>());
@@ -3853,8 +3853,8 @@ int rfdd_pivoted_cholesky(int64_t k, const double *G, double tol, int32_t polls,
     RFDD_CUDA(cudaMemcpy(Gd.p, G, (size_t)k * k * sizeof(double), cudaMemcpyHostToDevice));
     pd.alloc((size_t)k * sizeof(int));
     rd.alloc(sizeof(int));
-    status.alloc(sizeof(int));
-    RFDD_CUDA(cudaMemset(status.p, 0, sizeof(int)));
+    status.alloc(STATUS_WORDS * sizeof(int));
+    RFDD_CUDA(cudaMemset(status.p, 0, STATUS_WORDS * sizeof(int)));
     const int r = pivoted_cholesky(st, Gd.as<double>(), (int)k, pd.as<int>(), tol, rd.as<int>(), status.as<int>(), polls);
     int stt = 0;
     RFDD_CUDA(cudaMemcpy(&stt, status.p, sizeof(int), cudaMemcpyDeviceToHost));
@@ -3889,8 +3889,8 @@ int rfdd_cgemm(int64_t m, int64_t n, int64_t k, const float *A, int64_t lda, con
     std::vector<GemmItem<cx<float>>> it = {{a.as<cx<float>>(), b.as<cx<float>>(), c.as<cx<float>>(), (int)m, (int)n,
                                             (int)k, (int)lda, (int)ldb, (int)ldc}};
     Buf status;
-    status.alloc(sizeof(int));
-    RFDD_CUDA(cudaMemset(status.p, 0, sizeof(int)));
+    status.alloc(STATUS_WORDS * sizeof(int));
+    RFDD_CUDA(cudaMemset(status.p, 0, STATUS_WORDS * sizeof(int)));
     if (engine >= 1 && engine <= 3) {
       TcStatusScope tcs(status.as<int>());
       TcEngineScope eng(engine == 2 ? 1 : engine == 3 ? 2 : 0);
@@ -3924,8 +3924,8 @@ int rfdd_dgemm(int64_t m, int64_t n, int64_t k, int32_t ta, const double *A, int
     std::vector<GemmItem<double>> it = {
         {a.as<double>(), b.as<double>(), c.as<double>(), (int)m, (int)n, (int)k, (int)lda, (int)ldb, (int)ldc}};
     Buf status;
-    status.alloc(sizeof(int));
-    RFDD_CUDA(cudaMemset(status.p, 0, sizeof(int)));
+    status.alloc(STATUS_WORDS * sizeof(int));
+    RFDD_CUDA(cudaMemset(status.p, 0, STATUS_WORDS * sizeof(int)));
     {
       TcStatusScope tcs(status.as<int>());
       if (engine == 1) gemm_f64x2_batched(st, it, ta != 0, tb != 0, alpha, beta, {(char)(sym != 0)});

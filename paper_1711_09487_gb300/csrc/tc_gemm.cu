@@ -97,7 +97,7 @@ constexpr int TC_MAXB = 64;
 struct TcBatchP {
   TcItem it[TC_MAXB];
   int count, total_tiles;
-  int *err;    // status word of the launch (DS_WAIT_TIMEOUT on a wait that ran out)
+  int *err;    // status words of the launch (DS_WAIT_TIMEOUT on a wait that ran out; far scales, see far_launch)
 };
 
 __device__ __forceinline__ int find_item(const TcBatchP &b, int tile) {
@@ -152,15 +152,59 @@ struct ChunkC {
   }
 };
 
+// Scales that the usual order of the read-back (drain_tile: (x rr) (alpha rb)) cannot take: an accumulator is below 2^45 and
+// scales lie between 2^-126 and 2^114, so x rr stays in range up to rr = 2^80, and alpha rb for columns within 2^100 of 1 and an
+// alpha within 2^20 of 1.  The packing records others in the word after the status word; launches that find it set, or have
+// such an alpha, read back by drain_far.  Looked at tile by tile the check cost more than the read-back
+// gained, and with both orders in one body it spilled: K = 32 update of 8192 x 8192 0.27 ms, 0.30 and 0.36 with these.
+__device__ __forceinline__ bool far_row(float s) { return s > 0x1p80f; }
+__device__ __forceinline__ bool far_col(float s) { return !(s >= 0x1p-100f && s <= 0x1p100f); }
+__device__ __forceinline__ bool far_launch(const int *err, float alpha) {
+  const float a = fabsf(alpha);
+  return __ldcg(err + 1) != 0 || !(a >= 0x1p-20f && a <= 0x1p20f);
+}
+
+// Read-back of such launches: scales on one side of 1 one after the other, scales on different sides by their
+// product, then alpha.
+template <int NCH, typename W, typename F>
+__device__ __forceinline__ bool drain_far(const TcItem &it, uint32_t tacc, int mt, int col0, int q, int c0, int lane,
+                                          float *stg, float alpha, float beta, W &&wait, F &&done) {
+  const int row0 = mt * TC_BM + q * 32, nrows = min(32, it.m - row0);
+  if (!wait()) return false;
+#pragma unroll 1
+  for (int c = c0; c < c0 + NCH; ++c) {
+    uint32_t v[32];
+    TC_LD32(tacc + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32), v);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    if (c == c0 + NCH - 1) done();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) stg[lane * 32 + (j ^ lane)] = __uint_as_float(v[j]);
+    __syncwarp();
+    const int j = col0 + c * 32 + lane;
+    if (j < it.n2) {
+      const float rb = it.sB[j];
+#pragma unroll 1
+      for (int r = 0; r < nrows; ++r) {
+        const float rr = it.sA[row0 + r], x = stg[r * 32 + (lane ^ r)];
+        const float y = (rr >= 1.f) == (rb >= 1.f) ? (x * rr) * rb : x * (rr * rb);
+        float *p = it.C + (long long)(row0 + r) * it.ldc + j;
+        *p = fmaf(alpha, y, beta != 0.f ? beta * *p : 0.f);
+      }
+    }
+    __syncwarp();
+  }
+  return true;
+}
+
 // Epilogue of one output tile by one warp: TMEM lanes 32q..32q+31 (rows mt*128 + 32q ..), NCH column
 // chunks of 32 accumulator columns from chunk c0 on; C = alpha * scaled acc + beta * C, rows and columns
 // masked.  The accumulator's rows are turned into C's through shared memory (16-byte pieces of row r at
 // piece ^ (r & 7): no bank conflicts either way).  What bounds it is the latency of C: two chunks of C are in
 // flight from before the accumulator is ready (`wait` returns false if it never is), and each is
 // replaced by the chunk after the next as soon as it has been used.  `done` runs once the
-// accumulator has been read.  Measured, 8192 x 8192 complex: K = 32 0.28 ms (0.35 with one chunk in flight
-// and one float per access), K = 256 0.29 ms = 472 TFLOP/s (0.37; 0.49 with the TF32 split), K = 512 0.50 ms =
-// 547 TFLOP/s, 1.64 PFLOP/s of MMAs.
+// accumulator has been read.  Measured, 8192 x 8192 complex, C rows on 32 bytes, the best of four launches each: K = 32
+// 0.27 ms (0.35 with one chunk in flight and one float per access), K = 256 0.296 ms = 465 TFLOP/s (0.37 so; 0.49 with the
+// TF32 split).
 template <int NCH, bool SCALED, int V, typename W, typename F>
 __device__ __forceinline__ bool drain_tile(const TcItem &it, uint32_t tacc, int mt, int col0, int q, int c0, int lane,
                                            float *stg, float alpha, float beta, W &&wait, F &&done) {
@@ -170,7 +214,7 @@ __device__ __forceinline__ bool drain_tile(const TcItem &it, uint32_t tacc, int 
   float cb[NCH > 1 ? 2 : 1][32];
   CC::load(it, row0, nrows, col0 + c0 * 32, lane, beta, cb[0]);
   if (NCH > 1) CC::load(it, row0, nrows, col0 + c0 * 32 + 32, lane, beta, cb[NCH > 1 ? 1 : 0]);
-  // scale of the row this lane takes from the accumulator, times alpha
+  // scale of the row this lane takes from the accumulator
   const float ra = SCALED && lane < nrows ? it.sA[row0 + lane] : 1.f;
   if (!wait()) return false;
 #pragma unroll
@@ -180,7 +224,7 @@ __device__ __forceinline__ bool drain_tile(const TcItem &it, uint32_t tacc, int 
 #pragma unroll
     for (int t = 0; t < V; ++t) {
       const int j = cc + CC::col(lane) + t;
-      rb[t] = SCALED && j < it.n2 ? it.sB[j] : 1.f;
+      rb[t] = (SCALED && j < it.n2 ? it.sB[j] : 1.f) * alpha;
     }
     uint32_t v[32];
     TC_LD32(tacc + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32), v);
@@ -204,10 +248,10 @@ __device__ __forceinline__ bool drain_tile(const TcItem &it, uint32_t tacc, int 
       if (V == 4) *reinterpret_cast<float4 *>(x) = *reinterpret_cast<const float4 *>(sp);
       else x[0] = *sp;
       const float rr = SCALED ? __shfl_sync(0xffffffffu, ra, r) : 1.f;
-      // the two scales are powers of two: their product first, so that neither over- or underflows alone
+      // the row's scale, then alpha times the column's: the product of the two scales may leave the range of a float
+      // where the result does not (sums near 2^-126, huge rows and columns without common entries)
 #pragma unroll
-      for (int t = 0; t < V; ++t)
-        x[t] = fmaf(SCALED ? alpha * (rr * rb[t]) : alpha, x[t], beta * cv[i * V + t]);
+      for (int t = 0; t < V; ++t) x[t] = fmaf(rb[t], SCALED ? x[t] * rr : x[t], beta * cv[i * V + t]);
       if (r < nrows) CC::store(it, p, cc + cl, x);
     }
     __syncwarp();
@@ -217,7 +261,10 @@ __device__ __forceinline__ bool drain_tile(const TcItem &it, uint32_t tacc, int 
 }
 template <int NCH, bool SCALED, typename W, typename F>
 __device__ __forceinline__ bool drain_tile_vec(const TcItem &it, uint32_t tacc, int mt, int col0, int q, int c0,
-                                               int lane, float *stg, float alpha, float beta, W &&wait, F &&done) {
+                                               int lane, float *stg, float alpha, float beta, bool far, W &&wait,
+                                               F &&done) {
+  if (SCALED && far)
+    return drain_far<NCH>(it, tacc, mt, col0, q, c0, lane, stg, alpha, beta, wait, done);
   if (it.vec == 4) return drain_tile<NCH, SCALED, 4>(it, tacc, mt, col0, q, c0, lane, stg, alpha, beta, wait, done);
   return drain_tile<NCH, SCALED, 1>(it, tacc, mt, col0, q, c0, lane, stg, alpha, beta, wait, done);
 }
@@ -244,7 +291,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
   float *epi = reinterpret_cast<float *>(base + TC_RING_BYTES);
   __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], tfull_bar[2], tempty_bar[2];
   __shared__ uint32_t tmem_s;
-  __shared__ volatile int abort_s;
+  __shared__ volatile int abort_s, far_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -259,6 +306,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (threadIdx.x == 64) far_s = F16 && far_launch(err, alpha);  // in shared memory: the epilogue has no register to spare
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)),
                  "r"(2 * BN)
@@ -371,7 +419,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
       tile_pos(it, local, mt, nt);
       const int acc = lt & 1;
       const bool ok = drain_tile_vec<NCH, F16>(
-          it, tmem + (uint32_t)(acc * BN), mt, nt * BN, q, c0, lane, stg, alpha, beta,
+          it, tmem + (uint32_t)(acc * BN), mt, nt * BN, q, c0, lane, stg, alpha, beta, far_s != 0,
           [&] {
             const bool ready = mbar_wait(smem_u32(&tfull_bar[acc]), (uint32_t)((lt >> 1) & 1), &abort_s);
             // the whole warp takes the same branch (tcgen05.ld is a warp-collective)
@@ -620,6 +668,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
     constexpr int NCH = TC_BN / 64;
     const int c0 = ((warp - 2) >> 2) * NCH;
     float *stg = epi + (warp - 2) * EPI_TILE;
+    const bool far = far_launch(err, alpha);
     const uint32_t tempty_leader0 = map_to_rank(smem_u32(&tempty_bar[0]), 0);
     const uint32_t tempty_leader1 = map_to_rank(smem_u32(&tempty_bar[1]), 0);
     int lt = 0;
@@ -630,7 +679,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
       const int mt = 2 * mp + (int)rank;  // rows beyond m (a missing second row) are masked
       const int acc = lt & 1;
       const bool ok = drain_tile_vec<NCH, true>(
-          it, tmem + (uint32_t)(acc * TC_BN), mt, nt * TC_BN, q, c0, lane, stg, alpha, beta,
+          it, tmem + (uint32_t)(acc * TC_BN), mt, nt * TC_BN, q, c0, lane, stg, alpha, beta, far,
           [&] {
             const bool ready = mbar_wait_cl(smem_u32(&tfull_bar[acc]), (uint32_t)((lt >> 1) & 1), &abort_s);
             const bool go = __all_sync(0xffffffffu, ready && !abort_s);
@@ -768,25 +817,24 @@ struct PackItem {
 struct PackBatchP {
   PackItem a[TC_MAXB], b[TC_MAXB];
   int na, nb;
+  int *far;  // set where a scale is far (far_launch)
 };
 
 // A tiles: [mt][kt] 128 rows x 64 halves; 16-byte chunk c of row r stored at chunk c ^ (r & 7).  A row takes 32
 // lanes, or 8 or 16 when it has no more chunks than that (the 32-deep panel updates): its largest magnitude
 // first, then the split (the second read of the row comes from L1 / L2).
-template <bool CPLX, int NW>
-__device__ __forceinline__ void pack_a_rows(const PackItem &it) {
+template <bool CPLX, int NW, bool AL8>
+__device__ __forceinline__ void pack_a_rows(const PackItem &it, int *far) {
   constexpr int F = CPLX ? 2 : 1;
   const int kf = F * it.k, nq = it.nkt * 8, rows_pad = it.nblk * TC_BM;
   const int lpr = nq >= 32 ? 32 : nq >= 16 ? 16 : 8, per = 32 * NW / lpr, lane = threadIdx.x % lpr;
-  // complex entries in one access where they lie on 8 bytes; the caller's pointer is one to floats
-  const bool al8 = CPLX && (uintptr_t)it.src % 8 == 0;
   // rows_pad is a multiple of per, so the lanes of a warp stay together
   for (int row = blockIdx.x * per + (int)threadIdx.x / lpr; row < rows_pad; row += gridDim.x * per) {
     const float *src = it.src + (long long)row * F * it.ld;
     const bool live = row < it.rows;
     auto load8 = [&](int q, float (&x)[8]) {
       const int k0 = q * 8;
-      if (al8) {
+      if (AL8) {
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
           const float2 v = (live && k0 + 2 * t < kf) ? *reinterpret_cast<const float2 *>(src + k0 + 2 * t)
@@ -819,6 +867,7 @@ __device__ __forceinline__ void pack_a_rows(const PackItem &it) {
     row_scale(ml, fl, il);
     row_scale(mr, fr, ir);
     if (lane == 0) {
+      if (far_row(il) || far_row(ir)) *far = 1;
       if (it.side > 0) {
         it.scale[row] = il;
         it.scale[rows_pad + row] = ir;
@@ -847,15 +896,14 @@ __device__ __forceinline__ void pack_a_rows(const PackItem &it) {
 // in shared memory with reads along B's rows, takes the largest magnitude of every column, and writes
 // the packed rows with coalesced 16-byte stores.  Deeper B is staged twice, chunk by chunk.
 constexpr int PACK_KC = 256;
-template <bool CPLX, int NW>
-__device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
+template <bool CPLX, int NW, bool AL8>
+__device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb, int *far) {
   constexpr int F = CPLX ? 2 : 1;
   constexpr int CW = 64 / F;            // columns of B per block
   constexpr int PITCH = CPLX ? 66 : 65;  // floats per staged row
   __shared__ float smax[NW][64];
   __shared__ float mul_s[64];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool al8 = CPLX && (uintptr_t)it.src % 8 == 0;  // as in pack_a_rows
   const int nch = (it.k + PACK_KC - 1) / PACK_KC;
   for (int jb = blockIdx.x; jb < it.nblk; jb += gridDim.x) {
     const long long j0 = (long long)jb * CW;
@@ -867,7 +915,7 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
           const float *s = it.src + 2 * ((long long)(p0 + p) * it.ld + j0 + lane);
           float2 v = make_float2(0.f, 0.f);
           if (on) {
-            if (al8) v = *reinterpret_cast<const float2 *>(s);
+            if (AL8) v = *reinterpret_cast<const float2 *>(s);
             else v = make_float2(s[0], s[1]);
           }
           *reinterpret_cast<float2 *>(sb + p * PITCH + 2 * lane) = v;
@@ -902,6 +950,7 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb) {
       float mul, inv;
       row_scale(m, mul, inv);
       mul_s[tid] = mul;
+      if (far_col(inv)) *far = 1;
       it.scale[(long long)jb * 64 + tid] = inv;
     }
     __syncthreads();
@@ -951,12 +1000,21 @@ template <bool CPLX, int NW>
 __global__ void __launch_bounds__(32 * NW) pack_f16_kernel(const __grid_constant__ PackBatchP pb, int *zero) {
   extern __shared__ float pack_sb[];
   if (zero && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero = 0;
-  if ((int)blockIdx.y < pb.na) pack_a_rows<CPLX, NW>(pb.a[blockIdx.y]);
-  else pack_b_rows<CPLX, NW>(pb.b[blockIdx.y - pb.na], pack_sb);
+  // complex entries are read in one access where they lie on 8 bytes (the caller's pointer is one to floats)
+  const bool is_a = (int)blockIdx.y < pb.na;
+  const PackItem &it = is_a ? pb.a[blockIdx.y] : pb.b[blockIdx.y - pb.na];
+  if (CPLX && (uintptr_t)it.src % 8 == 0) {
+    if (is_a) pack_a_rows<CPLX, NW, true>(it, pb.far);
+    else pack_b_rows<CPLX, NW, true>(it, pack_sb, pb.far);
+  } else {
+    if (is_a) pack_a_rows<CPLX, NW, false>(it, pb.far);
+    else pack_b_rows<CPLX, NW, false>(it, pack_sb, pb.far);
+  }
 }
 
 template <bool CPLX>
-static void launch_pack(cudaStream_t st, const PackBatchP &pb, int *zero = nullptr) {
+static void launch_pack(cudaStream_t st, PackBatchP &pb, int *words, int *zero = nullptr) {
+  pb.far = words + 1;
   if (pb.na + pb.nb == 0) return;
   long long blocks = 1, all = 0;
   int kmax = 0;
@@ -1271,7 +1329,7 @@ static void tc_gemm_run(cudaStream_t st, const std::vector<GemmItem<T>> &items, 
     }
     const int tiles = set_tiles(tb, TC_BN);
     tb.err = g_tc_status;
-    launch_pack<CPLX>(st, pk);
+    launch_pack<CPLX>(st, pk, g_tc_status);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (profiling_enabled()) {
       e0 = profile_event();
@@ -1404,6 +1462,7 @@ TcPackedA tc_packed_view(const void *op, int64_t m, int64_t k_full, int64_t r0, 
 }
 
 void tc_pack_a_batched(cudaStream_t st, const std::vector<TcPackJob> &jobs) {
+  RFDD_REQUIRE(g_tc_status != nullptr, RFDD_ESTATE, "operands packed without a status word");
   tc_device_setup();
   for (size_t s0 = 0; s0 < jobs.size(); s0 += TC_MAXB) {
     const int cnt = (int)std::min<size_t>(TC_MAXB, jobs.size() - s0);
@@ -1417,7 +1476,7 @@ void tc_pack_a_batched(cudaStream_t st, const std::vector<TcPackJob> &jobs) {
       pk.a[pk.na++] = {reinterpret_cast<const float *>(j.A), j.lda, (int)j.m, (int)j.k, hi, lo,
                        reinterpret_cast<float *>(lo + mtc * nkt * A_TILE), (int)mtc, (int)nkt, j.side};
     }
-    launch_pack<true>(st, pk);
+    launch_pack<true>(st, pk, g_tc_status);
   }
 }
 
@@ -1482,8 +1541,8 @@ constexpr size_t NOALLOC_A_BYTES = noalloc_bytes(NOALLOC_MT * NOALLOC_KT, A_TILE
 constexpr size_t NOALLOC_B_BYTES = noalloc_bytes(NOALLOC_NT * NOALLOC_KT, B_TILE, NOALLOC_NT * TC_BN);
 
 static __device__ __align__(256) uint8_t g_noalloc_scratch[NOALLOC_A_BYTES + NOALLOC_B_BYTES];  // 3 MiB
-// status word of the allocation-free launches (DS_WAIT_TIMEOUT), beside the scratch
-static __device__ int g_noalloc_status;
+// status words of the allocation-free launches, beside the scratch
+static __device__ int g_noalloc_status[STATUS_WORDS];
 
 struct NoallocAddr {
   uint8_t *scratch = nullptr;
@@ -1542,13 +1601,14 @@ int tc_gemm_complex_noalloc(cudaStream_t st, const cx<float> *A, int64_t lda, co
   it.mtc = mtc;
   tb.count = 1;
   tb.err = na.status;
-  // the status word keeps the last call's value: the packing launch clears it
-  launch_pack<true>(st, pk, na.status);
+  // the status word keeps the last call's value: the packing launch clears it; that of the far scales is cleared here
+  launch_pack<true>(st, pk, na.status, na.status);
   launch_one_cta(st, tb, nsm, alpha, beta);
-  int status = 0;
-  RFDD_CUDA(cudaMemcpyAsync(&status, na.status, sizeof(int), cudaMemcpyDeviceToHost, st));
+  int status[STATUS_WORDS] = {};
+  RFDD_CUDA(cudaMemcpyAsync(status, na.status, sizeof(status), cudaMemcpyDeviceToHost, st));
   RFDD_CUDA(cudaStreamSynchronize(st));
-  return status;
+  if (status[1]) RFDD_CUDA(cudaMemsetAsync(na.status + 1, 0, sizeof(int), st));
+  return status[0];
 }
 
 }  // namespace rfdd

@@ -5,7 +5,7 @@
 #include <string>
 
 namespace rfdd {
-// Status word (device int) that the tensor-core launches issued by the calling host thread record
+// Status words (STATUS_WORDS device ints) that the tensor-core launches issued by the calling host thread record
 // a failed wait in (DS_WAIT_TIMEOUT), for the lifetime of the scope.  A launch outside any scope is
 // refused with RFDD_ESTATE.
 struct TcStatusScope {

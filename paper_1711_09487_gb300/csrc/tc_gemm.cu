@@ -1607,7 +1607,10 @@ int tc_gemm_complex_noalloc(cudaStream_t st, const cx<float> *A, int64_t lda, co
   int status[STATUS_WORDS] = {};
   RFDD_CUDA(cudaMemcpyAsync(status, na.status, sizeof(status), cudaMemcpyDeviceToHost, st));
   RFDD_CUDA(cudaStreamSynchronize(st));
-  if (status[1]) RFDD_CUDA(cudaMemsetAsync(na.status + 1, 0, sizeof(int), st));
+  if (status[1]) {  // cleared before this call returns: the next one may come on another stream
+    RFDD_CUDA(cudaMemsetAsync(na.status + 1, 0, sizeof(int), st));
+    RFDD_CUDA(cudaStreamSynchronize(st));
+  }
   return status[0];
 }
 

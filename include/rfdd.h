@@ -342,9 +342,12 @@ int rfdd_cgemm(int64_t m, int64_t n, int64_t k, const float *A, int64_t lda, con
  * matrices, the interior CholQR, the Rayleigh-Ritz Gram matrices and Ritz vector updates):
  * C = beta*C + alpha*op(A)*op(B) for FP64 host arrays, row-major; op(X) = X^T when the flag is 1
  * (A then stored k x m with leading dimension lda >= m; B stored n x k with ldb >= k).
- * engine 0 = FP64 CUDA-core kernel; 1 = the kernels the solver uses for these products: large ones by
- * exact digit products on the tensor cores (55-bit operands relative to the largest entry of their row of op(A) or
- * column of op(B)), the others in double-FP32 (each operand split into two floats, error-free products
+ * engine 0 = FP64 CUDA-core kernel; 1 = the kernels the solver uses for these products.  Large ones (m, n, k >= 48
+ * and m n k >= 6.4e7) are exact digit products on the tensor cores: column k of op(A) is divided and row k of
+ * op(B) multiplied by the power of two of the column's largest entry, and the operands so scaled are integers of 2^-62 of
+ * the largest entry of their row of op(A) or column of op(B); |error| within k 2^-57 of the product of those two largest
+ * entries, plus the roundings of the result.  An entry of a row that holds infinities or NaN is NaN.  The
+ * others are in double-FP32 (each operand split into two floats, error-free products
  * and compensated sums: |error| within about 2^-42 of sum_k |a_ik||b_kj|).  sym = 1 declares op(A)*op(B) symmetric
  * (m == n required): only the upper 64 x 64 tiles are formed and mirrored.
  * Deep K with few output tiles is split over CTAs and the partial tiles summed in a fixed order. */

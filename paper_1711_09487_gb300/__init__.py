@@ -507,7 +507,8 @@ def rfdd_polish(h: Handle, lam, X):
 
 def rfdd_dgemm(A: np.ndarray, B: np.ndarray, C: np.ndarray, alpha: float = 1.0, beta: float = 0.0,
                ta: bool = False, tb: bool = False, engine: int = 1, sym: bool = False) -> np.ndarray:
-    """beta*C + alpha*op(A)@op(B) for float64 row-major arrays on the GPU (engine 1: double-FP32)."""
+    """beta*C + alpha*op(A)@op(B) for float64 row-major arrays on the GPU (engine 0: FP64 on the CUDA cores; 1: the
+    solver's basis products, large ones by digit products, small ones in double-FP32; bounds in rfdd.h)."""
     A = np.ascontiguousarray(A, dtype=np.float64)
     B = np.ascontiguousarray(B, dtype=np.float64)
     C = np.array(C, dtype=np.float64, order="C", copy=True)

@@ -1,19 +1,26 @@
 // FP64 GEMM on the tensor cores by exact digit products.
 //
-// Every row of op(A) and every column of op(B) is scaled by a power of two and rounded to a 55-bit
-// fixed-point integer, which is cut into eight balanced base-128 digits (-64 .. 63), each exact in
-// fp16.  The products of digit planes with equal weight, i + j = g, are summed by tcgen05 kind::f16
-// MMAs into one of eight FP32 accumulators: all addends are integers and their sums stay below 2^24
-// (8 pairs x 512 x 2^12), so every accumulator is exact.  After at most 512 terms of K the eight are read back and
+// Every row of op(A) and every column of op(B) is scaled by a power of two and rounded to a 63-bit
+// fixed-point integer (entries down to 2^-9 of the largest are exact), which is cut into eight balanced base-256
+// digits (-128 .. 127), each exact in fp16.  The products of digit planes with equal weight, i + j = g, are summed by
+// tcgen05 kind::f16 MMAs into one of eight FP32 accumulators: all addends are integers and their sums stay within 2^24
+// (8 pairs x 128 x 2^14), so every accumulator is exact.  After at most 128 terms of K the eight are read back and
 // added into two 64-bit integers per entry, which hold the sum exactly up to the planes that are left out (i + j
-// > 7, below 2^-50 of the product of the two scales per term); one rounding to FP64 at the end.  This
-// is the splitting of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59, 2012) with integer digits.
+// > 7); one rounding to FP64 at the end.  This is the splitting of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms
+// 59, 2012) with integer digits.
+//
+// Before that, the terms of the sum are brought to one size: column k of op(A) is divided, and row k of op(B) multiplied, by the
+// power of two of the column's largest entry (exponents only, exact).  Rows and columns scaled by factors of their own
+// (D A D for a diagonal D, whose factors and bases are graded along the sums) then lose nothing.
+//
+// Error of an entry: k 2^-57 (largest |a| of its row) (largest |b| of its column) of the operands so scaled, and the
+// roundings of the result.  For operands within a few powers of two of their largest entries that is below the
+// error of the sum in FP64, whatever its order.  (Digits of seven bits, 512 terms to a read-back, left out planes of 2^-49 of the largest product: 7 ulp on
+// operands whose digits have one sign.)
 //
 // What bounds it: the 36 plane products of a 128 x 64 x 32 stage read 12 KB of shared memory per 32
-// cycles of MMA (128 bytes per cycle is the limit), so a stage takes about 3500 cycles; that
-// is the bound from a few hundred terms on; below that the read-back (FP64 conversions) is.  Measured with
-// the packing: symmetric 1920 x 1920 x 64000 13.2 ms (134 ms in double-FP32), 384 x 384 x 64000 0.57 ms,
-// the 1885 x 1885 x 8000 product 9.2 -> 0.9 ms; its error falls from 8.2e-14 to 1.1e-15 of the norm.
+// cycles of MMA, by the descriptors, and a stage takes about 3500 cycles; that
+// is the bound from a few hundred terms on; below that the read-back is.
 #include "dense.cuh"
 #include "tc_common.cuh"
 #include "tc_gemm.cuh"
@@ -30,7 +37,10 @@ constexpr int DG_ATILE = DG_BM * 128, DG_BTILE = DG_BN * 128;  // bytes of one p
 constexpr int DG_ABYTES = DG_PAIRS * DG_ATILE, DG_BBYTES = DG_PAIRS * DG_BTILE;
 constexpr int DG_STAGE = DG_ABYTES + DG_BBYTES;  // 96 KB
 constexpr int DG_STAGES = 2;
-constexpr int DG_CHUNK = 16;   // stages between two read-backs (512 terms)
+constexpr int DG_BITS = 8;     // bits of a digit
+constexpr int DG_CHUNK = 4;    // stages between two read-backs (128 terms)
+constexpr int DG_SPLIT = 16;   // stages of the shallowest share of a split K (512 terms)
+static_assert(DG_PLANES * DG_CHUNK * DG_KT << 2 * (DG_BITS - 1) <= 1 << 24, "the accumulators stay exact");
 constexpr int DG_SMEM = DG_STAGES * DG_STAGE + 1024;
 constexpr int DG_EPI_WARPS = 8;
 constexpr int DG_THREADS = 64 + 32 * DG_EPI_WARPS;
@@ -46,23 +56,76 @@ struct DigitItem {
   int vb;           // vectors per tile (128 or 64)
   int nkt;
   uint8_t *dst;
-  int *emax;        // per vector: largest high word of |x|
+  int *emax;        // per vector: largest scaled exponent (term_exp)
+  int *kexp;        // per K-value: exponent of the largest entry of the column of op(A)
+  int ksign;        // -1: op(A), which is divided by these powers of two; 1: op(B)
 };
 struct DigitBatch {
   DigitItem it[2 * DG_MAXB];
   int count;
 };
 
-// Largest high word (sign dropped) of every vector, into emax (zeroed before).
+constexpr int DG_INF = 1 << 20;          // "exponent" of infinities and NaN
+constexpr int DG_NONE_BYTE = 0x80;       // exponents start as words of this byte, below that of any entry (zeros)
+constexpr int DG_NONE = (int)0x80808080u;
+
+// Biased exponent of x (1 for subnormal numbers), DG_NONE for zero, DG_INF for infinities and NaN; integer instructions
+__device__ __forceinline__ int term_exp(double x) {
+  const int hi = __double2hiint(x) & 0x7fffffff;
+  if ((hi | __double2loint(x)) == 0) return DG_NONE;
+  const int ex = hi >> 20;
+  return ex == 0x7ff ? DG_INF : max(ex, 1);
+}
+// the same with off added to the exponent of a finite nonzero x
+__device__ __forceinline__ int term_exp(double x, int off) {
+  const int ex = term_exp(x);
+  return ex == DG_NONE || ex == DG_INF ? ex : ex + off;
+}
+
+// Largest exponent of every column of op(A), into kexp (DG_NONE before); entries that are not finite do not count.
+__global__ void __launch_bounds__(256) digit_kexp_kernel(const __grid_constant__ DigitBatch b) {
+  const DigitItem &it = b.it[blockIdx.y];
+  if (it.ksign > 0) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto e = [](double x) {
+    const int ex = term_exp(x);
+    return ex == DG_INF ? DG_NONE : ex;
+  };
+  if (it.mode == 0) {  // a column of op(A) is contiguous
+    for (int k = blockIdx.x * 8 + warp; k < it.k; k += gridDim.x * 8) {
+      const double *s = it.src + (long long)k * it.ld;
+      int m = DG_NONE;
+      for (int v = lane; v < it.nv; v += 32) m = max(m, e(s[v]));
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) it.kexp[k] = m;
+    }
+    return;
+  }
+  // 32 columns x 256 rows per block step
+  const int nkb = (it.k + 31) / 32, nvb = (it.nv + 255) / 256;
+  for (int u = blockIdx.x; u < nkb * nvb; u += gridDim.x) {
+    const int k = (u % nkb) * 32 + lane, v0 = (u / nkb) * 256 + warp;
+    int m = DG_NONE;
+    if (k < it.k)
+#pragma unroll 8
+      for (int q = 0; q < 32; ++q) {
+        const int v = v0 + 8 * q;
+        if (v < it.nv) m = max(m, e(it.src[(long long)v * it.ld + k]));
+      }
+    if (m != DG_NONE) atomicMax(it.kexp + k, m);
+  }
+}
+
+// Largest scaled exponent of every vector, into emax (DG_NONE before).
 __global__ void __launch_bounds__(256) digit_emax_kernel(const __grid_constant__ DigitBatch b) {
   const DigitItem &it = b.it[blockIdx.y];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (it.mode == 1) {
     for (int v = blockIdx.x * 8 + warp; v < it.nv; v += gridDim.x * 8) {
       const double *s = it.src + (long long)v * it.ld;
-      int m = 0;
-      for (int k = lane; k < it.k; k += 32) m = max(m, __double2hiint(s[k]) & 0x7fffffff);
-      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+      int m = DG_NONE;
+      for (int k = lane; k < it.k; k += 32) m = max(m, term_exp(s[k], it.ksign * it.kexp[k]));
+      m = __reduce_max_sync(0xffffffffu, m);
       if (lane == 0) it.emax[v] = m;
     }
     return;
@@ -73,43 +136,43 @@ __global__ void __launch_bounds__(256) digit_emax_kernel(const __grid_constant__
   const int nvb = (nc + 31) / 32, nkb = (kr + 255) / 256;
   for (int u = blockIdx.x; u < nvb * nkb; u += gridDim.x) {
     const int v = (u % nvb) * 32 + lane, k0 = (u / nvb) * 256 + warp;
-    int m = 0;
+    int m = DG_NONE, m1 = DG_NONE;
     if (v < nc)
 #pragma unroll 8
       for (int q = 0; q < 32; ++q) {
         const int k = k0 + 8 * q;
         if (k < kr) {
           const double *s = it.src + ((long long)k * it.ld + v) * f;
-          m = max(m, __double2hiint(s[0]) & 0x7fffffff);
-          if (f == 2) m = max(m, __double2hiint(s[1]) & 0x7fffffff);
+          if (f == 1) {
+            m = max(m, term_exp(s[0], it.ksign * it.kexp[k]));
+          } else {  // column 2 v: re, -im; column 2 v + 1: im, re
+            const int o0 = it.ksign * it.kexp[2 * k], o1 = it.ksign * it.kexp[2 * k + 1];
+            m = max(m, max(term_exp(s[0], o0), term_exp(s[1], o1)));
+            m1 = max(m1, max(term_exp(s[1], o0), term_exp(s[0], o1)));
+          }
         }
       }
-    if (m > 0) {
-      atomicMax(it.emax + v * f, m);
-      if (f == 2) atomicMax(it.emax + 2 * v + 1, m);
-    }
+    if (m != DG_NONE) atomicMax(it.emax + v * f, m);
+    if (m1 != DG_NONE) atomicMax(it.emax + 2 * v + 1, m1);
   }
 }
 
-// Fixed point of x for a vector whose largest high word is em: x 2^(54 - 1 - E), E the exponent of the largest
-// entry, rounded to nearest: |q| < 2^54.
-__device__ __forceinline__ long long fixed55(double x, int em) {
+// Fixed point of x, its exponent shifted by off, for a vector whose largest such exponent is em: the integer nearest to
+// x 2^(off + 1084 - em), |q| < 2^62.
+__device__ __forceinline__ long long fixed63(double x, int off, int em) {
   const long long bits = __double_as_longlong(x);
-  const int ex = (int)((bits >> 52) & 0x7ff), emx = em >> 20;
-  if (emx == 0x7ff || ex == 0x7ff) return 0;  // infinities and NaN: the vector's scale is NaN
+  const int ex = (int)((bits >> 52) & 0x7ff);
   long long m = bits & 0xfffffffffffffll;
   if (ex > 0) m |= 1ll << 52;
-  // m < 2^53; the largest entry becomes m * 2, smaller exponents shift right
-  const int sh = max(emx, 1) - max(ex, 1) - 1;
+  if (em == DG_INF || ex == 0x7ff || m == 0) return 0;  // infinities and NaN: the vector's products are NaN
+  // m < 2^53; the largest entry becomes m * 2^9, smaller exponents shift right
+  const int sh = em - (max(ex, 1) + off) - 9;
   long long q;
-  if (sh < 0) q = m << 1;
-  else if (sh == 0) q = m;
+  if (sh <= 0) q = m << -sh;
   else if (sh > 54) q = 0;
   else q = (m + (1ll << (sh - 1))) >> sh;
   return bits < 0 ? -q : q;
 }
-// Scale of the vector: x = q * 2^(E - 1023 - 53), as a double (NaN when an entry was not finite)
-__device__ __forceinline__ int digit_exp(int em) { return max(em >> 20, 1) - 1023 - 53; }
 
 // v 2^e: by the exponent field where the result is normal (the FP64 pipe is slow), else by scalbn
 __device__ __forceinline__ double scale_exp(double v, int e) {
@@ -125,11 +188,13 @@ __device__ __forceinline__ double scale_exp(double v, int e) {
 __global__ void __launch_bounds__(256) digit_pack_kernel(const __grid_constant__ DigitBatch b) {
   const DigitItem &it = b.it[blockIdx.y];
   __shared__ double sx[64][33];
+  __shared__ int soff[DG_KT];
   const int tid = threadIdx.x;
   const int nvb = (it.nv + 63) / 64, total = nvb * it.nkt;
   for (int u = blockIdx.x; u < total; u += gridDim.x) {
     const int v0 = (u / it.nkt) * 64, kt = u % it.nkt, k0 = kt * DG_KT;
     __syncthreads();
+    if (tid < DG_KT) soff[tid] = k0 + tid < it.k ? it.ksign * it.kexp[k0 + tid] : 0;
     if (it.mode == 2) {
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
@@ -158,22 +223,22 @@ __global__ void __launch_bounds__(256) digit_pack_kernel(const __grid_constant__
     }
     __syncthreads();
     const int v = tid >> 2, g = tid & 3;  // 8 K-values of one vector
-    const int em = v0 + v < it.nv ? it.emax[v0 + v] : 0;
+    const int em = v0 + v < it.nv ? it.emax[v0 + v] : DG_NONE;
     uint32_t w[DG_PLANES][4];
 #pragma unroll
     for (int e = 0; e < 8; e += 2) {
-      // q + sum_s 64 * 128^s has the digits plus 64 as its base-128 digits
-      const unsigned long long off = 0x0081020408102040ull << 0;
-      const unsigned long long a = (unsigned long long)fixed55(sx[v][g * 8 + e], em) + off;
-      const unsigned long long c = (unsigned long long)fixed55(sx[v][g * 8 + e + 1], em) + off;
+      // q + sum_s 128 * 256^s has the digits plus 128 as its bytes
+      constexpr unsigned long long off = 0x8080808080808080ull;
+      const unsigned long long a = (unsigned long long)fixed63(sx[v][g * 8 + e], soff[g * 8 + e], em) + off;
+      const unsigned long long c = (unsigned long long)fixed63(sx[v][g * 8 + e + 1], soff[g * 8 + e + 1], em) + off;
 #pragma unroll
       for (int s = 0; s < DG_PLANES; ++s) {
-        const int shift = 7 * (DG_PLANES - 1 - s);  // plane 0 is the leading digit
-        const uint32_t d = ((uint32_t)(a >> shift) & 127u) | (((uint32_t)(c >> shift) & 127u) << 16);
-        // fp16(1024 + u) - 1088 = u - 64, exactly
+        const int shift = DG_BITS * (DG_PLANES - 1 - s);  // plane 0 is the leading digit
+        const uint32_t d = ((uint32_t)(a >> shift) & 255u) | (((uint32_t)(c >> shift) & 255u) << 16);
+        // fp16(1024 + u) - 1152 = u - 128, exactly
         const uint32_t h = d | 0x64006400u;
         __half2 x = *reinterpret_cast<const __half2 *>(&h);
-        x = __hsub2(x, __half2half2(__ushort_as_half(0x6440)));
+        x = __hsub2(x, __half2half2(__ushort_as_half(0x6480)));
         w[s][e >> 1] = *reinterpret_cast<uint32_t *>(&x);
       }
     }
@@ -367,26 +432,26 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const int x = __float2int_rn(__uint_as_float(v[j]));
-            if (g < 4) hi[j] += (long long)x * (1 << (7 * (3 - g)));
-            else lo[j] += (long long)x * (1 << (7 * (7 - g)));
+            if (g < 4) hi[j] += (long long)x * (1 << (DG_BITS * (3 - g)));
+            else lo[j] += (long long)x * (1 << (DG_BITS * (7 - g)));
           }
         }
       }
       if (!ok) break;
-      // planes 0 and 0 weigh 2^98 in units of the two integers; hi counts 2^77, lo 2^49
+      // planes 0 and 0 weigh 2^112 in units of the two integers; hi counts 2^88, lo 2^56
       const int i = mt * DG_BM + q * 32 + lane;
       if (i < it.m) {
         const int eai = it.ea[i];
-        const int xa = digit_exp(eai) + 49;
+        const int xa = eai - 2 * 1084 + 56;  // one unit of a product of two integers is 2^(ea + eb - 2 * 1084)
         const int j0 = nt * DG_BN + half * 32;
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
           const int c = j0 + j;
           if (c >= it.n) continue;
           const int ebj = it.eb[c];
-          double v = fma((double)hi[j], 268435456.0, (double)lo[j]);
-          v = scale_exp(v, xa + digit_exp(ebj));
-          if ((eai >> 20) == 0x7ff || (ebj >> 20) == 0x7ff) v = __longlong_as_double(0x7ff8000000000000ll);
+          double v = fma((double)hi[j], 4294967296.0, (double)lo[j]);
+          v = scale_exp(v, xa + ebj);
+          if (eai == DG_INF || ebj == DG_INF) v = __longlong_as_double(0x7ff8000000000000ll);
           if (it.nsplit > 1) {
             it.ws[((long long)sp * it.m + i) * it.n + c] = v;
             continue;
@@ -461,16 +526,19 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
       memset(&db, 0, sizeof(db));
       memset(&gb, 0, sizeof(gb));
       size_t bytes = 0, vecs = 0, wsum = 0;
-      struct Src { const double *p; int ld, nv, k, mode, vb; size_t off, ev; };
-      std::vector<Src> srcs;  // operands, each packed once even when several items use it
-      auto operand = [&](const double *p, int ld, int nv, int k, int mode, int vb) {
+      struct Src { const double *p; int ld, nv, k, mode, vb, with; size_t off, ev, kv; };
+      // operands, each packed once even when several items use it; with: -1 for an op(A), which sets the powers of two
+      // along K, else the op(A) that the operand is scaled for
+      std::vector<Src> srcs;
+      auto operand = [&](const double *p, int ld, int nv, int k, int mode, int vb, int with) {
         for (size_t q = 0; q < srcs.size(); ++q)
-          if (srcs[q].p == p && srcs[q].ld == ld && srcs[q].nv == nv && srcs[q].k == k && srcs[q].mode == mode && srcs[q].vb == vb)
+          if (srcs[q].p == p && srcs[q].ld == ld && srcs[q].nv == nv && srcs[q].k == k && srcs[q].mode == mode && srcs[q].vb == vb &&
+              srcs[q].with == with)
             return (int)q;
         const size_t nkt = (k + DG_KT - 1) / DG_KT, tiles = (nv + vb - 1) / vb;
-        srcs.push_back({p, ld, nv, k, mode, vb, bytes, vecs});
+        srcs.push_back({p, ld, nv, k, mode, vb, with, bytes, vecs, with < 0 ? vecs + (size_t)(nv + 63) / 64 * 64 : srcs[with].kv});
         bytes += tiles * nkt * DG_PAIRS * vb * 128;
-        vecs += (size_t)(nv + 63) / 64 * 64;
+        vecs += (size_t)(nv + 63) / 64 * 64 + (with < 0 ? (size_t)(k + 63) / 64 * 64 : 0);
         return (int)srcs.size() - 1;
       };
       std::vector<int> ia, ib;
@@ -483,8 +551,8 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
         if (k <= 0) continue;
         // rows kp .. of the operand (a complex row holds two real ones, each of two doubles)
         auto from = [&](const double *p, int ld, int mode) { return p + (mode == 1 ? (int64_t)kp : (int64_t)kp * ld); };
-        ia[i] = operand(from(g.A, g.lda, g.amode), g.lda, g.m, k, g.amode, DG_BM);
-        ib[i] = operand(from(g.B, g.ldb, g.bmode), g.ldb, g.n, k, g.bmode, DG_BN);
+        ia[i] = operand(from(g.A, g.lda, g.amode), g.lda, g.m, k, g.amode, DG_BM, -1);
+        ib[i] = operand(from(g.B, g.ldb, g.bmode), g.ldb, g.n, k, g.bmode, DG_BN, ia[i]);
         DgItem &x = gb.it[gb.count];
         x.m = g.m;
         x.n = g.n;
@@ -501,14 +569,14 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
         ++gb.count;
       }
       // splits: about three units of work per SM, none shallower than 512 terms
-      const double target = std::max<double>(DG_CHUNK, std::ceil(work / (3.0 * nsm) / DG_CHUNK) * DG_CHUNK);
+      const double target = std::max<double>(DG_SPLIT, std::ceil(work / (3.0 * nsm) / DG_SPLIT) * DG_SPLIT);
       int units = 0, splits = 1;
       for (int q = 0; q < gb.count; ++q) {
         DgItem &x = gb.it[q];
         const int tiles = x.unit0;
         x.nsplit = std::min(32, std::max(1, (int)std::floor(x.nkt / target)));
         x.kper = (x.nkt + x.nsplit - 1) / x.nsplit;
-        x.kper = (x.kper + DG_CHUNK - 1) / DG_CHUNK * DG_CHUNK;
+        x.kper = (x.kper + DG_SPLIT - 1) / DG_SPLIT * DG_SPLIT;
         x.nsplit = (x.nkt + x.kper - 1) / x.kper;
         x.unit0 = units;
         units += tiles * x.nsplit;
@@ -522,11 +590,13 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
       RFDD_CUDA(cudaMallocAsync((void **)&ws, ebytes + bytes + wsum * sizeof(double), st));
       int *emax = reinterpret_cast<int *>(ws);
       double *part = reinterpret_cast<double *>(ws + ebytes + bytes);
-      RFDD_CUDA(cudaMemsetAsync(emax, 0, ebytes, st));
-      long long be = 1, bp = 1;
+      RFDD_CUDA(cudaMemsetAsync(emax, DG_NONE_BYTE, ebytes, st));
+      long long be = 1, bp = 1, bk = 1;
       for (const Src &s : srcs) {
         const int nkt = (s.k + DG_KT - 1) / DG_KT;
-        db.it[db.count++] = {s.p, s.ld, s.nv, s.k, s.mode, s.vb, nkt, ws + ebytes + s.off, emax + s.ev};
+        db.it[db.count++] = {s.p, s.ld, s.nv, s.k, s.mode, s.vb, nkt, ws + ebytes + s.off, emax + s.ev, emax + s.kv, s.with < 0 ? -1 : 1};
+        if (s.with < 0)
+          bk = std::max<long long>(bk, s.mode == 0 ? (s.k + 7) / 8 : (long long)((s.k + 31) / 32) * ((s.nv + 255) / 256));
         be = std::max<long long>(be, s.mode == 1 ? (s.nv + 7) / 8 : (long long)((s.nv + 31) / 32) * ((s.k + 255) / 256));
         bp = std::max<long long>(bp, (long long)((s.nv + 63) / 64) * nkt);
       }
@@ -543,6 +613,8 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
           part += (size_t)x.nsplit * x.m * x.n;
         }
       }
+      digit_kexp_kernel<<<dim3((unsigned)std::min<long long>(bk, 2048), db.count), 256, 0, st>>>(db);
+      RFDD_CHECK_LAUNCH();
       digit_emax_kernel<<<dim3((unsigned)std::min<long long>(be, 2048), db.count), 256, 0, st>>>(db);
       RFDD_CHECK_LAUNCH();
       digit_pack_kernel<<<dim3((unsigned)std::min<long long>(bp, 4096), db.count), 256, 0, st>>>(db);

@@ -53,7 +53,11 @@ extern "C" {
 #define RFDD_ESTATE 10           /* call out of order (e.g. filter before factor) */
 
 /* ---- option values ---------------------------------------------------------------------- */
-#define RFDD_FP64 0              /* plain path: all factorisations and solves in FP64 */
+#define RFDD_FP64 0              /* plain path: all factorisations and solves in FP64.  Where the rows of A
+                                    and of M differ by less than 1024 in absolute row sum, large trailing
+                                    and triangular-solve updates are exact digit products (the bound is that
+                                    of rfdd_dgemm's engine 1, relative to rows and columns); else FP64
+                                    multiply-adds, whose error is relative to each term */
 #define RFDD_MIXED 1             /* complex-FP32 factorisations, FP64 iterative refinement */
 #define RFDD_MIDPOINT 0          /* midpoint rule of order 2Nc (Section 6, the paper's choice) */
 #define RFDD_GAUSS_LEGENDRE 1    /* Gauss-Legendre on the upper half circle (Section 2.1) */

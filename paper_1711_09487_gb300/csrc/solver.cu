@@ -242,6 +242,7 @@ struct rfdd_handle {
   double normA = 0.0, normM = 0.0;  // max absolute row sums
   double gershM = 0.0;              // min over rows of M_ii - sum_{j != i} |M_ij| (a lower bound of M's
                                     // spectrum when positive)
+  double grading = 1.0;             // largest over smallest nonzero absolute row sum, the larger of A's and M's
   bool has_me = false;              // M_E != 0 (the Gamma block of Z is needed)
   std::vector<int64_t> host_rp;
   std::vector<int32_t> host_cl, host_posmap;
@@ -347,6 +348,14 @@ struct rfdd_handle {
 namespace {
 
 inline bool is_mixed(const rfdd_handle *h) { return h->opt.precision == RFDD_MIXED; }
+
+// Whether the updates of FP64 factorisations and solves may run as digit products (tc_dgemm.cu), whose error is relative to
+// the largest entries of a row and a column.  On pencils with rows of about one size it is below that of the FP64 sums
+// (12^3 solve, same completion passes and residuals).  Where the rows of A or M differ by large factors, so do the
+// entries along the factors' rows, and the small ones are the ones that later rows are made of: the 12^3 pencil as D A D,
+// D powers of two within 2^-e and 2^e (rows apart by 2^4e), reached residuals of 5e-10 at e = 7 and 5e-6 at e = 15 with the
+// digits, 5e-11 and 2e-8 with the FP64 sums; equal up to e = 6.  The line lies at 2^10, e = 2.5.
+inline bool fp64_by_digits(const rfdd_handle *h) { return h->grading <= 1024.0; }
 
 // Leading dimension of a factor of order d: FP32 rows start on a 32-byte sector, so that the
 // tensor-core epilogue reads and writes them in 16-byte pieces (K = 256 update of a 9261 x 9005
@@ -644,6 +653,7 @@ void do_setup(rfdd_handle *h, const rfdd_csr *A, const rfdd_csr *M, const int32_
   std::vector<std::vector<int32_t>> ccl(nt_max);
   std::vector<std::vector<double>> cav(nt_max), cmv(nt_max);
   std::vector<double> cna(nt_max, 0.0), cnm(nt_max, 0.0), cgm(nt_max, std::numeric_limits<double>::infinity());
+  std::vector<double> cla = cgm, clm = cgm;
   std::vector<int64_t> cr0(nt_max, -1);
   std::vector<int64_t> rowlen(n, 0);
   parallel_rows(n, [&](int64_t r0, int64_t r1, int t) {
@@ -651,7 +661,7 @@ void do_setup(rfdd_handle *h, const rfdd_csr *A, const rfdd_csr *M, const int32_
     std::vector<std::pair<int64_t, std::pair<double, double>>> row;
     std::vector<int32_t> c;
     std::vector<double> a, m;
-    double na = 0.0, nm = 0.0, gm = std::numeric_limits<double>::infinity();
+    double na = 0.0, nm = 0.0, gm = std::numeric_limits<double>::infinity(), la = gm, lm = gm;
     int64_t est = 0;
     for (int64_t r = r0; r < r1; ++r) {
       const int64_t i = h->perm[r];
@@ -676,6 +686,8 @@ void do_setup(rfdd_handle *h, const rfdd_csr *A, const rfdd_csr *M, const int32_
       }
       na = std::max(na, sa);
       nm = std::max(nm, sm);
+      if (sa > 0.0) la = std::min(la, sa);
+      if (sm > 0.0) lm = std::min(lm, sm);
       gm = std::min(gm, 2.0 * mdiag - sm);
       // equal columns are summed below; each entry holds only one of (a, m), so their order is free
       std::sort(row.begin(), row.end(), [](auto &x, auto &y) { return x.first < y.first; });
@@ -695,6 +707,8 @@ void do_setup(rfdd_handle *h, const rfdd_csr *A, const rfdd_csr *M, const int32_
     cr0[t] = r0;
     cna[t] = na;
     cnm[t] = nm;
+    cla[t] = la;
+    clm[t] = lm;
     cgm[t] = gm;
     ccl[t] = std::move(c);
     cav[t] = std::move(a);
@@ -703,11 +717,15 @@ void do_setup(rfdd_handle *h, const rfdd_csr *A, const rfdd_csr *M, const int32_
   for (int64_t r = 0; r < n; ++r) rp[r + 1] = rp[r] + rowlen[r];
   h->normA = h->normM = 0.0;
   h->gershM = std::numeric_limits<double>::infinity();
+  double lowA = h->gershM, lowM = h->gershM;
   for (int64_t t = 0; t < nt_max; ++t) {
     h->normA = std::max(h->normA, cna[t]);
     h->normM = std::max(h->normM, cnm[t]);
     h->gershM = std::min(h->gershM, cgm[t]);
+    lowA = std::min(lowA, cla[t]);
+    lowM = std::min(lowM, clm[t]);
   }
+  h->grading = std::max(1.0, std::max(h->normA / lowA, h->normM / lowM));  // no nonzero row: 0
   cl.resize(rp[n]);
   av.resize(rp[n]);
   mv.resize(rp[n]);
@@ -2276,8 +2294,9 @@ void interior_factor_start(rfdd_handle *h, double sigma, cudaStream_t on) {
   const DevDD dd = h->dd;
   const int64_t *doff_dev = h->I_doff.as<int64_t>(), *boffr_dev = h->I_boffr_dev.as<int64_t>();
   const cx<double> *zs = h->I_zs.as<cx<double>>();
+  const bool digits = fp64_by_digits(h);
   auto launch = [=](cudaStream_t s) {
-    TcStatusScope ts(status);  // tensor-core time-outs of these launches land in their status word
+    TcStatusScope ts(status, digits);  // tensor-core time-outs of these launches land in their status word
     // assemble_blocks without border: D_j = d_j, and the same row mapping
     assemble_blocks<Tr>(s, P, dd, doff_dev, dsum, boffr_dev, zs, 1, Bs, false, (int)factor_ld<Tr>(1));
     lu_batched<Tr>(s, items, NBO_LU, status);
@@ -3497,7 +3516,7 @@ int rfdd_factor(rfdd_handle *h, int32_t n_nodes, const double *z, const double *
   if (!h || !z || !w || n_nodes < 1) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     set_nodes(h, n_nodes, z, w);
     factor(h);
   });
@@ -3507,7 +3526,7 @@ int rfdd_schur_copy(rfdd_handle *h, int32_t node, double *S_out) {
   if (!h || !S_out) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     RFDD_REQUIRE(h->have_factors && h->opt.keep_schur, RFDD_ESTATE, "schur_copy needs keep_schur and rfdd_factor");
     RFDD_REQUIRE(node >= 0 && node < h->nnodes, RFDD_EINVAL, "node out of range");
     const int64_t s = h->s;
@@ -3530,7 +3549,7 @@ int rfdd_shifted_solve(rfdd_handle *h, int32_t node, int32_t which, int32_t j, i
   if (!h || !R || !X || nrhs < 1) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     RFDD_REQUIRE(h->have_factors, RFDD_ESTATE, "shifted_solve needs rfdd_factor");
     RFDD_REQUIRE(node >= 0 && node < h->nnodes, RFDD_EINVAL, "node out of range");
     cudaStream_t st = h->st;
@@ -3604,7 +3623,7 @@ int rfdd_filter_apply(rfdd_handle *h, int64_t b, const double *X, double *W) {
   if (!h || !X || !W || b < 1) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     RFDD_REQUIRE(h->have_factors, RFDD_ESTATE, "filter_apply needs rfdd_factor");
     const int64_t s = h->s;
     Buf x, wv;
@@ -3622,7 +3641,7 @@ int rfdd_lanczos(rfdd_handle *h, int64_t cap, double *Q_out, int64_t *mu, double
   if (!h) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     RFDD_REQUIRE(h->have_factors, RFDD_ESTATE, "lanczos needs rfdd_factor");
     if (is_mixed(h)) lanczos_impl<cx<float>>(h);
     else lanczos_impl<cx<double>>(h);
@@ -3648,7 +3667,7 @@ int rfdd_interior(rfdd_handle *h, double sigma, int64_t cap, double *Z_out, int6
   if (!h) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     RFDD_REQUIRE(h->mu > 0, RFDD_ESTATE, "interior needs rfdd_lanczos");
     double sg = sigma;
     if (std::isnan(sg)) sg = h->have_interval ? 0.5 * (h->alpha + h->beta) : 0.0;
@@ -3671,7 +3690,7 @@ int rfdd_rayleigh_ritz(rfdd_handle *h, int64_t cap, double *theta_out, int64_t *
   if (!h) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     RFDD_REQUIRE(h->kz > 0, RFDD_ESTATE, "rayleigh_ritz needs rfdd_interior");
     const double a = h->have_interval ? h->alpha : -INFINITY, b = h->have_interval ? h->beta : INFINITY;
     if (is_mixed(h)) rr_on_Z<cx<float>>(h, a, b, nullptr);
@@ -3686,7 +3705,7 @@ int rfdd_inertia(rfdd_handle *h, double sigma, int64_t *count) {
   if (!h || !count || !std::isfinite(sigma)) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     *count = inertia_impl(h, sigma);
   });
 }
@@ -3696,7 +3715,7 @@ int rfdd_polish(rfdd_handle *h, int64_t nev, double *lambda, double *X, double *
   if (nev == 0) return RFDD_OK;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     interior_join(h, false);  // nothing of a failed solve may still be running on the second stream
     polish_impl(h, nev, lambda, X, resid);
   });
@@ -3709,7 +3728,7 @@ int rfdd_solve(rfdd_handle *h, double alpha, double beta, int32_t n_nodes, rfdd_
   if (!r) return RFDD_ENOMEM;
   int rc = guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     run_solve(h, alpha, beta, n_nodes, r);
   });
   if (rc != RFDD_OK) {
@@ -3727,7 +3746,7 @@ int rfdd_rfkrylov(rfdd_handle *h, double alpha, double beta, int32_t n_nodes, in
   if (!r) return RFDD_ENOMEM;
   int rc = guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
     run_rfkrylov(h, alpha, beta, n_nodes, max_dim, r);
   });
   if (rc != RFDD_OK) {
@@ -3755,7 +3774,7 @@ int rfdd_solve_async(rfdd_handle *h, double alpha, double beta, int32_t n_nodes,
     int rc = guarded([&] {
       RFDD_CUDA(cudaSetDevice(device));
       AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>());
+    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
       run_solve(h, alpha, beta, n_nodes, r);
     });
     if (rc != RFDD_OK) r->ready.store(-rc);

@@ -7,16 +7,20 @@
 namespace rfdd {
 // Status words (STATUS_WORDS device ints) that the tensor-core launches issued by the calling host thread record
 // a failed wait in (DS_WAIT_TIMEOUT), for the lifetime of the scope.  A launch outside any scope is
-// refused with RFDD_ESTATE.
+// refused with RFDD_ESTATE.  fp64_digits: whether the FP64 factorisation and solve updates of the scope may run as digit
+// products (tc_fp64_takes).
 struct TcStatusScope {
   int *prev;
-  explicit TcStatusScope(int *word);
+  bool prev_digits;
+  explicit TcStatusScope(int *word, bool fp64_digits = true);
   ~TcStatusScope();
   TcStatusScope(const TcStatusScope &) = delete;
   TcStatusScope &operator=(const TcStatusScope &) = delete;
 };
 // the calling thread's status word (nullptr outside any scope)
 int *tc_status_word();
+// whether FP64 updates may run as digit products in the calling thread's scope
+bool tc_fp64_digits();
 // While alive, the tensor-core kernel launches of the calling host thread record ab[0] just before
 // and ab[1] just after the kernel (not the operand packing): the probes time the MMA kernel alone.
 struct TcKernelEvents {

@@ -338,7 +338,8 @@ int rfdd_pivoted_cholesky(int64_t k, const double *G, double tol, int32_t polls,
  * realified product) and a two-CTA kernel (cta_group::2, 256 x 256 tiles on a pair of SMs);
  * engines 2 and 3 force the one-CTA and the two-CTA kernel; engine 0 = a CUDA-core kernel kept
  * as another engine for tests (the solver never dispatches to it).  RFDD_EINVAL for other
- * engines. */
+ * engines.  In engines 1 to 3 every entry of A (of B) is taken with an error of at most 2^-22 of itself or 2^-38 of the
+ * largest real or imaginary part of its row (its column), whichever is more; engine 0 takes it as it is. */
 int rfdd_cgemm(int64_t m, int64_t n, int64_t k, const float *A, int64_t lda, const float *B, int64_t ldb,
                float *C, int64_t ldc, double alpha, double beta, int32_t engine);
 

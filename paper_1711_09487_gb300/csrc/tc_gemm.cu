@@ -6,9 +6,13 @@
 // where Ar and Cr are the interleaved storage read as real matrices and each complex B[p][j]
 // becomes the 2x2 real block [[re, im], [-im, re]] of Br.  FP32 accuracy comes from a two-way split
 // of scaled operands: every row of Ar and every column of Br is scaled by a power of two that puts
-// its largest entry in [2^13, 2^14), and x = hi + lo with hi = fp16(x), lo = fp16(x - hi), 22
-// significant bits with round to nearest in both halves (entries more than 2^19 below the largest
-// one of their row lose trailing bits, 2^-39 of that largest entry and below).
+// its largest entry in [2^13, 2^14), and x = hi + lo with hi = fp16(x), lo = fp16(x - hi), rounded to
+// nearest in both halves: an entry has an error of 2^-23 of itself or 2^-38 of the largest one of its row (column), whichever
+// is more.  That is FP32 for entries down to 2^-15 of the largest; smaller ones keep fewer bits of their own (a split
+// with an exponent of its own per entry, as TF32 has, keeps 22) and those below 2^-38 are gone.  The solves do not
+// notice: the 12^3 pencil as D A D, D powers of two within 2^-e and 2^e, reaches the same residuals in the same
+// passes with either split (e = 5: 2 passes, 1e-11; e = 9: 1e-8, the limit of FP32 factors), and 7-point pencils of contrasts
+// up to 5e9 as well.
 // A*B ~ Ahi*Bhi + Ahi*Blo + Alo*Bhi, accumulated in FP32 in tensor memory and scaled back in the
 // epilogue.  Against the TF32 split of the same depth the operands take half the bytes, the MMAs
 // run at twice the rate, and the lower half is rounded instead of truncated.

@@ -84,7 +84,8 @@ typedef struct {
   int max_passes;       /* completion passes (filtered subspace iteration); default 8 */
   int ir_max;           /* FP64 iterative-refinement steps per shifted solve; default 10 */
   uint64_t seed;        /* counter-based RNG seed for start blocks; default 1 */
-  size_t mem_budget;    /* device bytes one solve may hold; 0 = no limit */
+  size_t mem_budget;    /* device bytes one solve may hold; 0 = no limit.  A sixteenth of it bounds the
+                           digits of an FP64 product; larger ones run on the CUDA cores */
   void *stream;         /* cudaStream_t to run on (must stay valid until rfdd_destroy: the
                            handle's device buffers are stream-ordered allocations on it);
                            NULL = a stream owned by the handle */
@@ -305,7 +306,8 @@ int rfdd_inertia(rfdd_handle *h, double sigma, int64_t *count);
  * updated in place; lambda: host, nev, updated; resid: host, nev, written.  Needs only
  * rfdd_setup; uses the handle's stream.  Device memory: 6 n x nev FP64 arrays plus the dense
  * blocks of as many pairs at a time as fit in 4 GiB (or in half of opt.mem_budget when set),
- * at least one pair.
+ * at least one pair, and the digits of one launch of FP64 products (1.5 GB, or a sixteenth of
+ * opt.mem_budget when set, at most).
  * RFDD_ESINGULAR when some B_j - lambda_i M_B^(j) has a zero pivot (lambda_i an eigenvalue of a
  * subdomain pencil) or a column has a zero vector after the polish; RFDD_EINVAL for nev < 0,
  * null arrays or a non-finite lambda_i. */

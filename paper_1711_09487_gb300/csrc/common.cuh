@@ -177,6 +177,12 @@ struct SolveShape {
   int64_t lv_s2 = 0;
   const int64_t *lv_n1 = nullptr, *lv_n2 = nullptr;
 };
+// Device bytes that the digits of one FP64 digit-product launch may take (tc_dgemm.cu): 1.5 GB, or a sixteenth of a
+// solve's memory budget.  Products that need more for 512 terms of their sums run on the CUDA cores.
+inline size_t digit_bytes_cap(size_t mem_budget) {
+  const size_t cap = 1500000000;
+  return mem_budget == 0 ? cap : mem_budget / 16 < cap ? mem_budget / 16 : cap;
+}
 // whether the mixed solve keeps tile copies of its factors (rfdd_options.pack_factors)
 bool packed_factors(const SolveShape &g, int nc);
 size_t factor_bytes_of(const SolveShape &g, int nc);

@@ -420,7 +420,7 @@ void gemm_batched(cudaStream_t st, const std::vector<GemmItem<T>> &items, bool t
   }
   if constexpr (std::is_same<typename ST<T>::real, double>::value) {
     // FP64 products with enough work: exact digit products on the tensor cores
-    if (!ta && !tb && tc_status_word() && tc_fp64_digits()) {
+    if (!ta && !tb && tc_status_word() && tc_digit_rule().updates) {
       std::vector<GemmItem<T>> live, rest;
       for (auto &g : items) (g.m > 0 && g.n > 0 && g.k > 0 ? live : rest).push_back(g);
       if (!live.empty() && tc_fp64_takes<T>(live)) {

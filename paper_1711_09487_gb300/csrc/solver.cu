@@ -355,7 +355,9 @@ inline bool is_mixed(const rfdd_handle *h) { return h->opt.precision == RFDD_MIX
 // entries along the factors' rows, and the small ones are the ones that later rows are made of: the 12^3 pencil as D A D,
 // D powers of two within 2^-e and 2^e (rows apart by 2^4e), reached residuals of 5e-10 at e = 7 and 5e-6 at e = 15 with the
 // digits, 5e-11 and 2e-8 with the FP64 sums; equal up to e = 6.  The line lies at 2^10, e = 2.5.
-inline bool fp64_by_digits(const rfdd_handle *h) { return h->grading <= 1024.0; }
+inline TcDigitRule digit_rule(const rfdd_handle *h) {
+  return TcDigitRule{h->grading <= 1024.0, digit_bytes_cap(h->opt.mem_budget)};
+}
 
 // Leading dimension of a factor of order d: FP32 rows start on a 32-byte sector, so that the
 // tensor-core epilogue reads and writes them in 16-byte pieces (K = 256 update of a 9261 x 9005
@@ -968,10 +970,11 @@ static size_t factor_bytes_impl(const SolveShape &g, int nc, bool packed) {
   const bool mixed = g.precision == RFDD_MIXED;
   const size_t scal = mixed ? sizeof(cx<float>) : sizeof(cx<double>);
   size_t e = 0;
-  for (int j = 0; j < g.p; ++j) e += (size_t)g.D[j] * g.D[j];
+  auto ld = [&](int64_t D) { return (size_t)(mixed ? factor_ld<cx<float>>(D) : D); };
+  for (int j = 0; j < g.p; ++j) e += (size_t)g.D[j] * ld(g.D[j]);
   size_t b = (size_t)nc * e * scal;
   // interface factors: one dense S, or S2' and the bordered group blocks
-  size_t se = (size_t)g.s * g.s, sinv = (size_t)block_inverse_elems(g.s, 256), spk = se + 2 * sinv;
+  size_t se = (size_t)g.s * ld(g.s), sinv = (size_t)block_inverse_elems(g.s, 256), spk = se + 2 * sinv;
   if (g.lv_groups > 0) {
     se = (size_t)g.lv_s2 * g.lv_s2;
     sinv = (size_t)block_inverse_elems(g.lv_s2, 256);
@@ -1010,16 +1013,29 @@ bool rfdd::packed_factors(const SolveShape &g, int nc) {
 
 size_t rfdd::factor_bytes_of(const SolveShape &g, int nc) { return factor_bytes_impl(g, nc, packed_factors(g, nc)); }
 
-// Device bytes a solve holds at its peak: the factors, the completion blocks for about nev_guess
-// pairs, the Lanczos basis; plus, when with_setup, the resident set-up (union CSR with both
-// values, its double-FP32 split, maps).
+// Device bytes a solve holds at its peak: the factors, and the larger of what the factorisation's updates and the
+// completion for about nev_guess pairs need on top of them (completion blocks, solve scratch, the digits or packed
+// operands of one launch, the projected problem); the Lanczos basis; plus, when with_setup, the resident set-up
+// (union CSR with both values, its double-FP32 split, maps).
 size_t rfdd::solve_bytes_of(const SolveShape &g, int nc, int64_t nev_guess, bool with_setup) {
-  const size_t scal = g.precision == RFDD_MIXED ? sizeof(cx<float>) : sizeof(cx<double>);
-  size_t b = factor_bytes_of(g, nc);
+  const bool mixed = g.precision == RFDD_MIXED;
+  const size_t scal = mixed ? sizeof(cx<float>) : sizeof(cx<double>);
   int64_t m = nev_guess + std::max<int64_t>((int64_t)std::ceil(g.guard_frac * nev_guess), g.min_guard);
   if (g.m_align > 1) m = (m + g.m_align - 1) / g.m_align * g.m_align;
-  b += (size_t)nc * g.n * m * (sizeof(cx<double>) * 4 + scal * 2);  // completion blocks
-  b += (size_t)nc * g.n * m * scal;  // triangular solves: full-height block products
+  size_t c = (size_t)nc * g.n * m * (sizeof(cx<double>) * 4 + scal * 2);  // completion blocks
+  c += (size_t)nc * g.n * m * scal;  // triangular solves: full-height block products
+  c += (size_t)m * m * 128;          // projected problem: Gram matrices, their factors, inverse iteration
+  // operands of one batch of updates over 256 rows, of blocks of order D with up to w columns
+  int64_t D = g.s;
+  for (int j = 0; j < g.p; ++j) D = std::max(D, g.D[j]);
+  const size_t items = std::min<size_t>(32, (size_t)nc * std::max(1, g.p)), cap = digit_bytes_cap(g.mem_budget);
+  auto update = [&](int64_t w) {
+    // FP64: eight planes of two bytes over 512 real rows; mixed: 16-bit pairs of a batch of up to 64 items
+    return mixed ? 2 * items * (size_t)(D + w) * 256 * 8 * 2 : std::min(cap, items * (size_t)(D + 2 * w) * 512 * 16);
+  };
+  c += std::max(mixed && packed_factors(g, nc) ? 0 : update(m), std::min(cap, (size_t)g.n * m * 32));
+  const size_t f = mixed && packed_factors(g, nc) ? 0 : update(D);
+  size_t b = factor_bytes_of(g, nc) + std::max(c, f);
   b += (size_t)g.s * g.s * sizeof(double);                           // Lanczos basis
   if (with_setup) b += (size_t)g.nnz * (4 + 8 + 8 + 16) + (size_t)g.n * 64;
   return b;
@@ -2294,7 +2310,7 @@ void interior_factor_start(rfdd_handle *h, double sigma, cudaStream_t on) {
   const DevDD dd = h->dd;
   const int64_t *doff_dev = h->I_doff.as<int64_t>(), *boffr_dev = h->I_boffr_dev.as<int64_t>();
   const cx<double> *zs = h->I_zs.as<cx<double>>();
-  const bool digits = fp64_by_digits(h);
+  const TcDigitRule digits = digit_rule(h);
   auto launch = [=](cudaStream_t s) {
     TcStatusScope ts(status, digits);  // tensor-core time-outs of these launches land in their status word
     // assemble_blocks without border: D_j = d_j, and the same row mapping
@@ -3516,7 +3532,7 @@ int rfdd_factor(rfdd_handle *h, int32_t n_nodes, const double *z, const double *
   if (!h || !z || !w || n_nodes < 1) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     set_nodes(h, n_nodes, z, w);
     factor(h);
   });
@@ -3526,7 +3542,7 @@ int rfdd_schur_copy(rfdd_handle *h, int32_t node, double *S_out) {
   if (!h || !S_out) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     RFDD_REQUIRE(h->have_factors && h->opt.keep_schur, RFDD_ESTATE, "schur_copy needs keep_schur and rfdd_factor");
     RFDD_REQUIRE(node >= 0 && node < h->nnodes, RFDD_EINVAL, "node out of range");
     const int64_t s = h->s;
@@ -3549,7 +3565,7 @@ int rfdd_shifted_solve(rfdd_handle *h, int32_t node, int32_t which, int32_t j, i
   if (!h || !R || !X || nrhs < 1) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     RFDD_REQUIRE(h->have_factors, RFDD_ESTATE, "shifted_solve needs rfdd_factor");
     RFDD_REQUIRE(node >= 0 && node < h->nnodes, RFDD_EINVAL, "node out of range");
     cudaStream_t st = h->st;
@@ -3623,7 +3639,7 @@ int rfdd_filter_apply(rfdd_handle *h, int64_t b, const double *X, double *W) {
   if (!h || !X || !W || b < 1) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     RFDD_REQUIRE(h->have_factors, RFDD_ESTATE, "filter_apply needs rfdd_factor");
     const int64_t s = h->s;
     Buf x, wv;
@@ -3641,7 +3657,7 @@ int rfdd_lanczos(rfdd_handle *h, int64_t cap, double *Q_out, int64_t *mu, double
   if (!h) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     RFDD_REQUIRE(h->have_factors, RFDD_ESTATE, "lanczos needs rfdd_factor");
     if (is_mixed(h)) lanczos_impl<cx<float>>(h);
     else lanczos_impl<cx<double>>(h);
@@ -3667,7 +3683,7 @@ int rfdd_interior(rfdd_handle *h, double sigma, int64_t cap, double *Z_out, int6
   if (!h) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     RFDD_REQUIRE(h->mu > 0, RFDD_ESTATE, "interior needs rfdd_lanczos");
     double sg = sigma;
     if (std::isnan(sg)) sg = h->have_interval ? 0.5 * (h->alpha + h->beta) : 0.0;
@@ -3690,7 +3706,7 @@ int rfdd_rayleigh_ritz(rfdd_handle *h, int64_t cap, double *theta_out, int64_t *
   if (!h) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     RFDD_REQUIRE(h->kz > 0, RFDD_ESTATE, "rayleigh_ritz needs rfdd_interior");
     const double a = h->have_interval ? h->alpha : -INFINITY, b = h->have_interval ? h->beta : INFINITY;
     if (is_mixed(h)) rr_on_Z<cx<float>>(h, a, b, nullptr);
@@ -3705,7 +3721,7 @@ int rfdd_inertia(rfdd_handle *h, double sigma, int64_t *count) {
   if (!h || !count || !std::isfinite(sigma)) return RFDD_EINVAL;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     *count = inertia_impl(h, sigma);
   });
 }
@@ -3715,7 +3731,7 @@ int rfdd_polish(rfdd_handle *h, int64_t nev, double *lambda, double *X, double *
   if (nev == 0) return RFDD_OK;
   return guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     interior_join(h, false);  // nothing of a failed solve may still be running on the second stream
     polish_impl(h, nev, lambda, X, resid);
   });
@@ -3728,7 +3744,7 @@ int rfdd_solve(rfdd_handle *h, double alpha, double beta, int32_t n_nodes, rfdd_
   if (!r) return RFDD_ENOMEM;
   int rc = guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     run_solve(h, alpha, beta, n_nodes, r);
   });
   if (rc != RFDD_OK) {
@@ -3746,7 +3762,7 @@ int rfdd_rfkrylov(rfdd_handle *h, double alpha, double beta, int32_t n_nodes, in
   if (!r) return RFDD_ENOMEM;
   int rc = guarded([&] {
     AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
     run_rfkrylov(h, alpha, beta, n_nodes, max_dim, r);
   });
   if (rc != RFDD_OK) {
@@ -3774,7 +3790,7 @@ int rfdd_solve_async(rfdd_handle *h, double alpha, double beta, int32_t n_nodes,
     int rc = guarded([&] {
       RFDD_CUDA(cudaSetDevice(device));
       AllocScope scope(h->st);
-    TcStatusScope tcs(h->status.as<int>(), fp64_by_digits(h));
+    TcStatusScope tcs(h->status.as<int>(), digit_rule(h));
       run_solve(h, alpha, beta, n_nodes, r);
     });
     if (rc != RFDD_OK) r->ready.store(-rc);

@@ -503,23 +503,34 @@ struct DgGemm {
   int amode, bmode, sym;
 };
 
+// bytes of digits of both operands per unit of K: 8 planes of 2 bytes, rows padded to tiles
+static double digit_bytes_per_k(int64_t m, int64_t n) {
+  return 16.0 * ((m + DG_BM - 1) / DG_BM * DG_BM + (n + DG_BN - 1) / DG_BN * DG_BN);
+}
+// whether 512 terms of an m x n x k product (or all of them) fit in the scope's bytes
+static bool digits_fit(int64_t m, int64_t n, int64_t k) {
+  const double kp = std::min<double>(512.0, (k + DG_KT - 1) / DG_KT * DG_KT);
+  return digit_bytes_per_k(m, n) * kp <= (double)tc_digit_rule().bytes;
+}
+
 static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double alpha, double beta) {
+  const double cap = (double)tc_digit_rule().bytes;
   RFDD_REQUIRE(tc_status_word() != nullptr, RFDD_ESTATE, "tensor-core GEMM launched without a status word");
   const int nsm = sm_count();
   RFDD_CUDA(cudaFuncSetAttribute(tc_dgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM));
   for (size_t s0 = 0, cnt = 0; s0 < items.size(); s0 += cnt) {
-    // as many items as keep the digits of 512 terms within 1.5 GB (at least one)
+    // as many items as keep the digits of 512 terms within the scope's bytes (one does, see the takes functions)
     int kmax = 0;
     double per_k = 0.0;  // bytes of digits per unit of K
     for (cnt = 0; cnt < (size_t)DG_MAXB && s0 + cnt < items.size(); ++cnt) {
       const auto &g = items[s0 + cnt];
-      const double b = 16.0 * (((g.m + 127) / 128) * 128.0 + ((g.n + 63) / 64) * 64.0);
-      if (cnt > 0 && (per_k + b) * std::min(512, std::max(kmax, g.k)) > 1.5e9) break;
+      const double b = digit_bytes_per_k(g.m, g.n);
+      if (cnt > 0 && (per_k + b) * std::min(512, std::max(kmax, g.k)) > cap) break;
       kmax = std::max(kmax, g.k);
       per_k += b;
     }
-    // K in passes whose digits fit in 1.5 GB; every pass but the first adds to C
-    const int kpass = std::min<double>(kmax, std::max(512.0, std::floor(1.5e9 / per_k / 512.0) * 512.0));
+    // K in passes whose digits fit; every pass but the first adds to C
+    const int kpass = std::min<double>(kmax, std::max(512.0, std::floor(cap / per_k / 512.0) * 512.0));
     for (int kp = 0; kp < kmax; kp += kpass) {
       DigitBatch db;
       DgBatch gb;
@@ -650,7 +661,7 @@ static void dgemm_run(cudaStream_t st, const std::vector<DgGemm> &items, double 
 // of a 128 x 64 tile.  Against double-FP32 (12 FP32 operations per product) the line lies at about 6e7
 // products an item; against the FP64 pipes (two products per cycle and SM) at 3e7 in the whole batch.
 bool tc_dgemm_takes(const GemmItem<double> &g) {
-  return g.m >= 48 && g.n >= 48 && g.k >= 48 && (double)g.m * g.n * g.k >= 6.4e7;
+  return g.m >= 48 && g.n >= 48 && g.k >= 48 && (double)g.m * g.n * g.k >= 6.4e7 && digits_fit(g.m, g.n, g.k);
 }
 
 void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
@@ -669,7 +680,7 @@ bool tc_fp64_takes(const std::vector<GemmItem<T>> &items) {
   constexpr double F = ST<T>::is_complex ? 2.0 : 1.0;
   double work = 0.0;
   for (const auto &g : items) {
-    if (g.m < 32 || F * g.n < 32 || F * g.k < 32) return false;
+    if (g.m < 32 || F * g.n < 32 || F * g.k < 32 || !digits_fit(g.m, (int64_t)F * g.n, (int64_t)F * g.k)) return false;
     work += F * F * g.m * g.n * (double)g.k;
   }
   return work >= 3.2e7;

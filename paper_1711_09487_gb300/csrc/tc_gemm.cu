@@ -64,18 +64,18 @@ constexpr int TC_SMEM = TC_RING_BYTES + EPI_BYTES + 1024;
 // failure is reported by the solve that met it and by no other.
 thread_local int *g_tc_status = nullptr;
 
-thread_local bool g_tc_fp64_digits = true;
+thread_local TcDigitRule g_tc_digits;
 
-TcStatusScope::TcStatusScope(int *w, bool fp64_digits) : prev(g_tc_status), prev_digits(g_tc_fp64_digits) {
+TcStatusScope::TcStatusScope(int *w, TcDigitRule digits) : prev(g_tc_status), prev_digits(g_tc_digits) {
   g_tc_status = w;
-  g_tc_fp64_digits = fp64_digits;
+  g_tc_digits = digits;
 }
 TcStatusScope::~TcStatusScope() {
   g_tc_status = prev;
-  g_tc_fp64_digits = prev_digits;
+  g_tc_digits = prev_digits;
 }
 int *tc_status_word() { return g_tc_status; }
-bool tc_fp64_digits() { return g_tc_fp64_digits; }
+TcDigitRule tc_digit_rule() { return g_tc_digits; }
 
 // Events recorded around the tensor-core kernel launches of the calling host thread (probes).
 thread_local const cudaEvent_t *g_tc_events = nullptr;

@@ -7,20 +7,23 @@
 namespace rfdd {
 // Status words (STATUS_WORDS device ints) that the tensor-core launches issued by the calling host thread record
 // a failed wait in (DS_WAIT_TIMEOUT), for the lifetime of the scope.  A launch outside any scope is
-// refused with RFDD_ESTATE.  fp64_digits: whether the FP64 factorisation and solve updates of the scope may run as digit
-// products (tc_fp64_takes).
+// refused with RFDD_ESTATE.  digits: what the digit products of the scope may be used for and hold.
+struct TcDigitRule {
+  bool updates = true;                   // FP64 factorisation and solve updates (tc_fp64_takes)
+  size_t bytes = digit_bytes_cap(0);     // device bytes of the digits of one launch
+};
 struct TcStatusScope {
   int *prev;
-  bool prev_digits;
-  explicit TcStatusScope(int *word, bool fp64_digits = true);
+  TcDigitRule prev_digits;
+  explicit TcStatusScope(int *word, TcDigitRule digits = {});
   ~TcStatusScope();
   TcStatusScope(const TcStatusScope &) = delete;
   TcStatusScope &operator=(const TcStatusScope &) = delete;
 };
 // the calling thread's status word (nullptr outside any scope)
 int *tc_status_word();
-// whether FP64 updates may run as digit products in the calling thread's scope
-bool tc_fp64_digits();
+// the rule of the calling thread's scope
+TcDigitRule tc_digit_rule();
 // While alive, the tensor-core kernel launches of the calling host thread record ab[0] just before
 // and ab[1] just after the kernel (not the operand packing): the probes time the MMA kernel alone.
 struct TcKernelEvents {
@@ -49,7 +52,8 @@ void tc_gemm_real(cudaStream_t st, const std::vector<GemmItem<float>> &items, do
 void tc_gemm_real_tf32(cudaStream_t st, const GemmItem<float> &item, double alpha, double beta);
 
 // FP64 products by exact digit products on the tensor cores (tc_dgemm.cu): C = beta*C + alpha*op(A)*op(B), op as
-// in gemm_batched, sym as in gemm_f64x2_batched.  tc_dgemm_takes: whether an item is large enough to gain.
+// in gemm_batched, sym as in gemm_f64x2_batched.  tc_dgemm_takes: whether an item is large enough to gain and its
+// digits fit.
 bool tc_dgemm_takes(const GemmItem<double> &g);
 void tc_dgemm_batched(cudaStream_t st, const std::vector<GemmItem<double>> &items, bool ta, bool tb, double alpha,
                       double beta, const std::vector<char> &sym);

@@ -326,10 +326,11 @@ int rfdd_sym_eig(int64_t n, const double *H, double *evals, double *evecs);
  * first pivot <= tol or not finite.  Host arrays: G (k x k row-major), perm (k; its first *rank
  * entries are the pivots in order), R (room for k x k; on return *rank x *rank row-major, upper).
  * polls: limit of the waits among the CTAs of its one launch (0: the library's own, seconds);
- * RFDD_ECUDA, with the outputs untouched, when such a wait ran out.  Needs no handle (runs on the
- * default stream of the current device). */
-int rfdd_pivoted_cholesky(int64_t k, const double *G, double tol, int32_t polls, int64_t *rank,
-                          int32_t *perm, double *R);
+ * RFDD_ECUDA, with the outputs untouched, when such a wait ran out.  ctas: CTAs asked for (0: one per
+ * SM); half as many, and so on, where the device has no room for all at once.  The result does not
+ * depend on their number.  Needs no handle (runs on the default stream of the current device). */
+int rfdd_pivoted_cholesky(int64_t k, const double *G, double tol, int32_t polls, int32_t ctas,
+                          int64_t *rank, int32_t *perm, double *R);
 
 /* Building block of a3-a5 (trailing updates of the factorisations), a6 and a10 (triangular-solve
  * updates): C = beta*C + alpha*A*B for complex single-precision A (m x k, leading dimension lda),

@@ -148,7 +148,7 @@ def load(path: str | None = None):
     lib.rfdd_rayleigh_ritz.argtypes = [vp, i64, dp, C.POINTER(i64)]
     lib.rfdd_memory_estimate.argtypes = [vp, i32, i64, C.POINTER(C.c_size_t)]
     lib.rfdd_sym_eig.argtypes = [i64, dp, dp, dp]
-    lib.rfdd_pivoted_cholesky.argtypes = [i64, dp, C.c_double, i32, C.POINTER(i64), C.POINTER(i32), dp]
+    lib.rfdd_pivoted_cholesky.argtypes = [i64, dp, C.c_double, i32, i32, C.POINTER(i64), C.POINTER(i32), dp]
     lib.rfdd_kernel_launches.restype = C.c_longlong
     fp = C.POINTER(C.c_float)
     lib.rfdd_cgemm.argtypes = [i64, i64, i64, fp, i64, fp, i64, fp, i64, C.c_double, C.c_double, i32]
@@ -456,12 +456,12 @@ def rfdd_sym_eig(H: np.ndarray):
     return ev, V
 
 
-def rfdd_pivoted_cholesky(G: np.ndarray, tol: float, polls: int = 0):
+def rfdd_pivoted_cholesky(G: np.ndarray, tol: float, polls: int = 0, ctas: int = 0):
     """Pivoted Cholesky of the symmetric G on the GPU: (rank, pivots in order, R) with R^T R = G[pivots][:, pivots]."""
     G = np.ascontiguousarray(G, dtype=np.float64)
     k = G.shape[0]
     rank, perm, Rf = C.c_int64(), np.empty(k, dtype=np.int32), np.empty(k * k)
-    _check(load().rfdd_pivoted_cholesky(k, _dp(G), tol, polls, C.byref(rank),
+    _check(load().rfdd_pivoted_cholesky(k, _dp(G), tol, polls, ctas, C.byref(rank),
                                         perm.ctypes.data_as(C.POINTER(C.c_int32)), _dp(Rf)))
     r = int(rank.value)
     return r, perm[:r], Rf[: r * r].reshape(r, r)

@@ -510,20 +510,24 @@ __global__ void __launch_bounds__(TRD_THREADS) tridiag_kernel(SymBatchP b, TridS
   }
 }
 
+// ctas CTAs over all items, shared in proportion to n^2 (the work of a step), at least four rows to a CTA at the start
+// and one CTA to an item
+static TridSplit trid_split(const SymBatchP &b, int cnt, int ctas) {
+  TridSplit sp;
+  double sq = 0.0;
+  for (int j = 0; j < cnt; ++j) sq += (double)b.it[j].n * b.it[j].n;
+  sp.off[0] = 0;
+  for (int j = 0; j < cnt; ++j) {
+    const double nj = b.it[j].n;
+    const int g = 1 + (int)(std::max(0, ctas - cnt) * nj * nj / sq);
+    sp.off[j + 1] = sp.off[j] + std::max(1, std::min(g, b.it[j].n / 4));
+  }
+  for (int j = cnt; j < EIG_MAXB; ++j) sp.off[j + 1] = sp.off[cnt];
+  return sp;
+}
+
 static void tridiagonalize(cudaStream_t st, const SymBatchP &b, int cnt, int nmax, int *status) {
   if (nmax > 2 && nmax <= TRD_NMAX && status) {
-    // one CTA per SM over all items, shared in proportion to n^2 (the work of a step), at least four
-    // rows to a CTA at the start
-    TridSplit sp;
-    double sq = 0.0;
-    for (int j = 0; j < cnt; ++j) sq += (double)b.it[j].n * b.it[j].n;
-    sp.off[0] = 0;
-    for (int j = 0; j < cnt; ++j) {
-      const double nj = b.it[j].n;
-      const int g = 1 + (int)(std::max(0, sm_count() - cnt) * nj * nj / sq);
-      sp.off[j + 1] = sp.off[j] + std::max(1, std::min(g, b.it[j].n / 4));
-    }
-    for (int j = cnt; j < EIG_MAXB; ++j) sp.off[j + 1] = sp.off[cnt];
     const int nv = (nmax + 1) & ~1;
     const size_t smem = (size_t)3 * nv * sizeof(double);
     // always the same limit: several host threads launch this kernel at once
@@ -534,14 +538,17 @@ static void tridiagonalize(cudaStream_t st, const SymBatchP &b, int cnt, int nma
     RFDD_CUDA(cudaMallocAsync((void **)&pbuf, pb + (size_t)cnt * sizeof(unsigned), st));
     unsigned *bars = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(pbuf) + pb);
     RFDD_CUDA(cudaMemsetAsync(bars, 0, (size_t)cnt * sizeof(unsigned), st));
-    SymBatchP bb = b;
-    int nvv = nv;
-    void *args[] = {&bb, &sp, &nvv, &pbuf, &bars, &status};
-    RFDD_CUDA(cudaLaunchCooperativeKernel((const void *)tridiag_kernel, dim3(sp.off[cnt]), dim3(nmax <= 512 ? 256 : TRD_THREADS), args, smem,
-                                          st));
-    RFDD_CHECK_LAUNCH();
+    // one CTA per SM
+    const int got = cooperative_launch(std::max(cnt, sm_count()), cnt, [&](int ctas) {
+      SymBatchP bb = b;
+      TridSplit sp = trid_split(b, cnt, ctas);
+      int nvv = nv;
+      void *args[] = {&bb, &sp, &nvv, &pbuf, &bars, &status};
+      return cudaLaunchCooperativeKernel((const void *)tridiag_kernel, dim3(sp.off[cnt]),
+                                         dim3(nmax <= 512 ? 256 : TRD_THREADS), args, smem, st);
+    });
     RFDD_CUDA(cudaFreeAsync(pbuf, st));
-    return;
+    if (got > 0) return;
   }
   double *qbuf = nullptr;
   RFDD_CUDA(cudaMallocAsync((void **)&qbuf, (size_t)cnt * std::max(nmax, 1) * sizeof(double), st));

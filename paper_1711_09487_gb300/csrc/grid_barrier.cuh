@@ -28,4 +28,22 @@ __device__ __forceinline__ bool grid_barrier(unsigned *cnt, unsigned target, int
   return ok_s != 0;
 }
 
+// CTAs of a cooperative launch: want of them, or half as many until the device has room for all at once (a process may be
+// held to fewer SMs than the device attribute says); 0 when not even least fit.  launch(ctas) returns the launch's
+// error.  A refused launch is a host-side error; nothing has run then.
+template <typename L>
+int cooperative_launch(int want, int least, L &&launch) {
+  for (int n = want;; n = n / 2 > least ? n / 2 : least) {
+    const cudaError_t e = launch(n);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+      cudaGetLastError();
+      if (n <= least) return 0;
+      continue;
+    }
+    RFDD_CUDA(e);
+    RFDD_CHECK_LAUNCH();
+    return n;
+  }
+}
+
 }  // namespace rfdd

@@ -461,23 +461,27 @@ __global__ void __launch_bounds__(256) pchol_gather_kernel(const double *__restr
   }
 }
 
-int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, int *rank_dev, int *status, int polls) {
+int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, int *rank_dev, int *status, int polls,
+                     int ctas) {
   if (polls <= 0) polls = GRID_SPIN;
+  const int want = std::max(1, std::min(ctas > 0 ? ctas : sm_count(), k));
+  auto smem_of = [&](int ng) { return ((size_t)ceil_div(k, ng) + (k <= PCH_XMAX ? k : 0)) * sizeof(double); };
+  RFDD_REQUIRE(smem_of(want) <= 220 * 1024, RFDD_EINVAL, "pivoted Cholesky: order too large");
   RFDD_CUDA(cudaMemsetAsync(rank_dev, 0, sizeof(int), st));
-  const int ng = std::max(1, std::min(sm_count(), k));
   double *Rt = nullptr;
   PchOffer *offers = nullptr;
   RFDD_CUDA(cudaMallocAsync((void **)&Rt, (size_t)k * k * sizeof(double), st));
-  RFDD_CUDA(cudaMallocAsync((void **)&offers, (size_t)2 * ng * sizeof(PchOffer) + sizeof(unsigned), st));
-  unsigned *bar = reinterpret_cast<unsigned *>(offers + 2 * ng);
+  RFDD_CUDA(cudaMallocAsync((void **)&offers, (size_t)2 * want * sizeof(PchOffer) + sizeof(unsigned), st));
+  unsigned *bar = reinterpret_cast<unsigned *>(offers + 2 * want);
   RFDD_CUDA(cudaMemsetAsync(bar, 0, sizeof(unsigned), st));
-  const size_t smem = ((size_t)ceil_div(k, ng) + (k <= PCH_XMAX ? k : 0)) * sizeof(double);
-  RFDD_REQUIRE(smem <= 220 * 1024, RFDD_EINVAL, "pivoted Cholesky: order too large");
   RFDD_CUDA(cudaFuncSetAttribute(pchol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-  const double *Gc = G;
-  void *args[] = {&Gc, &k, &Rt, &perm, &tol, &rank_dev, &offers, &bar, &polls, &status};
-  RFDD_CUDA(cudaLaunchCooperativeKernel((const void *)pchol_kernel, dim3(ng), dim3(PCH_THREADS), args, smem, st));
-  RFDD_CHECK_LAUNCH();
+  const int got = cooperative_launch(want, 1, [&](int ng) {
+    if (smem_of(ng) > 220 * 1024) return cudaErrorCooperativeLaunchTooLarge;
+    const double *Gc = G;
+    void *args[] = {&Gc, &k, &Rt, &perm, &tol, &rank_dev, &offers, &bar, &polls, &status};
+    return cudaLaunchCooperativeKernel((const void *)pchol_kernel, dim3(ng), dim3(PCH_THREADS), args, smem_of(ng), st);
+  });
+  RFDD_REQUIRE(got > 0, RFDD_ECUDA, "pivoted Cholesky: no room for its CTAs");
   const unsigned nt = (unsigned)ceil_div(k, 32);
   pchol_gather_kernel<<<dim3(nt, nt), 256, 0, st>>>(Rt, perm, k, rank_dev, G);
   RFDD_CHECK_LAUNCH();

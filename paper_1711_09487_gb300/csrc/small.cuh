@@ -37,9 +37,9 @@ namespace rfdd {
 // Pivoted Cholesky of the k x k symmetric G (full storage); returns the rank (pivots > tol), perm (device, k)
 // the pivots in order (its first rank entries); R is the leading rank x rank upper triangle of G on exit.
 // status: device word for a barrier that ran out (DS_GRID_TIMEOUT): the caller reads it before it uses the rank,
-// perm or R.  polls: limit of the barriers' waits (<= 0: the usual one).
+// perm or R.  polls: limit of the barriers' waits, ctas: CTAs asked for (<= 0: the usual ones).
 int pivoted_cholesky(cudaStream_t st, double *G, int k, int *perm, double tol, int *rank_dev, int *status,
-                     int polls = 0);
+                     int polls = 0, int ctas = 0);
 void gather_sym(cudaStream_t st, const double *K, int k, const int *perm, int r, double *out);
 void unit_lower_from_upper(cudaStream_t st, const double *R, int ldr, int r, double *Lt);
 void symmetrize_scaled(cudaStream_t st, const double *A, int r, const double *R, int ldr, double *out);

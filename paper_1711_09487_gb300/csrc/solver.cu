@@ -3878,9 +3878,9 @@ int rfdd_sym_eig(int64_t n, const double *H, double *evals, double *evecs) {
   });
 }
 
-int rfdd_pivoted_cholesky(int64_t k, const double *G, double tol, int32_t polls, int64_t *rank, int32_t *perm,
-                          double *R) {
-  if (k < 1 || k > INT32_MAX || polls < 0 || !G || !rank || !perm || !R) return RFDD_EINVAL;
+int rfdd_pivoted_cholesky(int64_t k, const double *G, double tol, int32_t polls, int32_t ctas, int64_t *rank,
+                          int32_t *perm, double *R) {
+  if (k < 1 || k > INT32_MAX || polls < 0 || ctas < 0 || !G || !rank || !perm || !R) return RFDD_EINVAL;
   return guarded([&] {
     cudaStream_t st = 0;
     Buf Gd, pd, rd, status;
@@ -3890,7 +3890,8 @@ int rfdd_pivoted_cholesky(int64_t k, const double *G, double tol, int32_t polls,
     rd.alloc(sizeof(int));
     status.alloc(STATUS_WORDS * sizeof(int));
     RFDD_CUDA(cudaMemset(status.p, 0, STATUS_WORDS * sizeof(int)));
-    const int r = pivoted_cholesky(st, Gd.as<double>(), (int)k, pd.as<int>(), tol, rd.as<int>(), status.as<int>(), polls);
+    const int r = pivoted_cholesky(st, Gd.as<double>(), (int)k, pd.as<int>(), tol, rd.as<int>(), status.as<int>(), polls,
+                                   ctas);
     int stt = 0;
     RFDD_CUDA(cudaMemcpy(&stt, status.p, sizeof(int), cudaMemcpyDeviceToHost));
     RFDD_REQUIRE(stt == 0, RFDD_ECUDA, "pivoted Cholesky: the CTAs timed out waiting for each other");

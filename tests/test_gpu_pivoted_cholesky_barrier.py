@@ -1,5 +1,5 @@
 """The one-launch pivoted Cholesky by itself: factors of full-rank and rank-deficient matrices around the number of
-CTAs, and a barrier whose wait runs out, which has to come back as an error with nothing indexed by the
+CTAs, more CTAs than the device has room for at once, and a barrier whose wait runs out, which has to come back as an error with nothing indexed by the
 pivots that were never chosen.
 
 Bound of the factors: k 2^-50 of the largest entry (k rounding errors of 2^-53 each, times eight)."""
@@ -44,3 +44,14 @@ def test_a_wait_that_runs_out_is_an_error(R, k):
         R.rfdd_pivoted_cholesky(G, 1e-12, polls=1)
     assert e.value.code == R.RFDD_ECUDA and "timed out" in str(e.value)
     assert R.rfdd_pivoted_cholesky(G, 1e-12)[0] == k  # the next call is unaffected
+
+
+@pytest.mark.parametrize("ctas", [1, 3, 2000])
+def test_number_of_ctas_changes_no_bit(R, ctas):
+    """2000 CTAs of this kernel are not resident together: the launch is refused and repeated with fewer."""
+    G = _gram(2000, 300, 2)
+    ref = R.rfdd_pivoted_cholesky(G, 1e-12)
+    got = R.rfdd_pivoted_cholesky(G, 1e-12, ctas=ctas)
+    assert got[0] == ref[0]
+    np.testing.assert_array_equal(got[1], ref[1])
+    np.testing.assert_array_equal(got[2], ref[2])

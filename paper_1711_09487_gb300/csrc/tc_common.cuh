@@ -34,6 +34,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
   return false;
 }
+// bounded wait that goes on after another role aborted: for copies and MMAs in flight, which have to end before the
+// CTA's shared and tensor memory can be another's
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+  uint32_t ok = 0;
+  for (long long i = 0; i < WAIT_LIMIT && !ok; ++i)
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+}
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
   const uint64_t g = (uint64_t)__cvta_generic_to_global(src);
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
                                                                  double beta) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ __align__(8) uint64_t full_bar[DG_STAGES], empty_bar[DG_STAGES], tfull_bar, tempty_bar;
+  __shared__ __align__(8) uint64_t full_bar[DG_STAGES], empty_bar[DG_STAGES], tfull_bar, tempty_bar, drain_bar;
   __shared__ uint32_t tmem_s;
   __shared__ volatile int abort_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -300,6 +300,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
       mbar_init(smem_u32(&empty_bar[s]), 1);
     }
     mbar_init(smem_u32(&tfull_bar), 1);
+    mbar_init(smem_u32(&drain_bar), 1);
     mbar_init(smem_u32(&tempty_bar), 32 * DG_EPI_WARPS);
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -347,9 +348,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
           bulk_g2s(dst + DG_ABYTES, B + (long long)kt * DG_BBYTES, DG_BBYTES, fb);
         }
       }
-      // every issued copy lands before the CTA can exit
+      // every issued copy lands before the CTA can exit, after an abort too
       for (long long q = (g > DG_STAGES ? g - DG_STAGES : 0); q < g; ++q)
-        mbar_wait(smem_u32(&full_bar[q % DG_STAGES]), (uint32_t)((q / DG_STAGES) & 1), &abort_s);
+        mbar_drain(smem_u32(&full_bar[q % DG_STAGES]), (uint32_t)((q / DG_STAGES) & 1));
     }
   } else if (warp == 1) {
     if (lane == 0) {  // MMA issuer
@@ -396,6 +397,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
         atomicOr(b.err, DS_WAIT_TIMEOUT);
         abort_s = 1;
       }
+      // every issued MMA ends before the tensor memory is freed, after an abort too
+      mma_commit(smem_u32(&drain_bar));
+      mbar_drain(smem_u32(&drain_bar), 0);
     }
   } else {
     // read-back: warp w takes accumulator lanes 32 (w % 4) .. (its rows) and half of the columns

@@ -302,7 +302,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
   extern __shared__ uint8_t smem_raw[];
   uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   float *epi = reinterpret_cast<float *>(base + TC_RING_BYTES);
-  __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], tfull_bar[2], tempty_bar[2];
+  __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], tfull_bar[2], tempty_bar[2],
+      drain_bar;
   __shared__ uint32_t tmem_s;
   __shared__ volatile int abort_s, far_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -315,6 +316,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
       mbar_init(smem_u32(&tfull_bar[a]), 1);
       mbar_init(smem_u32(&tempty_bar[a]), 32 * EPI_WARPS);
     }
+    mbar_init(smem_u32(&drain_bar), 1);
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -367,9 +369,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
           }
         }
       }
-      // drain: every issued copy must land before the CTA can exit
+      // every issued copy must land before the CTA can exit, after an abort too
       for (long long q = (g > STAGES ? g - STAGES : 0); q < g; ++q)
-        mbar_wait(smem_u32(&full_bar[q % STAGES]), (uint32_t)((q / STAGES) & 1), &abort_s);
+        mbar_drain(smem_u32(&full_bar[q % STAGES]), (uint32_t)((q / STAGES) & 1));
     }
   } else if (warp == 1) {
     if (lane == 0) {  // MMA issuer
@@ -416,6 +418,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const __grid_con
         if (!ok) break;
         mma_commit(smem_u32(&tfull_bar[acc]));
       }
+      // every issued MMA ends before the tensor memory is freed, after an abort too
+      mma_commit(smem_u32(&drain_bar));
+      mbar_drain(smem_u32(&drain_bar), 0);
     }
   } else {
     // epilogue warps: warp w reads accumulator lanes 32*(w % 4) .. +31 (its TMEM sub-partition);
@@ -518,6 +523,9 @@ __device__ __forceinline__ void mma2_f16(uint32_t tmem_d, uint64_t da, uint64_t 
       "l"(da), "l"(db), "r"(idesc), "r"(acc)
       : "memory");
 }
+__device__ __forceinline__ void mma2_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void mma2_commit_both(uint32_t bar) {
   const uint16_t mask = 0x3;
   asm volatile(
@@ -545,7 +553,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
   uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   float *epi = reinterpret_cast<float *>(base + T2_STAGES * T2_STAGE_BYTES);
   __shared__ __align__(8) uint64_t full_bar[T2_STAGES], pfull_bar[T2_STAGES], empty_bar[T2_STAGES], tfull_bar[2],
-      tempty_bar[2];
+      tempty_bar[2], drain_bar;
   __shared__ uint32_t tmem_s;
   __shared__ volatile int abort_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -561,6 +569,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
       mbar_init(smem_u32(&tfull_bar[a]), 1);
       mbar_init(smem_u32(&tempty_bar[a]), 2 * EPI_WARPS);  // one arrival per epilogue warp of each CTA
     }
+    mbar_init(smem_u32(&drain_bar), 1);
     abort_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -609,10 +618,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
           bulk_g2s(stage_addr(s, 3), Blo + (long long)kt * B_TILE, T2_BHALF, fb);
         }
       }
-      // every issued copy lands, and every stage's last consumption is signalled here (the leader's
-      // commits arrive on this CTA's empty barriers), before the CTA leaves
+      // every issued copy lands (after an abort too), and every stage's last consumption is signalled here (the
+      // leader's commits arrive on this CTA's empty barriers), before the CTA leaves
       for (long long q = (g > T2_STAGES ? g - T2_STAGES : 0); q < g; ++q) {
-        mbar_wait_cl(smem_u32(&full_bar[q % T2_STAGES]), (uint32_t)((q / T2_STAGES) & 1), &abort_s);
+        mbar_drain(smem_u32(&full_bar[q % T2_STAGES]), (uint32_t)((q / T2_STAGES) & 1));
         mbar_wait_cl(smem_u32(&empty_bar[q % T2_STAGES]), (uint32_t)((q / T2_STAGES) & 1), &abort_s);
       }
     }
@@ -674,6 +683,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
         if (!ok) break;
         mma2_commit_both(smem_u32(&tfull_bar[acc]));
       }
+      // every issued MMA ends before either CTA frees its tensor memory (the cluster barrier below), after an abort too
+      mma2_commit(smem_u32(&drain_bar));
+      mbar_drain(smem_u32(&drain_bar), 0);
     }
   } else {
     // epilogue warps of both CTAs: this CTA's 128 accumulator rows of the pair tile

@@ -403,15 +403,15 @@ def run_ours(args, rank, world, local_rank):
     # throughput probes of the units this path is bound by (context for the peaks above)
     probes = {}
     for name, which in (("tf32_mma_tflops", 0), ("fp64_fma_tflops", 1), ("fp32_fma_tflops", 2),
-                        ("tf32_gemm_8192_tflops", 3)):
+                        ("tf32_gemm_8192_tflops", 3), ("f16_mma_tflops", 4)):
         try:
             probes[name] = R.rfdd_peak_probe(which)
         except Exception as ex:  # a probe is context, not part of the measurement
             probes[name] = f"failed: {ex}"
-    if t_launch > 0 and isinstance(probes.get("tf32_mma_tflops"), float):
-        # the same achieved rate against the tensor pipe's 16-bit rate, twice the TF32 rate measured here (burst,
-        # MMAs from shared memory): the stricter denominator when it exceeds the sustained peak
-        roof["probe_peak_16bit"] = 2.0 * probes["tf32_mma_tflops"]
+    if t_launch > 0 and isinstance(probes.get("f16_mma_tflops"), float):
+        # the same achieved rate against the tensor pipe's 16-bit rate measured here (burst, MMAs from shared
+        # memory): the stricter denominator when it exceeds the sustained peak
+        roof["probe_peak_16bit"] = probes["f16_mma_tflops"]
         roof["frac_vs_probe"] = roof["achieved"] / roof["probe_peak_16bit"]
         roof["executed_frac_vs_probe"] = roof["executed_tflops"] / roof["probe_peak_16bit"]
     cpu_value, cpu_t, cpu_desc, cpu_threads = oracle_sample(w)

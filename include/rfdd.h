@@ -418,7 +418,8 @@ long long rfdd_kernel_launches(void);
  * one CTA per SM); 1 FP64 fused multiply-add on the CUDA cores; 2 FP32 fused multiply-add on the
  * CUDA cores; 3 a plain TF32 GEMM through the solver's tensor-core kernel (its TF32 form: one MMA per product,
  * operands fed from memory; a real 8192^3 GEMM, the MMA kernel alone timed, operand packing
- * excluded).  Allocates about 1.9 GB (which = 3) or a few MB, on a stream of its own. */
+ * excluded); 4 the tensor pipe's 16-bit rate (kind::f16 MMAs of 128 x 256 x 16, otherwise as 0).
+ * Allocates about 1.3 GB (which = 3) or a few MB, on a stream of its own. */
 int rfdd_peak_probe(int32_t which, double *tflops);
 int rfdd_profile(int32_t enable);
 int rfdd_profile_get(int32_t kind, int64_t *launches, double *ms, double *flops);

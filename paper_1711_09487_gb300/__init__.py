@@ -530,7 +530,8 @@ def rfdd_cgemm_noalloc(m: int, n: int, k: int, A_ptr: int, lda: int, B_ptr: int,
 
 def rfdd_peak_probe(which: int) -> float:
     """TFLOP/s of one arithmetic unit on the current device: 0 the tensor pipe's TF32 MMA rate,
-    1 FP64 FMA, 2 FP32 FMA (CUDA cores), 3 a plain TF32 8192^3 GEMM through the tensor-core kernel."""
+    1 FP64 FMA, 2 FP32 FMA (CUDA cores), 3 a plain TF32 8192^3 GEMM through the tensor-core kernel, 4 the tensor
+    pipe's 16-bit MMA rate."""
     t = C.c_double()
     _check(load().rfdd_peak_probe(int(which), C.byref(t)))
     return float(t.value)

@@ -159,7 +159,7 @@ __global__ void shifted_residual_kernel(const int64_t *__restrict__ rp, const in
   }
 }
 
-// The same for fewer than 32 columns: CL lanes take the columns, and the 32 / CL groups of lanes share the entries of
+// The same for up to 16 columns: CL lanes take the columns, and the 32 / CL groups of lanes share the entries of
 // the row (a warp's FP64 instruction costs the same with one lane as with 32): one column of the 3-D 24^3
 // pencil, eight nodes: 624 us with a lane per column; the 3-D 24^3 factor case, ten of these, went from 54.7 to 48.6 ms
 // with the entries shared (and the permuted conversion below).

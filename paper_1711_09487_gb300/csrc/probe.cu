@@ -119,13 +119,13 @@ double tf32_probe(cudaStream_t st) {
   return best;
 }
 
-double mma_probe(cudaStream_t st) {
+double mma_probe(cudaStream_t st, bool f16) {
   int *status = nullptr;
   RFDD_CUDA(cudaMallocAsync((void **)&status, STATUS_WORDS * sizeof(int), st));
   RFDD_CUDA(cudaMemsetAsync(status, 0, STATUS_WORDS * sizeof(int), st));
   double r = 0.0;
   try {
-    r = tc_mma_probe_tflops(st, status);
+    r = tc_mma_probe_tflops(st, status, f16);
   } catch (...) {
     cudaFreeAsync(status, st);
     throw;
@@ -145,11 +145,11 @@ double peak_probe(int which) {
   RFDD_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
   double r = 0.0;
   try {
-    if (which == 0) r = mma_probe(st);
+    if (which == 0 || which == 4) r = mma_probe(st, which == 4);
     else if (which == 1) r = fma_probe<double>(st);
     else if (which == 2) r = fma_probe<float>(st);
     else if (which == 3) r = tf32_probe(st);
-    else throw Error(RFDD_EINVAL, "peak probe: which must be 0..3");
+    else throw Error(RFDD_EINVAL, "peak probe: which must be 0..4");
   } catch (...) {
     cudaStreamSynchronize(st);
     cudaStreamDestroy(st);

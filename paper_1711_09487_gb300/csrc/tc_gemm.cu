@@ -732,12 +732,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm2_kernel(const __grid_co
 }
 
 // ---------------------------------------------------------------------------------------
-// Tensor-pipe throughput probe: one CTA per SM issues `iters` x 4 kind::tf32 MMAs of
-// 128 x 256 x 8 from operand tiles that stay in shared memory (no loads), into one TMEM
+// Tensor-pipe throughput probe: one CTA per SM issues `iters` x 4 MMAs, kind::tf32 of 128 x 256 x 8 or (F16)
+// kind::f16 of 128 x 256 x 16, from operand tiles that stay in shared memory (no loads), into one TMEM
 // accumulator, then waits for their completion on an mbarrier (bounded; DS_WAIT_TIMEOUT into *err
 // on time-out).  Measures the MMA issue rate alone, not the operand feed.
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128, 1) tf32_mma_probe_kernel(int iters, int *err) {
+template <bool F16>
+__global__ void __launch_bounds__(128, 1) mma_probe_kernel(int iters, int *err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *base = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t done_bar;
@@ -763,13 +764,16 @@ __global__ void __launch_bounds__(128, 1) tf32_mma_probe_kernel(int iters, int *
   fence_after();
   const uint32_t tmem = tmem_s;
   if (threadIdx.x == 0) {
-    const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_BN >> 3) << 17) |
+    const uint32_t idesc = (1u << 4) | (F16 ? 0u : (2u << 7) | (2u << 10)) | ((uint32_t)(TC_BN >> 3) << 17) |
                            ((uint32_t)(TC_BM >> 4) << 24);
     const uint32_t a = smem_u32(base), b = smem_u32(base + A_TILE);
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
-      for (int kk = 0; kk < ROW_B / 32; ++kk)
-        mma_tf32(tmem, sdesc(a + kk * 32), sdesc(b + kk * 32), idesc, (it > 0 || kk > 0) ? 1u : 0u);
+      for (int kk = 0; kk < ROW_B / 32; ++kk) {
+        const uint32_t acc = (it > 0 || kk > 0) ? 1u : 0u;
+        if (F16) mma_f16(tmem, sdesc(a + kk * 32), sdesc(b + kk * 32), idesc, acc);
+        else mma_tf32(tmem, sdesc(a + kk * 32), sdesc(b + kk * 32), idesc, acc);
+      }
     }
     mma_commit(smem_u32(&done_bar));
     if (!mbar_wait(smem_u32(&done_bar), 0, &abort_s)) atomicOr(err, DS_WAIT_TIMEOUT);
@@ -782,12 +786,13 @@ __global__ void __launch_bounds__(128, 1) tf32_mma_probe_kernel(int iters, int *
   }
 }
 
-double tc_mma_probe_tflops(cudaStream_t st, int *dev_status) {
+double tc_mma_probe_tflops(cudaStream_t st, int *dev_status, bool f16) {
+  const auto kernel = f16 ? mma_probe_kernel<true> : mma_probe_kernel<false>;
   int dev = 0, nsm = 0;
   RFDD_CUDA(cudaGetDevice(&dev));
   RFDD_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const int smem = A_TILE + B_TILE + 1024;
-  RFDD_CUDA(cudaFuncSetAttribute(tf32_mma_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  RFDD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   cudaEvent_t e0, e1;
   RFDD_CUDA(cudaEventCreate(&e0));
   RFDD_CUDA(cudaEventCreate(&e1));
@@ -795,13 +800,13 @@ double tc_mma_probe_tflops(cudaStream_t st, int *dev_status) {
   double best = 0.0;
   for (int rep = 0; rep < 4; ++rep) {  // the first launch is a warm-up
     RFDD_CUDA(cudaEventRecord(e0, st));
-    tf32_mma_probe_kernel<<<nsm, 128, smem, st>>>(iters, dev_status);
+    kernel<<<nsm, 128, smem, st>>>(iters, dev_status);
     RFDD_CHECK_LAUNCH();
     RFDD_CUDA(cudaEventRecord(e1, st));
     RFDD_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;
     RFDD_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-    const double fl = 2.0 * TC_BM * TC_BN * 8.0 * (TC_BK32 / 8) * (double)iters * nsm;
+    const double fl = 2.0 * TC_BM * TC_BN * (double)(f16 ? TC_BK : TC_BK32) * (double)iters * nsm;
     if (rep > 0 && ms > 0.f) best = std::max(best, fl / (ms * 1e-3) / 1e12);
   }
   cudaEventDestroy(e0);
@@ -1064,19 +1069,18 @@ static void launch_pack(cudaStream_t st, PackBatchP &pb, int *words, int *zero =
 }
 
 // ---------------------------------------------------------------------------------------
-// operands of the plain TF32 probe: real, rounded to TF32, tiles of 32 floats of K (hi only is used)
+// operands of the plain TF32 probe: real, rounded to TF32, tiles of 32 floats of K
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ void split_tf32(float x, float &hi, float &lo) {
+__device__ __forceinline__ float round_tf32(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  hi = __uint_as_float(r);
-  lo = x - hi;
+  return __uint_as_float(r);
 }
 struct Tf32PackItem {
   const float *src;
   long long ld;
   int m, n, k;
-  float *hi, *lo;
+  float *dst;
   int mtc, ntc, nkt;
 };
 struct Tf32PackP {
@@ -1107,14 +1111,13 @@ __global__ void __launch_bounds__(256) pack_b_real_t_kernel(Tf32PackP pb) {
     for (int i = 0; i < 4; ++i) {
       const int id = threadIdx.x + 256 * i;
       const int rl = id >> 3, c = id & 7;
-      float h[4], l[4];
+      float h[4];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) split_tf32(sb[c * 4 + t][rl], h[t], l[t]);
+      for (int t = 0; t < 4; ++t) h[t] = round_tf32(sb[c * 4 + t][rl]);
       const long long row = j0 + rl;
       const int nt = (int)(row / TC_BN), r = (int)(row % TC_BN);
       const long long off = ((long long)nt * it.nkt + kt) * (B_TILE / 4) + r * TC_BK32 + ((c ^ (r & 7)) << 2);
-      *reinterpret_cast<float4 *>(it.hi + off) = make_float4(h[0], h[1], h[2], h[3]);
-      *reinterpret_cast<float4 *>(it.lo + off) = make_float4(l[0], l[1], l[2], l[3]);
+      *reinterpret_cast<float4 *>(it.dst + off) = make_float4(h[0], h[1], h[2], h[3]);
     }
   }
 }
@@ -1128,16 +1131,14 @@ __global__ void pack_a_real_kernel(Tf32PackP pb) {
     const int q = (int)(e % (it.nkt * 8));
     const int kt = q >> 3, c = q & 7;
     const int mt = (int)(row / TC_BM), r = (int)(row % TC_BM);
-    float h[4], l[4];
+    float h[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int kr = kt * TC_BK32 + c * 4 + t;
-      const float x = (row < it.m && kr < it.k) ? it.src[row * it.ld + kr] : 0.f;
-      split_tf32(x, h[t], l[t]);
+      h[t] = (row < it.m && kr < it.k) ? round_tf32(it.src[row * it.ld + kr]) : 0.f;
     }
     const long long off = ((long long)mt * it.nkt + kt) * (A_TILE / 4) + r * TC_BK32 + ((c ^ (r & 7)) << 2);
-    *reinterpret_cast<float4 *>(it.hi + off) = make_float4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<float4 *>(it.lo + off) = make_float4(l[0], l[1], l[2], l[3]);
+    *reinterpret_cast<float4 *>(it.dst + off) = make_float4(h[0], h[1], h[2], h[3]);
   }
 }
 // Per-device launch set-up of the tensor-core kernel: its dynamic shared-memory limit is raised
@@ -1515,10 +1516,10 @@ void tc_gemm_real_tf32(cudaStream_t st, const GemmItem<float> &g, double alpha, 
   const int mtc = ceil_div(g.m, TC_BM), ntc = ceil_div(g.n, TC_BN), nkt = ceil_div(g.k, TC_BK32);
   const size_t a_bytes = (size_t)mtc * nkt * A_TILE, b_bytes = (size_t)ntc * nkt * B_TILE;
   uint8_t *ws = nullptr;
-  RFDD_CUDA(cudaMallocAsync((void **)&ws, 2 * (a_bytes + b_bytes), st));
-  uint8_t *Bh = ws + 2 * a_bytes;
-  Tf32PackP pa{{g.A, g.lda, g.m, g.n, g.k, reinterpret_cast<float *>(ws), reinterpret_cast<float *>(ws + a_bytes), mtc, ntc, nkt}};
-  Tf32PackP pb{{g.B, g.ldb, g.m, g.n, g.k, reinterpret_cast<float *>(Bh), reinterpret_cast<float *>(Bh + b_bytes), mtc, ntc, nkt}};
+  RFDD_CUDA(cudaMallocAsync((void **)&ws, a_bytes + b_bytes, st));
+  uint8_t *Bt = ws + a_bytes;
+  Tf32PackP pa{{g.A, g.lda, g.m, g.n, g.k, reinterpret_cast<float *>(ws), mtc, ntc, nkt}};
+  Tf32PackP pb{{g.B, g.ldb, g.m, g.n, g.k, reinterpret_cast<float *>(Bt), mtc, ntc, nkt}};
   pack_a_real_kernel<<<4096, 256, 0, st>>>(pa);
   RFDD_CHECK_LAUNCH();
   pack_b_real_t_kernel<<<8192, 256, 0, st>>>(pb);
@@ -1529,7 +1530,7 @@ void tc_gemm_real_tf32(cudaStream_t st, const GemmItem<float> &g, double alpha, 
   tb.err = g_tc_status;
   TcItem &it = tb.it[0];
   it.Ahi = ws;
-  it.Bhi = Bh;
+  it.Bhi = Bt;
   it.C = g.C;
   it.ldc = g.ldc;
   it.m = g.m;

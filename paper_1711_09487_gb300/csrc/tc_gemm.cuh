@@ -96,9 +96,9 @@ void tc_pack_a_batched(cudaStream_t st, const std::vector<TcPackJob> &jobs);
 // the sub-matrix of a packed m x k_full operand starting at row r0 (a multiple of 128) and complex
 // column c0 (a multiple of 32); side: 0 the only scale, or that of the left part; 1 the right part's
 TcPackedA tc_packed_view(const void *op, int64_t m, int64_t k_full, int64_t r0 = 0, int64_t c0 = 0, int side = 0);
-// TFLOP/s of kind::tf32 MMAs issued back to back from operand tiles resident in shared memory
-// (one CTA per SM, no operand loads): the tensor pipe's own TF32 rate.  Time-outs go to *dev_status.
-double tc_mma_probe_tflops(cudaStream_t st, int *dev_status);
+// TFLOP/s of kind::tf32 or kind::f16 MMAs issued back to back from operand tiles resident in shared memory
+// (one CTA per SM, no operand loads): the tensor pipe's own rate.  Time-outs go to *dev_status.
+double tc_mma_probe_tflops(cudaStream_t st, int *dev_status, bool f16);
 // tile walk of a GEMM item with mtc x ntc output tiles and nkt K tiles: 1 down the columns, 0
 // along the rows (see tc_gemm.cu)
 int tc_tile_order(int mtc, int ntc, int nkt);

@@ -12,15 +12,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def R():
-    from paper_1711_09487_gb300 import build
-    build.build()
-    import paper_1711_09487_gb300 as pkg
-    pkg.load()
-    return pkg
-
-
 def _check(R, A, B, rows, cols):
     """A (m x k) B (k x n) at the given rows and columns."""
     C = R.rfdd_dgemm(A, B, np.zeros((A.shape[0], B.shape[1])))

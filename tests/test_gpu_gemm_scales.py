@@ -11,15 +11,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def R():
-    from paper_1711_09487_gb300 import build
-    build.build()
-    import paper_1711_09487_gb300 as pkg
-    pkg.load()
-    return pkg
-
-
 def _rnd(g, m, n, e):
     return ((g.standard_normal((m, n)) + 1j * g.standard_normal((m, n))) * 2.0 ** e).astype(np.complex64)
 

@@ -10,15 +10,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def R():
-    from paper_1711_09487_gb300 import build
-    build.build()
-    import paper_1711_09487_gb300 as pkg
-    pkg.load()
-    return pkg
-
-
 @pytest.mark.parametrize("engine", [1, 2, 3])
 @pytest.mark.parametrize("side", ["row of A", "column of B"])
 @pytest.mark.parametrize("below", [0, 8, 13, 14, 15, 16, 17, 20, 24, 30, 37, 41])

@@ -11,15 +11,6 @@ import rfdd_inputs as I
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def R():
-    from paper_1711_09487_gb300 import build
-    build.build()
-    import paper_1711_09487_gb300 as pkg
-    pkg.load()
-    return pkg
-
-
 def _csr(S):
     S = sp.csr_matrix(S)
     S.sort_indices()

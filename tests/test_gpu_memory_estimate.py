@@ -13,15 +13,6 @@ pytestmark = pytest.mark.gpu
 USED_CURRENT, USED_HIGH = 7, 8  # CUmemPool_attribute
 
 
-@pytest.fixture(scope="module")
-def R():
-    from paper_1711_09487_gb300 import build
-    build.build()
-    import paper_1711_09487_gb300 as pkg
-    pkg.load()
-    return pkg
-
-
 class Pool:
     def __init__(self):
         self.cu, self.pool = C.CDLL("libcuda.so.1"), C.c_void_p()

@@ -7,15 +7,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def R():
-    from paper_1711_09487_gb300 import build
-    build.build()
-    import paper_1711_09487_gb300 as pkg
-    pkg.load()
-    return pkg
-
-
 def _place(torch, X, shift):
     """The floats of X on the device, `shift` floats after a 256-byte boundary."""
     buf = torch.zeros(X.size * 2 + 8, dtype=torch.float32, device="cuda")

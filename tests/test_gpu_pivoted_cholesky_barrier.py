@@ -9,15 +9,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def R():
-    from paper_1711_09487_gb300 import build
-    build.build()
-    import paper_1711_09487_gb300 as pkg
-    pkg.load()
-    return pkg
-
-
 def _gram(k, rank, seed):
     Y = np.random.default_rng(seed).standard_normal((rank, k))
     d = 1.0 / np.sqrt((Y * Y).sum(0))

@@ -5,15 +5,6 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def R():
-    from paper_1711_09487_gb300 import build
-    build.build()
-    import paper_1711_09487_gb300 as pkg
-    pkg.load()
-    return pkg
-
-
 def test_16bit_rate(R):
     tf32, f16 = R.rfdd_peak_probe(0), R.rfdd_peak_probe(4)
     assert 1.3 * tf32 < f16 < 2.6 * tf32

@@ -166,15 +166,20 @@ struct ChunkC {
 };
 
 // Scales that the usual order of the read-back (drain_tile: (x rr) (alpha rb)) cannot take: an accumulator is below 2^45 and
-// scales lie between 2^-126 and 2^114, so x rr stays in range up to rr = 2^80, and alpha rb for columns within 2^100 of 1 and an
-// alpha within 2^20 of 1.  The packing records others in the word after the status word; launches that find it set, or have
-// such an alpha, read back by drain_far.  Looked at tile by tile the check cost more than the read-back
+// scales lie between 2^-126 and 2^114, so x rr stays in range up to rr = 2^80, and alpha rb is exact for an alpha that is a
+// power of two within 2^13 of 1 (the solver's are 1 and -1), for others where the column is within 2^100 and alpha within
+// 2^20 of 1.  The packing records other rows and columns in the word after the status word; launches that they concern
+// read back by drain_far.  (Columns below 2^-87 are ordinary: factors of wide 2-D subdomains decay that far.  Rows beyond
+// 2^93 are not.)  Looked at tile by tile the check cost more than the read-back
 // gained, and with both orders in one body it spilled: K = 32 update of 8192 x 8192 0.27 ms, 0.30 and 0.36 with these.
 __device__ __forceinline__ bool far_row(float s) { return s > 0x1p80f; }
 __device__ __forceinline__ bool far_col(float s) { return !(s >= 0x1p-100f && s <= 0x1p100f); }
+constexpr int FAR_ROW = 1, FAR_COL = 2;
 __device__ __forceinline__ bool far_launch(const int *err, float alpha) {
   const float a = fabsf(alpha);
-  return __ldcg(err + 1) != 0 || !(a >= 0x1p-20f && a <= 0x1p20f);
+  const bool plain = (__float_as_uint(a) & 0x7fffffu) == 0 && a >= 0x1p-13f && a <= 0x1p13f;
+  const int far = __ldcg(err + 1);
+  return (far & FAR_ROW) || (!plain && (far || !(a >= 0x1p-20f && a <= 0x1p20f)));
 }
 
 // Read-back of such launches: scales on one side of 1 one after the other, scales on different sides by their
@@ -897,7 +902,7 @@ __device__ __forceinline__ void pack_a_rows(const PackItem &it, int *far) {
     row_scale(ml, fl, il);
     row_scale(mr, fr, ir);
     if (lane == 0) {
-      if (far_row(il) || far_row(ir)) *far = 1;
+      if (far_row(il) || far_row(ir)) atomicOr(far, FAR_ROW);
       if (it.side > 0) {
         it.scale[row] = il;
         it.scale[rows_pad + row] = ir;
@@ -980,7 +985,7 @@ __device__ __forceinline__ void pack_b_rows(const PackItem &it, float *sb, int *
       float mul, inv;
       row_scale(m, mul, inv);
       mul_s[tid] = mul;
-      if (far_col(inv)) *far = 1;
+      if (far_col(inv) && (__ldcg(far) & FAR_COL) == 0) atomicOr(far, FAR_COL);
       it.scale[(long long)jb * 64 + tid] = inv;
     }
     __syncthreads();

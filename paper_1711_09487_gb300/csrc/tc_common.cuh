@@ -92,4 +92,11 @@ __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::aft
         "=r"(v[30]), "=r"(v[31])                                                                              \
       : "r"(taddr))
 
+#define TC_LD16(taddr, v)                                                                                      \
+  asm volatile(                                                                                                \
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];" \
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),       \
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])  \
+      : "r"(taddr))
+
 }  // namespace rfdd

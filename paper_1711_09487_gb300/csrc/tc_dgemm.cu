@@ -4,8 +4,8 @@
 // fixed-point integer (entries down to 2^-9 of the largest are exact), which is cut into eight balanced base-256
 // digits (-128 .. 127), each exact in fp16.  The products of digit planes with equal weight, i + j = g, are summed by
 // tcgen05 kind::f16 MMAs into one of eight FP32 accumulators: all addends are integers and their sums stay within 2^24
-// (8 pairs x 128 x 2^14), so every accumulator is exact.  After at most 128 terms of K the eight are read back and
-// added into two 64-bit integers per entry, which hold the sum exactly up to the planes that are left out (i + j
+// (8 pairs x 128 x 2^14), so every accumulator is exact.  After at most 128 terms of K (256 for the four of the leading
+// planes, which sum fewer products) they are read back and added into two 64-bit integers per entry, which hold the sum exactly up to the planes that are left out (i + j
 // > 7); one rounding to FP64 at the end.  This is the splitting of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms
 // 59, 2012) with integer digits.
 //
@@ -19,8 +19,11 @@
 // operands whose digits have one sign.)
 //
 // What bounds it: the 36 plane products of a 128 x 64 x 32 stage read 12 KB of shared memory per 32
-// cycles of MMA, by the descriptors, and a stage takes about 3500 cycles; that
-// is the bound from a few hundred terms on; below that the read-back is.
+// cycles of MMA, by the descriptors, and a stage takes about 3500 cycles; the read-back (conversions and 64-bit
+// additions of 64 k sums, about 7000 cycles for all eight accumulators) comes on top, because they fill the tensor
+// memory.  Measured, without the packing: symmetric 1920 x 1920 x 64000 10.0 ms, 1885 x 1885 x 8000 1.27 ms (symmetric)
+// and 1.90; with seven-bit digits, one read-back in 512 terms, 8.9, 1.12 and 1.67; with eight warps for the read-back and all
+// accumulators every 128 terms 11.0, 1.39 and 2.07.
 #include "dense.cuh"
 #include "tc_common.cuh"
 #include "tc_gemm.cuh"
@@ -40,9 +43,14 @@ constexpr int DG_STAGES = 2;
 constexpr int DG_BITS = 8;     // bits of a digit
 constexpr int DG_CHUNK = 4;    // stages between two read-backs (128 terms)
 constexpr int DG_SPLIT = 16;   // stages of the shallowest share of a split K (512 terms)
+// Accumulator g sums g + 1 plane products: the four of the upper half stay exact for two chunks and are read back, and
+// start anew, with every second one.
 static_assert(DG_PLANES * DG_CHUNK * DG_KT << 2 * (DG_BITS - 1) <= 1 << 24, "the accumulators stay exact");
+static_assert(DG_PLANES / 2 * 2 * DG_CHUNK * DG_KT << 2 * (DG_BITS - 1) <= 1 << 24, "the upper ones for two chunks");
 constexpr int DG_SMEM = DG_STAGES * DG_STAGE + 1024;
-constexpr int DG_EPI_WARPS = 8;
+constexpr int DG_EPI_WARPS = 16;  // four to each lane quarter of the accumulators
+constexpr int DG_EC = DG_BN / (DG_EPI_WARPS / 4);  // columns a read-back warp takes
+static_assert(DG_EC == 16, "tcgen05.ld x16");
 constexpr int DG_THREADS = 64 + 32 * DG_EPI_WARPS;
 constexpr int DG_MAXB = 32;
 
@@ -369,6 +377,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
           }
           fence_after();
           const int k1 = min(ke, k0 + DG_CHUNK);
+          const bool second = ((k0 - kb) / DG_CHUNK & 1) != 0;  // the upper accumulators go on
           for (int kt = k0; kt < k1; ++kt, ++g) {
             const int s = (int)(g % DG_STAGES);
             if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)((g / DG_STAGES) & 1), &abort_s)) {
@@ -385,7 +394,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
 #pragma unroll
                 for (int j = 0; j < DG_PLANES - i; ++j)
                   mma_f16(tmem + (uint32_t)((i + j) * DG_BN), da, sdesc(sb + (j >> 1) * DG_BTILE + (j & 1) * 64 + kk * 32),
-                          idesc, (kt > k0 || kk > 0 || i > 0) ? 1u : 0u);
+                          idesc, (kt > k0 || kk > 0 || i > 0 || (second && i + j < DG_PLANES / 2)) ? 1u : 0u);
               }
             }
             mma_commit(smem_u32(&empty_bar[s]));
@@ -402,8 +411,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
       mbar_drain(smem_u32(&drain_bar), 0);
     }
   } else {
-    // read-back: warp w takes accumulator lanes 32 (w % 4) .. (its rows) and half of the columns
-    const int q = warp & 3, half = (warp - 2) >> 2;
+    // read-back: warp w takes accumulator lanes 32 (w % 4) .. (its rows) and a quarter of the columns
+    const int q = warp & 3, part = (warp - 2) >> 2;
     long long ch = 0;
     bool ok = true;
     for (int u = blockIdx.x; u < b.units && ok; u += gridDim.x) {
@@ -411,9 +420,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
       int mt, nt, sp;
       dg_unit(it, u - it.unit0, mt, nt, sp);
       const int kb = sp * it.kper, ke = min(it.nkt, kb + it.kper);
-      long long hi[32], lo[32];
+      long long hi[DG_EC], lo[DG_EC];
 #pragma unroll
-      for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0;
+      for (int j = 0; j < DG_EC; ++j) hi[j] = lo[j] = 0;
       for (int k0 = kb; k0 < ke; k0 += DG_CHUNK, ++ch) {
         const bool ready = mbar_wait(smem_u32(&tfull_bar), (uint32_t)(ch & 1), &abort_s);
         if (!__all_sync(0xffffffffu, ready && !abort_s)) {
@@ -423,18 +432,20 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
           break;
         }
         fence_after();
-        const uint32_t t0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 32);
+        const uint32_t t0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(part * DG_EC);
+        const bool all = ((k0 - kb) / DG_CHUNK & 1) != 0 || k0 + DG_CHUNK >= ke;
 #pragma unroll
         for (int g = 0; g < DG_PLANES; ++g) {
-          uint32_t v[32];
-          TC_LD32(t0 + (uint32_t)(g * DG_BN), v);
+          if (g < DG_PLANES / 2 && !all) continue;
+          uint32_t v[DG_EC];
+          TC_LD16(t0 + (uint32_t)(g * DG_BN), v);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (g == DG_PLANES - 1) {
             fence_before();
             mbar_arrive(smem_u32(&tempty_bar));
           }
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
+          for (int j = 0; j < DG_EC; ++j) {
             const int x = __float2int_rn(__uint_as_float(v[j]));
             if (g < 4) hi[j] += (long long)x * (1 << (DG_BITS * (3 - g)));
             else lo[j] += (long long)x * (1 << (DG_BITS * (7 - g)));
@@ -447,9 +458,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1) tc_dgemm_kernel(const __grid_co
       if (i < it.m) {
         const int eai = it.ea[i];
         const int xa = eai - 2 * 1084 + 56;  // one unit of a product of two integers is 2^(ea + eb - 2 * 1084)
-        const int j0 = nt * DG_BN + half * 32;
+        const int j0 = nt * DG_BN + part * DG_EC;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
+        for (int j = 0; j < DG_EC; ++j) {
           const int c = j0 + j;
           if (c >= it.n) continue;
           const int ebj = it.eb[c];

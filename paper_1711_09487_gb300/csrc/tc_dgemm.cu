@@ -5,9 +5,9 @@
 // digits (-128 .. 127), each exact in fp16.  The products of digit planes with equal weight, i + j = g, are summed by
 // tcgen05 kind::f16 MMAs into one of eight FP32 accumulators: all addends are integers and their sums stay within 2^24
 // (8 pairs x 128 x 2^14), so every accumulator is exact.  After at most 128 terms of K (256 for the four of the leading
-// planes, which sum fewer products) they are read back and added into two 64-bit integers per entry, which hold the sum exactly up to the planes that are left out (i + j
-// > 7); one rounding to FP64 at the end.  This is the splitting of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms
-// 59, 2012) with integer digits.
+// planes, which sum fewer products) they are read back and added into two 64-bit integers per entry, which hold the sum
+// exactly up to the planes that are left out (i + j > 7); one rounding to FP64 at the end.  This is the splitting of
+// Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59, 2012) with integer digits.
 //
 // Before that, the terms of the sum are brought to one size: column k of op(A) is divided, and row k of op(B) multiplied, by the
 // power of two of the column's largest entry (exponents only, exact).  Rows and columns scaled by factors of their own
@@ -15,8 +15,8 @@
 //
 // Error of an entry: k 2^-57 (largest |a| of its row) (largest |b| of its column) of the operands so scaled, and the
 // roundings of the result.  For operands within a few powers of two of their largest entries that is below the
-// error of the sum in FP64, whatever its order.  (Digits of seven bits, 512 terms to a read-back, left out planes of 2^-49 of the largest product: 7 ulp on
-// operands whose digits have one sign.)
+// error of the sum in FP64, whatever its order.  (Digits of seven bits, 512 terms to a read-back, left out planes of
+// 2^-49 of the largest product: 7 ulp on operands whose digits have one sign.)
 //
 // What bounds it: the 36 plane products of a 128 x 64 x 32 stage read 12 KB of shared memory per 32
 // cycles of MMA, by the descriptors, and a stage takes about 3500 cycles; the read-back (conversions and 64-bit
